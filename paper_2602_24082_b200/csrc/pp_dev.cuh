@@ -97,29 +97,20 @@ inline bool encode_thd_f32(CUtensorMap* m, const void* base, int T, int H, int D
 
 constexpr uint32_t kBoxBytes = 128 * 128;  // one {64 x 128 rows} bf16 box
 
-// K-major operand descriptor for k-step `k16` (16 elements of the contraction = 32 bytes
-// inside a 128-byte row; four steps per box).
-__device__ __forceinline__ uint64_t kmajor_desc(uint32_t tile_base, int k16) {
-  return make_sdesc(tile_base + (k16 >> 2) * kBoxBytes + (k16 & 3) * 32, 16, 1024);
+// Operand descriptors (low words, see make_sdesc_lo): the descriptor for k-step k16 (16
+// elements of the contraction) is the tile's base descriptor plus a compile-time constant in its
+// address field (shared-memory addresses stay below 2^18, so the 14-bit field cannot overflow).
+// K-major: a k-step is 32 bytes inside a 128-byte row, four steps per box.  MN-major: a k-step
+// is 16 rows = 2048 bytes; the next 64 elements of the M / N index live in the next box.
+__device__ __forceinline__ uint32_t kmajor_base(uint32_t tile_base) {
+  return make_sdesc_lo(tile_base, 16);
 }
-// MN-major operand descriptor for k-step `k16` (16 rows = 2048 bytes); the next 64 elements
-// of the M/N index live in the next box.
-__device__ __forceinline__ uint64_t mnmajor_desc(uint32_t tile_base, int k16) {
-  return make_sdesc(tile_base + k16 * 2048, kBoxBytes, 1024);
+__device__ __forceinline__ uint32_t mnmajor_base(uint32_t tile_base) {
+  return make_sdesc_lo(tile_base, kBoxBytes);
 }
-
-// Descriptor arithmetic for unrolled k-loops: a descriptor for k-step k16 is the tile's base
-// descriptor plus a compile-time constant in its address field (shared-memory addresses stay
-// below 2^18, so the 14-bit field cannot overflow).
-__device__ __forceinline__ uint64_t kmajor_base(uint32_t tile_base) {
-  return make_sdesc(tile_base, 16, 1024);
+__host__ __device__ constexpr uint32_t kmajor_off(int k16) {
+  return uint32_t(((k16 >> 2) * kBoxBytes + (k16 & 3) * 32) >> 4);
 }
-__device__ __forceinline__ uint64_t mnmajor_base(uint32_t tile_base) {
-  return make_sdesc(tile_base, kBoxBytes, 1024);
-}
-__host__ __device__ constexpr uint64_t kmajor_off(int k16) {
-  return uint64_t(((k16 >> 2) * kBoxBytes + (k16 & 3) * 32) >> 4);
-}
-__host__ __device__ constexpr uint64_t mnmajor_off(int k16) { return uint64_t((k16 * 2048) >> 4); }
+__host__ __device__ constexpr uint32_t mnmajor_off(int k16) { return uint32_t((k16 * 2048) >> 4); }
 
 }  // namespace pp

@@ -127,7 +127,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
            const __grid_constant__ CUtensorMap tm_v, FwdParams prm) {
   using L = FwdSmem<D>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // (known to be uniform in the warp)
 
   if (prm.header[0] != kStatusOk) return;
   const int ntiles_total = prm.header[2];
@@ -208,7 +209,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       uint32_t kc = 0, qc[2] = {0, 0};
       Unit un;
       for (uint32_t un_i = 0; fetch_unit(un_i, un); ++un_i) {
@@ -250,21 +251,25 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    // tcgen05.mma issue blocks this thread for about one MMA duration, so the tensor pipe is
-    // idle whenever the thread executes anything else for longer than that: the loop below
-    // keeps the work between two groups of MMAs to a minimum (descriptors and instruction
-    // descriptors precomputed, barrier addresses and parities kept in registers, one branch
-    // for the common case of full 128-key tiles).
-    if (lane == 0) {
+    // The tensor pipe takes about two MMAs ahead of the one it executes, so whatever the issuing
+    // thread does between two groups of MMAs beyond that is idle tensor-pipe time: the loop
+    // below keeps it to a minimum (descriptors and instruction descriptors precomputed, barrier
+    // addresses and parities kept in registers, one branch for the common case of full 128-key
+    // tiles).  The branch is an elect.sync and not `lane == 0`: with the latter eight MMAs took
+    // the thread 494 cycles to issue whatever their N (62 each: operands moved to uniform
+    // registers one by one), with the former 402 at N = 128 and 322 at N = 64.  A launch on two
+    // rows of 32768 tokens (Hq / Hkv 32 / 8, D 128) went from 11.3 to 10.4 M cycles, eight
+    // 1100-token rows from 143 to 132 us, head_dim 64 from 248 to 227 us.
+    if (elect_one()) {
       uint32_t kc = 0, tc0 = 0, tc1 = 0, uc0 = 0, uc1 = 0;
       constexpr uint32_t idesc_o = make_idesc(128, DV, 0, 1);
       constexpr uint32_t idesc_full = make_idesc(128, 128, 0, 0);
-      constexpr uint64_t kStageStep = uint64_t(L::kTileBytes >> 4);
-      const uint64_t dq0 = kmajor_base(sQ), dk0 = kmajor_base(sK), dv0 = mnmajor_base(sV);
+      constexpr uint32_t kStageStep = uint32_t(L::kTileBytes >> 4);
+      const uint32_t dq0 = kmajor_base(sQ), dk0 = kmajor_base(sK), dv0 = mnmajor_base(sV);
       // length of key tile j of a unit: only the last tile of each visible range and the
       // diagonal tile can be shorter than 128
       auto issue_qk = [&](int s, uint32_t kstage, int k_len) {
-        const uint64_t a = dq0 + s * kStageStep, b = dk0 + kstage * kStageStep;
+        const uint32_t a = dq0 + s * kStageStep, b = dk0 + kstage * kStageStep;
         const uint32_t tS = tmem + s * 128;
         if (k_len == kTile) {
 #pragma unroll
@@ -279,7 +284,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         mma_commit(bar(kSFull + s));
       };
       auto issue_pv = [&](int s, uint32_t vstage, int k_len, bool first, bool last) {
-        const uint64_t b = dv0 + vstage * kStageStep;
+        const uint32_t b = dv0 + vstage * kStageStep;
         const uint32_t tS = tmem + s * 128, tO = tmem + 256 + s * 128;
         if (k_len == kTile && !first) {
 #pragma unroll

@@ -13,6 +13,22 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// One lane of a converged warp, chosen by the hardware.  Code that issues tcgen05 or TMA
+// instructions from one thread enters through this predicate and not through `lane == 0`: the
+// compiler then knows that exactly one thread is active and feeds the instructions' uniform
+// operands directly.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "elect.sync _|p, 0xffffffff;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(ok));
+  return ok != 0;
+}
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
@@ -129,28 +145,50 @@ __device__ __forceinline__ void tmem_wait_st() {
 }
 
 // ---------------------------------------------------------------- tcgen05: MMA
+// Shared-memory matrix descriptor for 128-byte-swizzled tiles whose rows are 128 bytes
+// (64 bf16) and whose 8-row groups are 1024 bytes apart -- the layout a TMA box of
+// {64 elements, rows} with SWIZZLE_128B produces.
+//   [0,14) address >> 4   [16,30) leading byte offset >> 4   [32,46) stride byte offset >> 4
+//   [46,48) version = 1   [61,64) swizzle mode (2 = 128 B)
+// K-major operand (rows = M or N index, the 64 contiguous elements = K): stride offset = 1024,
+//   leading offset unused.  MN-major operand (rows = K index, contiguous elements = M or N):
+//   stride offset = 1024 (next 8 K rows), leading offset = distance to the next 64 M/N elements.
+// The stride offset is 1024 for both, which leaves one high word for all descriptors.
+constexpr uint32_t kSdescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t make_sdesc_lo(uint32_t smem_addr, uint32_t lbo_bytes) {
+  return ((smem_addr & 0x3FFFFu) >> 4) | (((lbo_bytes >> 4) & 0x3FFFu) << 16);
+}
+
+// Shared-memory operands are given by the LOW word of their matrix descriptor (see make_sdesc):
+// the high word is the same for every tile here, so the issuing thread handles one register per
+// operand and k-step instead of two.
 // D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate, one CTA.
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
+__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint32_t a_desc, uint32_t b_desc,
                                        uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n"
       ".reg .pred p;\n"
+      ".reg .b64 a, b;\n"
       "setp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
+      "mov.b64 a, {%1, %5};\n"
+      "mov.b64 b, {%2, %5};\n"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n"
       "}\n" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "r"(a_desc), "r"(b_desc), "r"(idesc), "r"(accumulate), "n"(kSdescHi)
       : "memory");
 }
 // D[tmem] (+)= A[tmem] * B[smem]
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
+__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_desc,
                                        uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n"
       ".reg .pred p;\n"
+      ".reg .b64 b;\n"
       "setp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n"
+      "mov.b64 b, {%2, %5};\n"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %3, p;\n"
       "}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "r"(a_tmem), "r"(b_desc), "r"(idesc), "r"(accumulate), "n"(kSdescHi)
       : "memory");
 }
 // mbarrier arrives once every MMA issued so far by this thread has finished.
@@ -165,25 +203,6 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
 __host__ __device__ constexpr uint32_t make_idesc(int M, int N, int a_mn_major, int b_mn_major) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(a_mn_major) << 15) |
          (uint32_t(b_mn_major) << 16) | (uint32_t(N >> 3) << 17) | (uint32_t(M >> 4) << 24);
-}
-
-// Shared-memory matrix descriptor for 128-byte-swizzled tiles whose rows are 128 bytes
-// (64 bf16) and whose 8-row groups are 1024 bytes apart -- the layout a TMA box of
-// {64 elements, rows} with SWIZZLE_128B produces.
-//   [0,14) address >> 4   [16,30) leading byte offset >> 4   [32,46) stride byte offset >> 4
-//   [46,48) version = 1   [61,64) swizzle mode (2 = 128 B)
-// K-major operand (rows = M or N index, the 64 contiguous elements = K): stride offset = 1024,
-//   leading offset unused.  MN-major operand (rows = K index, contiguous elements = M or N):
-//   stride offset = 1024 (next 8 K rows), leading offset = distance to the next 64 M/N elements.
-__device__ __forceinline__ uint64_t make_sdesc(uint32_t smem_addr, uint32_t lbo_bytes,
-                                               uint32_t sbo_bytes) {
-  uint64_t d = 0;
-  d |= uint64_t((smem_addr & 0x3FFFF) >> 4);
-  d |= uint64_t((lbo_bytes >> 4) & 0x3FFF) << 16;
-  d |= uint64_t((sbo_bytes >> 4) & 0x3FFF) << 32;
-  d |= uint64_t(1) << 46;
-  d |= uint64_t(2) << 61;
-  return d;
 }
 
 // ---------------------------------------------------------------- tcgen05: TMEM <-> registers
