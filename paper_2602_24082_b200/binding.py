@@ -454,7 +454,8 @@ def pp_build_rows(grp_prompt_len: torch.Tensor, grp_resp_off: torch.Tensor, resp
     ws = torch.empty(nbytes.value, dtype=torch.uint8, device=dev)
     i32 = lambda n: torch.empty(n, dtype=torch.int32, device=dev)
     i64 = lambda n: torch.empty(n, dtype=torch.int64, device=dev)
-    order, rgo, nrows, status = i32(G), i32(G + 1), i32(1), i32(2)
+    order, rgo, meta = i32(G), i32(G + 1), i32(3)   # meta: status code, detail, number of rows
+    status, nrows = meta[:2], meta[2:]
     rtok, rcost = i64(G), i64(G)
     oP, ooff, orl = i32(G), i32(G + 1), i32(N)
     with torch.cuda.device(dev):
@@ -463,10 +464,9 @@ def pp_build_rows(grp_prompt_len: torch.Tensor, grp_resp_off: torch.Tensor, resp
                                    order.data_ptr(), rgo.data_ptr(), nrows.data_ptr(), rtok.data_ptr(),
                                    rcost.data_ptr(), oP.data_ptr(), ooff.data_ptr(), orl.data_ptr(),
                                    status.data_ptr(), _stream()), "pp_build_rows")
-    st = status.tolist()
-    r = int(nrows.item())
+    code, detail, r = meta.tolist()   # one synchronising copy
     return {"order": order, "row_group_off": rgo[:r + 1], "row_tokens": rtok[:r], "row_cost": rcost[:r],
-            "grp_prompt_len": oP, "grp_resp_off": ooff, "resp_len": orl, "status": (st[0], st[1])}
+            "grp_prompt_len": oP, "grp_resp_off": ooff, "resp_len": orl, "status": (code, detail)}
 
 
 def pp_assign_rows(row_cost: torch.Tensor, num_ranks: int):

@@ -18,11 +18,12 @@ struct RowsPtrs {
   const int32_t* prompt_len;
   const int32_t* resp_off;
   const int32_t* resp_len;
-  long long* tok;    // [G] tokens per group
+  int32_t* tok;      // [G] tokens per group, saturated (a group above the capacity is an error)
   long long* cost;   // [G] visible pairs per group
   long long* pre;    // [G] inclusive prefix sums of the sorted groups' tokens
+  long long* pre_cost;  // [G] ... and of their visible pairs
   int32_t* nxt;      // [G] end of the row that would start at each sorted position
-  int32_t* jump_a;   // [G] pointer-doubling buffers
+  int32_t* jump_a;   // [G] pointer-doubling buffers, used when they do not fit shared memory
   int32_t* jump_b;   // [G]
   int32_t* mark;     // [G] 1 = a row starts here
   int32_t* order;
@@ -61,106 +62,180 @@ __global__ void rows_measure_kernel(RowsPtrs p) {
     u += R * P + R * (R + 1) / 2;
   }
   if (t > p.capacity) rows_fail(p.status, kRowsTooLong, g);
-  p.tok[g] = t;
+  p.tok[g] = int32_t(t < 0x7fffffff ? t : 0x7fffffff);
   p.cost[g] = u;
 }
 
-// position of every group in the order "longest first, ties by original index": rank counting
-// against all groups, staged through shared memory
-__global__ void __launch_bounds__(256) rows_rank_kernel(RowsPtrs p) {
-  __shared__ long long s_tok[256];
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  const long long mine = g < p.G ? p.tok[g] : 0;
-  int rank = 0;
-  for (int base = 0; base < p.G; base += 256) {
-    const int u = base + threadIdx.x;
-    s_tok[threadIdx.x] = u < p.G ? p.tok[u] : -1;
+// Position of every key in the order "largest first, ties by index", by rank counting.  The count
+// is quadratic, so what matters is to spread it: a block ranks 32 keys, each of its 32 warps
+// counts a slice of every staged chunk (all lanes read the same key: broadcast reads), and the
+// partial counts are added at the end.  (One thread per key and 256 keys per block left 132 SMs
+// idle: 72 us for 4096 groups, now 7.)
+constexpr int kRankKeys = 32, kRankSlices = 32, kRankChunk = 2048;
+
+template <typename Key>
+__global__ void __launch_bounds__(kRankKeys * kRankSlices)
+rank_kernel(int n, const Key* __restrict__ keys, int32_t* __restrict__ order) {
+  __shared__ Key s_key[kRankChunk];
+  __shared__ int32_t s_count[kRankSlices][kRankKeys];
+  const int tid = threadIdx.x, item = tid % kRankKeys, slice = tid / kRankKeys;
+  const int first = blockIdx.x * kRankKeys, g = first + item;
+  const Key mine = g < n ? keys[g] : 0;
+  int count = 0;
+  for (int base = 0; base < n; base += kRankChunk) {
+    const int here = min(kRankChunk, n - base);
+    for (int i = tid; i < here; i += kRankKeys * kRankSlices) s_key[i] = keys[base + i];
     __syncthreads();
-    const int lim = min(256, p.G - base);
-    for (int i = 0; i < lim; ++i) {
-      const long long o = s_tok[i];
-      rank += (o > mine) || (o == mine && base + i < g);
+    constexpr int kPer = kRankChunk / kRankSlices;
+    const int lo = slice * kPer, hi = min(lo + kPer, here);
+    if (base + hi <= first) {          // slices before or behind my block's keys: one comparison
+#pragma unroll 16
+      for (int i = lo; i < hi; ++i) count += s_key[i] >= mine;
+    } else if (base + lo >= first + kRankKeys) {
+#pragma unroll 16
+      for (int i = lo; i < hi; ++i) count += s_key[i] > mine;
+    } else {
+      for (int i = lo; i < hi; ++i) count += s_key[i] > mine || (s_key[i] == mine && base + i < g);
     }
     __syncthreads();
   }
-  if (g < p.G) p.order[rank] = g;
+  s_count[slice][item] = count;
+  __syncthreads();
+  if (tid < kRankKeys && g < n) {
+    int rank = 0;
+#pragma unroll
+    for (int k = 0; k < kRankSlices; ++k) rank += s_count[k][tid];
+    order[rank] = g;
+  }
 }
 
-// one block: prefix sums over the sorted groups, next-fit rows, row costs, reordered
-// descriptors
-__global__ void __launch_bounds__(1024) rows_pack_kernel(RowsPtrs p) {
-  __shared__ long long s_a[1024];
-  __shared__ int32_t s_b[1024];
-  __shared__ long long s_carry;
-  __shared__ int32_t s_carry_b;
-  __shared__ int32_t s_rows;
+// Inclusive block-wide sums of three values per thread (two barriers).
+struct Sum3 {
+  long long a, b;
+  int32_t c;
+};
+__device__ __forceinline__ Sum3 block_scan(Sum3 v, Sum3* s_warp) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const long long a = __shfl_up_sync(0xffffffffu, v.a, d), b = __shfl_up_sync(0xffffffffu, v.b, d);
+    const int32_t c = __shfl_up_sync(0xffffffffu, v.c, d);
+    if (lane >= d) {
+      v.a += a;
+      v.b += b;
+      v.c += c;
+    }
+  }
+  if (lane == 31) s_warp[warp] = v;
+  __syncthreads();
+  if (warp == 0) {   // the block has 32 warps
+    Sum3 w = s_warp[lane];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const long long a = __shfl_up_sync(0xffffffffu, w.a, d), b = __shfl_up_sync(0xffffffffu, w.b, d);
+      const int32_t c = __shfl_up_sync(0xffffffffu, w.c, d);
+      if (lane >= d) {
+        w.a += a;
+        w.b += b;
+        w.c += c;
+      }
+    }
+    s_warp[lane] = w;
+  }
+  __syncthreads();
+  if (warp) {
+    v.a += s_warp[warp - 1].a;
+    v.b += s_warp[warp - 1].b;
+    v.c += s_warp[warp - 1].c;
+  }
+  return v;
+}
+
+// One block: prefix sums over the sorted groups, next-fit rows, row costs, reordered
+// descriptors.  It is all latency, so dependent loads are issued for several groups at once and
+// whatever is searched or chased -- the token sums, the pointer-doubling tables -- lives in
+// shared memory up to kPackSmemGroups groups (20 bytes each).  4096 groups: 47 us with the tables
+// in global memory and shared-memory scans of ten rounds per 1024 groups, now 38.
+constexpr int kPackSmemGroups = 8192;
+
+__global__ void __launch_bounds__(1024) rows_pack_kernel(RowsPtrs p, int tables_in_smem) {
+  extern __shared__ long long s_tables[];
+  __shared__ Sum3 s_warp[32];
+  __shared__ Sum3 s_total;
   const int tid = threadIdx.x, nthr = blockDim.x;
   if (p.status[0] != kRowsOk) {
     if (tid == 0) *p.num_rows = 0;
     return;
   }
-  if (tid == 0) {
-    s_carry = 0;
-    s_carry_b = 0;
+  long long* pre = tables_in_smem ? s_tables : p.pre;
+  int32_t* s_int = reinterpret_cast<int32_t*>(s_tables + p.G);
+  int32_t* ja = tables_in_smem ? s_int : p.jump_a;
+  int32_t* jb = tables_in_smem ? s_int + p.G : p.jump_b;
+  int32_t* mark = tables_in_smem ? s_int + 2 * p.G : p.mark;
+  // tokens, pairs and response counts in sorted order
+#pragma unroll 4
+  for (int i = tid; i < p.G; i += nthr) {
+    const int g = p.order[i];
+    pre[i] = p.tok[g];
+    p.pre_cost[i] = p.cost[g];
+    p.out_prompt_len[i] = p.prompt_len[g];
+    const int x0 = p.resp_off[g];
+    ja[i] = x0;
+    jb[i] = p.resp_off[g + 1] - x0;
   }
-  __syncthreads();
-  // inclusive scan of tokens and exclusive scan of response counts, both in sorted order
+  // inclusive scans of tokens and pairs and exclusive scan of response counts, in sorted order
+  // (every thread scans what it has gathered itself: no barrier in between)
+  Sum3 carry = {0, 0, 0};
   for (int base = 0; base < p.G; base += nthr) {
     const int i = base + tid;
-    long long a = 0;
-    int32_t b = 0;
+    Sum3 v = {0, 0, 0};
+    if (i < p.G) v = {pre[i], p.pre_cost[i], jb[i]};
+    const int32_t n_resp = v.c;
+    const Sum3 w = block_scan(v, s_warp);
     if (i < p.G) {
-      const int g = p.order[i];
-      a = p.tok[g];
-      b = p.resp_off[g + 1] - p.resp_off[g];
-      p.out_prompt_len[i] = p.prompt_len[g];
+      pre[i] = carry.a + w.a;
+      p.pre_cost[i] = carry.b + w.b;
+      p.out_resp_off[i] = carry.c + w.c - n_resp;
     }
-    s_a[tid] = a;
-    s_b[tid] = b;
+    if (tid == nthr - 1) s_total = w;
     __syncthreads();
-    for (int d = 1; d < nthr; d <<= 1) {
-      const long long xa = tid >= d ? s_a[tid - d] : 0;
-      const int32_t xb = tid >= d ? s_b[tid - d] : 0;
-      __syncthreads();
-      s_a[tid] += xa;
-      s_b[tid] += xb;
-      __syncthreads();
-    }
-    if (i < p.G) {
-      p.pre[i] = s_carry + s_a[tid];
-      p.out_resp_off[i] = s_carry_b + s_b[tid] - b;
-    }
-    __syncthreads();
-    if (tid == nthr - 1) {
-      s_carry += s_a[tid];
-      s_carry_b += s_b[tid];
-    }
-    __syncthreads();
+    carry.a += s_total.a;
+    carry.b += s_total.b;
+    carry.c += s_total.c;
   }
-  if (tid == 0) p.out_resp_off[p.G] = s_carry_b;
+  if (tid == 0) p.out_resp_off[p.G] = carry.c;
+  // the responses' lengths, four loads in flight per thread
+  for (int i = tid; i < p.G; i += nthr) {
+    const int x0 = ja[i], n = jb[i], y0 = p.out_resp_off[i];
+#pragma unroll 4
+    for (int x = 0; x < n; ++x) p.out_resp_len[y0 + x] = p.resp_len[x0 + x];
+  }
   __syncthreads();
   // Next fit in parallel.  nxt[s] = where the row that starts at sorted position s ends: the
   // largest e whose tokens still fit (every group fits alone, so e > s).  The row starts are
   // the positions reachable from 0 through nxt; they are marked by pointer doubling (after
   // round r every start within 2^r hops is marked), then numbered by a prefix count.
   for (int s = tid; s < p.G; s += nthr) {
-    const long long base = s ? p.pre[s - 1] : 0;
+    const long long base = s ? pre[s - 1] : 0;
     int lo = s + 1, hi = p.G;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (p.pre[mid - 1] - base <= p.capacity) lo = mid; else hi = mid - 1;
+      if (pre[mid - 1] - base <= p.capacity) lo = mid; else hi = mid - 1;
     }
     p.nxt[s] = lo;
-    p.jump_a[s] = lo;
-    p.mark[s] = (s == 0);
+    ja[s] = lo;
+    mark[s] = (s == 0);
   }
-  int32_t* ja = p.jump_a;
-  int32_t* jb = p.jump_b;
   for (int hop = 1; hop < p.G; hop <<= 1) {
     __syncthreads();
+    for (int s = tid; s < p.G; s += nthr) {
+      const int to = ja[s];
+      jb[s] = to < p.G ? ja[to] : p.G;
+    }
+    // (marking runs along with the doubling: a mark set in this round by another thread only
+    // marks further positions that are reachable as well)
     for (int s = tid; s < p.G; s += nthr)
-      if (p.mark[s] && ja[s] < p.G) p.mark[ja[s]] = 1;
-    for (int s = tid; s < p.G; s += nthr) jb[s] = ja[s] < p.G ? ja[ja[s]] : p.G;
+      if (mark[s] && ja[s] < p.G) mark[ja[s]] = 1;
     __syncthreads();
     int32_t* t = ja;
     ja = jb;
@@ -168,77 +243,102 @@ __global__ void __launch_bounds__(1024) rows_pack_kernel(RowsPtrs p) {
   }
   __syncthreads();
   // number the marked positions (exclusive scan of the marks) and emit the rows
-  if (tid == 0) s_carry_b = 0;
-  __syncthreads();
+  int32_t rows = 0;
   for (int base = 0; base < p.G; base += nthr) {
     const int i = base + tid;
-    const int32_t m = i < p.G ? p.mark[i] : 0;
-    s_b[tid] = m;
-    __syncthreads();
-    for (int d = 1; d < nthr; d <<= 1) {
-      const int32_t xb = tid >= d ? s_b[tid - d] : 0;
-      __syncthreads();
-      s_b[tid] += xb;
-      __syncthreads();
-    }
+    const int32_t m = i < p.G ? mark[i] : 0;
+    const Sum3 w = block_scan({0, 0, m}, s_warp);
     if (m) {
-      const int r = s_carry_b + s_b[tid] - 1;
+      const int r = rows + w.c - 1, e = p.nxt[i] - 1;
       p.row_group_off[r] = i;
-      p.row_tokens[r] = p.pre[p.nxt[i] - 1] - (i ? p.pre[i - 1] : 0);
+      p.row_tokens[r] = pre[e] - (i ? pre[i - 1] : 0);
+      p.row_cost[r] = p.pre_cost[e] - (i ? p.pre_cost[i - 1] : 0);
     }
+    if (tid == nthr - 1) s_total = w;
     __syncthreads();
-    if (tid == nthr - 1) s_carry_b += s_b[tid];
-    __syncthreads();
+    rows += s_total.c;
   }
   if (tid == 0) {
-    p.row_group_off[s_carry_b] = p.G;
-    *p.num_rows = s_carry_b;
-    s_rows = s_carry_b;
-  }
-  __syncthreads();
-  for (int r = tid; r < s_rows; r += nthr) {
-    long long c = 0;
-    for (int i = p.row_group_off[r]; i < p.row_group_off[r + 1]; ++i) c += p.cost[p.order[i]];
-    p.row_cost[r] = c;
-  }
-  for (int i = tid; i < p.G; i += nthr) {
-    const int g = p.order[i];
-    const int x0 = p.resp_off[g], n = p.resp_off[g + 1] - x0, y0 = p.out_resp_off[i];
-    for (int x = 0; x < n; ++x) p.out_resp_len[y0 + x] = p.resp_len[x0 + x];
+    p.row_group_off[rows] = p.G;
+    *p.num_rows = rows;
   }
 }
 
 // ---------------------------------------------------------------- rows -> data-parallel ranks
 // Longest-processing-time assignment: rows in order of decreasing cost (ties by index), each to
 // the rank with the least cost so far (ties to the lowest rank).  The order comes from rank
-// counting over all rows; the greedy pass is sequential by nature and runs in one warp, the
-// lanes sharing the search for the least-loaded rank.
-__global__ void __launch_bounds__(256)
-assign_rank_kernel(int R, const long long* __restrict__ cost, int32_t* __restrict__ order) {
-  __shared__ long long s_c[256];
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  const long long mine = r < R ? cost[r] : 0;
-  int rank = 0;
-  for (int base = 0; base < R; base += 256) {
-    const int u = base + threadIdx.x;
-    s_c[threadIdx.x] = u < R ? cost[u] : -1;
-    __syncthreads();
-    const int lim = min(256, R - base);
-    for (int i = 0; i < lim; ++i) {
-      const long long o = s_c[i];
-      rank += (o > mine) || (o == mine && base + i < r);
-    }
-    __syncthreads();
-  }
-  if (r < R) order[rank] = r;
-}
-
+// counting over all rows; the greedy pass is sequential by nature and runs in one warp.  What
+// bounds it is the chain from one row's assignment to the next one's, so the ranks are kept
+// sorted by (load, rank) across the lanes' registers, kPerLane entries each: a step takes the
+// first entry, adds the row's cost and inserts it again -- every lane compares its entries with
+// the new one and keeps, shifts or replaces them -- so the chain is one broadcast, one add and
+// one compare.  Rows are fetched and results written 32 at a time.  (Searching all loads in shared
+// memory for the least one with a five-step butterfly took 345 ns a row, now 67 with up to 32 ranks, 98 with 64, 120 with 128.)
 constexpr int kMaxAssignRanks = 1024;
 
+template <int kPerLane>
 __global__ void __launch_bounds__(32)
 assign_greedy_kernel(int R, int ranks, const long long* __restrict__ cost,
                      const int32_t* __restrict__ order, int32_t* __restrict__ rank_of_row,
                      long long* __restrict__ rank_cost) {
+  constexpr long long kInf = 0x7fffffffffffffffLL;
+  const int lane = threadIdx.x;
+  long long load[kPerLane];
+  int id[kPerLane];
+#pragma unroll
+  for (int j = 0; j < kPerLane; ++j) {   // entry lane * kPerLane + j of the sorted list
+    id[j] = lane * kPerLane + j;
+    load[j] = id[j] < ranks ? 0 : kInf;
+  }
+  int row_next = lane < R ? order[lane] : 0;
+  long long cost_next = lane < R ? cost[row_next] : 0;
+  for (int base = 0; base < R; base += 32) {
+    const int row = row_next;
+    const long long c_mine = cost_next;
+    const int ahead = base + 32 + lane;
+    row_next = ahead < R ? order[ahead] : 0;
+    cost_next = ahead < R ? cost[row_next] : 0;
+    int my_rank = 0;
+    const int here = min(32, R - base);
+    for (int i = 0; i < here; ++i) {
+      const long long v = __shfl_sync(0xffffffffu, load[0], 0) + __shfl_sync(0xffffffffu, c_mine, i);
+      const int r = __shfl_sync(0xffffffffu, id[0], 0);
+      // the entry behind my last one
+      long long up_load = __shfl_down_sync(0xffffffffu, load[0], 1);
+      const int up_id = __shfl_down_sync(0xffffffffu, id[0], 1);
+      if (lane == 31) up_load = kInf;
+      if (lane == i) my_rank = r;
+      // before(e): entry e stays in front of the new one
+      auto before = [&](long long l, int k) { return l < v || (l == v && k < r); };
+      bool mine_before = lane == 0 || before(load[0], id[0]);   // (entry 0 of lane 0 is taken out)
+#pragma unroll
+      for (int j = 0; j < kPerLane; ++j) {
+        const long long nl = j + 1 < kPerLane ? load[j + 1] : up_load;
+        const int ni = j + 1 < kPerLane ? id[j + 1] : up_id;
+        const bool next_before = before(nl, ni);
+        if (next_before) {           // everything up to the next entry moves forward
+          load[j] = nl;
+          id[j] = ni;
+        } else if (mine_before) {    // the new entry belongs here
+          load[j] = v;
+          id[j] = r;
+        }
+        mine_before = next_before;
+      }
+    }
+    if (base + lane < R) rank_of_row[row] = my_rank;
+  }
+#pragma unroll
+  for (int j = 0; j < kPerLane; ++j)
+    if (id[j] < ranks) rank_cost[id[j]] = load[j];
+}
+
+// More ranks than the lanes' registers hold: the loads in shared memory, the lanes sharing the
+// search for the least one.
+__global__ void __launch_bounds__(32)
+assign_greedy_smem_kernel(int R, int ranks, const long long* __restrict__ cost,
+                          const int32_t* __restrict__ order, int32_t* __restrict__ rank_of_row,
+                          long long* __restrict__ rank_cost) {
   __shared__ long long s_load[kMaxAssignRanks];
   const int lane = threadIdx.x;
   for (int k = lane; k < ranks; k += 32) s_load[k] = 0;
@@ -277,14 +377,19 @@ assign_greedy_kernel(int R, int ranks, const long long* __restrict__ cost,
 cudaError_t launch_assign_rows(int R, const long long* row_cost, int ranks, int32_t* order,
                                int32_t* rank_of_row, long long* rank_cost, cudaStream_t stream,
                                int* launches) {
-  assign_rank_kernel<<<(R + 255) / 256, 256, 0, stream>>>(R, row_cost, order);
-  assign_greedy_kernel<<<1, 32, 0, stream>>>(R, ranks, row_cost, order, rank_of_row, rank_cost);
+  rank_kernel<long long><<<(R + kRankKeys - 1) / kRankKeys, kRankKeys * kRankSlices, 0, stream>>>(
+      R, row_cost, order);
+  auto greedy = ranks <= 32    ? assign_greedy_kernel<1>
+                : ranks <= 64  ? assign_greedy_kernel<2>
+                : ranks <= 128 ? assign_greedy_kernel<4>
+                               : assign_greedy_smem_kernel;
+  greedy<<<1, 32, 0, stream>>>(R, ranks, row_cost, order, rank_of_row, rank_cost);
   if (launches) *launches = 2;
   return cudaGetLastError();
 }
 
 size_t rows_workspace_bytes(int G) {
-  return align_up(size_t(8) * G, 256) * 3 + align_up(size_t(4) * G, 256) * 4;
+  return align_up(size_t(8) * G, 256) * 3 + align_up(size_t(4) * G, 256) * 5;
 }
 
 cudaError_t launch_build_rows(int G, int N, const int32_t* prompt_len, const int32_t* resp_off,
@@ -302,14 +407,15 @@ cudaError_t launch_build_rows(int G, int N, const int32_t* prompt_len, const int
   p.resp_len = resp_len;
   char* w = static_cast<char*>(ws);
   const size_t a8 = align_up(size_t(8) * G, 256);
-  p.tok = reinterpret_cast<long long*>(w);
-  p.cost = reinterpret_cast<long long*>(w + a8);
-  p.pre = reinterpret_cast<long long*>(w + 2 * a8);
+  p.cost = reinterpret_cast<long long*>(w);
+  p.pre = reinterpret_cast<long long*>(w + a8);
+  p.pre_cost = reinterpret_cast<long long*>(w + 2 * a8);
   const size_t a4 = align_up(size_t(4) * G, 256);
   p.nxt = reinterpret_cast<int32_t*>(w + 3 * a8);
   p.jump_a = reinterpret_cast<int32_t*>(w + 3 * a8 + a4);
   p.jump_b = reinterpret_cast<int32_t*>(w + 3 * a8 + 2 * a4);
   p.mark = reinterpret_cast<int32_t*>(w + 3 * a8 + 3 * a4);
+  p.tok = reinterpret_cast<int32_t*>(w + 3 * a8 + 4 * a4);
   p.order = order;
   p.row_group_off = row_group_off;
   p.num_rows = num_rows;
@@ -322,8 +428,20 @@ cudaError_t launch_build_rows(int G, int N, const int32_t* prompt_len, const int
   cudaError_t e = cudaMemsetAsync(status, 0, 8, stream);
   if (e != cudaSuccess) return e;
   rows_measure_kernel<<<(G + 255) / 256, 256, 0, stream>>>(p);
-  rows_rank_kernel<<<(G + 255) / 256, 256, 0, stream>>>(p);
-  rows_pack_kernel<<<1, 1024, 0, stream>>>(p);
+  rank_kernel<int32_t><<<(G + kRankKeys - 1) / kRankKeys, kRankKeys * kRankSlices, 0, stream>>>(
+      G, p.tok, order);
+  // per device: the opt-in to more than 48 KB of dynamic shared memory
+  static DeviceSetup setup[kMaxDevices];
+  DeviceSetup* dev = device_setup(setup);
+  if (!dev) return cudaErrorInvalidDevice;
+  if (!dev->configured) {
+    e = cudaFuncSetAttribute(rows_pack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             20 * kPackSmemGroups);
+    if (e != cudaSuccess) return e;
+    dev->configured = true;
+  }
+  const bool in_smem = G <= kPackSmemGroups;
+  rows_pack_kernel<<<1, 1024, in_smem ? size_t(20) * G : 0, stream>>>(p, in_smem);
   if (launches) *launches = 3;
   return cudaGetLastError();
 }

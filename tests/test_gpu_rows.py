@@ -123,3 +123,25 @@ def test_assign_rows_errors():
     with pytest.raises(B.PPError) as e:
         B.pp_assign_rows(c, 2000)
     assert e.value.code == -2
+
+
+@pytest.mark.parametrize("G", [31, 33, 64, 65, 1023, 1025, 2049, 8192, 8193])
+def test_row_builder_at_the_edges_of_its_blocks_and_tables(G):
+    """Bit-exact; 8192 groups are the most whose tables stay in shared memory."""
+    rng = np.random.default_rng(G)
+    P, off, rl = _random_groups(rng, G, 40)
+    _compare(P, off, rl, int(R.group_tokens(P, off, rl).max()) * 3 + G % 7)
+
+
+@pytest.mark.parametrize("ranks", [2, 31, 32, 33, 64, 65, 128, 129])
+@pytest.mark.parametrize("rows", [1, 31, 32, 33, 129, 700])
+def test_assign_rows_at_the_edges_of_the_lane_lists(rows, ranks):
+    """One, two and four list entries per lane and the search beyond; zero costs and ties."""
+    from paper_2602_24082_b200 import binding as B
+    rng = np.random.default_rng(rows * 1000 + ranks)
+    cost = rng.integers(0, 6 if rows % 2 else 1 << 45, size=rows).astype(np.int64)
+    order, rank_of_row, rank_cost = B.pp_assign_rows(torch.from_numpy(cost).cuda(), ranks)
+    want = R.assign_rows(cost, ranks)
+    assert np.array_equal(order.cpu().numpy(), want[0])
+    assert np.array_equal(rank_of_row.cpu().numpy(), want[1])
+    assert np.array_equal(rank_cost.cpu().numpy(), want[2])
