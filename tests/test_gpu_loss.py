@@ -14,6 +14,12 @@ CASES = [
     W.Workload("single", [[(97, (64,)), (128, (128, 128, 7, 9, 40))], [(700, (1, 1))]], 2, 2, 64, seed=5),
     W.config2(),
     W.config4(3),
+    # every team width of the kernel (mean segment 1 .. 4096 tokens), more responses than teams
+    W.Workload("ones", [[(1, (1,) * 37)] for _ in range(9)], 1, 1, 64, seed=6),
+    W.Workload("mean200", [[(200, (190, 210, 1, 399) * 5)]], 1, 1, 64, seed=7),
+    W.Workload("mean400", [[(400, (511, 289, 400))], [(1, (799,))]], 1, 1, 64, seed=8),
+    W.Workload("mean900", [[(900, (1023, 1, 1577))]], 1, 1, 64, seed=9),
+    W.Workload("mean4096", [[(4096, (4095, 4097))]], 1, 1, 64, seed=10),
 ] + [W.random_structure(s) for s in range(8)]
 
 
