@@ -40,80 +40,68 @@ struct BwdParams {
 // ---------------------------------------------------------------- preprocess
 // Delta = sum_d dO * O per (token, query head) row, the LSE in base-2 units, and the row of
 // the fp32 dQ accumulator cleared (so no separate memset pass over it is needed) unless the
-// forward has already cleared it (kClear = false).  D / 8 lanes per row with 16-byte loads,
-// four row groups per warp in flight: the pass is a pure stream over O and dO.  The rows
-// [T][Hq] and the statistics [Hq][T] are transposed to each other, so one side is strided:
-// kTokenMajor walks memory order (contiguous O / dO, scattered 4-byte statistics), otherwise
-// rows are walked head by head (contiguous statistics, one row per Hq * D * 2 bytes).  The
-// second measured about 5 us faster where a token's heads span 8 KB (Hq = 32, D = 128,
-// T = 9241), the first about 60 us faster at 16 KB (Hq = 64, T = 16384); the launcher picks by
-// that size.
+// forward has already cleared it (kClear = false).  A pure stream over O and dO, bound by
+// memory: D / 8 lanes per row with 16-byte loads, kUnroll rows per lane group in flight.  A warp
+// takes kUnroll * kRows consecutive tokens of one head, so that the statistics [Hq][T] leave as
+// one store of consecutive words; the block index runs over the heads fastest, so that the blocks
+// running at the same time read whole tokens of [T][Hq][D].  No row index is divided: a version
+// that derived (token, head) from a 64-bit row number, two divisions per row and lane, took 40 us
+// where this takes 30 (T = 9241, Hq = 32, D = 128: 151 MB), 129 against 92 at T = 16384, Hq = 64,
+// and with the clearing 488 against 330 at T = 65536, Hq = 32 (2.1 GB, 6.5 TB/s).
 // lanes that share a row: D / 8 (16 bytes of bf16 per lane), rounded up to a power of two
 __host__ __device__ constexpr int pre_lanes(int d) { return d == 96 ? 16 : d / 8; }
+constexpr int kPreUnroll = 4, kPreWarps = 8;
+// tokens per block
+__host__ __device__ constexpr int pre_tokens(int d) { return kPreWarps * kPreUnroll * (32 / pre_lanes(d)); }
 
-template <int D, bool kClear, bool kTokenMajor>
-__global__ void __launch_bounds__(256)
+template <int D, bool kClear>
+__global__ void __launch_bounds__(32 * kPreWarps)
 bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o,
                       const float* __restrict__ lse, float* __restrict__ delta,
                       float* __restrict__ lse2, float* __restrict__ dq_acc, int T, int Hq) {
   constexpr int kLanes = pre_lanes(D);    // lanes per row (D / 8 of them hold data)
   constexpr int kRows = 32 / kLanes;      // rows per warp and step
-  constexpr int kUnroll = 4;
   const int lane = threadIdx.x & 31, sub = lane % kLanes, rin = lane / kLanes;
-  const long long rows = (long long)T * Hq;
-  const long long warp0 = ((long long)blockIdx.x * 8 + (threadIdx.x >> 5)) * (kRows * kUnroll);
-  const long long stride = (long long)gridDim.x * 8 * (kRows * kUnroll);
-  for (long long base = warp0; base < rows; base += stride) {
-    uint4 a[kUnroll], b[kUnroll];
+  const int chunk = blockIdx.x / Hq, h = blockIdx.x - chunk * Hq;
+  const int t0 = chunk * pre_tokens(D) + (threadIdx.x >> 5) * (kPreUnroll * kRows);
+  // lane (rin, sub = u) writes the statistics of token t0 + u * kRows + rin
+  const int t_stat = t0 + sub * kRows + rin;
+  const bool writes = sub < kPreUnroll && t_stat < T;
+  const size_t stat = size_t(h) * T + t_stat;
+  const float my_lse = writes ? lse[stat] : 0.f;
+  const size_t row0 = (size_t(t0 + rin) * Hq + h) * D + sub * 8, step = size_t(kRows) * Hq * D;
+  uint4 a[kPreUnroll], b[kPreUnroll];
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      // rows are walked head by head, tokens fastest: the per-row statistics [Hq][T] are then
-      // written to consecutive addresses (each O / dO row is one contiguous piece anyway)
-      const long long idx = base + u * kRows + rin;
-      a[u] = b[u] = make_uint4(0u, 0u, 0u, 0u);
-      if (idx < rows && sub < D / 8) {
-        long long row = idx;
-        if (!kTokenMajor) {
-          const int h = int(idx / T), t = int(idx - (long long)h * T);
-          row = (long long)t * Hq + h;
-        }
-        a[u] = reinterpret_cast<const uint4*>(o + row * D)[sub];
-        b[u] = reinterpret_cast<const uint4*>(d_o + row * D)[sub];
-      }
+  for (int u = 0; u < kPreUnroll; ++u) {
+    a[u] = b[u] = make_uint4(0u, 0u, 0u, 0u);
+    if (t0 + u * kRows + rin < T && sub < D / 8) {
+      a[u] = *reinterpret_cast<const uint4*>(o + row0 + u * step);
+      b[u] = *reinterpret_cast<const uint4*>(d_o + row0 + u * step);
+    }
+  }
+  float mine = 0.f;
+#pragma unroll
+  for (int u = 0; u < kPreUnroll; ++u) {
+    const uint32_t aw[4] = {a[u].x, a[u].y, a[u].z, a[u].w}, bw[4] = {b[u].x, b[u].y, b[u].z, b[u].w};
+    float acc = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[i]));
+      const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw[i]));
+      acc = fmaf(x.x, y.x, fmaf(x.y, y.y, acc));
     }
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      const long long idx = base + u * kRows + rin;
-      const uint32_t aw[4] = {a[u].x, a[u].y, a[u].z, a[u].w}, bw[4] = {b[u].x, b[u].y, b[u].z, b[u].w};
-      float acc = 0.f;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[i]));
-        const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw[i]));
-        acc = fmaf(x.x, y.x, fmaf(x.y, y.y, acc));
-      }
-#pragma unroll
-      for (int sft = kLanes / 2; sft > 0; sft >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, sft);
-      if (idx < rows) {
-        long long row = idx, stat = idx;  // position in [T][Hq] and in [Hq][T]
-        if (kTokenMajor) {
-          const int t = int(idx / Hq), h = int(idx - (long long)t * Hq);
-          stat = (long long)h * T + t;
-        } else {
-          const int h = int(idx / T), t = int(idx - (long long)h * T);
-          row = (long long)t * Hq + h;
-        }
-        if (kClear && sub < D / 8) {
-          float4* z = reinterpret_cast<float4*>(dq_acc + row * D + sub * 8);
-          z[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-          z[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        if (sub == 0) {
-          delta[stat] = acc;
-          lse2[stat] = lse[stat] * 1.4426950408889634f;
-        }
-      }
+    for (int sft = kLanes / 2; sft > 0; sft >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, sft);
+    if (sub == u) mine = acc;
+    if (kClear && t0 + u * kRows + rin < T && sub < D / 8) {
+      float4* z = reinterpret_cast<float4*>(dq_acc + row0 + u * step);
+      z[0] = make_float4(0.f, 0.f, 0.f, 0.f);
+      z[1] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
+  }
+  if (writes) {
+    delta[stat] = mine;
+    lse2[stat] = my_lse * 1.4426950408889634f;
   }
 }
 
@@ -876,25 +864,12 @@ cudaError_t launch_bwd_t(const pp_plan* plan, const void* o, const float* lse, c
   }
   const pp_problem& pb = plan->prob;
   const size_t T = pb.total_tokens, Hq = pb.num_q_heads;
-  const long long pairs = (long long)T * Hq;
   const int num_sms = dev->num_sms;
-  constexpr int kRowsPerBlock = 8 * (32 / pre_lanes(DV)) * 4;  // warps x rows per warp x unroll
-  const unsigned pre_blocks = unsigned(
-      std::min<long long>((pairs + kRowsPerBlock - 1) / kRowsPerBlock, (long long)num_sms * 16));
-  auto pre = [&](auto clear, auto token_major) {
-    bwd_preprocess_kernel<DV, decltype(clear)::value, decltype(token_major)::value>
-        <<<pre_blocks, 256, 0, stream>>>(
-            static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse,
-            const_cast<float*>(prm.delta), const_cast<float*>(prm.lse2), prm.dq_acc, int(T), int(Hq));
-  };
-  const bool token_major = Hq * DV * 2 >= 16384;
-  if (dq_cleared) {
-    if (token_major) pre(std::false_type{}, std::true_type{});
-    else pre(std::false_type{}, std::false_type{});
-  } else {
-    if (token_major) pre(std::true_type{}, std::true_type{});
-    else pre(std::true_type{}, std::false_type{});
-  }
+  const unsigned pre_blocks = unsigned(Hq * ((T + pre_tokens(DV) - 1) / pre_tokens(DV)));
+  auto pre = dq_cleared ? bwd_preprocess_kernel<DV, false> : bwd_preprocess_kernel<DV, true>;
+  pre<<<pre_blocks, 32 * kPreWarps, 0, stream>>>(
+      static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse,
+      const_cast<float*>(prm.delta), const_cast<float*>(prm.lse2), prm.dq_acc, int(T), int(Hq));
   const long long units = (long long)plan->max_tiles * pb.num_kv_heads;
   dim3 grid(unsigned(std::min<long long>(units, num_sms)));
   ProfileEvents& ev = profile_events();
