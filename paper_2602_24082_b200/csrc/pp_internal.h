@@ -222,7 +222,9 @@ bool profile_read(float* fwd_ms, float* bwd_ms);
 bool profile_read_all(float* fwd_ms, float* bwd_ms, int capacity, int* n_fwd, int* n_bwd);
 
 // launchers (defined in the .cu files); all return a cudaError_t
-cudaError_t launch_plan(const pp_plan* plan, cudaStream_t stream, int* launches);
+// host_desc: the four descriptor arrays on the host, or null when they are on the device
+cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cudaStream_t stream,
+                        int* launches);
 cudaError_t launch_fwd(const pp_plan* plan, const void* q, const void* k, const void* v, float scale,
                        void* o, float* lse, float* dq_clear, cudaStream_t stream, int* launches);
 cudaError_t launch_bwd(const pp_plan* plan, const void* q, const void* k, const void* v,

@@ -9,7 +9,10 @@
 // backward has its own key tiles, cut per group (see BTile): its masks are two comparisons per
 // element with per-key bounds, so straddling costs nothing there and short segments leave no
 // ragged tiles.
+#include <string.h>
+
 #include <algorithm>
+#include <type_traits>
 
 #include "pp_internal.h"
 
@@ -382,111 +385,434 @@ __global__ void plan_units_kernel(PlanPtrs p) {
   if (t < n) plan_units_body(p, t, n);
 }
 
-// The whole plan in one block: used when the problem is small enough that one block's
-// latency beats eight dependent launches (every stage only needs block-level ordering).  The
-// per-tile keys of the rank-counting stages are kept in shared memory, so that the O(n^2)
-// loops do not go through global memory, and key_end is filled tile by tile (every key of a
-// forward tile ends its visibility at the tile's vis_end) instead of by a search per token.
-constexpr int kFusedMaxTiles = 2048;
+// ---------------------------------------------------------------- host descriptors
+template <size_t N>
+struct DescBlock {
+  int32_t v[N];
+};
+constexpr size_t kDescSmall = 960, kDescFused = 4104, kDescLarge = 7168;
 
-__global__ void __launch_bounds__(1024) plan_fused_kernel(PlanPtrs p) {
-  __shared__ uint16_t s_wf[kFusedMaxTiles];   // forward work of the forward tiles
-  __shared__ uint16_t s_wb[kFusedMaxTiles];   // work of the backward tiles
-  __shared__ int32_t s_gs[kFusedMaxTiles];    // group id of the backward tiles
-  __shared__ int32_t s_gw[kFusedMaxTiles];    // backward work of the tile's whole group
-  __shared__ uint16_t s_sg[kFusedMaxTiles];   // super-group
-  if (!plan_scan_body(p)) return;
-  const int n = p.header[kHdrNumTiles], nb = p.header[kHdrNumBTiles];
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  for (int t = tid; t < n; t += nthr) {
-    plan_tile_body(p, t);
-    s_wf[t] = uint16_t(p.tiles[t].work);  // own write
+void fill_desc(const int32_t* const* src, const size_t (&n)[4], int32_t* dst) {
+  for (int i = 0; i < 4; ++i) {
+    memcpy(dst, src[i], n[i] * sizeof(int32_t));
+    dst += n[i];
   }
-  for (int t = tid; t < nb; t += nthr) {
-    plan_btile_body(p, t);
-    const BTile b = p.btiles[t];  // own write
-    s_wb[t] = uint16_t(b.work);
-    s_gs[t] = b.grp_start;
-  }
-  __syncthreads();
-  // key_end: one warp per forward tile, coalesced
-  for (int t = tid >> 5; t < n; t += nthr >> 5) {
-    const Tile tl = p.tiles[t];
-    for (int i = tid & 31; i < tl.len; i += 32) p.key_end[tl.start + i] = tl.vis_end;
-  }
-  // Longest-work-first orders by rank counting, and the work of each backward tile's group.
-  // One warp per tile: the lanes stride over the other tiles and the partial counts are
-  // summed with shuffles (a thread per tile would walk the whole list alone, a few
-  // microseconds of dependent shared-memory reads per pass on a 100-tile plan).
-  const int lane = tid & 31, wid = tid >> 5, nwarp = nthr >> 5;
-  auto warp_sum = [](int x) {
+}
+
+template <size_t N>
+__global__ void stage_desc_kernel(const __grid_constant__ DescBlock<N> blk, int n, int32_t* dst) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = blk.v[i];
+}
+
+// ---------------------------------------------------------------- the whole plan in one block
+// Used when the problem is small enough that one block's latency beats eight dependent launches.
+// It is all latency: a few thousand integers through a chain of dependent steps.  So everything
+// that is read back -- descriptors, segment and tile offsets, works -- stays in shared memory (a
+// dependent read costs 30 cycles there instead of 300 - 700), host descriptors arrive as a kernel
+// argument without a staging kernel in front, scans are two barriers, the block has no more
+// threads than the plan has use for (idle warps take issue slots from the others), and the orders
+// come from 32-bit keys, work and index in one word: up to kRankTiles tiles by counting the
+// smaller keys (n^2 comparisons spread over the block: 300 cycles for 128 keys), beyond by a
+// bitonic sort (66 steps for 2048).  Eight 1100-token groups 17.4 -> 8.2 us, four 4800-token
+// groups 27 -> 12, two rows of 32768 tokens 118 -> 32, 40000 tokens in 1330 short segments
+// 194 -> 52.
+constexpr int kRankTiles = 512;
+constexpr int kFusedSmallTiles = 256;  // blocks of 256 threads up to here, 1024 beyond
+constexpr int kFusedMaxTiles = 2048;   // tiles; also bounds the segments, and twice the groups
+
+struct FusedSmem {
+  union alignas(16) {   // (keys are read as uint4)
+    uint32_t sort[2][3][kFusedMaxTiles];
+    struct {
+      uint32_t key[4][kRankTiles];      // forward tiles, backward tiles, groups, backward units
+      int32_t rank[4][kRankTiles];      // (groups: backward tiles of the groups ranked before)
+    } r;
+  } o;
+  int32_t desc[kDescFused];
+  int32_t seg_start[kFusedMaxTiles + 1];
+  int32_t seg_tile0[kFusedMaxTiles + 1];
+  int32_t btile0[kFusedMaxTiles / 2 + 1];
+  int32_t tile[3][kFusedMaxTiles];      // start, end, vis_end of the forward tiles
+  int32_t gwork[kFusedMaxTiles / 2];    // backward work of each group
+  int32_t before[kFusedMaxTiles / 2];   // backward tiles of the groups ranked before it
+  uint16_t seg_grp[kFusedMaxTiles];
+  uint16_t wb[kFusedMaxTiles];          // work and group of the backward tiles
+  uint16_t bgrp[kFusedMaxTiles];
+  uint16_t unit_tile[kFusedMaxTiles];   // backward tiles in the order of their units
+  int32_t warp_sum[2][32];
+  int32_t status, detail;
+};
+
+// Inclusive sums of two values over the block.
+__device__ __forceinline__ void block_scan2(int& a, int& b, int32_t (&s_warp)[2][32]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto warp_scan = [&](int& x, int& y) {
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(0xffffffffu, x, d);
-    return x;
+    for (int d = 1; d < 32; d <<= 1) {
+      const int xa = __shfl_up_sync(0xffffffffu, x, d), yb = __shfl_up_sync(0xffffffffu, y, d);
+      if (lane >= d) {
+        x += xa;
+        y += yb;
+      }
+    }
   };
-  for (int t = wid; t < n; t += nwarp) {
-    const int wf = s_wf[t];
-    int rf = 0;
-    for (int u = lane; u < n; u += 32) {
-      const int of = s_wf[u];
-      rf += (of > wf) || (of == wf && u < t);
-    }
-    rf = warp_sum(rf);
-    if (lane == 0) p.fwd_order[rf] = t;
+  warp_scan(a, b);
+  if (lane == 31) {
+    s_warp[0][warp] = a;
+    s_warp[1][warp] = b;
   }
-  for (int t = wid; t < nb; t += nwarp) {
-    const int wb = s_wb[t], gs = s_gs[t];
-    int rb = 0, gw = 0;
-    for (int u = lane; u < nb; u += 32) {
-      const int ob = s_wb[u];
-      rb += (ob > wb) || (ob == wb && u < t);
-      gw += (s_gs[u] == gs) ? ob : 0;
+  __syncthreads();
+  if (warp == 0) {
+    const bool there = lane < int(blockDim.x >> 5);
+    int x = there ? s_warp[0][lane] : 0, y = there ? s_warp[1][lane] : 0;
+    warp_scan(x, y);
+    s_warp[0][lane] = x;
+    s_warp[1][lane] = y;
+  }
+  __syncthreads();
+  if (warp) {
+    a += s_warp[0][warp - 1];
+    b += s_warp[1][warp - 1];
+  }
+}
+
+// rank[t] += (weight of the) keys below key t, for m <= kRankTiles keys: the block's threads form
+// slices of a power of two >= m threads, each counts over its part of the keys (read four at a
+// time, the same ones by all lanes of a warp).  Keys are padded to a multiple of four with ~0.
+template <bool kWeighted>
+__device__ __forceinline__ void rank_count(const uint32_t* key, int m, int32_t* rank, const int32_t* off) {
+  int lg = 5;
+  while ((1 << lg) < m) ++lg;
+  const int t = threadIdx.x & ((1 << lg) - 1), slice = threadIdx.x >> lg, slices = blockDim.x >> lg;
+  const int quads = (m + 3) >> 2, per = (quads + slices - 1) / slices;
+  const int lo = slice * per, hi = min(lo + per, quads);
+  if (t >= m || lo >= hi) return;
+  const uint32_t mine = key[t];
+  int count = 0;
+#pragma unroll 2
+  for (int i = lo; i < hi; ++i) {
+    const uint4 k = reinterpret_cast<const uint4*>(key)[i];
+    const uint32_t kk[4] = {k.x, k.y, k.z, k.w};
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      if (kk[c] < mine) count += kWeighted ? off[4 * i + c + 1] - off[4 * i + c] : 1;
+  }
+  if (count) atomicAdd(&rank[t], count);
+}
+
+// Ascending bitonic sort of kArrays arrays of `n2` (1024 or 2048) keys in a block of 1024 threads,
+// key tid + 1024 r of each in v[.][r].  Distances below 32 are shuffles, 1024 is inside the thread,
+// the others go through shared memory (two buffers in turn: one barrier per distance).
+template <int kArrays>
+__device__ __forceinline__ void bitonic_sort(uint32_t (&v)[kArrays][2], int n2,
+                                             uint32_t (&buf)[2][3][kFusedMaxTiles]) {
+  const int tid = threadIdx.x;
+  const bool two = n2 > 1024;
+  int turn = 0;
+  for (int k = 2; k <= n2; k <<= 1) {
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      if (j == 1024) {   // k = 2048: ascending throughout
+#pragma unroll
+        for (int a = 0; a < kArrays; ++a) {
+          const uint32_t lo = min(v[a][0], v[a][1]), hi = max(v[a][0], v[a][1]);
+          v[a][0] = lo;
+          v[a][1] = hi;
+        }
+        continue;
+      }
+      // the lower key of a pair keeps the smaller one where the run ascends, and vice versa
+      const bool small0 = ((tid & j) == 0) == ((tid & k) == 0);
+      const bool small1 = ((tid & j) == 0) == (((tid + 1024) & k) == 0);
+      if (j >= 32) {
+#pragma unroll
+        for (int a = 0; a < kArrays; ++a) {
+          buf[turn][a][tid] = v[a][0];
+          if (two) buf[turn][a][tid + 1024] = v[a][1];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int a = 0; a < kArrays; ++a) {
+          const uint32_t o = buf[turn][a][tid ^ j];
+          v[a][0] = small0 ? min(v[a][0], o) : max(v[a][0], o);
+          if (two) {
+            const uint32_t q = buf[turn][a][(tid ^ j) + 1024];
+            v[a][1] = small1 ? min(v[a][1], q) : max(v[a][1], q);
+          }
+        }
+        turn ^= 1;
+      } else {
+#pragma unroll
+        for (int a = 0; a < kArrays; ++a) {
+          const uint32_t o = __shfl_xor_sync(0xffffffffu, v[a][0], j);
+          v[a][0] = small0 ? min(v[a][0], o) : max(v[a][0], o);
+          if (two) {
+            const uint32_t q = __shfl_xor_sync(0xffffffffu, v[a][1], j);
+            v[a][1] = small1 ? min(v[a][1], q) : max(v[a][1], q);
+          }
+        }
+      }
     }
-    rb = warp_sum(rb);
-    gw = warp_sum(gw);
-    if (lane == 0) {
-      p.bwd_order[rb] = t;
-      p.tile_gwork[t] = gw;
-      s_gw[t] = gw;
+  }
+}
+
+template <size_t kDesc>
+__global__ void __launch_bounds__(1024)
+plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  FusedSmem& sm = *reinterpret_cast<FusedSmem*>(smem_raw);
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nthr = blockDim.x;
+  const int n_rgo = p.num_rows + 1, n_all = n_rgo + p.G + p.G + 1 + p.N;
+  // ---- descriptors -> shared memory, and the copy that later kernels read
+  if (kDesc > 1) {
+    for (int i = tid; i < n_all; i += nthr) sm.desc[i] = blk.v[i];
+  } else {
+    const int n[4] = {n_rgo, p.G, p.G + 1, p.N};
+    int at = 0;
+    for (int a = 0; a < 4; ++a) {
+      for (int i = tid; i < n[a]; i += nthr) sm.desc[at + i] = p.src_desc[a][i];
+      at += n[a];
+    }
+  }
+  if (tid == 0) {
+    sm.status = kStatusOk;
+    sm.detail = 0;
+  }
+  __syncthreads();
+  for (int i = tid; i < n_all; i += nthr) p.desc_copy[i] = sm.desc[i];
+  const int32_t* rgo = sm.desc;
+  const int32_t* gpl = rgo + n_rgo;
+  const int32_t* gro = gpl + p.G;
+  const int32_t* rlen = gro + p.G + 1;
+  auto fail = [&](int32_t status, int32_t detail) {
+    if (atomicCAS(&sm.status, kStatusOk, status) == kStatusOk) sm.detail = detail;
+  };
+  auto give_up = [&]() {   // the header of a plan that was refused
+    if (tid < 16)
+      p.header[tid] = tid == kHdrStatus ? sm.status
+                      : tid == kHdrDetail ? sm.detail : tid == kHdrNumSegments ? p.nseg : 0;
+  };
+  // ---- validation, segment lengths
+  if (tid == 0) {
+    if (rgo[0] != 0 || rgo[p.num_rows] != p.G) fail(kStatusBadDescriptor, -1);
+    if (gro[0] != 0 || gro[p.G] != p.N) fail(kStatusBadDescriptor, -2);
+  }
+  __syncthreads();
+  for (int r = tid; r < p.num_rows; r += nthr)
+    if (rgo[r + 1] < rgo[r]) fail(kStatusBadDescriptor, r);
+  for (int g = tid; g < p.G; g += nthr) {
+    const int lo = gro[g], hi = gro[g + 1];
+    if (!(gpl[g] >= 1 && hi > lo && lo >= 0 && hi <= p.N)) {
+      fail(kStatusBadDescriptor, g);
+      continue;
+    }
+    sm.seg_start[g + lo] = gpl[g];
+    sm.seg_grp[g + lo] = uint16_t(g);
+    for (int x = lo; x < hi; ++x) {
+      const int len = rlen[x];
+      if (len < 1) fail(kStatusBadDescriptor, p.G + x);
+      sm.seg_start[g + 1 + x] = len;
+      sm.seg_grp[g + 1 + x] = uint16_t(g);
     }
   }
   __syncthreads();
-  for (int t = wid; t < nb; t += nwarp) {
-    const int gs = s_gs[t], gw = s_gw[t];
-    int rest = 0;  // tiles of this group and of the groups that come later
-    for (int u = lane; u < nb; u += 32) {
-      const int ogs = s_gs[u], ow = s_gw[u];
-      rest += (ogs == gs) || (ow < gw) || (ow == gw && ogs > gs);
+  if (sm.status != kStatusOk) {
+    give_up();
+    return;
+  }
+  // ---- first token and first tile of every segment: two segments per thread
+  {
+    const int s0 = 2 * tid, s1 = s0 + 1;
+    // (a length beyond T is a mismatch anyway; clamped, 2048 of them cannot overflow)
+    const int l0 = s0 < p.nseg ? min(sm.seg_start[s0], p.T + 1) : 0;
+    const int l1 = s1 < p.nseg ? min(sm.seg_start[s1], p.T + 1) : 0;
+    const int c0 = (l0 + kTile - 1) / kTile, c1 = (l1 + kTile - 1) / kTile;
+    int tok = l0 + l1, til = c0 + c1;
+    block_scan2(tok, til, sm.warp_sum);
+    // (the barriers inside the scan order these writes behind the reads above)
+    if (s0 <= p.nseg) {
+      sm.seg_start[s0] = tok - l0 - l1;
+      sm.seg_tile0[s0] = til - c0 - c1;
     }
-    rest = warp_sum(rest);
-    if (lane == 0) {
-      const int sg = (p.Hkv * rest - 1) / kSuperGroupUnits;
-      p.tile_sgroup[t] = sg;
-      s_sg[t] = uint16_t(sg);
+    if (s1 <= p.nseg) {
+      sm.seg_start[s1] = tok - l1;
+      sm.seg_tile0[s1] = til - c1;
+    }
+    if (tid == nthr - 1) {
+      if (p.nseg == 2 * nthr) {   // (entry nseg is past the last pair)
+        sm.seg_start[p.nseg] = tok;
+        sm.seg_tile0[p.nseg] = til;
+      }
+      if (tok != p.T) fail(kStatusTokenMismatch, tok);
     }
   }
   __syncthreads();
-  for (int t = wid; t < nb; t += nwarp) {
-    const int sg = s_sg[t], wb = s_wb[t], gs = s_gs[t], gw = s_gw[t];
-    int pos = 0, before = 0, ng = 0, k_rel = 0;
-    for (int u = lane; u < nb; u += 32) {
-      const int osg = s_sg[u], ob = s_wb[u], ogs = s_gs[u], ow = s_gw[u];
-      pos += (osg > sg) || (osg == sg && ((ob > wb) || (ob == wb && u < t)));
-      before += (ow > gw) || (ow == gw && ogs < gs);
-      ng += (ogs == gs);
-      k_rel += (ogs == gs && u < t);   // tiles of a group are consecutive
+  if (sm.status != kStatusOk) {
+    give_up();
+    return;
+  }
+  const int n = sm.seg_tile0[p.nseg];
+  // ---- first backward tile of every group
+  {
+    int til = 0, unused = 0;
+    if (tid < p.G)
+      til = (sm.seg_start[tid + 1 + gro[tid + 1]] - sm.seg_start[tid + gro[tid]] + kTile - 1) / kTile;
+    const int mine = til;
+    block_scan2(til, unused, sm.warp_sum);
+    if (tid < p.G) sm.btile0[tid] = til - mine;
+    if (tid == p.G - 1) sm.btile0[p.G] = til;
+  }
+  // ---- forward tiles
+  const bool by_rank = n <= kRankTiles;   // (there are at most as many backward tiles as forward
+                                          // tiles, and fewer groups)
+  // keys of tile (group) tid + nthr r: forward tiles, backward tiles, groups
+  uint32_t key[3][2] = {{~0u, ~0u}, {~0u, ~0u}, {~0u, ~0u}};
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int t = tid + nthr * r;
+    if (t < n) {
+      const int s = upper_segment(sm.seg_tile0, p.nseg, t), g = sm.seg_grp[s];
+      const int sp = g + gro[g], gs = sm.seg_start[sp];
+      const int ss = sm.seg_start[s], se = sm.seg_start[s + 1];
+      Tile tl;
+      tl.start = ss + (t - sm.seg_tile0[s]) * kTile;
+      tl.len = min(kTile, se - tl.start);
+      tl.kv0_start = gs;
+      if (s == sp) {
+        tl.kv0_len = tl.start - gs;
+        tl.kv1_start = tl.start;
+        tl.kv1_len = 0;
+        tl.vis_end = sm.seg_start[g + 1 + gro[g + 1]];
+      } else {
+        tl.kv0_len = gpl[g];
+        tl.kv1_start = ss;
+        tl.kv1_len = tl.start - ss;
+        tl.vis_end = se;
+      }
+      tl.work = (tl.kv0_len + kTile - 1) / kTile + (tl.kv1_len + kTile - 1) / kTile + 1;
+      p.tiles[t] = tl;
+      sm.tile[0][t] = tl.start;
+      sm.tile[1][t] = tl.start + tl.len;
+      sm.tile[2][t] = tl.vis_end;
+      key[0][r] = uint32_t(0xffff - tl.work) << 16 | uint32_t(t);
     }
-    pos = warp_sum(pos);
-    before = warp_sum(before);
-    ng = warp_sum(ng);
-    k_rel = warp_sum(k_rel);
+  }
+  for (int s = tid; s <= p.nseg; s += nthr) p.seg_start[s] = sm.seg_start[s];
+  __syncthreads();
+  const int nb = sm.btile0[p.G];
+  // ---- backward tiles; key_end (every key of a forward tile ends its visibility at vis_end)
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int t = tid + nthr * r;
+    if (t >= nb) break;
+    const int g = upper_segment(sm.btile0, p.G, t);
+    const int sp = g + gro[g], s_end = g + 1 + gro[g + 1];   // the group's segments [sp, s_end)
+    const int gs = sm.seg_start[sp], pe = sm.seg_start[sp + 1], ge = sm.seg_start[s_end];
+    const int k_rel = t - sm.btile0[g];
+    BTile b;
+    b.start = gs + k_rel * kTile;
+    b.len = min(kTile, ge - b.start);
+    b.grp_start = gs;
+    b.grp_end = ge;
+    // (key_end and query-tile readings: see plan_btile_body)
+    const int s_first = sp + upper_segment(sm.seg_start + sp, s_end - sp, b.start);
+    const int s_last = sp + upper_segment(sm.seg_start + sp, s_end - sp, b.start + b.len - 1);
+    b.vis_end = s_first == sp ? ge : sm.seg_start[s_last + 1];
+    b.work = 1 + (b.vis_end - (b.start + b.len) + kTile - 1) / kTile;
+    b.npc = (pe - gs + kTile - 1) / kTile;
+    b.dep_lo = b.start >= pe ? max(b.npc, (sm.seg_start[s_first] - gs) / kTile) : k_rel;
+    p.btiles[t] = b;
+    sm.wb[t] = uint16_t(b.work);
+    sm.bgrp[t] = uint16_t(g);
+    key[1][r] = uint32_t(0xffff - b.work) << 16 | uint32_t(t);
+  }
+  for (int t = wid; t < n; t += nthr >> 5) {
+    const int left = sm.tile[1][t] - sm.tile[0][t] - lane, vis_end = sm.tile[2][t];
+    int32_t* at = p.key_end + sm.tile[0][t] + lane;
+#pragma unroll
+    for (int c = 0; c < kTile; c += 32)
+      if (c < left) at[c] = vis_end;
+  }
+  __syncthreads();
+  // ---- work of every group (a warp each), groups in order of decreasing work
+  for (int g = wid; g < p.G; g += nthr >> 5) {
+    int w = 0;
+    for (int t = sm.btile0[g] + lane; t < sm.btile0[g + 1]; t += 32) w += sm.wb[t];
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) w += __shfl_xor_sync(0xffffffffu, w, d);
+    if (lane == 0) sm.gwork[g] = w;
+  }
+  __syncthreads();
+  // at most 2048 * 2049 / 2 < 2^22 units of work in a group, at most 1024 groups
+  if (tid < p.G) key[2][0] = uint32_t(0x3fffff - sm.gwork[tid]) << 10 | uint32_t(tid);
+  // super-groups (see above), inside one the longest tiles first; Hkv * nb / 600 < 512
+  auto unit_key = [&](int t, int ranked_before) {
+    const int sg = (p.Hkv * (nb - ranked_before) - 1) / kSuperGroupUnits;
+    return uint32_t(511 - sg) << 23 | uint32_t(4095 - sm.wb[t]) << 11 | uint32_t(t);
+  };
+  if (by_rank) {   // (blocks of 256 threads have at most 256 tiles: one per thread)
+    for (int t = tid; t < kRankTiles; t += nthr) {
+      sm.o.r.key[0][t] = t == tid ? key[0][0] : ~0u;
+      sm.o.r.key[1][t] = t == tid ? key[1][0] : ~0u;
+      sm.o.r.key[2][t] = t == tid ? key[2][0] : ~0u;
+      sm.o.r.key[3][t] = ~0u;
+      sm.o.r.rank[0][t] = sm.o.r.rank[1][t] = sm.o.r.rank[2][t] = sm.o.r.rank[3][t] = 0;
+    }
+    __syncthreads();
+    rank_count<false>(sm.o.r.key[0], n, sm.o.r.rank[0], nullptr);
+    rank_count<false>(sm.o.r.key[1], nb, sm.o.r.rank[1], nullptr);
+    rank_count<true>(sm.o.r.key[2], p.G, sm.o.r.rank[2], sm.btile0);
+    __syncthreads();
+    if (tid < n) p.fwd_order[sm.o.r.rank[0][tid]] = tid;
+    if (tid < nb) {
+      p.bwd_order[sm.o.r.rank[1][tid]] = tid;
+      sm.o.r.key[3][tid] = unit_key(tid, sm.o.r.rank[2][sm.bgrp[tid]]);
+    }
+    if (tid < p.G) sm.before[tid] = sm.o.r.rank[2][tid];
+    __syncthreads();
+    rank_count<false>(sm.o.r.key[3], nb, sm.o.r.rank[3], nullptr);
+    __syncthreads();
+    if (tid < nb) sm.unit_tile[sm.o.r.rank[3][tid]] = uint16_t(tid);
+    __syncthreads();
+  } else {
+    int n2 = 1024;
+    while (n2 < n) n2 <<= 1;
+    bitonic_sort<3>(key, n2, sm.o.sort);
+    // tiles of the groups ranked before each group
+    int cnt = 0, unused = 0, g = 0;
+    if (tid < p.G) {
+      g = int(key[2][0] & 1023u);
+      cnt = sm.btile0[g + 1] - sm.btile0[g];
+    }
+    const int mine = cnt;
+    block_scan2(cnt, unused, sm.warp_sum);
+    if (tid < p.G) sm.before[g] = cnt - mine;
+    __syncthreads();
+    uint32_t ukey[1][2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int t = tid + nthr * r;
+      if (t < n) p.fwd_order[t] = int32_t(key[0][r] & 0xffffu);
+      if (t < nb) p.bwd_order[t] = int32_t(key[1][r] & 0xffffu);
+      ukey[0][r] = t < nb ? unit_key(t, sm.before[sm.bgrp[t]]) : ~0u;
+    }
+    bitonic_sort<1>(ukey, n2, sm.o.sort);
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+      if (tid + nthr * r < nb) sm.unit_tile[tid + nthr * r] = uint16_t(ukey[0][r] & 2047u);
+    __syncthreads();
+  }
+  // ---- backward units, in both orders
+  for (int e = tid; e < nb * p.Hkv; e += nthr) {
+    const int i = e / p.Hkv, kvh = e - i * p.Hkv;
+    p.bwd_units[e] = (kvh << 24) | int(sm.unit_tile[i]);
     // deterministic backward: set after set (see plan_units_body)
+    const int g = sm.bgrp[i], ng = sm.btile0[g + 1] - sm.btile0[g], k_rel = i - sm.btile0[g];
     const int slot = ng <= p.det_asc_max ? k_rel : ng - 1 - k_rel;
-    for (int kvh = lane; kvh < p.Hkv; kvh += 32) {
-      p.bwd_units[p.Hkv * pos + kvh] = (kvh << 24) | t;
-      p.bwd_units_det[p.Hkv * before + kvh * ng + slot] = (kvh << 24) | t;
-    }
+    p.bwd_units_det[p.Hkv * sm.before[g] + kvh * ng + slot] = (kvh << 24) | i;
   }
+  if (tid < 16)   // (words from 4 on, except the backward tile count: dynamic-scheduling counters)
+    p.header[tid] = tid == kHdrNumTiles ? n
+                    : tid == kHdrNumSegments ? p.nseg : tid == kHdrNumBTiles ? nb : 0;
 }
 
 }  // namespace
@@ -557,7 +883,8 @@ bool profile_read(float* fwd_ms, float* bwd_ms) {
   return ok;
 }
 
-cudaError_t launch_plan(const pp_plan* plan, cudaStream_t stream, int* launches) {
+cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cudaStream_t stream,
+                        int* launches) {
   PlanPtrs p;
   char* ws = plan->ws;
   const PlanLayout& l = plan->lay;
@@ -581,12 +908,11 @@ cudaError_t launch_plan(const pp_plan* plan, cudaStream_t stream, int* launches)
   p.bwd_units_det = reinterpret_cast<int32_t*>(ws + l.bwd_units_det);
   p.Hkv = plan->prob.num_kv_heads;
   p.key_end = reinterpret_cast<int32_t*>(ws + l.key_end);
-  {
-    // a third of the SMs (the backward runs one CTA per SM), at most 48 tiles = 6144 tokens
-    static DeviceSetup setup[kMaxDevices];
-    DeviceSetup* dev = device_setup(setup);
-    p.det_asc_max = dev ? std::min(48, dev->num_sms / 3) : 0;
-  }
+  // a third of the SMs (the backward runs one CTA per SM), at most 48 tiles = 6144 tokens
+  static DeviceSetup setup[kMaxDevices];
+  DeviceSetup* dev = device_setup(setup);
+  if (!dev) return cudaErrorInvalidDevice;
+  p.det_asc_max = std::min(48, dev->num_sms / 3);
   p.num_rows = plan->prob.num_rows;
   p.G = plan->prob.num_groups;
   p.N = plan->prob.num_responses;
@@ -594,11 +920,54 @@ cudaError_t launch_plan(const pp_plan* plan, cudaStream_t stream, int* launches)
   p.nseg = plan->nseg;
   p.max_tiles = plan->max_tiles;
 
-  int mt = plan->max_tiles;
+  const int mt = plan->max_tiles;
+  // Host descriptors: up to kDescLarge entries travel as a kernel argument, which keeps the call
+  // asynchronous (a cudaMemcpyAsync from pageable host memory would first wait on the host for
+  // everything already in the stream); longer sets are copied into the workspace.
+  const size_t n_desc[4] = {size_t(p.num_rows) + 1, size_t(p.G), size_t(p.G) + 1, size_t(p.N)};
+  const size_t n_all = n_desc[0] + n_desc[1] + n_desc[2] + n_desc[3];
   if (mt <= kFusedMaxTiles && p.T <= (1 << 18)) {
-    plan_fused_kernel<<<1, 1024, 0, stream>>>(p);
+    // rows <= G <= N and G + N <= 2048: kDescFused entries always suffice
+    if (!dev->configured) {
+      cudaError_t e = cudaSuccess;
+      auto opt_in = [&](auto kern) {
+        if (e == cudaSuccess)
+          e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(FusedSmem));
+      };
+      opt_in(plan_fused_kernel<1>);
+      opt_in(plan_fused_kernel<kDescSmall>);
+      opt_in(plan_fused_kernel<kDescFused>);
+      if (e != cudaSuccess) return e;
+      dev->configured = true;
+    }
+    auto go = [&](auto n_c) {
+      constexpr size_t kN = decltype(n_c)::value;
+      DescBlock<kN> blk;
+      if (host_desc) fill_desc(host_desc, n_desc, blk.v);
+      plan_fused_kernel<kN><<<1, mt <= kFusedSmallTiles ? 256 : 1024, sizeof(FusedSmem), stream>>>(blk, p);
+    };
+    if (!host_desc) go(std::integral_constant<size_t, 1>{});
+    else if (n_all <= kDescSmall) go(std::integral_constant<size_t, kDescSmall>{});
+    else go(std::integral_constant<size_t, kDescFused>{});
     if (launches) *launches = 1;
     return cudaGetLastError();
+  }
+  int n_launch = 8;
+  if (host_desc) {
+    if (n_all <= kDescLarge) {
+      DescBlock<kDescLarge> blk;
+      fill_desc(host_desc, n_desc, blk.v);
+      stage_desc_kernel<kDescLarge><<<1, 256, 0, stream>>>(blk, int(n_all), p.desc_copy);
+      ++n_launch;
+    } else {
+      int32_t* at = p.desc_copy;
+      for (int i = 0; i < 4; ++i) {
+        cudaError_t e = cudaMemcpyAsync(at, host_desc[i], n_desc[i] * sizeof(int32_t),
+                                        cudaMemcpyHostToDevice, stream);
+        if (e != cudaSuccess) return e;
+        at += n_desc[i];
+      }
+    }
   }
   plan_scan_kernel<<<1, 1024, 0, stream>>>(p);
   plan_tiles_kernel<<<(mt + 255) / 256, 256, 0, stream>>>(p);
@@ -608,7 +977,7 @@ cudaError_t launch_plan(const pp_plan* plan, cudaStream_t stream, int* launches)
   plan_gwork_kernel<<<(mt + 127) / 128, 128, 0, stream>>>(p);
   plan_sgroup_kernel<<<(mt + 127) / 128, 128, 0, stream>>>(p);
   plan_units_kernel<<<(mt + 127) / 128, 128, 0, stream>>>(p);
-  if (launches) *launches = 8;
+  if (launches) *launches = n_launch;
   return cudaGetLastError();
 }
 

@@ -192,6 +192,34 @@ def test_device_side_validation_reports_status():
     assert (o == 3.0).all()
 
 
+@pytest.mark.parametrize("segs,length", [(127, 1), (128, 1), (256, 1), (257, 1), (129, 130), (512, 1), (513, 1),
+                                         (1024, 1), (1025, 1), (300, 300), (2040, 1)])
+def test_one_block_plan_at_the_edges_of_its_sorts_and_blocks(segs, length):
+    """Blocks of 256 and 1024 threads, orders by rank counting (up to 512 tiles) and by sorting:
+    the multi-kernel path's orders are reproduced exactly (longest first, ties by index)."""
+    from paper_2602_24082_b200 import binding as B
+    rng = np.random.default_rng(segs)
+    rows, left = [], segs
+    while left >= 2:
+        n = min(left - 1, int(rng.integers(1, 4)))
+        if left - 1 - n == 1:
+            n = min(n + 1, left - 1)
+        pick = lambda: int(rng.integers(1, 2 * length))
+        rows.append([(pick(), tuple(pick() for _ in range(n)))])
+        left -= 1 + n
+    w = W.Workload("edges", rows, 6, 3, 64, seed=1)
+    plan = B.plan_for(w)
+    assert plan.status() == (0, 0)
+    tiles, fwd_order, bwd_order, key_end = plan.read()
+    btiles = plan.read_bwd_tiles()
+    nb = len(btiles)
+    assert fwd_order.tolist() == sorted(range(len(tiles)), key=lambda t: (-tiles[t, 7], t))
+    assert bwd_order[:nb].tolist() == sorted(range(nb), key=lambda t: (-btiles[t, 6], t))
+    for (start, ln, _, _, _, _, vis_end, _) in tiles.tolist():
+        assert (key_end[start:start + ln] == vis_end).all()
+    test_backward_units_order(w)
+
+
 @pytest.mark.parametrize("groups", [40, 1100, 2500], ids=["small-block", "large-block", "copied"])
 def test_host_descriptors_reach_the_device_unchanged(groups):
     """Host descriptors travel as a kernel argument (two block sizes) or, beyond that, by
