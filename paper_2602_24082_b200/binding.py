@@ -95,7 +95,7 @@ def lib() -> ctypes.CDLL:
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _check(rc: int, where: str):
@@ -103,16 +103,42 @@ def _check(rc: int, where: str):
         raise PPError(rc, where)
 
 
+def _call(index: int, where: str, fn, *args):
+    """``fn(*args, current stream of device index)`` with that device current.  (On small problems
+    the time a call spends here is the time it takes: 14 us of Python around each of 8 us of plan,
+    4 us of forward and 12 us of backward, before the device guard was limited to calls that need
+    it, the stream came as a raw handle, and shapes and sizes were kept as plain integers.)"""
+    if torch.cuda.current_device() == index:
+        rc = fn(*args, torch._C._cuda_getCurrentRawStream(index))
+    else:
+        with torch.cuda.device(index):
+            rc = fn(*args, torch._C._cuda_getCurrentRawStream(index))
+    if rc != 0:
+        raise PPError(rc, where)
+
+
 class Plan:
     """Owns the host handle, the device workspace and the backward scratch of one problem."""
 
-    def __init__(self, handle: int, problem: _Problem, workspace: torch.Tensor, keep, sizes):
+    def __init__(self, handle: int, problem: _Problem, workspace: torch.Tensor, keep):
         self.handle = handle
         self.problem = problem
         self.workspace = workspace
         self._keep = keep
-        self.plan_bytes, self.fwd_scratch_bytes, self.bwd_scratch_bytes = sizes
+        self._sizes: Optional[Tuple[int, int, int]] = None
         self._bwd_scratch: Optional[torch.Tensor] = None
+        T, Hq, Hkv, D = (problem.total_tokens, problem.num_q_heads, problem.num_kv_heads,
+                         problem.head_dim)
+        self.q_shape, self.kv_shape, self.lse_shape = (T, Hq, D), (T, Hkv, D), (Hq, T)
+
+    def _size(self, i: int) -> int:
+        if self._sizes is None:
+            self._sizes = pp_plan_workspace_bytes(self.problem)
+        return self._sizes[i]
+
+    plan_bytes = property(lambda self: self._size(0))
+    fwd_scratch_bytes = property(lambda self: self._size(1))
+    bwd_scratch_bytes = property(lambda self: self._size(2))
 
     @property
     def total_tokens(self) -> int:
@@ -173,19 +199,12 @@ def make_problem(desc: Sequence[np.ndarray], num_q_heads: int, num_kv_heads: int
                  total_tokens: int, device_arrays: Optional[Sequence[torch.Tensor]] = None):
     """Fills a pp_problem.  ``desc`` = (row_group_off, grp_prompt_len, grp_resp_off, resp_len)."""
     arrs = [np.ascontiguousarray(a, dtype=np.int32) for a in desc]
-    p = _Problem()
-    p.num_rows = len(arrs[0]) - 1
-    p.num_groups = len(arrs[1])
-    p.num_responses = len(arrs[3])
     if device_arrays is not None:
         ptrs = [t.data_ptr() for t in device_arrays]
-        p.desc_on_device = 1
     else:
-        ptrs = [a.ctypes.data for a in arrs]
-        p.desc_on_device = 0
-    p.row_group_off, p.grp_prompt_len, p.grp_resp_off, p.resp_len = ptrs
-    p.num_q_heads, p.num_kv_heads, p.head_dim = num_q_heads, num_kv_heads, head_dim
-    p.total_tokens = total_tokens
+        ptrs = [a.__array_interface__["data"][0] for a in arrs]
+    p = _Problem(len(arrs[0]) - 1, *ptrs, len(arrs[1]), len(arrs[3]), int(device_arrays is not None),
+                 num_q_heads, num_kv_heads, head_dim, total_tokens)
     return p, (arrs, device_arrays)
 
 
@@ -208,19 +227,27 @@ def pp_build_plan(desc: Sequence[np.ndarray], num_q_heads: int, num_kv_heads: in
     if desc_on_device and dev_arrays is None:
         dev_arrays = [torch.from_numpy(np.ascontiguousarray(a, dtype=np.int32)).to(device) for a in desc]
     problem, keep = make_problem(desc, num_q_heads, num_kv_heads, head_dim, total_tokens, dev_arrays)
-    sizes = pp_plan_workspace_bytes(problem)
-    ws = workspace if workspace is not None else torch.empty(sizes[0], dtype=torch.uint8, device=device)
-    if ws.numel() < sizes[0]:
-        raise ValueError("workspace too small")
+    if workspace is None:
+        workspace = torch.empty(pp_plan_workspace_bytes(problem)[0], dtype=torch.uint8, device=device)
+    elif not workspace.is_cuda:
+        raise ValueError("workspace: expected a CUDA tensor")
     handle = ctypes.c_void_p(0)
-    with torch.cuda.device(ws.device):
-        _check(lib().pp_build_plan(ctypes.byref(problem), ws.data_ptr(), sizes[0], _stream(),
-                                   ctypes.byref(handle)), "pp_build_plan")
-    return Plan(handle.value, problem, ws, keep, sizes)
+    try:
+        _call(workspace.get_device(), "pp_build_plan", _build_plan, problem, workspace.data_ptr(),
+              workspace.numel(), handle)
+    except PPError as e:
+        if e.code == -3:
+            raise ValueError("workspace too small") from None
+        raise
+    return Plan(handle.value, problem, workspace, keep)
+
+
+def _build_plan(problem, ws_ptr, ws_bytes, handle, stream):
+    return lib().pp_build_plan(ctypes.byref(problem), ws_ptr, ws_bytes, stream, ctypes.byref(handle))
 
 
 def _chk(t: torch.Tensor, shape, dtype, name):
-    if t.dtype != dtype or tuple(t.shape) != tuple(shape) or not t.is_contiguous() or not t.is_cuda:
+    if t.dtype is not dtype or t.shape != shape or not t.is_contiguous() or not t.is_cuda:
         raise ValueError(f"{name}: expected contiguous CUDA {dtype} {tuple(shape)}, got "
                          f"{t.dtype} {tuple(t.shape)} on {t.device}")
 
@@ -230,49 +257,47 @@ def pp_attn_fwd(plan: Plan, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor,
                 lse: Optional[torch.Tensor] = None, for_backward: bool = False):
     """``for_backward``: also hand the plan's backward scratch to the forward, which then clears
     the fp32 dQ accumulator in it (the following ``pp_attn_bwd`` skips its own clearing)."""
-    p = plan.problem
-    T, Hq, Hkv, D = p.total_tokens, p.num_q_heads, p.num_kv_heads, p.head_dim
-    _chk(q, (T, Hq, D), torch.bfloat16, "q")
-    _chk(k, (T, Hkv, D), torch.bfloat16, "k")
-    _chk(v, (T, Hkv, D), torch.bfloat16, "v")
+    bf16 = torch.bfloat16
+    _chk(q, plan.q_shape, bf16, "q")
+    _chk(k, plan.kv_shape, bf16, "k")
+    _chk(v, plan.kv_shape, bf16, "v")
     if o is None:
         o = torch.empty_like(q)
+    else:
+        _chk(o, plan.q_shape, bf16, "o")
     if lse is None:
-        lse = torch.empty(Hq, T, dtype=torch.float32, device=q.device)
-    _chk(o, (T, Hq, D), torch.bfloat16, "o")
-    _chk(lse, (Hq, T), torch.float32, "lse")
+        lse = q.new_empty(plan.lse_shape, dtype=torch.float32)
+    else:
+        _chk(lse, plan.lse_shape, torch.float32, "lse")
     sc_ptr, sc_bytes = None, 0
     if for_backward:
         sc = plan.bwd_scratch()
         sc_ptr, sc_bytes = sc.data_ptr(), sc.numel()
-    with torch.cuda.device(q.device):
-        _check(lib().pp_attn_fwd(plan.handle, q.data_ptr(), k.data_ptr(), v.data_ptr(),
-                                 float(softmax_scale), o.data_ptr(), lse.data_ptr(), sc_ptr, sc_bytes,
-                                 _stream()), "pp_attn_fwd")
+    _call(q.get_device(), "pp_attn_fwd", lib().pp_attn_fwd, plan.handle, q.data_ptr(), k.data_ptr(),
+          v.data_ptr(), float(softmax_scale), o.data_ptr(), lse.data_ptr(), sc_ptr, sc_bytes)
     return o, lse
 
 
 def pp_attn_bwd(plan: Plan, q, k, v, o, lse, d_o, softmax_scale: float, d_q=None, d_k=None, d_v=None,
                 deterministic: bool = False):
     """``deterministic``: pp_attn_bwd_deterministic (bit-reproducible dQ; key tiles take turns)."""
-    p = plan.problem
-    T, Hq, Hkv, D = p.total_tokens, p.num_q_heads, p.num_kv_heads, p.head_dim
-    _chk(q, (T, Hq, D), torch.bfloat16, "q")
-    _chk(k, (T, Hkv, D), torch.bfloat16, "k")
-    _chk(v, (T, Hkv, D), torch.bfloat16, "v")
-    _chk(o, (T, Hq, D), torch.bfloat16, "o")
-    _chk(d_o, (T, Hq, D), torch.bfloat16, "d_o")
-    _chk(lse, (Hq, T), torch.float32, "lse")
+    bf16 = torch.bfloat16
+    q_shape, kv_shape = plan.q_shape, plan.kv_shape
+    _chk(q, q_shape, bf16, "q")
+    _chk(k, kv_shape, bf16, "k")
+    _chk(v, kv_shape, bf16, "v")
+    _chk(o, q_shape, bf16, "o")
+    _chk(d_o, q_shape, bf16, "d_o")
+    _chk(lse, plan.lse_shape, torch.float32, "lse")
     d_q = torch.empty_like(q) if d_q is None else d_q
     d_k = torch.empty_like(k) if d_k is None else d_k
     d_v = torch.empty_like(v) if d_v is None else d_v
     scratch = plan.bwd_scratch()
-    fn = lib().pp_attn_bwd_deterministic if deterministic else lib().pp_attn_bwd
-    with torch.cuda.device(q.device):
-        _check(fn(plan.handle, q.data_ptr(), k.data_ptr(), v.data_ptr(),
-                  o.data_ptr(), lse.data_ptr(), d_o.data_ptr(), float(softmax_scale),
-                  d_q.data_ptr(), d_k.data_ptr(), d_v.data_ptr(), scratch.data_ptr(),
-                  scratch.numel(), _stream()), "pp_attn_bwd")
+    L = lib()
+    _call(q.get_device(), "pp_attn_bwd", L.pp_attn_bwd_deterministic if deterministic else L.pp_attn_bwd,
+          plan.handle, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(),
+          d_o.data_ptr(), float(softmax_scale), d_q.data_ptr(), d_k.data_ptr(), d_v.data_ptr(),
+          scratch.data_ptr(), scratch.numel())
     return d_q, d_k, d_v
 
 
@@ -281,19 +306,16 @@ def pp_position_ids(plan: Plan, out: Optional[torch.Tensor] = None) -> torch.Ten
     if out is None:
         out = torch.empty(plan.total_tokens, dtype=torch.int32, device=plan.workspace.device)
     _chk(out, (plan.total_tokens,), torch.int32, "position_ids")
-    with torch.cuda.device(out.device):
-        _check(lib().pp_position_ids(plan.handle, out.data_ptr(), _stream()), "pp_position_ids")
+    _call(out.get_device(), "pp_position_ids", lib().pp_position_ids, plan.handle, out.data_ptr())
     return out
 
 
 def pp_rope_qk(plan: Plan, q: torch.Tensor, k: torch.Tensor, rope_base: float = 10000.0):
     """Rotary embedding with the packed positions, in place on q [T,Hq,D] and k [T,Hkv,D]."""
-    p = plan.problem
-    _chk(q, (p.total_tokens, p.num_q_heads, p.head_dim), torch.bfloat16, "q")
-    _chk(k, (p.total_tokens, p.num_kv_heads, p.head_dim), torch.bfloat16, "k")
-    with torch.cuda.device(q.device):
-        _check(lib().pp_rope_qk(plan.handle, q.data_ptr(), k.data_ptr(), float(rope_base), _stream()),
-               "pp_rope_qk")
+    _chk(q, plan.q_shape, torch.bfloat16, "q")
+    _chk(k, plan.kv_shape, torch.bfloat16, "k")
+    _call(q.get_device(), "pp_rope_qk", lib().pp_rope_qk, plan.handle, q.data_ptr(), k.data_ptr(),
+          float(rope_base))
     return q, k
 
 
@@ -310,12 +332,10 @@ def pp_preference_loss(plan: Plan, token_logp: torch.Tensor, ref_token_logp: Opt
     resp_reward = torch.empty(N, dtype=torch.float32, device=dev)
     grp_loss = torch.empty(G, dtype=torch.float32, device=dev)
     grad = torch.empty(T, dtype=torch.float32, device=dev) if want_grad else None
-    with torch.cuda.device(dev):
-        _check(lib().pp_preference_loss(plan.handle, token_logp.data_ptr(),
-                                        ref_token_logp.data_ptr() if ref_token_logp is not None else None,
-                                        float(beta), resp_logp.data_ptr(), resp_reward.data_ptr(),
-                                        grp_loss.data_ptr(), grad.data_ptr() if want_grad else None,
-                                        _stream()), "pp_preference_loss")
+    _call(token_logp.get_device(), "pp_preference_loss", lib().pp_preference_loss, plan.handle,
+          token_logp.data_ptr(), ref_token_logp.data_ptr() if ref_token_logp is not None else None,
+          float(beta), resp_logp.data_ptr(), resp_reward.data_ptr(), grp_loss.data_ptr(),
+          grad.data_ptr() if want_grad else None)
     return resp_logp, resp_reward, grp_loss, grad
 
 
@@ -330,18 +350,15 @@ def pp_attn_bwd_noalloc(plan: Plan, q, k, v, o, lse, d_o, softmax_scale: float, 
     library (32 MiB per GPU), so the outputs have to be passed in and nothing is allocated
     here either.  Problems whose scratch exceeds pp_attn_bwd_noalloc_max_bytes() raise
     PPError(-7).  Calls on one stream may follow each other; overlapping calls race."""
-    p = plan.problem
-    T, Hq, Hkv, D = p.total_tokens, p.num_q_heads, p.num_kv_heads, p.head_dim
-    for t, shape, name in ((q, (T, Hq, D), "q"), (k, (T, Hkv, D), "k"), (v, (T, Hkv, D), "v"),
-                           (o, (T, Hq, D), "o"), (d_o, (T, Hq, D), "d_o"), (d_q, (T, Hq, D), "d_q"),
-                           (d_k, (T, Hkv, D), "d_k"), (d_v, (T, Hkv, D), "d_v")):
+    q_shape, kv_shape = plan.q_shape, plan.kv_shape
+    for t, shape, name in ((q, q_shape, "q"), (k, kv_shape, "k"), (v, kv_shape, "v"), (o, q_shape, "o"),
+                           (d_o, q_shape, "d_o"), (d_q, q_shape, "d_q"), (d_k, kv_shape, "d_k"),
+                           (d_v, kv_shape, "d_v")):
         _chk(t, shape, torch.bfloat16, name)
-    _chk(lse, (Hq, T), torch.float32, "lse")
-    with torch.cuda.device(q.device):
-        _check(lib().pp_attn_bwd_noalloc(plan.handle, q.data_ptr(), k.data_ptr(), v.data_ptr(),
-                                         o.data_ptr(), lse.data_ptr(), d_o.data_ptr(),
-                                         float(softmax_scale), d_q.data_ptr(), d_k.data_ptr(),
-                                         d_v.data_ptr(), _stream()), "pp_attn_bwd_noalloc")
+    _chk(lse, plan.lse_shape, torch.float32, "lse")
+    _call(q.get_device(), "pp_attn_bwd_noalloc", lib().pp_attn_bwd_noalloc, plan.handle, q.data_ptr(),
+          k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(), d_o.data_ptr(),
+          float(softmax_scale), d_q.data_ptr(), d_k.data_ptr(), d_v.data_ptr())
     return d_q, d_k, d_v
 
 
@@ -388,13 +405,10 @@ class HostStep:
         for t in (q, k, v, d_o):
             if t.is_cuda or not t.is_contiguous() or t.dtype != torch.bfloat16:
                 raise ValueError("pp_attn_step_host takes contiguous CPU bf16 tensors")
-        with torch.cuda.device(self.arena.device):
-            _check(lib().pp_attn_step_host(ctypes.byref(self.problem), q.data_ptr(), k.data_ptr(),
-                                           v.data_ptr(), d_o.data_ptr(), float(self.scale),
-                                           self.o.data_ptr(), self.lse.data_ptr(), self.dq.data_ptr(),
-                                           self.dk.data_ptr(), self.dv.data_ptr(),
-                                           self.arena.data_ptr(), self.arena.numel(), _stream()),
-                   "pp_attn_step_host")
+        _call(self.arena.get_device(), "pp_attn_step_host", lib().pp_attn_step_host,
+              ctypes.byref(self.problem), q.data_ptr(), k.data_ptr(), v.data_ptr(), d_o.data_ptr(),
+              float(self.scale), self.o.data_ptr(), self.lse.data_ptr(), self.dq.data_ptr(),
+              self.dk.data_ptr(), self.dv.data_ptr(), self.arena.data_ptr(), self.arena.numel())
         return self.o, self.lse, self.dq, self.dk, self.dv
 
 
@@ -458,12 +472,10 @@ def pp_build_rows(grp_prompt_len: torch.Tensor, grp_resp_off: torch.Tensor, resp
     status, nrows = meta[:2], meta[2:]
     rtok, rcost = i64(G), i64(G)
     oP, ooff, orl = i32(G), i32(G + 1), i32(N)
-    with torch.cuda.device(dev):
-        _check(lib().pp_build_rows(G, N, grp_prompt_len.data_ptr(), grp_resp_off.data_ptr(),
-                                   resp_len.data_ptr(), int(row_capacity), ws.data_ptr(), ws.numel(),
-                                   order.data_ptr(), rgo.data_ptr(), nrows.data_ptr(), rtok.data_ptr(),
-                                   rcost.data_ptr(), oP.data_ptr(), ooff.data_ptr(), orl.data_ptr(),
-                                   status.data_ptr(), _stream()), "pp_build_rows")
+    _call(order.get_device(), "pp_build_rows", lib().pp_build_rows, G, N, grp_prompt_len.data_ptr(),
+          grp_resp_off.data_ptr(), resp_len.data_ptr(), int(row_capacity), ws.data_ptr(), ws.numel(),
+          order.data_ptr(), rgo.data_ptr(), nrows.data_ptr(), rtok.data_ptr(), rcost.data_ptr(),
+          oP.data_ptr(), ooff.data_ptr(), orl.data_ptr(), status.data_ptr())
     code, detail, r = meta.tolist()   # one synchronising copy
     return {"order": order, "row_group_off": rgo[:r + 1], "row_tokens": rtok[:r], "row_cost": rcost[:r],
             "grp_prompt_len": oP, "grp_resp_off": ooff, "resp_len": orl, "status": (code, detail)}
@@ -478,10 +490,8 @@ def pp_assign_rows(row_cost: torch.Tensor, num_ranks: int):
     order = torch.empty(R, dtype=torch.int32, device=dev)
     rank_of_row = torch.empty(R, dtype=torch.int32, device=dev)
     rank_cost = torch.empty(int(num_ranks), dtype=torch.int64, device=dev)
-    with torch.cuda.device(dev):
-        _check(lib().pp_assign_rows(R, row_cost.data_ptr(), int(num_ranks), order.data_ptr(),
-                                    rank_of_row.data_ptr(), rank_cost.data_ptr(), _stream()),
-               "pp_assign_rows")
+    _call(order.get_device(), "pp_assign_rows", lib().pp_assign_rows, R, row_cost.data_ptr(),
+          int(num_ranks), order.data_ptr(), rank_of_row.data_ptr(), rank_cost.data_ptr())
     return order, rank_of_row, rank_cost
 
 
