@@ -30,7 +30,7 @@ struct BwdParams {
   const float* delta;  // [Hq][T]
   const float* lse2;   // [Hq][T]  LSE * log2(e)
   float* dq_acc;       // [T][Hq][D] fp32
-  int32_t* dq_sem;     // deterministic variant: turn counters [backward tile][Hq]; else null
+  int32_t* dq_sem;     // deterministic variant: turn counters [backward tile][Hq][4 row quarters]; else null
   __nv_bfloat16* dk;
   __nv_bfloat16* dv;
   int T, Hq, Hkv;
@@ -120,23 +120,37 @@ bwd_finalize_kernel(const float4* __restrict__ acc, uint2* __restrict__ dq, size
 }
 
 // ---------------------------------------------------------------- main
-// Persistent, warp-specialised CTA (one per SM), 448 threads:
+// Persistent, warp-specialised CTA (one per SM), 512 threads in four warpgroups:
 //   warp 0       producer: K, V once per unit; per query tile Q and dO by TMA (two-stage rings)
 //                and the tile's LSE*log2(e) / Delta into shared memory
-//   warp 1       MMA issuer (one thread)
-//   warps 2-5    compute warpgroup 0: thread = key row, query columns 0..63 of the tile
-//   warps 6-9    compute warpgroup 1: query columns 64..127
-//   warps 10-13  dQ warpgroup: thread = query row; moves each dQ tile from tensor memory
-//                through a swizzled shared-memory staging buffer into the fp32 accumulator
-//                with TMA reduce-add (whole 128-byte lines per row instead of per-thread
-//                16-byte reductions, which saturate the L2 atomic units)
+//   warp 1       MMA issuer (one thread); warps 2, 3 idle
+//   warps 4-7    compute warpgroup 0: thread = key row, query columns 0..63 of the tile
+//   warps 8-11   compute warpgroup 1: query columns 64..127
+//   warps 12-15  dQ warpgroup: thread = query row; takes each dQ tile out of tensor memory as a
+//                whole and adds it to the fp32 accumulator, every warp its own 32 rows through its
+//                own two swizzled staging boxes with TMA reduce-adds (whole 128-byte lines per
+//                row instead of per-thread 16-byte reductions, which saturate the L2 atomic units)
+// What bounds it (two rows of 32768 tokens, Hq / Hkv 32 / 8, D 128; cycles per query tile and
+// head): 2560 of MMAs; 3100 - 3400 with every load and reduction taken out, the MMA thread's own
+// waits; 3850 as it is, because an iteration moves 64 KB of Q and dO and 64 KB of reductions
+// between the SM and L2.  Before, at 4070, the thread waited for two chains on top: dQ drained in
+// two halves with the staging of the first in between (1015 cycles to 200 now that 152 registers
+// hold the tile), and dS (1350 to 1000: P kept in fp32 registers instead of unpacked from bf16, no
+// selects on full tiles, the next columns loaded under the arithmetic of these).  The kernel went
+// from 26.9 to 25.8 M cycles there, 2.64 to 2.49 on four 4800-token groups (28 / 4 heads), 2.13 to
+// 2.01 on sixteen thousand tokens (64 / 8 heads), 757 to 726 thousand at D 64.
 // Tensor-memory map (columns): [0,128) S^T, overwritten by P^T (bf16: columns [0,32) and
 // [64,96), each warpgroup inside the columns it has read itself); [128,256) dP^T, then the
 // dQ tile; [256,256+D) dV; [384,384+D) dK.
 // MMA order per query tile i:  dP(i)  dV(i)  S(i+1)  dQ(i)  dK(i).  The exponentials of tile
 // i+1 run under dQ(i), dK(i), dP(i+1); dS(i) is computed under dV(i), S(i+1); the dQ tile is
 // drained under dK(i), so the dP/dQ columns are free again when dP(i+1) is issued.
-constexpr int kBwdThreads = 448;
+constexpr int kBwdThreads = 512;
+// Registers per thread behind the split: warpgroup 0 (producer, MMA issuer), 1 and 2 (compute), 3
+// (dQ).  They have to add up to what the launch allocates.
+constexpr int kBwdRegsLaunch = 65536 / kBwdThreads;  // 128
+constexpr int kBwdRegsIssue = 104, kBwdRegsCompute = 128, kBwdRegsDq = 152;
+static_assert(kBwdRegsIssue + 2 * kBwdRegsCompute + kBwdRegsDq == 4 * kBwdRegsLaunch, "register split");
 constexpr uint32_t kBwdTmemCols = 512;
 
 enum BwdBar : int {
@@ -147,13 +161,13 @@ enum BwdBar : int {
   kDoFull = 6,   // dO is single-buffered: free after dV(i), needed again at dP(i+1)
   kDoEmpty = 8,
   kSFullB = 10,
-  kPReady,       // 256
+  kPReady,       // 8: one arrival per compute warp
   kDpFull,
-  kDsReady,      // 256
+  kDsReady,      // 8
   kDqFull,
-  kDqDrained,    // 128
+  kDqDrained,    // 4: one arrival per dQ warp
   kDkvFull,
-  kDkvFree,      // 256
+  kDkvFree,      // 8
   kSchedFull,    // [2]  unit ids handed from the producer warp to the other roles
   kSchedEmpty = kSchedFull + 2,  // [2]  13 arrivals: MMA thread + 8 compute warps + 4 dQ warps
   kNumBwdBars = kSchedEmpty + 2
@@ -162,9 +176,9 @@ enum BwdBar : int {
 template <int D>
 struct BwdSmem {
   static constexpr int kTileBytes = 128 * D * 2;
-  static constexpr int kStageBytes = 128 * 128;  // one {32 floats x 128 rows} box of a dQ tile
+  static constexpr int kStageBytes = 32 * 128;  // one {32 floats x 32 rows} box of a dQ tile; two per dQ warp
   static constexpr int kK = 0, kV = kTileBytes, kQ = 2 * kTileBytes, kdO = 4 * kTileBytes,
-                       kStg = 5 * kTileBytes, kdS = kStg + 2 * kStageBytes,
+                       kStg = 5 * kTileBytes, kdS = kStg + 8 * kStageBytes,
                        kStats = kdS + 128 * 128 * 2, kBars = kStats + 2 * 256 * 4;
   static constexpr int kUsed = kBars + 8 * kNumBwdBars + 32;
   // The declared 1024-byte alignment of the dynamic shared memory leaves no slack to spend at
@@ -263,8 +277,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     for (int i = 0; i < kNumBwdBars; ++i) {
       uint32_t cnt = 1;
       if (i == kQFullB || i == kQFullB + 1) cnt = 33;
-      if (i == kPReady || i == kDsReady || i == kDkvFree) cnt = 256;
-      if (i == kDqDrained) cnt = 128;
+      if (i == kPReady || i == kDsReady || i == kDkvFree) cnt = 8;
+      if (i == kDqDrained) cnt = 4;
       if (i == kSchedEmpty || i == kSchedEmpty + 1) cnt = 13;
       mbar_init(bar(i), cnt);
     }
@@ -311,7 +325,9 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     return u;
   };
 
-  if (warp == 0) {
+  if (warp < 4) {
+    set_max_registers<kBwdRegsIssue, kBwdRegsLaunch>();
+    if (warp == 0) {
     // ------------------------------------------------------------ producer
     uint32_t qc = 0, ucnt = 0;
     BwdUnit un;
@@ -361,7 +377,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         }
       }
     }
-  } else if (warp == 1) {
+    } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
     // (elect.sync, not `lane == 0`: see the forward's issuer.  Here two rows of 32768 tokens went
     // from 32.8 to 26.9 M cycles and from 21.2 to 19.4 ms -- the clock settles lower under the
@@ -484,12 +500,16 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         gc += un.n_it;
       }
     }
-  } else if (warp < 10) {
+    }
+  } else if (warp < 12) {
     // ------------------------------------------------------------ compute warpgroups
-    const int wg = (warp - 2) >> 2;       // column half
+    set_max_registers<kBwdRegsCompute, kBwdRegsLaunch>();
+    const int wg = (warp - 4) >> 2;       // column half
     const int row = 32 * (warp & 3) + lane;
     const uint32_t lane_base = tmem + (uint32_t(32 * (warp & 3)) << 16);
     const int cb = 64 * wg;
+    const uint64_t sc2 = pack2(prm.scale_log2, prm.scale_log2);
+    const uint32_t ds_row = sdS + wg * kBoxBytes + row * 128;   // dS^T row `row` in box wg
     uint32_t gc = 0, ucnt = 0;
     BwdUnit un;
     for (; get_bwd_unit(prm, take_unit(ucnt, true), ntiles_total, un); ++ucnt) {
@@ -514,84 +534,106 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         wait_bar(bar(kQFullB + st), (g >> 1) & 1, abort_flag, prm.header, 70);
         wait_bar(bar(kSFullB), par, abort_flag, prm.header, 71);
         tc_fence_after();
-        uint32_t v[64];
-        tmem_ld32(lane_base + tS + cb, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
-        tmem_ld32(lane_base + tS + cb + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
-        tmem_wait_ld();
-        uint32_t pk[32];
+        // P stays in fp32 registers for dS; its bf16 form goes to tensor memory
+        float p[64];
         const float4* sl4 = reinterpret_cast<const float4*>(sl);
-        const uint64_t sc2 = pack2(prm.scale_log2, prm.scale_log2);
-        if (full) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const float4 l = sl4[i];   // -LSE * log2(e)
-            float x0, x1, x2, x3;
-            unpack2(fma2(pack2(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1])), sc2,
-                         pack2(l.x, l.y)), x0, x1);
-            unpack2(fma2(pack2(__uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3])), sc2,
-                         pack2(l.z, l.w)), x2, x3);
-            pk[2 * i] = pack_bf16(ex2(x0), ex2(x1));
-            pk[2 * i + 1] = pack_bf16(ex2(x2), ex2(x3));
-          }
-          if (!row_all) {
+        for (int hf = 0; hf < 2; ++hf) {
+          uint32_t v[32], pk[16];
+          tmem_ld32(lane_base + tS + cb + 32 * hf, v);
+          tmem_wait_ld();
+          float* ph = p + 32 * hf;
+          if (full) {
 #pragma unroll
-            for (int i = 0; i < 32; ++i) pk[i] = 0u;
-          }
-        } else {
-          // query column c is visible iff key_lo <= qt.start + c < key_hi (an absent key row
-          // has an empty range; key_hi never exceeds the group's end, so c < qt.len follows)
+            for (int i = 0; i < 8; ++i) {
+              const float4 l = sl4[8 * hf + i];   // -LSE * log2(e)
+              float x0, x1, x2, x3;
+              unpack2(fma2(pack2(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1])), sc2,
+                           pack2(l.x, l.y)), x0, x1);
+              unpack2(fma2(pack2(__uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3])), sc2,
+                           pack2(l.z, l.w)), x2, x3);
+              ph[4 * i] = ex2(x0);
+              ph[4 * i + 1] = ex2(x1);
+              ph[4 * i + 2] = ex2(x2);
+              ph[4 * i + 3] = ex2(x3);
+            }
+            if (!row_all) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const int c0 = cb + 2 * i;
-            float p0 = ex2(fmaf(__uint_as_float(v[2 * i]), prm.scale_log2, sl[2 * i]));
-            float p1 = ex2(fmaf(__uint_as_float(v[2 * i + 1]), prm.scale_log2, sl[2 * i + 1]));
-            p0 = (c0 >= lo && c0 < hi) ? p0 : 0.f;
-            p1 = (c0 + 1 >= lo && c0 + 1 < hi) ? p1 : 0.f;
-            pk[i] = pack_bf16(p0, p1);
+              for (int i = 0; i < 32; ++i) ph[i] = 0.f;
+            }
+          } else {
+            // query column c is visible iff key_lo <= qt.start + c < key_hi (an absent key row
+            // has an empty range; key_hi never exceeds the group's end, so c < qt.len follows)
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+              const int c = cb + 32 * hf + i;
+              const float e = ex2(fmaf(__uint_as_float(v[i]), prm.scale_log2, sl[32 * hf + i]));
+              ph[i] = (c >= lo && c < hi) ? e : 0.f;
+            }
           }
+#pragma unroll
+          for (int i = 0; i < 16; ++i) pk[i] = pack_bf16(ph[2 * i], ph[2 * i + 1]);
+          tmem_st16(lane_base + tS + cb + 16 * hf, pk);
         }
-        tmem_st32(lane_base + tS + cb, pk);
         tmem_wait_st();
         tc_fence_before();
-        mbar_arrive(bar(kPReady));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(kPReady));
 
         wait_bar(bar(kDpFull), par, abort_flag, prm.header, 72);
         tc_fence_after();
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          uint32_t d[32];
-          tmem_ld32(lane_base + tdP + cb + 32 * half, d);
-          tmem_wait_ld();
-          uint32_t ds[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const uint32_t pp = pk[16 * half + i];
-            const float p0 = __uint_as_float(pp << 16), p1 = __uint_as_float(pp & 0xffff0000u);
-            const float2 dl = reinterpret_cast<const float2*>(sl + 128 + 32 * half)[i];   // -Delta
-            float d0, d1;
-            unpack2(fma2(pack2(p0, p1),
-                         add2(pack2(__uint_as_float(d[2 * i]), __uint_as_float(d[2 * i + 1])),
-                              pack2(dl.x, dl.y)),
-                         pack2(0.f, 0.f)),
-                    d0, d1);
-            if (!full) {  // stale tensor-memory columns may hold anything
-              d0 = (pp & 0xffffu) ? d0 : 0.f;
-              d1 = (pp & 0xffff0000u) ? d1 : 0.f;
-            }
-            ds[i] = pack_bf16(d0, d1);
-          }
-          // dS^T row `row`, columns [cb + 32 half, +32): box wg, 16-byte chunks 4 half .. +3
-          const uint32_t row_addr = sdS + wg * kBoxBytes + row * 128;
+        // dS = P (dP - Delta), in pieces of 16 columns: the load of the next one in flight under
+        // the arithmetic of this one
+        auto ds16 = [&](const uint32_t (&d)[16], int piece, auto masked_c) {
+          uint32_t ds[8];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const uint32_t chunk = uint32_t(half * 4 + i) ^ uint32_t(row & 7);
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row_addr + chunk * 16),
+            const float4 dl = sl4[32 + 4 * piece + i];   // -Delta
+            const float* pp = p + 16 * piece + 4 * i;
+            float d0, d1, d2, d3;
+            unpack2(mul2(pack2(pp[0], pp[1]),
+                         add2(pack2(__uint_as_float(d[4 * i]), __uint_as_float(d[4 * i + 1])),
+                              pack2(dl.x, dl.y))), d0, d1);
+            unpack2(mul2(pack2(pp[2], pp[3]),
+                         add2(pack2(__uint_as_float(d[4 * i + 2]), __uint_as_float(d[4 * i + 3])),
+                              pack2(dl.z, dl.w))), d2, d3);
+            if (decltype(masked_c)::value) {  // stale tensor-memory columns may hold anything
+              d0 = pp[0] != 0.f ? d0 : 0.f;
+              d1 = pp[1] != 0.f ? d1 : 0.f;
+              d2 = pp[2] != 0.f ? d2 : 0.f;
+              d3 = pp[3] != 0.f ? d3 : 0.f;
+            }
+            ds[2 * i] = pack_bf16(d0, d1);
+            ds[2 * i + 1] = pack_bf16(d2, d3);
+          }
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const uint32_t chunk = uint32_t(piece * 2 + i) ^ uint32_t(row & 7);
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ds_row + chunk * 16),
                          "r"(ds[4 * i]), "r"(ds[4 * i + 1]), "r"(ds[4 * i + 2]), "r"(ds[4 * i + 3])
                          : "memory");
           }
-        }
+        };
+        auto ds_all = [&](auto masked_c) {
+          const uint32_t t = lane_base + tdP + cb;
+          uint32_t da[16], db[16];
+          tmem_ld16(t, da);
+          tmem_wait_ld();
+          tmem_ld16(t + 16, db);
+          ds16(da, 0, masked_c);
+          tmem_wait_ld();
+          tmem_ld16(t + 32, da);
+          ds16(db, 1, masked_c);
+          tmem_wait_ld();
+          tmem_ld16(t + 48, db);
+          ds16(da, 2, masked_c);
+          tmem_wait_ld();
+          ds16(db, 3, masked_c);
+        };
+        if (full) ds_all(std::false_type{}); else ds_all(std::true_type{});
         fence_proxy_async_smem();
-        mbar_arrive(bar(kDsReady));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(kDsReady));
       }
       gc += un.n_it;
       // ---- unit epilogue: warpgroup 0 stores dV, warpgroup 1 stores scale * dK
@@ -615,7 +657,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
           ob[c * 16 + i] = pack_bf16(__uint_as_float(w[2 * i]) * f, __uint_as_float(w[2 * i + 1]) * f);
       }
       tc_fence_before();
-      mbar_arrive(bar(kDkvFree));
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(kDkvFree));
       // A thread holds one row as 16-byte chunks; transposing each group of eight chunks
       // (128 bytes) inside groups of eight lanes gives every lane the same chunk of eight
       // consecutive rows, so that one store instruction of the warp writes four whole
@@ -663,10 +706,12 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     }
   } else {
     // ------------------------------------------------------------ dQ warpgroup
+    set_max_registers<kBwdRegsDq, kBwdRegsLaunch>();
     const int row = 32 * (warp & 3) + lane;
-    const bool leader = (warp == 10 && lane == 0);
+    const int quarter = warp & 3;   // rows [32 quarter, + 32) of the tile
+    const bool leader = lane == 0;
     const uint32_t lane_base = tmem + (uint32_t(32 * (warp & 3)) << 16);
-    const uint32_t stg = base + L::kStg;
+    const uint32_t stg = base + L::kStg + (warp - 12) * (2 * L::kStageBytes);
     uint32_t gc = 0, chunk = 0, ucnt = 0;
     BwdUnit un;
     for (; get_bwd_unit(prm, take_unit(ucnt, true), ntiles_total, un); ++ucnt) {
@@ -689,9 +734,13 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
       // same query tile a whole query tile's worth of iterations later -- or at once whenever
       // this unit finds that it has to wait for its own turn.
       int32_t* pend = nullptr;
-      auto publish = [&](int32_t* p) {   // (the release store orders it behind the completed adds)
+      // What the turns order are reductions performed in L2: ours are complete (waited for, so
+      // performed) before the store below is issued, and the next unit issues its own behind the
+      // load that sees it.  Nobody reads the sums before the kernel ends, so neither side needs
+      // a fence -- which would cost this warp about a thousand cycles per tile.
+      auto publish = [&](int32_t* p) {
         const int mine = k_rel + 1;
-        asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(mine) : "memory");
+        asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(mine) : "memory");
       };
       for (int it = 0; it < un.n_it; ++it, q_advance(qi, prm.Hq / prm.Hkv)) {
         const QTile qt = q_tile_at(prm, un, qi);
@@ -699,95 +748,85 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         int32_t* sem = nullptr;
         int seen_early = -1;
         if (kDet && leader) {
-          sem = prm.dq_sem + size_t(un.tidx + qi.qt) * prm.Hq + qt.h;
+          sem = prm.dq_sem + (size_t(un.tidx + qi.qt) * prm.Hq + qt.h) * 4 + quarter;
           // the last prompt tile follows the lowest response tile that adds to this query tile
           if (qi.hh == 0 && qi.qt > 0 && k_rel == un.tile.npc - 1 && k_rel + qi.qt >= un.tile.npc)
             dep_lo = prm.tiles[un.tidx + qi.qt].dep_lo;
           // read the counter now: the answer (normally already the expected one) is back by the
           // time the first box of the tile is staged
-          asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen_early) : "l"(sem) : "memory");
+          asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(seen_early) : "l"(sem) : "memory");
         }
         wait_bar(bar(kDqFull), g & 1, abort_flag, prm.header, 80);
         tc_fence_after();
-        // Two halves of D/2 columns.  The second half is read out of tensor memory (and the
-        // dP/dQ columns handed back to the MMA warp) before any wait on the reductions issued
-        // for the first half, so the MMA pipeline never waits for TMA reads of the staging.
+        // The whole tile goes to registers at once and the dP/dQ columns back to the MMA thread,
+        // before any wait on the staging buffers: the next dP has to wait for this.
+        uint32_t w[D];
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          uint32_t w[D / 2];
-#pragma unroll
-          for (int c = 0; c < D / 64; ++c) {
-            if (DV == D || half * (D / 2) + c * 32 < DV) {
-              tmem_ld32(lane_base + tdP + half * (D / 2) + c * 32,
-                        *reinterpret_cast<uint32_t(*)[32]>(&w[c * 32]));
-            } else {  // no such columns in global memory: the box is not reduced either
-#pragma unroll
-              for (int i = 0; i < 32; ++i) w[c * 32 + i] = 0u;
-            }
+        for (int c = 0; c < D / 32; ++c) {
+          if (c * 32 < DV) {   // (no such columns in global memory: the box is not reduced either)
+            tmem_ld32(lane_base + tdP + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&w[c * 32]));
           }
-          tmem_wait_ld();
-          if (half == 1) {
-            tc_fence_before();
-            mbar_arrive(bar(kDqDrained));
+        }
+        tmem_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(kDqDrained));
+        if (row >= qt.len) {  // rows past the tile's end belong to other tokens: add zero
+#pragma unroll
+          for (int i = 0; i < DV; ++i) w[i] = 0u;
+        }
+#pragma unroll
+        for (int c = 0; c < DV / 32; ++c, ++chunk) {
+          const uint32_t buf = stg + (chunk & 1) * L::kStageBytes;
+          // the reduce issued two boxes ago must have finished reading this buffer
+          if (leader) bulk_wait_group_read<1>();
+          __syncwarp();
+          const uint32_t row_addr = buf + lane * 128;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const uint32_t ch = uint32_t(i) ^ uint32_t(lane & 7);
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row_addr + ch * 16),
+                         "r"(w[c * 32 + 4 * i]), "r"(w[c * 32 + 4 * i + 1]),
+                         "r"(w[c * 32 + 4 * i + 2]), "r"(w[c * 32 + 4 * i + 3])
+                         : "memory");
           }
-          if (row >= qt.len) {  // rows past the tile's end belong to other tokens: add zero
-#pragma unroll
-            for (int i = 0; i < D / 2; ++i) w[i] = 0u;
-          }
-#pragma unroll
-          for (int c = 0; c < D / 64; ++c, ++chunk) {
-            const uint32_t buf = stg + (chunk & 1) * L::kStageBytes;
-            // the reduce issued two chunks ago must have finished reading this buffer
-            if (leader) bulk_wait_group_read<1>();
-            named_barrier_sync(1, 128);
-            const uint32_t row_addr = buf + row * 128;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const uint32_t ch = uint32_t(i) ^ uint32_t(row & 7);
-              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row_addr + ch * 16),
-                           "r"(w[c * 32 + 4 * i]), "r"(w[c * 32 + 4 * i + 1]),
-                           "r"(w[c * 32 + 4 * i + 2]), "r"(w[c * 32 + 4 * i + 3])
-                           : "memory");
-            }
-            fence_proxy_async_smem();
-            named_barrier_sync(1, 128);
-            if (leader) {
-              if (kDet && sem && half == 0 && c == 0) {  // wait for this unit's turn (bounded)
-                const int expect =
-                    qi.qt == 0 ? 0
-                               : ((k_rel == un.tile.npc - 1 && k_rel + qi.qt >= un.tile.npc) ? dep_lo + 1
-                                                                                            : k_rel + 2);
-                bool ok = seen_early == expect;
-                for (uint32_t spin = 0; !ok && spin < (1u << 22); ++spin) {
-                  int seen;
-                  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(sem) : "memory");
-                  if (seen == expect) {
-                    ok = true;
-                    break;
-                  }
-                  if (pend) {  // about to wait: do not keep the unit below waiting for us
-                    bulk_wait_group<0>();
-                    publish(pend);
-                    pend = nullptr;
-                  }
-                  if ((spin & 0xff) == 0xff && *abort_flag) break;
-                  __nanosleep(20);
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (leader) {
+            if (kDet && sem && c == 0) {  // wait for this unit's turn (bounded)
+              const int expect =
+                  qi.qt == 0 ? 0
+                             : ((k_rel == un.tile.npc - 1 && k_rel + qi.qt >= un.tile.npc) ? dep_lo + 1
+                                                                                          : k_rel + 2);
+              bool ok = seen_early == expect;
+              for (uint32_t spin = 0; !ok && spin < (1u << 22); ++spin) {
+                int seen;
+                asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(sem) : "memory");
+                if (seen == expect) {
+                  ok = true;
+                  break;
                 }
-                if (!ok && !*abort_flag) {
-                  if (atomicCAS(&prm.header[0], kStatusOk, kStatusWaitExpired) == kStatusOk)
-                    prm.header[1] = 81;
-                  *abort_flag = 1;
+                if (pend) {  // about to wait: do not keep the unit below waiting for us
+                  bulk_wait_group<0>();
+                  publish(pend);
+                  pend = nullptr;
                 }
+                if ((spin & 0xff) == 0xff && *abort_flag) break;
+                __nanosleep(20);
               }
-              if (DV == D || half * (D / 2) + c * 32 < DV)
-                tma_reduce_add_3d(&tm_dq, buf, half * (D / 2) + c * 32, qt.h, qt.start);
-              bulk_commit_group();
+              if (!ok && !*abort_flag) {
+                if (atomicCAS(&prm.header[0], kStatusOk, kStatusWaitExpired) == kStatusOk)
+                  prm.header[1] = 81;
+                *abort_flag = 1;
+              }
             }
+            if (32 * quarter < qt.len) tma_reduce_add_3d(&tm_dq, buf, c * 32, qt.h, qt.start + 32 * quarter);
+            bulk_commit_group();
           }
         }
         if (kDet && sem) {
-          if (pend) {  // the previous tile's boxes (all but this tile's D / 32 groups) have landed
-            bulk_wait_group<D / 32>();
+          if (pend) {  // the previous tile's boxes (all but this tile's DV / 32 groups) have landed
+            bulk_wait_group<DV / 32>();
             publish(pend);
           }
           pend = sem;

@@ -81,14 +81,14 @@ inline bool encode_thd(CUtensorMap* m, const void* base, int T, int H, int D, in
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// fp32 tensor [T][H][D] for TMA reductions: one box = 32 floats x 1 head x 128 tokens,
+// fp32 tensor [T][H][D] for TMA reductions: one box = 32 floats x 1 head x 32 tokens,
 // 128-byte swizzled (row r at r * 128 bytes, 16-byte chunks XOR-ed with r mod 8).
 inline bool encode_thd_f32(CUtensorMap* m, const void* base, int T, int H, int D) {
   EncodeTiledFn fn = encode_tiled_fn();
   if (!fn) return false;
   cuuint64_t dims[3] = {cuuint64_t(D), cuuint64_t(H), cuuint64_t(T)};
   cuuint64_t strides[2] = {cuuint64_t(D) * 4, cuuint64_t(H) * D * 4};
-  cuuint32_t box[3] = {32, 1, 128};
+  cuuint32_t box[3] = {32, 1, 32};
   cuuint32_t estr[3] = {1, 1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box,
             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,

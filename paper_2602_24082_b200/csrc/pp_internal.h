@@ -127,8 +127,8 @@ inline PlanLayout plan_layout(const pp_problem& p) {
 }
 
 // Backward scratch: fp32 dQ accumulator [T][Hq][D], Delta [Hq][T], LSE*log2(e) [Hq][T], and
-// the turn counters of the deterministic variant, one per (query tile of the backward grid,
-// query head)
+// the turn counters of the deterministic variant, four per (query tile of the backward grid,
+// query head): one for each warp's 32 rows
 struct BwdScratch {
   size_t dq_acc, delta, lse2, sem, sem_bytes, total;
 };
@@ -140,7 +140,7 @@ inline BwdScratch bwd_scratch_layout(const pp_problem& p) {
   s.delta = off;  off = align_up(off + 4 * T * Hq, 256);
   s.lse2 = off;   off = align_up(off + 4 * T * Hq, 256);
   s.sem = off;
-  s.sem_bytes = 4 * size_t(max_tiles_of(p)) * Hq;
+  s.sem_bytes = 16 * size_t(max_tiles_of(p)) * Hq;
   off = align_up(off + s.sem_bytes, 256);
   s.total = off;
   return s;

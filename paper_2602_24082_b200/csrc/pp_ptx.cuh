@@ -108,14 +108,13 @@ __device__ __forceinline__ void named_barrier_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
-// Per-warpgroup register re-allocation (all four warps of the warpgroup execute it).
-template <int N>
-__device__ __forceinline__ void setmaxnreg_inc() {
-  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
-}
-template <int N>
-__device__ __forceinline__ void setmaxnreg_dec() {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+// Per-warpgroup register re-allocation (all four warps of the warpgroup execute it) from the
+// kLaunch registers per thread the kernel was launched with to kTo: taking and giving back are two
+// instructions, and either one in the wrong direction is illegal.
+template <int kTo, int kLaunch>
+__device__ __forceinline__ void set_max_registers() {
+  if constexpr (kTo > kLaunch) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kTo));
+  if constexpr (kTo < kLaunch) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kTo));
 }
 
 // ---------------------------------------------------------------- tcgen05: TMEM management
@@ -292,6 +291,11 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   uint64_t r;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
 __device__ __forceinline__ float max3(float a, float b, float c) {
