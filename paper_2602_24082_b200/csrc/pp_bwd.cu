@@ -59,6 +59,7 @@ __global__ void __launch_bounds__(32 * kPreWarps)
 bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o,
                       const float* __restrict__ lse, float* __restrict__ delta,
                       float* __restrict__ lse2, float* __restrict__ dq_acc, int T, int Hq) {
+  launch_dependents();
   constexpr int kLanes = pre_lanes(D);    // lanes per row (D / 8 of them hold data)
   constexpr int kRows = 32 / kLanes;      // rows per warp and step
   const int lane = threadIdx.x & 31, sub = lane % kLanes, rin = lane / kLanes;
@@ -108,6 +109,7 @@ bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* 
 // ---------------------------------------------------------------- finalize
 __global__ void __launch_bounds__(256)
 bwd_finalize_kernel(const float4* __restrict__ acc, uint2* __restrict__ dq, size_t n4, float scale) {
+  launch_dependents();
   size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
   const size_t stride = size_t(gridDim.x) * blockDim.x;
   for (; i < n4; i += stride) {
@@ -193,15 +195,14 @@ struct BwdUnit {
 
 // Units are handed out dynamically: the producer warp draws the next index of the plan's
 // longest-work-first order from a global counter whenever the CTA is ready for more (list
-// scheduling), and passes it to the other roles through a two-entry shared-memory ring.
+// scheduling), and passes its entry to the other roles through a two-entry shared-memory ring.
 // header[5] is that counter, header[7] counts finished CTAs; the last one resets both, so a
 // plan can be used by any number of launches without a memset in between.
 constexpr int kHdrBwdNext = 5, kHdrBwdDone = 7;
 
-__device__ __forceinline__ bool get_bwd_unit(const BwdParams& prm, int u, int ntiles_total,
-                                             BwdUnit& un) {
-  if (u < 0 || u >= ntiles_total * prm.Hkv) return false;
-  const int packed = prm.order[u];  // (kv head << 24) | backward tile
+// `packed` = (kv head << 24) | backward tile, negative at the end of the work list.
+__device__ __forceinline__ bool get_bwd_unit(const BwdParams& prm, int packed, BwdUnit& un) {
+  if (packed < 0) return false;
   un.kvh = packed >> 24;
   un.tidx = packed & 0xffffff;
   un.tile = prm.tiles[un.tidx];
@@ -250,8 +251,6 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // (known to be uniform in the warp)
 
-  if (prm.header[0] != kStatusOk) return;
-  const int ntiles_total = prm.header[kHdrNumBTiles];
 #ifdef PP_DEBUG_COUNTERS
   const long long t_kernel0 = clock64();
 #endif
@@ -259,6 +258,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   if (base - raw + L::kUsed > L::kTotal) {  // cannot happen with an aligned base
+    dependency_wait();
     if (tid == 0 && atomicCAS(&prm.header[0], kStatusOk, kStatusWaitExpired) == kStatusOk)
       prm.header[1] = 99;
     return;
@@ -298,24 +298,13 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot_p;
+  dependency_wait();
   constexpr uint32_t tS = 0, tdP = 128, tdV = 256, tdK = 384;
   volatile int* sched = reinterpret_cast<volatile int*>(gbase + L::kBars + 8 * kNumBwdBars + 16);
-  // producer warp (all lanes): draw the n-th unit of this CTA and publish it
-  auto fetch_unit = [&](uint32_t n) -> int {
-    int u = 0;
-    if (lane == 0) {
-      wait_bar(bar(kSchedEmpty + (n & 1)), ((n >> 1) & 1) ^ 1, abort_flag, prm.header, 90);
-      // after a wait has given up, no more work is drawn: an out-of-range id ends every role
-      u = *abort_flag ? 0x7fffffff : atomicAdd(&prm.header[kHdrBwdNext], 1);
-      sched[n & 1] = u;
-      mbar_arrive(bar(kSchedFull + (n & 1)));
-    }
-    return __shfl_sync(0xffffffffu, u, 0);
-  };
   // other roles: read the n-th unit; `whole_warp` = all 32 lanes are calling
   auto take_unit = [&](uint32_t n, bool whole_warp) -> int {
     const bool ok = wait_bar(bar(kSchedFull + (n & 1)), (n >> 1) & 1, abort_flag, prm.header, 91);
-    const int u = ok ? sched[n & 1] : 0x7fffffff;
+    const int u = ok ? sched[n & 1] : -1;
     if (whole_warp) {
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(kSchedEmpty + (n & 1)));
@@ -331,7 +320,26 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     // ------------------------------------------------------------ producer
     uint32_t qc = 0, ucnt = 0;
     BwdUnit un;
-    for (; get_bwd_unit(prm, fetch_unit(ucnt), ntiles_total, un); ++ucnt) {
+    // (a refused plan has no work)
+    const int num_units = prm.header[0] == kStatusOk ? prm.header[kHdrNumBTiles] * prm.Hkv : 0;
+    // all lanes: draw the n-th unit of this CTA, publish it to the other roles
+    auto fetch_unit = [&](uint32_t n) -> int {
+      int packed = -1;
+      if (lane == 0) {
+        wait_bar(bar(kSchedEmpty + (n & 1)), ((n >> 1) & 1) ^ 1, abort_flag, prm.header, 90);
+        // after a wait has given up, no more work is drawn: the end marker goes out instead
+        // (The first unit is the one of the CTA's own index.  Not in the deterministic variant: a
+        // CTA that starts late must not hold a unit that running CTAs wait for.)
+        const int u = *abort_flag        ? num_units
+                      : !kDet && n == 0 ? int(blockIdx.x)
+                                         : (kDet ? 0 : int(gridDim.x)) + atomicAdd(&prm.header[kHdrBwdNext], 1);
+        if (u < num_units) packed = prm.order[u];
+        sched[n & 1] = packed;
+        mbar_arrive(bar(kSchedFull + (n & 1)));
+      }
+      return __shfl_sync(0xffffffffu, packed, 0);
+    };
+    for (; get_bwd_unit(prm, fetch_unit(ucnt), un); ++ucnt) {
       if (lane == 0) {
         wait_bar(bar(kKvEmpty), (ucnt & 1) ^ 1, abort_flag, prm.header, 50);
         mbar_expect_tx(bar(kKvFull), 2 * L::kTileBytes);
@@ -398,7 +406,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
           mma_ss(tmem + tS, dK_k + kmajor_off(k), dq_k + kmajor_off(k), idesc, k > 0);
         mma_commit(bar(kSFullB));
       };
-      for (; get_bwd_unit(prm, take_unit(ucnt, false), ntiles_total, un); ++ucnt) {
+      for (; get_bwd_unit(prm, take_unit(ucnt, false), un); ++ucnt) {
         const int ksteps = (un.tile.len + 15) >> 4;
         wait_bar(bar(kKvFull), ucnt & 1, abort_flag, prm.header, 60);
         QIter qi;
@@ -512,7 +520,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const uint32_t ds_row = sdS + wg * kBoxBytes + row * 128;   // dS^T row `row` in box wg
     uint32_t gc = 0, ucnt = 0;
     BwdUnit un;
-    for (; get_bwd_unit(prm, take_unit(ucnt, true), ntiles_total, un); ++ucnt) {
+    for (; get_bwd_unit(prm, take_unit(ucnt, true), un); ++ucnt) {
       const bool row_ok = row < un.tile.len;
       // my key j = tile.start + row is seen by the queries [j, key_end[j])
       const int key_lo = un.tile.start + row;
@@ -714,7 +722,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const uint32_t stg = base + L::kStg + (warp - 12) * (2 * L::kStageBytes);
     uint32_t gc = 0, chunk = 0, ucnt = 0;
     BwdUnit un;
-    for (; get_bwd_unit(prm, take_unit(ucnt, true), ntiles_total, un); ++ucnt) {
+    for (; get_bwd_unit(prm, take_unit(ucnt, true), un); ++ucnt) {
       QIter qi;
       // Deterministic variant: the key tiles that add to a (query tile, head) do so in
       // DESCENDING tile order: the query tile's own key tile first, then the tiles below it
@@ -909,12 +917,15 @@ cudaError_t launch_bwd_t(const pp_plan* plan, const void* o, const float* lse, c
   pre<<<pre_blocks, 32 * kPreWarps, 0, stream>>>(
       static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse,
       const_cast<float*>(prm.delta), const_cast<float*>(prm.lse2), prm.dq_acc, int(T), int(Hq));
+  cudaError_t e = cudaGetLastError();
   const long long units = (long long)plan->max_tiles * pb.num_kv_heads;
   dim3 grid(unsigned(std::min<long long>(units, num_sms)));
   ProfileEvents& ev = profile_events();
   const int slot = int(ev.bwd_count % kProfileRing);
   if (ev.on) profile_record(ev.bwd0[slot], stream);
-  kern<<<grid, kBwdThreads, BwdSmem<D>::kTotal, stream>>>(tq, tk, tv, tdo, tdq, prm);
+  if (e == cudaSuccess)
+    e = launch_kernel(units <= (long long)kOverlapUnits * num_sms, kern, grid, dim3(kBwdThreads),
+                      BwdSmem<D>::kTotal, stream, tq, tk, tv, tdo, tdq, prm);
   if (ev.on) {
     profile_record(ev.bwd1[slot], stream);
     ++ev.bwd_count;
@@ -923,8 +934,9 @@ cudaError_t launch_bwd_t(const pp_plan* plan, const void* o, const float* lse, c
   unsigned fb = unsigned(std::min<size_t>((n4 + 255) / 256, size_t(num_sms) * 16));
   bwd_finalize_kernel<<<fb, 256, 0, stream>>>(reinterpret_cast<const float4*>(prm.dq_acc),
                                               static_cast<uint2*>(dq), n4, prm.scale);
+  if (e == cudaSuccess) e = cudaGetLastError();
   if (launches) *launches += 3;
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace

@@ -95,9 +95,9 @@ struct Unit {
   int h0, kvh, nslots, n0, n1, ntiles;
 };
 
-// Units are handed out dynamically in the plan's longest-work-first order: the producer
-// draws the next index from a global counter (header[4]) when the CTA is ready for more and
-// passes it on through a two-entry shared-memory ring; header[6] counts finished CTAs and the
+// Units are handed out dynamically in the plan's longest-work-first order: a CTA starts with the
+// unit of its own index, for later ones the producer draws from a global counter (header[4]) when
+// the CTA is ready for more; it passes them on through a two-entry shared-memory ring; header[6] counts finished CTAs and the
 // last one resets both counters for the next launch.
 constexpr int kHdrFwdNext = 4, kHdrFwdDone = 6;
 
@@ -130,6 +130,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // (known to be uniform in the warp)
 
+  dependency_wait();
   if (prm.header[0] != kStatusOk) return;
   const int ntiles_total = prm.header[2];
 #ifdef PP_DEBUG_COUNTERS
@@ -173,7 +174,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   auto fetch_unit = [&](uint32_t n, Unit& un) -> bool {  // producer thread
     wait_bar(bar(kSchedEmptyF + (n & 1)), ((n >> 1) & 1) ^ 1, abort_flag, prm.header, 90);
     // after a wait has given up, no more work is drawn: the end marker goes out instead
-    const int u = *abort_flag ? 0x7fffffff : atomicAdd(&prm.header[kHdrFwdNext], 1);
+    const int u = *abort_flag ? 0x7fffffff
+                  : n == 0    ? int(blockIdx.x)
+                              : int(gridDim.x) + atomicAdd(&prm.header[kHdrFwdNext], 1);
     const bool ok = get_unit(prm, u, ntiles_total, un);
     volatile int* e = sched + (n & 1) * 8;
     e[0] = un.tile.start;
@@ -707,12 +710,13 @@ cudaError_t launch_fwd_t(const pp_plan* plan, const CUtensorMap& tq, const CUten
   ProfileEvents& ev = profile_events();
   const int slot = int(ev.fwd_count % kProfileRing);
   if (ev.on && ev.fwd_on) profile_record(ev.fwd0[slot], stream);
-  kern<<<grid, kFwdThreads, FwdSmem<D>::kTotal, stream>>>(tq, tk, tv, prm);
+  const cudaError_t le = launch_kernel(units <= (long long)kOverlapUnits * num_sms, kern, grid,
+                                       dim3(kFwdThreads), FwdSmem<D>::kTotal, stream, tq, tk, tv, prm);
   if (ev.on && ev.fwd_on) {
     profile_record(ev.fwd1[slot], stream);
     ++ev.fwd_count;
   }
-  return cudaGetLastError();
+  return le;
 }
 
 }  // namespace

@@ -15,6 +15,7 @@
 #include <type_traits>
 
 #include "pp_internal.h"
+#include "pp_ptx.cuh"
 
 namespace pp {
 namespace {
@@ -562,10 +563,12 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
   FusedSmem& sm = *reinterpret_cast<FusedSmem*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nthr = blockDim.x;
   const int n_rgo = p.num_rows + 1, n_all = n_rgo + p.G + p.G + 1 + p.N;
+  launch_dependents();
   // ---- descriptors -> shared memory, and the copy that later kernels read
   if (kDesc > 1) {
     for (int i = tid; i < n_all; i += nthr) sm.desc[i] = blk.v[i];
   } else {
+    dependency_wait();
     const int n[4] = {n_rgo, p.G, p.G + 1, p.N};
     int at = 0;
     for (int a = 0; a < 4; ++a) {
@@ -577,6 +580,7 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
     sm.status = kStatusOk;
     sm.detail = 0;
   }
+  if (kDesc > 1) dependency_wait();   // (the workspace may still be in use up to here)
   __syncthreads();
   for (int i = tid; i < n_all; i += nthr) p.desc_copy[i] = sm.desc[i];
   const int32_t* rgo = sm.desc;
@@ -928,8 +932,8 @@ cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cu
   const size_t n_all = n_desc[0] + n_desc[1] + n_desc[2] + n_desc[3];
   if (mt <= kFusedMaxTiles && p.T <= (1 << 18)) {
     // rows <= G <= N and G + N <= 2048: kDescFused entries always suffice
+    cudaError_t e = cudaSuccess;
     if (!dev->configured) {
-      cudaError_t e = cudaSuccess;
       auto opt_in = [&](auto kern) {
         if (e == cudaSuccess)
           e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(FusedSmem));
@@ -944,13 +948,14 @@ cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cu
       constexpr size_t kN = decltype(n_c)::value;
       DescBlock<kN> blk;
       if (host_desc) fill_desc(host_desc, n_desc, blk.v);
-      plan_fused_kernel<kN><<<1, mt <= kFusedSmallTiles ? 256 : 1024, sizeof(FusedSmem), stream>>>(blk, p);
+      e = launch_kernel(true, plan_fused_kernel<kN>, dim3(1), dim3(mt <= kFusedSmallTiles ? 256 : 1024),
+                            sizeof(FusedSmem), stream, blk, p);
     };
     if (!host_desc) go(std::integral_constant<size_t, 1>{});
     else if (n_all <= kDescSmall) go(std::integral_constant<size_t, kDescSmall>{});
     else go(std::integral_constant<size_t, kDescFused>{});
     if (launches) *launches = 1;
-    return cudaGetLastError();
+    return e;
   }
   int n_launch = 8;
   if (host_desc) {

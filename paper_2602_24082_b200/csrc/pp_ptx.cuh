@@ -29,6 +29,16 @@ __device__ __forceinline__ bool elect_one() {
   return ok != 0;
 }
 
+// ---------------------------------------------------------------- dependent launch
+// The next kernel on the stream may be launched once every block has got here.
+__device__ __forceinline__ void launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// Waits until the kernels in front on the stream are complete and their writes visible.
+__device__ __forceinline__ void dependency_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
