@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libpp_attn.so: argument marshalling only.
+"""Thin binding of libpp_attn.so: argument marshalling only (the calls of a step -- plan,
+forward, backward -- through the CPython module _pp_torch, everything else through ctypes).
 
 Every step of the path (plan building, forward, backward) runs in the library's CUDA
 kernels; PyTorch only provides device memory and the current stream.  There is no CPU
@@ -19,6 +20,7 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libpp_attn.so")
 _lib: Optional[ctypes.CDLL] = None
+_ext = None
 
 EXPORTS = ["pp_plan_workspace_bytes", "pp_build_plan", "pp_plan_status", "pp_destroy_plan",
            "pp_plan_max_tiles", "pp_plan_read", "pp_attn_fwd", "pp_attn_bwd",
@@ -104,10 +106,7 @@ def _check(rc: int, where: str):
 
 
 def _call(index: int, where: str, fn, *args):
-    """``fn(*args, current stream of device index)`` with that device current.  (On small problems
-    the time a call spends here is the time it takes: 14 us of Python around each of 8 us of plan,
-    4 us of forward and 12 us of backward, before the device guard was limited to calls that need
-    it, the stream came as a raw handle, and shapes and sizes were kept as plain integers.)"""
+    """``fn(*args, current stream of device index)`` with that device current."""
     if torch.cuda.current_device() == index:
         rc = fn(*args, torch._C._cuda_getCurrentRawStream(index))
     else:
@@ -117,19 +116,46 @@ def _call(index: int, where: str, fn, *args):
         raise PPError(rc, where)
 
 
+def _step_calls():
+    """The CPython module with the calls of a step, bound to the library ``lib`` has loaded."""
+    global _ext
+    if _ext is None:
+        lib()
+        try:
+            from . import _pp_torch
+        except ImportError as e:
+            raise RuntimeError("_pp_torch.so is missing or does not load: build it with "
+                               "`python -m paper_2602_24082_b200.build`") from e
+        _pp_torch.bind(LIB_PATH, PPError, _chk)
+        _ext = _pp_torch
+    return _ext
+
+
 class Plan:
     """Owns the host handle, the device workspace and the backward scratch of one problem."""
 
-    def __init__(self, handle: int, problem: _Problem, workspace: torch.Tensor, keep):
+    def __init__(self, handle: int, workspace: torch.Tensor, keep, num_q_heads: int, num_kv_heads: int,
+                 head_dim: int, total_tokens: int):
         self.handle = handle
-        self.problem = problem
         self.workspace = workspace
-        self._keep = keep
+        self._keep = keep          # (descriptor arrays, device arrays or None)
+        self._problem: Optional[_Problem] = None
         self._sizes: Optional[Tuple[int, int, int]] = None
         self._bwd_scratch: Optional[torch.Tensor] = None
-        T, Hq, Hkv, D = (problem.total_tokens, problem.num_q_heads, problem.num_kv_heads,
-                         problem.head_dim)
-        self.q_shape, self.kv_shape, self.lse_shape = (T, Hq, D), (T, Hkv, D), (Hq, T)
+        self.total_tokens = total_tokens
+        # the arguments every call of a step starts with
+        self._head = (handle, total_tokens, num_q_heads, num_kv_heads, head_dim)
+
+    @property
+    def problem(self) -> _Problem:
+        if self._problem is None:
+            _, T, Hq, Hkv, D = self._head
+            self._problem, self._keep = make_problem(self._keep[0], Hq, Hkv, D, T, self._keep[1])
+        return self._problem
+
+    q_shape = property(lambda self: (self._head[1], self._head[2], self._head[4]))
+    kv_shape = property(lambda self: (self._head[1], self._head[3], self._head[4]))
+    lse_shape = property(lambda self: (self._head[2], self._head[1]))
 
     def _size(self, i: int) -> int:
         if self._sizes is None:
@@ -139,10 +165,6 @@ class Plan:
     plan_bytes = property(lambda self: self._size(0))
     fwd_scratch_bytes = property(lambda self: self._size(1))
     bwd_scratch_bytes = property(lambda self: self._size(2))
-
-    @property
-    def total_tokens(self) -> int:
-        return self.problem.total_tokens
 
     def bwd_scratch(self) -> torch.Tensor:
         if self._bwd_scratch is None:
@@ -221,8 +243,16 @@ def pp_build_plan(desc: Sequence[np.ndarray], num_q_heads: int, num_kv_heads: in
                   workspace: Optional[torch.Tensor] = None) -> Plan:
     """Builds a plan.  ``device_arrays`` (int32 CUDA tensors) and ``workspace`` (uint8 CUDA
     tensor of at least the queried size) let a caller re-plan every step without allocating."""
-    if not torch.cuda.is_available():
-        raise RuntimeError("pp_build_plan needs a CUDA device (there is no CPU fallback)")
+    ext = _ext
+    if ext is None:
+        if not torch.cuda.is_available():
+            raise RuntimeError("pp_build_plan needs a CUDA device (there is no CPU fallback)")
+        ext = _step_calls()
+    if workspace is not None and device_arrays is None and not desc_on_device:
+        # (None: the arrays have to be converted first, below)
+        handle = ext.build_plan(tuple(desc), num_q_heads, num_kv_heads, head_dim, total_tokens, workspace)
+        if handle is not None:
+            return Plan(handle, workspace, (desc, None), num_q_heads, num_kv_heads, head_dim, total_tokens)
     dev_arrays = device_arrays
     if desc_on_device and dev_arrays is None:
         dev_arrays = [torch.from_numpy(np.ascontiguousarray(a, dtype=np.int32)).to(device) for a in desc]
@@ -239,7 +269,7 @@ def pp_build_plan(desc: Sequence[np.ndarray], num_q_heads: int, num_kv_heads: in
         if e.code == -3:
             raise ValueError("workspace too small") from None
         raise
-    return Plan(handle.value, problem, workspace, keep)
+    return Plan(handle.value, workspace, keep, num_q_heads, num_kv_heads, head_dim, total_tokens)
 
 
 def _build_plan(problem, ws_ptr, ws_bytes, handle, stream):
@@ -257,48 +287,14 @@ def pp_attn_fwd(plan: Plan, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor,
                 lse: Optional[torch.Tensor] = None, for_backward: bool = False):
     """``for_backward``: also hand the plan's backward scratch to the forward, which then clears
     the fp32 dQ accumulator in it (the following ``pp_attn_bwd`` skips its own clearing)."""
-    bf16 = torch.bfloat16
-    _chk(q, plan.q_shape, bf16, "q")
-    _chk(k, plan.kv_shape, bf16, "k")
-    _chk(v, plan.kv_shape, bf16, "v")
-    if o is None:
-        o = torch.empty_like(q)
-    else:
-        _chk(o, plan.q_shape, bf16, "o")
-    if lse is None:
-        lse = q.new_empty(plan.lse_shape, dtype=torch.float32)
-    else:
-        _chk(lse, plan.lse_shape, torch.float32, "lse")
-    sc_ptr, sc_bytes = None, 0
-    if for_backward:
-        sc = plan.bwd_scratch()
-        sc_ptr, sc_bytes = sc.data_ptr(), sc.numel()
-    _call(q.get_device(), "pp_attn_fwd", lib().pp_attn_fwd, plan.handle, q.data_ptr(), k.data_ptr(),
-          v.data_ptr(), float(softmax_scale), o.data_ptr(), lse.data_ptr(), sc_ptr, sc_bytes)
-    return o, lse
+    return _ext.fwd(*plan._head, q, k, v, softmax_scale, o, lse, plan.bwd_scratch() if for_backward else None)
 
 
 def pp_attn_bwd(plan: Plan, q, k, v, o, lse, d_o, softmax_scale: float, d_q=None, d_k=None, d_v=None,
                 deterministic: bool = False):
     """``deterministic``: pp_attn_bwd_deterministic (bit-reproducible dQ; key tiles take turns)."""
-    bf16 = torch.bfloat16
-    q_shape, kv_shape = plan.q_shape, plan.kv_shape
-    _chk(q, q_shape, bf16, "q")
-    _chk(k, kv_shape, bf16, "k")
-    _chk(v, kv_shape, bf16, "v")
-    _chk(o, q_shape, bf16, "o")
-    _chk(d_o, q_shape, bf16, "d_o")
-    _chk(lse, plan.lse_shape, torch.float32, "lse")
-    d_q = torch.empty_like(q) if d_q is None else d_q
-    d_k = torch.empty_like(k) if d_k is None else d_k
-    d_v = torch.empty_like(v) if d_v is None else d_v
-    scratch = plan.bwd_scratch()
-    L = lib()
-    _call(q.get_device(), "pp_attn_bwd", L.pp_attn_bwd_deterministic if deterministic else L.pp_attn_bwd,
-          plan.handle, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(),
-          d_o.data_ptr(), float(softmax_scale), d_q.data_ptr(), d_k.data_ptr(), d_v.data_ptr(),
-          scratch.data_ptr(), scratch.numel())
-    return d_q, d_k, d_v
+    return _ext.bwd(*plan._head, q, k, v, o, lse, d_o, softmax_scale, d_q, d_k, d_v, plan.bwd_scratch(),
+                    deterministic)
 
 
 def pp_position_ids(plan: Plan, out: Optional[torch.Tensor] = None) -> torch.Tensor:

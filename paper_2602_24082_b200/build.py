@@ -1,4 +1,5 @@
-"""Builds the CUDA library in-tree: paper_2602_24082_b200/libpp_attn.so (sm_100a only)."""
+"""Builds in-tree the CUDA library libpp_attn.so (sm_100a only) and the CPython module _pp_torch.so
+through which the binding makes the calls of a step."""
 from __future__ import annotations
 
 import os
@@ -8,6 +9,8 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpp_attn.so")
+EXT = os.path.join(HERE, "_pp_torch.so")
+EXT_SOURCE = "pp_torch.cpp"
 SOURCES = ["pp_api.cu", "pp_plan.cu", "pp_fwd.cu", "pp_bwd.cu", "pp_rope.cu", "pp_loss.cu", "pp_rows.cu"]
 HEADERS = ["pp_internal.h", "pp_dev.cuh", "pp_ptx.cuh", os.path.join("..", "..", "include", "pp_attn.h")]
 
@@ -19,19 +22,51 @@ def _nvcc() -> str:
     return "nvcc"
 
 
-def needs_build() -> bool:
-    if not os.path.exists(LIB):
+def _outdated(target: str, deps) -> bool:
+    if not os.path.exists(target):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS]
-    return any(os.path.getmtime(d) > t for d in deps)
+    t = os.path.getmtime(target)
+    return any(os.path.getmtime(os.path.join(CSRC, d)) > t for d in deps)
+
+
+def needs_build() -> bool:
+    return _outdated(LIB, SOURCES + HEADERS)
+
+
+def _start_ext(force: bool):
+    """Starts the compiler for _pp_torch.so if it has to be built."""
+    if not force and not _outdated(EXT, [EXT_SOURCE, HEADERS[-1]]):
+        return None
+    import sysconfig
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.isabs(_nvcc()) else "/usr/local/cuda"
+    include = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+               sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    cmd += ["-I" + d for d in include] + [os.path.join(CSRC, EXT_SOURCE), "-o", EXT,
+                                          "-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda",
+                                          "-ltorch_cpu", "-ltorch_python"]
+    return cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+
+
+def _finish(procs, verbose: bool):
+    for cmd, p in procs:
+        out, _ = p.communicate()
+        if verbose or p.returncode:
+            sys.stderr.write(out)
+        if p.returncode:
+            raise RuntimeError("compiler failed: " + " ".join(cmd))
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and not needs_build():
-        return LIB
+    ext = _start_ext(force)
+    procs = [ext] if ext else []
     objs = []
-    procs = []
+    if not force and not needs_build():
+        _finish(procs, verbose)
+        return LIB
     for s in SOURCES:
         obj = os.path.join(CSRC, s.replace(".cu", ".o"))
         cmd = [_nvcc(), "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
@@ -41,12 +76,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         cmd[1:1] = os.environ.get("PP_EXTRA_NVCC_FLAGS", "").split()
         procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
         objs.append(obj)
-    for cmd, p in procs:
-        out, _ = p.communicate()
-        if verbose or p.returncode:
-            sys.stderr.write(out)
-        if p.returncode:
-            raise RuntimeError("nvcc failed: " + " ".join(cmd))
+    _finish(procs, verbose)
     link = [_nvcc(), "-shared", "-o", LIB] + objs
     subprocess.run(link, check=True)
     return LIB
