@@ -163,7 +163,7 @@ int pp_attn_fwd(const pp_plan* plan, const void* q, const void* k, const void* v
  * the forward's O and LSE, writes dQ, dK, dV (bf16).  Prompt keys receive contributions from
  * the prompt's own queries and from every response's queries; dK and dV are summed over the
  * query heads that share a KV head.  dQ is accumulated in fp32 inside d_scratch and rounded
- * once at the end.
+ * once at the end; so are dK and dV where a small batch's work is cut into parts by query head.
  */
 int pp_attn_bwd(const pp_plan* plan, const void* q, const void* k, const void* v, const void* o,
                 const float* lse, const void* d_o, float softmax_scale, void* d_q, void* d_k,
@@ -227,7 +227,8 @@ int pp_preference_loss(const pp_plan* plan, const float* token_logp, const float
  * allocating routine; the caller still passes every input and output tensor.
  *
  *  - Limit: the scratch pp_plan_workspace_bytes reports for the plan's problem must not exceed
- *    pp_attn_bwd_noalloc_max_bytes (32 MiB, i.e. about T * Hq * D <= 8.2 M elements);
+ *    pp_attn_bwd_noalloc_max_bytes (32 MiB, i.e. about T * Hq * D <= 8.2 M elements), not
+ *    counting the room for partial dK and dV sums, which are only used where they fit too;
  *    larger problems are rejected with PP_ERR_STATIC_SCRATCH_LIMIT and nothing is launched.
  *  - Cost: every GPU on which the library is loaded holds those 32 MiB until the process exits.
  *  - The array used is the one on the device that holds the plan's workspace, and that device

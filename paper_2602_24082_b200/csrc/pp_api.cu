@@ -114,7 +114,8 @@ int pp_build_plan(const pp_problem* problem, void* d_workspace, size_t workspace
   plan->ws = static_cast<char*>(d_workspace);
   plan->lay = lay;
   plan->fwd_scratch = 0;
-  plan->bwd_scratch = pp::bwd_scratch_layout(*problem).total;
+  plan->lg_split = pp::bwd_split_log2(*problem);
+  plan->bwd_scratch = pp::bwd_scratch_layout(*problem, plan->lg_split).total;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
 
   // The four arrays, back to back in the workspace, are what the plan (plan kernels, position
@@ -237,7 +238,7 @@ int pp_attn_fwd(const pp_plan* plan, const void* q, const void* k, const void* v
     const pp_problem& pb = plan->prob;
     if (size_t(4) * pb.total_tokens * pb.num_q_heads * pb.head_dim <= kFwdClearMaxBytes)
       dq_clear = reinterpret_cast<float*>(static_cast<char*>(d_scratch) +
-                                          pp::bwd_scratch_layout(pb).dq_acc);
+                                          pp::bwd_scratch_layout(pb, plan->lg_split).dq_acc);
   }
   cudaError_t e = pp::launch_fwd(plan, q, k, v, softmax_scale, o, lse, dq_clear,
                                  reinterpret_cast<cudaStream_t>(stream), &g_last_launches);
@@ -262,7 +263,7 @@ static int attn_bwd_common(const pp_plan* plan, const void* q, const void* k, co
   const bool dq_cleared = plan->cleared_scratch == d_scratch;
   plan->cleared_scratch = nullptr;
   cudaError_t e = pp::launch_bwd(plan, q, k, v, o, lse, d_o, softmax_scale, d_q, d_k, d_v,
-                                 d_scratch, dq_cleared, deterministic,
+                                 d_scratch, plan->lg_split, dq_cleared, deterministic,
                                  reinterpret_cast<cudaStream_t>(stream), &g_last_launches);
   return e == cudaSuccess ? PP_OK : (e == cudaErrorNotSupported ? PP_ERR_UNSUPPORTED : PP_ERR_CUDA);
 }
@@ -295,7 +296,8 @@ int pp_attn_bwd_noalloc(const pp_plan* plan, const void* q, const void* k, const
   if (!plan || !q || !k || !v || !o || !lse || !d_o || !d_q || !d_k || !d_v)
     return PP_ERR_INVALID_ARG;
   if (!(softmax_scale > 0.f) || softmax_scale > 1e30f) return PP_ERR_INVALID_ARG;
-  if (plan->bwd_scratch > pp::kStaticScratchBytes) return PP_ERR_STATIC_SCRATCH_LIMIT;
+  // (units stay whole where the parts do not fit)
+  if (pp::bwd_scratch_layout(plan->prob, 0).total > pp::kStaticScratchBytes) return PP_ERR_STATIC_SCRATCH_LIMIT;
   const void* ptrs[] = {q, k, v, o, lse, d_o, d_q, d_k, d_v};
   for (const void* p : ptrs)
     if (!aligned16(p)) return PP_ERR_ALIGNMENT;
@@ -448,14 +450,14 @@ int step_runs_wanted(const pp_problem& p) {
 }
 
 // Places the chunks' private blocks; false if they do not fit the arena's regions.
-bool place_step(std::vector<StepChunk>& chunks, const pp::StepArena& a, size_t heads_q) {
+bool place_step(std::vector<StepChunk>& chunks, const pp::StepArena& a, size_t heads_q, int lg_split) {
   size_t po = a.plan, so = a.scratch, lo = a.lse;
   for (StepChunk& ch : chunks) {
     ch.plan_off = po;
     ch.plan_bytes = pp::plan_layout(ch.prob).total;
     po += pp::align_up(ch.plan_bytes, 256);
     ch.scratch_off = so;
-    ch.scratch_bytes = pp::bwd_scratch_layout(ch.prob).total;
+    ch.scratch_bytes = pp::bwd_scratch_layout(ch.prob, lg_split).total;
     so += pp::align_up(ch.scratch_bytes, 256);
     ch.lse_off = lo;
     lo += pp::align_up(size_t(ch.prob.total_tokens) * heads_q * 4, 256);
@@ -518,9 +520,11 @@ int pp_attn_step_host(const pp_problem* problem, const void* h_q, const void* h_
   // directions) while the kernels of run c execute.  Inside a run dO still goes up behind
   // the forward and O / LSE come down behind the backward.
   std::vector<StepChunk> chunks = cut_step(*problem, step_runs_wanted(*problem));
-  if (!place_step(chunks, a, Hq)) {
+  // (the parts of backward units are those of the whole problem: same sums, bit for bit)
+  const int lg_split = pp::bwd_split_log2(*problem);
+  if (!place_step(chunks, a, Hq, lg_split)) {
     chunks = cut_step(*problem, 1);
-    if (!place_step(chunks, a, Hq)) return PP_ERR_WORKSPACE_TOO_SMALL;
+    if (!place_step(chunks, a, Hq, lg_split)) return PP_ERR_WORKSPACE_TOO_SMALL;
   }
   auto ok = [](cudaError_t e) { return e == cudaSuccess; };
   if (!ok(cudaEventRecord(ss->e_start, s)) || !ok(cudaStreamWaitEvent(ss->up, ss->e_start, 0)) ||
@@ -554,6 +558,8 @@ int pp_attn_step_host(const pp_problem* problem, const void* h_q, const void* h_
     rc = pp_build_plan(&ch.prob, base + ch.plan_off, ch.plan_bytes, stream, &plan);
     if (rc) break;
     launches += g_last_launches;
+    plan->lg_split = lg_split;
+    plan->bwd_scratch = ch.scratch_bytes;
     if (!ok(cudaStreamWaitEvent(s, ss->e_qkv[c], 0))) rc = PP_ERR_CUDA;
     if (rc == PP_OK) {
       rc = pp_attn_fwd(plan, base + a.q + qo, base + a.k + ko, base + a.v + ko, softmax_scale,

@@ -35,6 +35,9 @@ struct BwdParams {
   __nv_bfloat16* dv;
   int T, Hq, Hkv;
   float scale, scale_log2;
+  // where units are cut into parts
+  float4* parts;       // dV, dK of the parts [part][2][D / 4][128 rows]
+  int lg_split;        // log2 of the parts per unit
 };
 
 // ---------------------------------------------------------------- preprocess
@@ -107,17 +110,62 @@ bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* 
 }
 
 // ---------------------------------------------------------------- finalize
+// dQ = bf16(scale * accumulator) in the first `dq_blocks` blocks; where units are cut into parts,
+// the blocks behind them add up the parts of a (backward tile, KV head), 32 rows of dV or dK each.
+struct SumParts {
+  const float4* parts;
+  const int32_t* header;
+  const BTile* tiles;
+  __nv_bfloat16* dk;
+  __nv_bfloat16* dv;
+  int lg_split, Hkv, D;
+};
+
 __global__ void __launch_bounds__(256)
-bwd_finalize_kernel(const float4* __restrict__ acc, uint2* __restrict__ dq, size_t n4, float scale) {
+bwd_finalize_kernel(const float4* __restrict__ acc, uint2* __restrict__ dq, size_t n4, float scale,
+                    unsigned dq_blocks, SumParts sp) {
   launch_dependents();
-  size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const size_t stride = size_t(gridDim.x) * blockDim.x;
-  for (; i < n4; i += stride) {
-    float4 a = acc[i];
-    uint2 w;
-    w.x = pack_bf16(a.x * scale, a.y * scale);
-    w.y = pack_bf16(a.z * scale, a.w * scale);
-    dq[i] = w;
+  if (blockIdx.x < dq_blocks) {
+    size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    const size_t stride = size_t(dq_blocks) * blockDim.x;
+    for (; i < n4; i += stride) {
+      float4 a = acc[i];
+      uint2 w;
+      w.x = pack_bf16(a.x * scale, a.y * scale);
+      w.y = pack_bf16(a.z * scale, a.w * scale);
+      dq[i] = w;
+    }
+    return;
+  }
+  __shared__ uint2 s_out[32][33];
+  const int b = int(blockIdx.x - dq_blocks), quarter = b & 3, which = (b >> 2) & 1, unit = b >> 3;
+  const int tidx = unit / sp.Hkv, kvh = unit - tidx * sp.Hkv;
+  if (sp.header[0] != kStatusOk || tidx >= sp.header[kHdrNumBTiles]) return;
+  const BTile tile = sp.tiles[tidx];
+  const int rows = min(32, tile.len - 32 * quarter), c4s = sp.D / 4;
+  if (rows <= 0) return;
+  const int lane = threadIdx.x & 31;
+  const float f = which ? scale : 1.f;
+  for (int c = threadIdx.x >> 5; c < c4s; c += 8) {
+    const float4* src = sp.parts + ((size_t(unit) << sp.lg_split) * 2 + which) * (c4s * kTile) +
+                        c * kTile + 32 * quarter + lane;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int p = 0; p < (1 << sp.lg_split); ++p) {
+      const float4 x = src[size_t(p) * 2 * c4s * kTile];
+      s.x += x.x;
+      s.y += x.y;
+      s.z += x.z;
+      s.w += x.w;
+    }
+    s_out[lane][c] = make_uint2(pack_bf16(s.x * f, s.y * f), pack_bf16(s.z * f, s.w * f));
+  }
+  __syncthreads();
+  __nv_bfloat16* out = which ? sp.dk : sp.dv;
+  for (int i = threadIdx.x; i < rows * c4s; i += blockDim.x) {
+    const int r = i / c4s, c = i - r * c4s;
+    *reinterpret_cast<uint2*>(out + ((size_t(tile.start) + 32 * quarter + r) * sp.Hkv + kvh) * sp.D + 4 * c) =
+        s_out[r][c];
   }
 }
 
@@ -191,6 +239,7 @@ struct BwdSmem {
 struct BwdUnit {
   BTile tile;
   int kvh, nq, n_it, tidx;
+  int part, h0, nh;   // part of the unit: query heads [h0, h0 + nh) of the KV head
 };
 
 // Units are handed out dynamically: the producer warp draws the next index of the plan's
@@ -200,15 +249,33 @@ struct BwdUnit {
 // plan can be used by any number of launches without a memset in between.
 constexpr int kHdrBwdNext = 5, kHdrBwdDone = 7;
 
-// `packed` = (kv head << 24) | backward tile, negative at the end of the work list.
+// `packed` = (kv head << 24) | backward tile, negative at the end of the work list; with units cut
+// into parts also (part << kPartShift).  (kSplit is a template parameter all the way down: with the
+// parts' heads worked out at run time, steps whose units stay whole lost 1 - 4 % to other code
+// around the issue loops.)
+template <bool kSplit>
 __device__ __forceinline__ bool get_bwd_unit(const BwdParams& prm, int packed, BwdUnit& un) {
   if (packed < 0) return false;
   un.kvh = packed >> 24;
-  un.tidx = packed & 0xffffff;
+  un.tidx = packed & (kSplit ? (1 << kPartShift) - 1 : 0xffffff);
   un.tile = prm.tiles[un.tidx];
   un.nq = un.tile.work;
-  un.n_it = un.nq * (prm.Hq / prm.Hkv);
+  if (kSplit) {
+    const int heads = prm.Hq / prm.Hkv;
+    un.part = (packed >> kPartShift) & ((1 << (24 - kPartShift)) - 1);
+    un.h0 = (heads * un.part) >> prm.lg_split;
+    un.nh = ((heads * (un.part + 1)) >> prm.lg_split) - un.h0;
+    un.h0 += un.kvh * heads;
+    un.n_it = un.nq * un.nh;
+  } else {
+    un.n_it = un.nq * (prm.Hq / prm.Hkv);
+  }
   return true;
+}
+// query heads the (part of the) unit walks
+template <bool kSplit>
+__device__ __forceinline__ int unit_heads(const BwdParams& prm, const BwdUnit& un) {
+  return kSplit ? un.nh : prm.Hq / prm.Hkv;
 }
 
 // Query tile qt of a unit: tile qt of the group's 128-token grid counted from the key tile
@@ -244,9 +311,10 @@ __device__ __forceinline__ void q_advance(QIter& s, int heads, int nq) {
     }
   }
 }
+template <bool kSplit>
 __device__ __forceinline__ QTile q_tile_at(const BwdParams& prm, const BwdUnit& un, const QIter& s) {
   QTile q;
-  q.h = un.kvh * (prm.Hq / prm.Hkv) + s.hh;
+  q.h = kSplit ? un.h0 + s.hh : un.kvh * (prm.Hq / prm.Hkv) + s.hh;
   q.start = un.tile.start + s.qt * kTile;
   q.len = min(kTile, un.tile.grp_end - q.start);
   return q;
@@ -255,7 +323,7 @@ __device__ __forceinline__ QTile q_tile_at(const BwdParams& prm, const BwdUnit& 
 // D: head dimension of the shared-memory tiles; DV <= D: head dimension of the tensors in
 // global memory (96 in tiles of 128: the TMA loads zero-fill the columns past DV, so only the
 // loops over the head dimension, the N of dV / dK / dQ and global addressing know about DV).
-template <int D, bool kDet, int DV = D>
+template <int D, bool kDet, bool kSplit, int DV = D>
 __global__ void __launch_bounds__(kBwdThreads, 1)
 bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
            const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
@@ -336,7 +404,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     BwdUnit un;
     // (a refused plan has no work)
     const int num_units = prm.header[0] == kStatusOk ? prm.header[kHdrNumBTiles] * prm.Hkv : 0;
-    // all lanes: draw the n-th unit of this CTA, publish it to the other roles
+    const int num_parts = kSplit ? num_units << prm.lg_split : num_units;
+    // all lanes: draw the n-th (part of a) unit of this CTA, publish it to the other roles
     auto fetch_unit = [&](uint32_t n) -> int {
       int packed = -1;
       if (lane == 0) {
@@ -344,16 +413,18 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         // after a wait has given up, no more work is drawn: the end marker goes out instead
         // (The first unit is the one of the CTA's own index.  Not in the deterministic variant: a
         // CTA that starts late must not hold a unit that running CTAs wait for.)
-        const int u = *abort_flag        ? num_units
+        const int u = *abort_flag        ? num_parts
                       : !kDet && n == 0 ? int(blockIdx.x)
                                          : (kDet ? 0 : int(gridDim.x)) + atomicAdd(&prm.header[kHdrBwdNext], 1);
-        if (u < num_units) packed = prm.order[u];
+        if (u < num_parts)
+          packed = kSplit ? prm.order[u >> prm.lg_split] | (u & ((1 << prm.lg_split) - 1)) << kPartShift
+                          : prm.order[u];
         sched[n & 1] = packed;
         mbar_arrive(bar(kSchedFull + (n & 1)));
       }
       return __shfl_sync(0xffffffffu, packed, 0);
     };
-    for (; get_bwd_unit(prm, fetch_unit(ucnt), un); ++ucnt) {
+    for (; get_bwd_unit<kSplit>(prm, fetch_unit(ucnt), un); ++ucnt) {
       if (lane == 0) {
         wait_bar(bar(kKvEmpty), (ucnt & 1) ^ 1, abort_flag, prm.header, 50);
         mbar_expect_tx(bar(kKvFull), 2 * L::kTileBytes);
@@ -363,8 +434,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         }
       }
       QIter qi;
-      for (int it = 0; it < un.n_it && !*abort_flag; ++it, ++qc, q_advance<kDet>(qi, prm.Hq / prm.Hkv, un.nq)) {
-        const QTile qt = q_tile_at(prm, un, qi);
+      for (int it = 0; it < un.n_it && !*abort_flag; ++it, ++qc, q_advance<kDet>(qi, unit_heads<kSplit>(prm, un), un.nq)) {
+        const QTile qt = q_tile_at<kSplit>(prm, un, qi);
         const uint32_t st = qc & 1, par = ((qc >> 1) & 1) ^ 1;
         // per-query statistics, fetched before the stage is known to be free and handed on
         // NEGATED (the compute warps add them in packed two-lane instructions);
@@ -420,11 +491,11 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
           mma_ss(tmem + tS, dK_k + kmajor_off(k), dq_k + kmajor_off(k), idesc, k > 0);
         mma_commit(bar(kSFullB));
       };
-      for (; get_bwd_unit(prm, take_unit(ucnt, false), un); ++ucnt) {
+      for (; get_bwd_unit<kSplit>(prm, take_unit(ucnt, false), un); ++ucnt) {
         const int ksteps = (un.tile.len + 15) >> 4;
         wait_bar(bar(kKvFull), ucnt & 1, abort_flag, prm.header, 60);
         QIter qi;
-        QTile qt = q_tile_at(prm, un, qi);
+        QTile qt = q_tile_at<kSplit>(prm, un, qi);
         wait_bar(bar(kQFullB + (gc & 1)), (gc >> 1) & 1, abort_flag, prm.header, 61);
         tc_fence_after();
         issue_s(gc & 1, qt.len);
@@ -449,8 +520,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
           QTile nx = qt;
           const bool has_next = it + 1 < un.n_it;
           if (has_next) {
-            q_advance<kDet>(qi, prm.Hq / prm.Hkv, un.nq);
-            nx = q_tile_at(prm, un, qi);
+            q_advance<kDet>(qi, unit_heads<kSplit>(prm, un), un.nq);
+            nx = q_tile_at<kSplit>(prm, un, qi);
           }
           const uint32_t idesc_s_next = make_idesc(128, ((nx.len + 15) >> 4) << 4, 0, 0);
           const uint32_t dq_k_next = kmajor_base(sQ) + ((g + 1) & 1) * kStageStep;
@@ -534,14 +605,14 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const uint32_t ds_row = sdS + wg * kBoxBytes + row * 128;   // dS^T row `row` in box wg
     uint32_t gc = 0, ucnt = 0;
     BwdUnit un;
-    for (; get_bwd_unit(prm, take_unit(ucnt, true), un); ++ucnt) {
+    for (; get_bwd_unit<kSplit>(prm, take_unit(ucnt, true), un); ++ucnt) {
       const bool row_ok = row < un.tile.len;
       // my key j = tile.start + row is seen by the queries [j, key_end[j])
       const int key_lo = un.tile.start + row;
       const int key_hi = row_ok ? prm.key_end[key_lo] : key_lo;
       QIter qi;
-      for (int it = 0; it < un.n_it; ++it, q_advance<kDet>(qi, prm.Hq / prm.Hkv, un.nq)) {
-        const QTile qt = q_tile_at(prm, un, qi);
+      for (int it = 0; it < un.n_it; ++it, q_advance<kDet>(qi, unit_heads<kSplit>(prm, un), un.nq)) {
+        const QTile qt = q_tile_at<kSplit>(prm, un, qi);
         const uint32_t g = gc + it, st = g & 1, par = g & 1;
         const float* sl = stats + st * 256 + cb;
         // Fast path: both tiles complete and every key row of this warp sees either the whole
@@ -661,6 +732,24 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
       // ---- unit epilogue: warpgroup 0 stores dV, warpgroup 1 stores scale * dK
       wait_bar(bar(kDkvFull), ucnt & 1, abort_flag, prm.header, 73);
       tc_fence_after();
+      if constexpr (kSplit) {   // a part: fp32, 128 rows side by side per four columns
+        const size_t slot = (size_t(un.tidx) * prm.Hkv + un.kvh) << prm.lg_split | size_t(un.part);
+        float4* dst = prm.parts + (slot * 2 + wg) * (DV / 4 * kTile) + row;
+#pragma unroll 1
+        for (int c = 0; c < DV / 16; ++c) {
+          uint32_t w[16];
+          tmem_ld16(lane_base + (wg ? tdK : tdV) + c * 16, w);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            dst[(c * 4 + i) * kTile] = make_float4(__uint_as_float(w[4 * i]), __uint_as_float(w[4 * i + 1]),
+                                                   __uint_as_float(w[4 * i + 2]), __uint_as_float(w[4 * i + 3]));
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(kDkvFree));
+        continue;
+      }
       const uint32_t tsrc = wg ? tdK : tdV;
       const float f = wg ? prm.scale : 1.f;
       uint32_t ob[D / 2];
@@ -736,7 +825,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const uint32_t stg = base + L::kStg + (warp - 12) * (2 * L::kStageBytes);
     uint32_t gc = 0, chunk = 0, ucnt = 0;
     BwdUnit un;
-    for (; get_bwd_unit(prm, take_unit(ucnt, true), un); ++ucnt) {
+    for (; get_bwd_unit<kSplit>(prm, take_unit(ucnt, true), un); ++ucnt) {
       QIter qi;
       // Deterministic variant: the key tiles that add to a (query tile, head) do so in
       // DESCENDING tile order: the query tile's own key tile first, then the tiles below it
@@ -764,8 +853,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         const int mine = k_rel + 1;
         asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(mine) : "memory");
       };
-      for (int it = 0; it < un.n_it; ++it, q_advance<kDet>(qi, prm.Hq / prm.Hkv, un.nq)) {
-        const QTile qt = q_tile_at(prm, un, qi);
+      for (int it = 0; it < un.n_it; ++it, q_advance<kDet>(qi, unit_heads<kSplit>(prm, un), un.nq)) {
+        const QTile qt = q_tile_at<kSplit>(prm, un, qi);
         const uint32_t g = gc + it;
         int32_t* sem = nullptr;
         int seen_early = -1;
@@ -912,15 +1001,15 @@ cudaError_t launch_bwd_t(const pp_plan* plan, const void* o, const float* lse, c
   DeviceSetup* dev = device_setup(setup);
   if (!dev) return cudaErrorInvalidDevice;
   if (dev->cc_major != 10) return cudaErrorNotSupported;
-  auto kern = prm.dq_sem ? bwd_kernel<D, true, DV> : bwd_kernel<D, false, DV>;
+  using Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, BwdParams);
+  const Kernel kerns[4] = {bwd_kernel<D, false, false, DV>, bwd_kernel<D, false, true, DV>,
+                           bwd_kernel<D, true, false, DV>, bwd_kernel<D, true, true, DV>};
+  const Kernel kern = kerns[(prm.dq_sem ? 2 : 0) + (prm.lg_split ? 1 : 0)];
   if (!dev->configured) {
-    cudaError_t e = cudaFuncSetAttribute(bwd_kernel<D, false, DV>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         BwdSmem<D>::kTotal);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(bwd_kernel<D, true, DV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               BwdSmem<D>::kTotal);
-    if (e != cudaSuccess) return e;
+    for (Kernel k : kerns) {
+      cudaError_t ce = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<D>::kTotal);
+      if (ce != cudaSuccess) return ce;
+    }
     dev->configured = true;
   }
   const pp_problem& pb = plan->prob;
@@ -932,7 +1021,7 @@ cudaError_t launch_bwd_t(const pp_plan* plan, const void* o, const float* lse, c
       static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse,
       const_cast<float*>(prm.delta), const_cast<float*>(prm.lse2), prm.dq_acc, int(T), int(Hq));
   cudaError_t e = cudaGetLastError();
-  const long long units = (long long)plan->max_tiles * pb.num_kv_heads;
+  const long long units = ((long long)plan->max_tiles * pb.num_kv_heads) << prm.lg_split;
   dim3 grid(unsigned(std::min<long long>(units, num_sms)));
   ProfileEvents& ev = profile_events();
   const int slot = int(ev.bwd_count % kProfileRing);
@@ -946,8 +1035,10 @@ cudaError_t launch_bwd_t(const pp_plan* plan, const void* o, const float* lse, c
   }
   const size_t n4 = T * Hq * DV / 4;
   unsigned fb = unsigned(std::min<size_t>((n4 + 255) / 256, size_t(num_sms) * 16));
-  bwd_finalize_kernel<<<fb, 256, 0, stream>>>(reinterpret_cast<const float4*>(prm.dq_acc),
-                                              static_cast<uint2*>(dq), n4, prm.scale);
+  const SumParts sp = {prm.parts, prm.header, prm.tiles, prm.dk, prm.dv, prm.lg_split, pb.num_kv_heads, DV};
+  const unsigned sum_blocks = prm.lg_split ? unsigned(plan->max_tiles) * pb.num_kv_heads * 8 : 0;
+  bwd_finalize_kernel<<<fb + sum_blocks, 256, 0, stream>>>(
+      reinterpret_cast<const float4*>(prm.dq_acc), static_cast<uint2*>(dq), n4, prm.scale, fb, sp);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (launches) *launches += 3;
   return e;
@@ -957,8 +1048,8 @@ cudaError_t launch_bwd_t(const pp_plan* plan, const void* o, const float* lse, c
 
 cudaError_t launch_bwd(const pp_plan* plan, const void* q, const void* k, const void* v,
                        const void* o, const float* lse, const void* d_o, float scale, void* dq,
-                       void* dk, void* dv, void* scratch, bool dq_cleared, bool deterministic,
-                       cudaStream_t stream, int* launches) {
+                       void* dk, void* dv, void* scratch, int lg_split, bool dq_cleared,
+                       bool deterministic, cudaStream_t stream, int* launches) {
   const pp_problem& pb = plan->prob;
   CUtensorMap tq, tk, tv, tdo;
   if (!encode_thd(&tq, q, pb.total_tokens, pb.num_q_heads, pb.head_dim, kTile) ||
@@ -966,7 +1057,7 @@ cudaError_t launch_bwd(const pp_plan* plan, const void* q, const void* k, const 
       !encode_thd(&tv, v, pb.total_tokens, pb.num_kv_heads, pb.head_dim, kTile) ||
       !encode_thd(&tdo, d_o, pb.total_tokens, pb.num_q_heads, pb.head_dim, kTile))
     return cudaErrorNotSupported;
-  BwdScratch sl = bwd_scratch_layout(pb);
+  const BwdScratch sl = bwd_scratch_layout(pb, lg_split);
   char* sc = static_cast<char*>(scratch);
   BwdParams prm;
   prm.header = reinterpret_cast<int32_t*>(plan->ws + plan->lay.header);
@@ -977,6 +1068,8 @@ cudaError_t launch_bwd(const pp_plan* plan, const void* q, const void* k, const 
   prm.delta = reinterpret_cast<float*>(sc + sl.delta);
   prm.lse2 = reinterpret_cast<float*>(sc + sl.lse2);
   prm.dq_acc = reinterpret_cast<float*>(sc + sl.dq_acc);
+  prm.parts = reinterpret_cast<float4*>(sc + sl.parts);
+  prm.lg_split = lg_split;
   prm.dq_sem = nullptr;
   if (deterministic) {
     prm.dq_sem = reinterpret_cast<int32_t*>(sc + sl.sem);
@@ -1045,8 +1138,9 @@ cudaError_t launch_bwd_static(const pp_plan* plan, const void* q, const void* k,
   if (e != cudaSuccess) return e;
   // launch_bwd zeroes the fp32 dQ accumulator inside the scratch on every call and rewrites
   // Delta and the scaled LSE, so nothing of an earlier call's contents is read.
-  return launch_bwd(plan, q, k, v, o, lse, d_o, scale, dq, dk, dv, scratch, false, false, stream,
-                    launches);
+  const int lg_split = plan->bwd_scratch <= kStaticScratchBytes ? plan->lg_split : 0;
+  return launch_bwd(plan, q, k, v, o, lse, d_o, scale, dq, dk, dv, scratch, lg_split, false, false,
+                    stream, launches);
 }
 
 }  // namespace pp

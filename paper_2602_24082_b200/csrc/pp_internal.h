@@ -87,6 +87,7 @@ struct pp_plan {
   pp::PlanLayout lay;
   // scratch sizes
   size_t fwd_scratch, bwd_scratch;
+  int lg_split;   // log2 of the parts each backward unit is cut into (bwd_split_log2)
   // backward scratch whose dQ accumulator the latest forward on this plan has cleared
   mutable const void* cleared_scratch = nullptr;
 };
@@ -128,11 +129,45 @@ inline PlanLayout plan_layout(const pp_problem& p) {
 
 // Backward scratch: fp32 dQ accumulator [T][Hq][D], Delta [Hq][T], LSE*log2(e) [Hq][T], and
 // the turn counters of the deterministic variant, four per (query tile of the backward grid,
-// query head): one for each warp's 32 rows
+// query head): one for each warp's 32 rows; and, where units are cut into
+// parts (below), the parts' fp32 dV and dK tiles.
 struct BwdScratch {
-  size_t dq_acc, delta, lse2, sem, sem_bytes, total;
+  size_t dq_acc, delta, lse2, sem, sem_bytes, parts, total;
 };
-inline BwdScratch bwd_scratch_layout(const pp_problem& p) {
+
+// A backward unit (a key tile and KV head against every (query tile, query head) that sees them)
+// is a serial chain, so in small batches a few CTAs run long ones while the others idle: eight heads
+// on one KV head and a 276-token group make three units of up to 24 iterations.  There each unit is
+// cut into 2^n parts by query heads, which CTAs process independently; each part leaves its dV and
+// dK in fp32 in the scratch and the finalize kernel adds them up in order.  n minimises the
+// estimated time in iterations, the longer of the longest part and everything's share per SM, with
+// two iterations of overhead for a unit and three for a part; it depends on sizes alone, so that
+// every way of running a problem sums in the same order.  Whole steps, units whole -> cut (us):
+// 276 tokens, 8 heads on 1 KV head 99 -> 56; 573, 32 on 4 102 -> 53; 8999, 7 on 1 183 -> 114; 3999,
+// 4 on 1 in one group 251 -> 113; 2753, 2 on 1 50 -> 44.  From about 148 units' worth of balanced
+// work on, parts only add their overhead and fp32 traffic, and the rule leaves units whole.
+constexpr int kPartShift = 21;   // tile, part and KV head of a part in one word: 21, 3 and 7 bits
+inline int bwd_split_log2(const pp_problem& p) {
+  const int heads = p.num_q_heads / p.num_kv_heads;
+  const double r = heads, groups = p.num_groups;
+  const double m = double((p.total_tokens / p.num_groups + kTile - 1) / kTile);   // tiles of a mean group
+  const double units = (p.total_tokens / double(kTile) + groups / 2) * p.num_kv_heads;
+  const double longest = r * m * (p.num_groups > 1 ? 1.5 : 1.0);
+  const double total = units * r * (m + 1) / 2;
+  int best = 0;
+  double best_time = 0;
+  for (int n = 0; n <= 3 && (1 << n) <= heads && max_tiles_of(p) < (1 << kPartShift); ++n) {
+    const double parts = units * (1 << n), share = (total + (n ? 3 : 2) * parts) / 148;
+    const double time = share > longest / (1 << n) + 2 ? share : longest / (1 << n) + 2;
+    if (n == 0 || time < 0.95 * best_time) {
+      best = n;
+      best_time = time;
+    }
+  }
+  return best;
+}
+
+inline BwdScratch bwd_scratch_layout(const pp_problem& p, int lg_split) {
   BwdScratch s{};
   size_t T = p.total_tokens, Hq = p.num_q_heads, D = p.head_dim;
   size_t off = 0;
@@ -142,9 +177,15 @@ inline BwdScratch bwd_scratch_layout(const pp_problem& p) {
   s.sem = off;
   s.sem_bytes = 16 * size_t(max_tiles_of(p)) * Hq;
   off = align_up(off + s.sem_bytes, 256);
+  s.parts = off;
+  if (lg_split) {
+    const size_t parts = size_t(max_tiles_of(p)) * p.num_kv_heads << lg_split;
+    off = align_up(off + parts * 2 * kTile * D * 4, 256);
+  }
   s.total = off;
   return s;
 }
+inline BwdScratch bwd_scratch_layout(const pp_problem& p) { return bwd_scratch_layout(p, bwd_split_log2(p)); }
 
 // Device arena of pp_attn_step_host: inputs, outputs, plan workspace, backward scratch.  The
 // step is cut into at most kStepChunks runs of whole groups, each with its own plan, scratch and
@@ -256,8 +297,8 @@ cudaError_t launch_fwd(const pp_plan* plan, const void* q, const void* k, const 
                        void* o, float* lse, float* dq_clear, cudaStream_t stream, int* launches);
 cudaError_t launch_bwd(const pp_plan* plan, const void* q, const void* k, const void* v,
                        const void* o, const float* lse, const void* d_o, float scale, void* dq,
-                       void* dk, void* dv, void* scratch, bool dq_cleared, bool deterministic,
-                       cudaStream_t stream, int* launches);
+                       void* dk, void* dv, void* scratch, int lg_split, bool dq_cleared,
+                       bool deterministic, cudaStream_t stream, int* launches);
 
 // Row builder (csrc/pp_rows.cu).
 size_t rows_workspace_bytes(int num_groups);

@@ -916,7 +916,8 @@ cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cu
   static DeviceSetup setup[kMaxDevices];
   DeviceSetup* dev = device_setup(setup);
   if (!dev) return cudaErrorInvalidDevice;
-  p.det_asc_max = std::min(48, dev->num_sms / 3);
+  // (a set of the backward is held up with all its parts)
+  p.det_asc_max = std::min(48, dev->num_sms / 3) >> plan->lg_split;
   p.num_rows = plan->prob.num_rows;
   p.G = plan->prob.num_groups;
   p.N = plan->prob.num_responses;
