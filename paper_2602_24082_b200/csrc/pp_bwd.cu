@@ -47,7 +47,11 @@ struct BwdParams {
 // memory: D / 8 lanes per row with 16-byte loads, kUnroll rows per lane group in flight.  A warp
 // takes kUnroll * kRows consecutive tokens of one head, so that the statistics [Hq][T] leave as
 // one store of consecutive words; the block index runs over the heads fastest, so that the blocks
-// running at the same time read whole tokens of [T][Hq][D].  No row index is divided: a version
+// running at the same time read whole tokens of [T][Hq][D].  Without the clearing the
+// tokens go from the last to the first, so that the end of O that the forward left in L2 is read
+// before it is evicted, and O, not read again in the step, is marked evict-first: in a step, 33.8
+// -> 27.6 us at T = 9241, Hq = 32, D = 128 (151 MB, part of it from L2), 101 -> 92 at T = 16384,
+// Hq = 64 (with the clearing, beyond 640 MB, either cost 2 %).  No row index is divided: a version
 // that derived (token, head) from a 64-bit row number, two divisions per row and lane, took 40 us
 // where this takes 30 (T = 9241, Hq = 32, D = 128: 151 MB), 129 against 92 at T = 16384, Hq = 64,
 // and with the clearing 488 against 330 at T = 65536, Hq = 32 (2.1 GB, 6.5 TB/s).
@@ -66,7 +70,7 @@ bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* 
   constexpr int kLanes = pre_lanes(D);    // lanes per row (D / 8 of them hold data)
   constexpr int kRows = 32 / kLanes;      // rows per warp and step
   const int lane = threadIdx.x & 31, sub = lane % kLanes, rin = lane / kLanes;
-  const int chunk = blockIdx.x / Hq, h = blockIdx.x - chunk * Hq;
+  const int block = int(kClear ? blockIdx.x : gridDim.x - 1 - blockIdx.x), chunk = block / Hq, h = block - chunk * Hq;
   const int t0 = chunk * pre_tokens(D) + (threadIdx.x >> 5) * (kPreUnroll * kRows);
   // lane (rin, sub = u) writes the statistics of token t0 + u * kRows + rin
   const int t_stat = t0 + sub * kRows + rin;
@@ -79,7 +83,8 @@ bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* 
   for (int u = 0; u < kPreUnroll; ++u) {
     a[u] = b[u] = make_uint4(0u, 0u, 0u, 0u);
     if (t0 + u * kRows + rin < T && sub < D / 8) {
-      a[u] = *reinterpret_cast<const uint4*>(o + row0 + u * step);
+      const uint4* po = reinterpret_cast<const uint4*>(o + row0 + u * step);
+      a[u] = kClear ? *po : __ldcs(po);
       b[u] = *reinterpret_cast<const uint4*>(d_o + row0 + u * step);
     }
   }
@@ -110,8 +115,14 @@ bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* 
 }
 
 // ---------------------------------------------------------------- finalize
-// dQ = bf16(scale * accumulator) in the first `dq_blocks` blocks; where units are cut into parts,
-// the blocks behind them add up the parts of a (backward tile, KV head), 32 rows of dV or dK each.
+// dQ = bf16(scale * accumulator) in the first `dq_blocks` blocks: a stream bound by memory, four
+// 16-byte loads per thread in flight and, as neither side is read again here, both marked
+// evict-first, which leaves more of the accumulator's tail from the backward in L2.  T = 9241,
+// Hq = 32, D = 128 (227 MB): 44 us with one load per thread and a grid-stride loop, 38 / 33 with
+// 2 / 4 loads, 30 with the hints (7.5 TB/s, part of it from L2); T = 16384, Hq = 64: 154 -> 116.
+// Where units are cut into parts, the blocks behind these add up the parts of a (backward tile, KV
+// head), 32 rows of dV or dK each.
+constexpr int kFinUnroll = 4;
 struct SumParts {
   const float4* parts;
   const int32_t* header;
@@ -126,15 +137,19 @@ bwd_finalize_kernel(const float4* __restrict__ acc, uint2* __restrict__ dq, size
                     unsigned dq_blocks, SumParts sp) {
   launch_dependents();
   if (blockIdx.x < dq_blocks) {
-    size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    const size_t stride = size_t(dq_blocks) * blockDim.x;
-    for (; i < n4; i += stride) {
-      float4 a = acc[i];
-      uint2 w;
-      w.x = pack_bf16(a.x * scale, a.y * scale);
-      w.y = pack_bf16(a.z * scale, a.w * scale);
-      dq[i] = w;
-    }
+    const size_t i0 = size_t(blockIdx.x) * (256 * kFinUnroll) + threadIdx.x;
+    float4 a[kFinUnroll];
+#pragma unroll
+    for (int u = 0; u < kFinUnroll; ++u)
+      if (i0 + u * 256 < n4) a[u] = __ldcs(acc + i0 + u * 256);
+#pragma unroll
+    for (int u = 0; u < kFinUnroll; ++u)
+      if (i0 + u * 256 < n4) {
+        uint2 w;
+        w.x = pack_bf16(a[u].x * scale, a[u].y * scale);
+        w.y = pack_bf16(a[u].z * scale, a[u].w * scale);
+        __stcs(dq + i0 + u * 256, w);
+      }
     return;
   }
   __shared__ uint2 s_out[32][33];
@@ -1034,7 +1049,7 @@ cudaError_t launch_bwd_t(const pp_plan* plan, const void* o, const float* lse, c
     ++ev.bwd_count;
   }
   const size_t n4 = T * Hq * DV / 4;
-  unsigned fb = unsigned(std::min<size_t>((n4 + 255) / 256, size_t(num_sms) * 16));
+  unsigned fb = unsigned((n4 + 256 * kFinUnroll - 1) / (256 * kFinUnroll));
   const SumParts sp = {prm.parts, prm.header, prm.tiles, prm.dk, prm.dv, prm.lg_split, pb.num_kv_heads, DV};
   const unsigned sum_blocks = prm.lg_split ? unsigned(plan->max_tiles) * pb.num_kv_heads * 8 : 0;
   bwd_finalize_kernel<<<fb + sum_blocks, 256, 0, stream>>>(
