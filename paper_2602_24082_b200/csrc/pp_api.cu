@@ -87,8 +87,10 @@ int pp_plan_workspace_bytes(const pp_problem* problem, size_t* plan_bytes,
   return PP_OK;
 }
 
-int pp_build_plan(const pp_problem* problem, void* d_workspace, size_t workspace_bytes,
-                  pp_stream_t stream, pp_plan** out_plan) {
+// `whole`: the problem whose sizes choose how the kernels cut their work (a run of the host step
+// takes the choices of the step, so that its sums are the same, bit for bit).
+static int build_plan(const pp_problem* problem, const pp_problem* whole, void* d_workspace,
+                      size_t workspace_bytes, pp_stream_t stream, pp_plan** out_plan) {
   if (!out_plan) return PP_ERR_INVALID_ARG;
   *out_plan = nullptr;
   int rc = check_problem_shape(problem);
@@ -114,7 +116,8 @@ int pp_build_plan(const pp_problem* problem, void* d_workspace, size_t workspace
   plan->ws = static_cast<char*>(d_workspace);
   plan->lay = lay;
   plan->fwd_scratch = 0;
-  plan->lg_split = pp::bwd_split_log2(*problem);
+  plan->mixed = pp::fwd_mixed_tiles(*whole);
+  plan->lg_split = pp::bwd_split_log2(*whole);
   plan->bwd_scratch = pp::bwd_scratch_layout(*problem, plan->lg_split).total;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
 
@@ -139,6 +142,11 @@ int pp_build_plan(const pp_problem* problem, void* d_workspace, size_t workspace
   }
   *out_plan = plan;
   return PP_OK;
+}
+
+int pp_build_plan(const pp_problem* problem, void* d_workspace, size_t workspace_bytes,
+                  pp_stream_t stream, pp_plan** out_plan) {
+  return build_plan(problem, problem, d_workspace, workspace_bytes, stream, out_plan);
 }
 
 int pp_plan_status(const pp_plan* plan, pp_stream_t stream, int32_t* status, int32_t* detail) {
@@ -520,7 +528,6 @@ int pp_attn_step_host(const pp_problem* problem, const void* h_q, const void* h_
   // directions) while the kernels of run c execute.  Inside a run dO still goes up behind
   // the forward and O / LSE come down behind the backward.
   std::vector<StepChunk> chunks = cut_step(*problem, step_runs_wanted(*problem));
-  // (the parts of backward units are those of the whole problem: same sums, bit for bit)
   const int lg_split = pp::bwd_split_log2(*problem);
   if (!place_step(chunks, a, Hq, lg_split)) {
     chunks = cut_step(*problem, 1);
@@ -555,11 +562,9 @@ int pp_attn_step_host(const pp_problem* problem, const void* h_q, const void* h_
     const size_t qb = tc * Hq * D * 2, kb = tc * Hkv * D * 2;
     float* d_lse = reinterpret_cast<float*>(base + ch.lse_off);
     pp_plan* plan = nullptr;
-    rc = pp_build_plan(&ch.prob, base + ch.plan_off, ch.plan_bytes, stream, &plan);
+    rc = build_plan(&ch.prob, problem, base + ch.plan_off, ch.plan_bytes, stream, &plan);
     if (rc) break;
     launches += g_last_launches;
-    plan->lg_split = lg_split;
-    plan->bwd_scratch = ch.scratch_bytes;
     if (!ok(cudaStreamWaitEvent(s, ss->e_qkv[c], 0))) rc = PP_ERR_CUDA;
     if (rc == PP_OK) {
       rc = pp_attn_fwd(plan, base + a.q + qo, base + a.k + ko, base + a.v + ko, softmax_scale,

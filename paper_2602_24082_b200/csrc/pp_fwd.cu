@@ -19,6 +19,7 @@
 // its MN-major B operand straight from the TMA layout.  O is rescaled lazily: only when a
 // row's running maximum grew by more than 2^8 since the value used for scaling.
 // TMEM: S0 | S1 | O0 | O1, 128 columns each.
+// Query tiles are those of the segments or, with many short ones, mixed tiles (kMixed below).
 #include <algorithm>
 #include <type_traits>
 
@@ -29,8 +30,10 @@ namespace {
 
 struct FwdParams {
   int32_t* header;
-  const Tile* tiles;
-  const int32_t* order;
+  const Tile* tiles;       // tiles of the segments
+  const QTile* qtiles;     // (mixed tiles)
+  const int32_t* key_end;  // (mixed tiles)
+  const int32_t* order;    // the tiles, longest work first
   __nv_bfloat16* o;
   float* lse;
   float* dq_clear;  // optional: the backward's fp32 dQ accumulator [T][Hq][D], cleared here
@@ -72,7 +75,8 @@ struct KvTile {
   bool diag;
 };
 
-__device__ __forceinline__ KvTile kv_tile_of(const Tile& t, int j, int n0, int n1) {
+template <typename T>
+__device__ __forceinline__ KvTile kv_tile_of(const T& t, int j, int n0, int n1) {
   KvTile k;
   if (j < n0) {
     k.start = t.kv0_start + j * kTile;
@@ -90,8 +94,9 @@ __device__ __forceinline__ KvTile kv_tile_of(const Tile& t, int j, int n0, int n
   return k;
 }
 
+template <bool kMixed>
 struct Unit {
-  Tile tile;
+  std::conditional_t<kMixed, QTile, Tile> tile;
   int h0, kvh, nslots, n0, n1, ntiles;
 };
 
@@ -101,7 +106,8 @@ struct Unit {
 // last one resets both counters for the next launch.
 constexpr int kHdrFwdNext = 4, kHdrFwdDone = 6;
 
-__device__ __forceinline__ bool get_unit(const FwdParams& prm, int u, int ntiles_total, Unit& un) {
+template <bool kMixed>
+__device__ __forceinline__ bool get_unit(const FwdParams& prm, int u, int ntiles_total, Unit<kMixed>& un) {
   const int r = prm.Hq / prm.Hkv, npairs = (r + 1) >> 1, per_tile = prm.Hkv * npairs;
   const int ord = u / per_tile;
   if (ord >= ntiles_total) return false;
@@ -110,7 +116,8 @@ __device__ __forceinline__ bool get_unit(const FwdParams& prm, int u, int ntiles
   const int pair = rem - un.kvh * npairs;
   un.h0 = un.kvh * r + 2 * pair;
   un.nslots = (2 * pair + 1 < r) ? 2 : 1;
-  un.tile = prm.tiles[prm.order[ord]];
+  if constexpr (kMixed) un.tile = prm.qtiles[prm.order[ord]];
+  else un.tile = prm.tiles[prm.order[ord]];
   un.n0 = (un.tile.kv0_len + kTile - 1) / kTile;
   un.n1 = (un.tile.kv1_len + kTile - 1) / kTile;
   un.ntiles = un.n0 + un.n1 + 1;
@@ -121,7 +128,10 @@ __device__ __forceinline__ bool get_unit(const FwdParams& prm, int u, int ntiles
 // tensors in global memory.  For DV < D (96 in tiles of 128) the TMA loads fill the columns
 // past DV with zeros, so only the loops over the head dimension, the N of the second GEMM and
 // everything that addresses global memory know about DV.
-template <int D, int DV = D>
+// kMixed: the rows of a query tile may belong to several segments, which changes the masks of its
+// own keys and of the first rows' response.  (A template parameter because the more general masks
+// take registers from the loop: 3.5 % on two rows of 32768 tokens in one instance for all.)
+template <int D, bool kMixed, int DV = D>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
            const __grid_constant__ CUtensorMap tm_v, FwdParams prm) {
@@ -132,7 +142,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
 
   dependency_wait();
   if (prm.header[0] != kStatusOk) return;
-  const int ntiles_total = prm.header[2];
+  const int ntiles_total = prm.header[kMixed ? kHdrNumQTiles : kHdrNumTiles];
 #ifdef PP_DEBUG_COUNTERS
   const long long t_kernel0 = clock64();
 #endif
@@ -171,7 +181,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   // Ring of two decoded unit records (producer -> MMA thread and softmax warps): the producer
   // alone reads the plan's tile list; the other roles get what they need from shared memory.
   volatile int* sched = reinterpret_cast<volatile int*>(gbase + L::kSched);
-  auto fetch_unit = [&](uint32_t n, Unit& un) -> bool {  // producer thread
+  auto fetch_unit = [&](uint32_t n, Unit<kMixed>& un) -> bool {  // producer thread
     wait_bar(bar(kSchedEmptyF + (n & 1)), ((n >> 1) & 1) ^ 1, abort_flag, prm.header, 90);
     // after a wait has given up, no more work is drawn: the end marker goes out instead
     const int u = *abort_flag ? 0x7fffffff
@@ -180,7 +190,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const bool ok = get_unit(prm, u, ntiles_total, un);
     volatile int* e = sched + (n & 1) * 8;
     e[0] = un.tile.start;
-    e[1] = un.tile.len;
+    if constexpr (kMixed) e[1] = un.tile.len | un.tile.first_rows << 8;
+    else e[1] = un.tile.len;
     e[2] = un.h0;
     e[3] = ok ? un.nslots : 0;  // 0 slots marks the end of the work list
     e[4] = un.n0;
@@ -194,7 +205,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
 #define PP_TAKE_UNIT(n, whole_warp)                                                              \
   const bool u_ok = wait_bar(bar(kSchedFullF + ((n) & 1)), ((n) >> 1) & 1, abort_flag, prm.header, 91); \
   const volatile int* u_e = sched + ((n) & 1) * 8;                                               \
-  const int u_start = u_e[0], u_len = u_e[1], u_h0 = u_e[2], u_nslots = u_ok ? u_e[3] : 0;       \
+  const int u_start = u_e[0], u_len1 = u_e[1], u_len = kMixed ? u_len1 & 255 : u_len1, u_h0 = u_e[2], u_nslots = u_ok ? u_e[3] : 0;       \
   const int u_n0 = u_e[4], u_n1 = u_e[5], u_last0 = u_e[6], u_last1 = u_e[7];                    \
   const int u_ntiles = u_n0 + u_n1 + 1;                                                          \
   if (whole_warp) {                                                                              \
@@ -214,7 +225,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     // ------------------------------------------------------------ TMA producer
     if (elect_one()) {
       uint32_t kc = 0, qc[2] = {0, 0};
-      Unit un;
+      Unit<kMixed> un;
       for (uint32_t un_i = 0; fetch_unit(un_i, un); ++un_i) {
         for (int s = 0; s < un.nslots; ++s) {
           wait_bar(bar(kQEmpty + s), (qc[s] & 1) ^ 1, abort_flag, prm.header, 20 + s);
@@ -404,15 +415,48 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
       if (u_nslots == 0) break;
       if (s >= u_nslots) continue;
       float m_used = -INFINITY, l_part = 0.f;
+      // Rows of several segments: of the tile's own keys up to its own position, a row sees the
+      // prompt's, [0, pr), and those of its own segment, from `lo` on.  A segment ends where the
+      // visibility of its keys does.
+      const int u_first = kMixed ? (u_len1 >> 8) & (kQTilePrompt - 1) : u_len;
+      const bool one_segment = !kMixed || u_first == u_len;
+      int pr = 0, lo = 0;
+      if (!one_segment) {
+        int end[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+          end[b] = prm.key_end[u_start + min(32 * b + lane, u_len - 1)];
+        lo = pr = (u_len1 >> 8) & kQTilePrompt ? u_first : 0;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          uint32_t m = __ballot_sync(0xffffffffu, 32 * b + lane < u_len && end[b] == u_start + 32 * b + lane + 1);
+          if (b == qd) m &= (1u << lane) - 1u;   // segments that end before this row
+          if (b <= qd && m) lo = max(lo, 32 * (b + 1) - __clz(m));
+        }
+      }
       for (int j = 0; j < u_ntiles; ++j) {
         KvTile kt;
         kt.len = u_klen(j);
         kt.diag = j + 1 == u_ntiles;
         wait_bar(bar(kSFull + s), tcS & 1, abort_flag, prm.header, 40 + s);
         tc_fence_after();
-        const bool full = !kt.diag && kt.len == kTile;
+        const bool full = !kt.diag && kt.len == kTile && (one_segment || j < u_n0);
         // visible columns of this half: [0, col_lim) in the half's own numbering
-        const int col_lim = (kt.diag ? min(kt.len, row + 1) : kt.len) - 64 * half;
+        const int col_lim = (kt.diag ? min(kt.len, row + 1) : kMixed && j >= u_n0 && row >= u_first ? 0 : kt.len) -
+                            64 * half;
+        uint32_t vis[2];   // mixed tiles: one bit each
+        if (kMixed) {
+          auto below = [&](int x) { return ~__funnelshift_lc(0u, ~0u, max(x, 0)); };   // bits below x
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const int at = 64 * half + 32 * c;
+            vis[c] = below(col_lim - 32 * c);
+            if (kt.diag) vis[c] &= below(pr - at) | ~below(lo - at);
+          }
+        }
+        auto visible = [&](int col) -> bool {
+          return kMixed ? (vis[col >> 5] >> (col & 31)) & 1u : col < col_lim;
+        };
         float* xb = xch + (tcS & 1) * 256 + row * 2;
         // The 64 scores of this thread are handled as two chunks of 32 (fewer live registers).
         // max over the visible scores of one chunk
@@ -427,7 +471,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             return fmaxf(m, m1);
           }
 #pragma unroll
-          for (int i = 0; i < 32; ++i) m = fmaxf(m, 32 * c + i < col_lim ? __uint_as_float(w[i]) : -INFINITY);
+          for (int i = 0; i < 32; ++i) m = fmaxf(m, visible(32 * c + i) ? __uint_as_float(w[i]) : -INFINITY);
           return m;
         };
         float mx = -INFINITY;
@@ -474,9 +518,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
               float x0, x1;
               unpack2(fma2(pack2(__uint_as_float(w[2 * i]), __uint_as_float(w[2 * i + 1])), sc2, nm2), x0, x1);
               float p0 = ex2(x0), p1 = ex2(x1);
-              if (kMasked) {   // columns at and past col_lim are not visible
-                p0 = (16 * piece + 2 * i < col_lim) ? p0 : 0.f;
-                p1 = (16 * piece + 2 * i + 1 < col_lim) ? p1 : 0.f;
+              if (kMasked) {
+                p0 = visible(16 * piece + 2 * i) ? p0 : 0.f;
+                p1 = visible(16 * piece + 2 * i + 1) ? p1 : 0.f;
               }
               sum2 = add2(sum2, pack2(p0, p1));
               if (i & 1) pm1 = max3(pm1, p0, p1); else pm0 = max3(pm0, p0, p1);
@@ -536,8 +580,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
               for (int i = 0; i < 16; ++i) {
                 float p0 = ex2(fmaf(__uint_as_float(w[2 * i]), prm.scale_log2, neg_m));
                 float p1 = ex2(fmaf(__uint_as_float(w[2 * i + 1]), prm.scale_log2, neg_m));
-                p0 = (32 * c + 2 * i < col_lim) ? p0 : 0.f;
-                p1 = (32 * c + 2 * i + 1 < col_lim) ? p1 : 0.f;
+                p0 = visible(32 * c + 2 * i) ? p0 : 0.f;
+                p1 = visible(32 * c + 2 * i + 1) ? p1 : 0.f;
                 sum2 = add2(sum2, pack2(p0, p1));
                 pk[16 * c + i] = pack_bf16(p0, p1);
               }
@@ -695,11 +739,14 @@ cudaError_t launch_fwd_t(const pp_plan* plan, const CUtensorMap& tq, const CUten
   DeviceSetup* dev = device_setup(setup);
   if (!dev) return cudaErrorInvalidDevice;
   if (dev->cc_major != 10) return cudaErrorNotSupported;
-  auto kern = fwd_kernel<D, DV>;
+  using Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, FwdParams);
+  const Kernel kerns[2] = {fwd_kernel<D, false, DV>, fwd_kernel<D, true, DV>};
+  const Kernel kern = kerns[plan->mixed];
   if (!dev->configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         FwdSmem<D>::kTotal);
-    if (e != cudaSuccess) return e;
+    for (Kernel k : kerns) {
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<D>::kTotal);
+      if (e != cudaSuccess) return e;
+    }
     dev->configured = true;
   }
   const int num_sms = dev->num_sms;
@@ -732,7 +779,9 @@ cudaError_t launch_fwd(const pp_plan* plan, const void* q, const void* k, const 
   FwdParams prm;
   prm.header = reinterpret_cast<int32_t*>(plan->ws + plan->lay.header);
   prm.tiles = reinterpret_cast<const Tile*>(plan->ws + plan->lay.tiles);
-  prm.order = reinterpret_cast<const int32_t*>(plan->ws + plan->lay.fwd_order);
+  prm.qtiles = reinterpret_cast<const QTile*>(plan->ws + plan->lay.qtiles);
+  prm.key_end = reinterpret_cast<const int32_t*>(plan->ws + plan->lay.key_end);
+  prm.order = reinterpret_cast<const int32_t*>(plan->ws + (plan->mixed ? plan->lay.qorder : plan->lay.fwd_order));
   prm.o = static_cast<__nv_bfloat16*>(o);
   prm.lse = lse;
   prm.dq_clear = dq_clear;

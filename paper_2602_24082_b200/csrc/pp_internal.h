@@ -42,9 +42,21 @@ struct BTile {
 };
 static_assert(sizeof(BTile) == 32, "backward tile record is 32 bytes");
 
+// One query tile of the forward where it does not run over the tiles of the segments
+// (fwd_mixed_tiles below): a tile of the group's grid, whose rows may belong to several segments,
+// or a copy of a segment's tile.
+struct QTile {
+  int32_t start, len;
+  int32_t kv0_start, kv0_len;  // prompt keys before the tile: every row sees them
+  int32_t kv1_start, kv1_len;  // the first rows' own response before the tile: only they see it
+  int32_t first_rows;          // rows of the first segment, and kQTilePrompt if it is the prompt
+  int32_t work;                // key tiles of both ranges, and the tile itself
+};
+constexpr int kQTilePrompt = 256;
+
 // Words of the plan header (int32[16]).
 constexpr int kHdrStatus = 0, kHdrDetail = 1, kHdrNumTiles = 2, kHdrNumSegments = 3,
-              kHdrNumBTiles = 8;
+              kHdrNumBTiles = 8, kHdrNumQTiles = 9;
 
 // Status word values written by device code.
 enum : int32_t {
@@ -71,6 +83,10 @@ struct PlanLayout {
   size_t bwd_units_det;  // the same units, one (group, KV head) set after the other and inside a
                          //   set by descending tile index: the order of the deterministic backward
   size_t key_end;    // int32[T]
+  // only where the forward runs over mixed tiles
+  size_t qtiles;     // QTile[max_tiles]  a group's tiles from its first segment tile's index on
+  size_t qorder;     // int32[max_tiles]  the query tiles, longest work first
+  size_t grid_gain;  // int64[G]  forward work over the segments' tiles less that over the grid's
   size_t total;
 };
 
@@ -87,6 +103,7 @@ struct pp_plan {
   pp::PlanLayout lay;
   // scratch sizes
   size_t fwd_scratch, bwd_scratch;
+  bool mixed;     // the forward runs over mixed query tiles (fwd_mixed_tiles)
   int lg_split;   // log2 of the parts each backward unit is cut into (bwd_split_log2)
   // backward scratch whose dQ accumulator the latest forward on this plan has cleared
   mutable const void* cleared_scratch = nullptr;
@@ -99,6 +116,22 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 inline int max_tiles_of(const pp_problem& p) {
   // sum over segments of ceil(len / 128) <= T / 128 + number of segments
   return p.total_tokens / kTile + p.num_groups + p.num_responses;
+}
+
+// The forward's query tiles: those of the segments, or tiles of each group's 128-token grid, whose
+// rows may belong to several segments (a group keeps its segments' tiles where they are less
+// work).  Short segments leave their own tiles nearly empty: 41 groups of 106 tokens in 5 segments
+// have 165 tiles and 297 key tiles to visit, on the grid 52 and 89.  The plan then takes one more
+// order and the forward the more general masks, 2 - 4 us a step, which pays where segments add
+// more than 0.3 to the number of tiles and there are more units than run in two waves anyway.
+// Whole steps, segments -> grid, at (added tiles, units per SM): (2.6, 5) 139 -> 97 us, (1.4, 8)
+// 148 -> 118, (0.42, 54) 1805 -> 1524, (0.45, 13) 326 -> 289, (0.72, 1.8) 66 -> 63; but (0.27, 9)
+// 170 -> 173, (0.36, 1.6) 105 -> 112, (1.25, 0.4) 49 -> 52.  By sizes alone, so that every way of
+// running a problem sums in the same order.
+inline bool fwd_mixed_tiles(const pp_problem& p) {
+  const int pairs = (p.num_q_heads / p.num_kv_heads + 1) / 2;
+  const double grid = p.total_tokens / double(kTile) + 0.5 * p.num_groups, added = 0.5 * p.num_responses;
+  return added > 0.3 * grid && (grid + added) * p.num_kv_heads * pairs > 1.75 * 148;
 }
 
 inline PlanLayout plan_layout(const pp_problem& p) {
@@ -123,6 +156,9 @@ inline PlanLayout plan_layout(const pp_problem& p) {
   l.bwd_units_det = off;
   off = align_up(off + sizeof(int32_t) * size_t(mt) * size_t(p.num_kv_heads), 256);
   l.key_end = off;   off = align_up(off + sizeof(int32_t) * size_t(p.total_tokens), 256);
+  l.qtiles = off;    off = align_up(off + sizeof(QTile) * size_t(mt), 256);
+  l.qorder = off;    off = align_up(off + sizeof(int32_t) * size_t(mt), 256);
+  l.grid_gain = off; off = align_up(off + sizeof(int64_t) * size_t(p.num_groups), 256);
   l.total = off;
   return l;
 }

@@ -43,6 +43,9 @@ struct PlanPtrs {
   int32_t* bwd_units_det;
   int Hkv;
   int32_t* key_end;
+  QTile* qtiles;        // null: not wanted
+  int32_t* qorder;
+  long long* grid_gain;
   int det_asc_max;  // deterministic order: sets of at most this many tiles are handed out longest first
   int num_rows, G, N, T, nseg, max_tiles;
 };
@@ -144,7 +147,7 @@ __device__ __forceinline__ bool plan_scan_body(const PlanPtrs& p) {
     if (s_carry[0] != p.T) {
       set_status(p.header, kStatusTokenMismatch, s_carry[0]);
     } else {
-      p.header[2] = s_carry[1];  // number of tiles
+      p.header[2] = p.header[kHdrNumQTiles] = s_carry[1];  // number of tiles
     }
   }
   __syncthreads();
@@ -152,6 +155,8 @@ __device__ __forceinline__ bool plan_scan_body(const PlanPtrs& p) {
 
   // backward tiles: ceil(group length / 128) per group, exclusive scan over the groups
   if (tid == 0) s_carry[1] = 0;
+  if (p.qtiles)
+    for (int g = tid; g < p.G; g += blockDim.x) p.grid_gain[g] = 0;
   __syncthreads();
   for (int base = 0; base < p.G; base += blockDim.x) {
     const int g = base + tid;
@@ -204,6 +209,33 @@ __device__ __forceinline__ int group_of_segment(const PlanPtrs& p, int s) {
   return lo;
 }
 
+// Query tile of the grid, from the group's start, the prompt's end, and start and end of the
+// segment of the first row.
+__device__ __forceinline__ QTile grid_query_tile(int start, int len, int gs, int pe, int ss, int se) {
+  const bool prompt = start < pe;
+  QTile q;
+  q.start = start;
+  q.len = len;
+  q.kv0_start = gs;
+  q.kv0_len = prompt ? start - gs : pe - gs;
+  q.kv1_start = prompt ? start : ss;
+  q.kv1_len = prompt ? 0 : start - ss;
+  q.first_rows = min(len, se - start) + (prompt ? kQTilePrompt : 0);
+  q.work = (q.kv0_len + kTile - 1) / kTile + (q.kv1_len + kTile - 1) / kTile + 1;
+  return q;
+}
+// a segment's tile as query tile: rows of one segment
+__device__ __forceinline__ QTile segment_query_tile(const Tile& t) {
+  return {t.start, t.len, t.kv0_start, t.kv0_len, t.kv1_start, t.kv1_len, t.len, t.work};
+}
+// Work of a query tile in the choice between the two: its key tiles, and one for its beginning and
+// end.
+__device__ __forceinline__ int tile_cost(int work) { return work + 1; }
+__device__ __forceinline__ void add_grid_gain(const PlanPtrs& p, int g, int gain) {
+  atomicAdd(reinterpret_cast<unsigned long long*>(p.grid_gain + g),
+            static_cast<unsigned long long>(static_cast<long long>(gain)));
+}
+
 __device__ __forceinline__ void plan_tile_body(const PlanPtrs& p, int t) {
   int s = upper_segment(p.seg_tile0, p.nseg, t);
   // segments with zero tiles cannot exist (len >= 1), so seg_tile0 is strictly increasing
@@ -228,6 +260,7 @@ __device__ __forceinline__ void plan_tile_body(const PlanPtrs& p, int t) {
   }
   tl.work = (tl.kv0_len + kTile - 1) / kTile + (tl.kv1_len + kTile - 1) / kTile + 1;
   p.tiles[t] = tl;
+  if (p.qtiles) add_grid_gain(p, g, tile_cost(tl.work));
 }
 
 __global__ void plan_tiles_kernel(PlanPtrs p) {
@@ -276,6 +309,29 @@ __device__ __forceinline__ void plan_btile_body(const PlanPtrs& p, int t) {
   b.dep_lo = k_rel;
   if (b.start >= pe) b.dep_lo = max(b.npc, (p.seg_start[s_first] - gs) / kTile);
   p.btiles[t] = b;
+  if (p.qtiles)
+    add_grid_gain(p, g, -tile_cost(grid_query_tile(b.start, b.len, gs, pe, p.seg_start[s_first],
+                                                   p.seg_start[s_first + 1]).work));
+}
+
+// Query tile t: a group's tiles stand where the tiles of its segments do, those of the grid (never
+// more of them) followed by empty ones of no work.
+__device__ __forceinline__ void plan_qtile_body(const PlanPtrs& p, int t) {
+  const int g = group_of_segment(p, upper_segment(p.seg_tile0, p.nseg, t));
+  if (p.grid_gain[g] <= 0) {
+    p.qtiles[t] = segment_query_tile(p.tiles[t]);
+    return;
+  }
+  const int sp = g + p.grp_resp_off[g], i = t - p.seg_tile0[sp];
+  QTile q{};
+  if (i < p.grp_btile0[g + 1] - p.grp_btile0[g]) {
+    const BTile b = p.btiles[p.grp_btile0[g] + i];
+    const int s = upper_segment(p.seg_start, p.nseg, b.start);
+    q = grid_query_tile(b.start, b.len, b.grp_start, p.seg_start[sp + 1], p.seg_start[s], p.seg_start[s + 1]);
+  } else {
+    atomicSub(&p.header[kHdrNumQTiles], 1);
+  }
+  p.qtiles[t] = q;
 }
 
 __global__ void plan_btiles_kernel(PlanPtrs p) {
@@ -285,21 +341,23 @@ __global__ void plan_btiles_kernel(PlanPtrs p) {
 }
 
 // Longest-work-first orders by rank counting (tile counts are small: T/128 + segments).
-__device__ __forceinline__ void plan_fwd_order_body(const PlanPtrs& p, int t, int n) {
-  const int wf = p.tiles[t].work;
+template <typename T>
+__device__ __forceinline__ void plan_fwd_order_body(const T* tiles, int32_t* order, int t, int n) {
+  const int wf = tiles[t].work;
   int rf = 0;
   for (int u = 0; u < n; ++u) {
-    const int of = p.tiles[u].work;
+    const int of = tiles[u].work;
     rf += (of > wf) || (of == wf && u < t);
   }
-  p.fwd_order[rf] = t;
+  order[rf] = t;
 }
 
 __global__ void plan_fwd_order_kernel(PlanPtrs p) {
   if (p.header[0] != kStatusOk) return;
   const int n = p.header[kHdrNumTiles];
   int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n) plan_fwd_order_body(p, t, n);
+  if (t < n) plan_fwd_order_body(p.tiles, p.fwd_order, t, n);
+  if (t < n && p.qtiles) plan_qtile_body(p, t);
 }
 
 // Backward processing order, built for L2 reuse and balance.  Key tiles of one group stream
@@ -367,9 +425,10 @@ __device__ __forceinline__ void plan_units_body(const PlanPtrs& p, int t, int n)
 
 __global__ void plan_gwork_kernel(PlanPtrs p) {
   if (p.header[0] != kStatusOk) return;
-  const int n = p.header[kHdrNumBTiles];
+  const int n = p.header[kHdrNumBTiles], nq = p.header[kHdrNumTiles];
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < n) plan_gwork_body(p, t, n);
+  if (t < nq && p.qtiles) plan_fwd_order_body(p.qtiles, p.qorder, t, nq);
 }
 
 __global__ void plan_sgroup_kernel(PlanPtrs p) {
@@ -421,12 +480,15 @@ constexpr int kRankTiles = 512;
 constexpr int kFusedSmallTiles = 256;  // blocks of 256 threads up to here, 1024 beyond
 constexpr int kFusedMaxTiles = 2048;   // tiles; also bounds the segments, and twice the groups
 
+// kMixed: with the forward's mixed query tiles (an instance of its own: carried along, their code
+// and space cost the plans without them 1 us)
+template <bool kMixed>
 struct FusedSmem {
   union alignas(16) {   // (keys are read as uint4)
-    uint32_t sort[2][3][kFusedMaxTiles];
+    uint32_t sort[2][kMixed ? 4 : 3][kFusedMaxTiles];
     struct {
-      uint32_t key[4][kRankTiles];      // forward tiles, backward tiles, groups, backward units
-      int32_t rank[4][kRankTiles];      // (groups: backward tiles of the groups ranked before)
+      uint32_t key[kMixed ? 5 : 4][kRankTiles];      // forward tiles, backward tiles, groups, backward units,
+      int32_t rank[kMixed ? 5 : 4][kRankTiles];      //   query tiles (groups: backward tiles of the groups before)
     } r;
   } o;
   int32_t desc[kDescFused];
@@ -439,9 +501,11 @@ struct FusedSmem {
   uint16_t seg_grp[kFusedMaxTiles];
   uint16_t wb[kFusedMaxTiles];          // work and group of the backward tiles
   uint16_t bgrp[kFusedMaxTiles];
+  int32_t grid_gain[kMixed ? kFusedMaxTiles / 2 : 1];
+  uint16_t qwork[kMixed ? kFusedMaxTiles : 2];       // work of the query tiles, 0 where there is none
   uint16_t unit_tile[kFusedMaxTiles];   // backward tiles in the order of their units
   int32_t warp_sum[2][32];
-  int32_t status, detail;
+  int32_t status, detail, no_qtile;
 };
 
 // Inclusive sums of two values over the block.
@@ -504,9 +568,9 @@ __device__ __forceinline__ void rank_count(const uint32_t* key, int m, int32_t* 
 // Ascending bitonic sort of kArrays arrays of `n2` (1024 or 2048) keys in a block of 1024 threads,
 // key tid + 1024 r of each in v[.][r].  Distances below 32 are shuffles, 1024 is inside the thread,
 // the others go through shared memory (two buffers in turn: one barrier per distance).
-template <int kArrays>
+template <int kArrays, int kBufs>
 __device__ __forceinline__ void bitonic_sort(uint32_t (&v)[kArrays][2], int n2,
-                                             uint32_t (&buf)[2][3][kFusedMaxTiles]) {
+                                             uint32_t (&buf)[2][kBufs][kFusedMaxTiles]) {
   const int tid = threadIdx.x;
   const bool two = n2 > 1024;
   int turn = 0;
@@ -556,11 +620,11 @@ __device__ __forceinline__ void bitonic_sort(uint32_t (&v)[kArrays][2], int n2,
   }
 }
 
-template <size_t kDesc>
+template <size_t kDesc, bool kMixed>
 __global__ void __launch_bounds__(1024)
 plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  FusedSmem& sm = *reinterpret_cast<FusedSmem*>(smem_raw);
+  FusedSmem<kMixed>& sm = *reinterpret_cast<FusedSmem<kMixed>*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nthr = blockDim.x;
   const int n_rgo = p.num_rows + 1, n_all = n_rgo + p.G + p.G + 1 + p.N;
   launch_dependents();
@@ -578,7 +642,7 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
   }
   if (tid == 0) {
     sm.status = kStatusOk;
-    sm.detail = 0;
+    sm.detail = sm.no_qtile = 0;
   }
   if (kDesc > 1) dependency_wait();   // (the workspace may still be in use up to here)
   __syncthreads();
@@ -662,14 +726,20 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
       til = (sm.seg_start[tid + 1 + gro[tid + 1]] - sm.seg_start[tid + gro[tid]] + kTile - 1) / kTile;
     const int mine = til;
     block_scan2(til, unused, sm.warp_sum);
-    if (tid < p.G) sm.btile0[tid] = til - mine;
+    if (tid < p.G) {
+      sm.btile0[tid] = til - mine;
+      if (kMixed) sm.grid_gain[tid] = 0;
+    }
     if (tid == p.G - 1) sm.btile0[p.G] = til;
   }
+  if constexpr (kMixed) __syncthreads();
   // ---- forward tiles
   const bool by_rank = n <= kRankTiles;   // (there are at most as many backward tiles as forward
                                           // tiles, and fewer groups)
-  // keys of tile (group) tid + nthr r: forward tiles, backward tiles, groups
-  uint32_t key[3][2] = {{~0u, ~0u}, {~0u, ~0u}, {~0u, ~0u}};
+  // keys of tile (group) tid + nthr r: forward tiles, backward tiles, groups, query tiles
+  constexpr int kOrders = kMixed ? 4 : 3;
+  uint32_t key[kOrders][2];
+  for (int a = 0; a < kOrders; ++a) key[a][0] = key[a][1] = ~0u;
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     const int t = tid + nthr * r;
@@ -698,11 +768,13 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
       sm.tile[1][t] = tl.start + tl.len;
       sm.tile[2][t] = tl.vis_end;
       key[0][r] = uint32_t(0xffff - tl.work) << 16 | uint32_t(t);
+      if constexpr (kMixed) atomicAdd(&sm.grid_gain[g], tile_cost(tl.work));
     }
   }
   for (int s = tid; s <= p.nseg; s += nthr) p.seg_start[s] = sm.seg_start[s];
   __syncthreads();
   const int nb = sm.btile0[p.G];
+  QTile q[2];
   // ---- backward tiles; key_end (every key of a forward tile ends its visibility at vis_end)
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
@@ -728,6 +800,10 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
     sm.wb[t] = uint16_t(b.work);
     sm.bgrp[t] = uint16_t(g);
     key[1][r] = uint32_t(0xffff - b.work) << 16 | uint32_t(t);
+    if constexpr (kMixed) {
+      q[r] = grid_query_tile(b.start, b.len, gs, pe, sm.seg_start[s_first], sm.seg_start[s_first + 1]);
+      atomicSub(&sm.grid_gain[g], tile_cost(q[r].work));
+    }
   }
   for (int t = wid; t < n; t += nthr >> 5) {
     const int left = sm.tile[1][t] - sm.tile[0][t] - lane, vis_end = sm.tile[2][t];
@@ -737,6 +813,38 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
       if (c < left) at[c] = vis_end;
   }
   __syncthreads();
+  // ---- query tiles (see plan_qtile_body)
+  if constexpr (kMixed) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int t = tid + nthr * r;
+      if (t < n) {
+        const int g = sm.seg_grp[upper_segment(sm.seg_tile0, p.nseg, t)];
+        const int i = t - sm.seg_tile0[g + gro[g]], ng = sm.btile0[g + 1] - sm.btile0[g];
+        if (sm.grid_gain[g] <= 0) {
+          const QTile own = segment_query_tile(p.tiles[t]);
+          p.qtiles[t] = own;
+          sm.qwork[t] = uint16_t(own.work);
+        } else if (i >= ng) {
+          sm.qwork[t] = 0;
+          atomicAdd(&sm.no_qtile, 1);
+        }
+      }
+      if (t < nb) {
+        const int g = sm.bgrp[t], at = sm.seg_tile0[g + gro[g]] + t - sm.btile0[g];
+        if (sm.grid_gain[g] > 0) {
+          p.qtiles[at] = q[r];
+          sm.qwork[at] = uint16_t(q[r].work);
+        }
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int t = tid + nthr * r;
+      if (t < n) key[3][r] = uint32_t(0xffff - sm.qwork[t]) << 16 | uint32_t(t);
+    }
+  }
   // ---- work of every group (a warp each), groups in order of decreasing work
   for (int g = wid; g < p.G; g += nthr >> 5) {
     int w = 0;
@@ -760,13 +868,20 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
       sm.o.r.key[2][t] = t == tid ? key[2][0] : ~0u;
       sm.o.r.key[3][t] = ~0u;
       sm.o.r.rank[0][t] = sm.o.r.rank[1][t] = sm.o.r.rank[2][t] = sm.o.r.rank[3][t] = 0;
+      if constexpr (kMixed) {
+        sm.o.r.key[4][t] = t == tid ? key[3][0] : ~0u;
+        sm.o.r.rank[4][t] = 0;
+      }
     }
     __syncthreads();
     rank_count<false>(sm.o.r.key[0], n, sm.o.r.rank[0], nullptr);
     rank_count<false>(sm.o.r.key[1], nb, sm.o.r.rank[1], nullptr);
     rank_count<true>(sm.o.r.key[2], p.G, sm.o.r.rank[2], sm.btile0);
+    if constexpr (kMixed) rank_count<false>(sm.o.r.key[4], n, sm.o.r.rank[4], nullptr);
     __syncthreads();
     if (tid < n) p.fwd_order[sm.o.r.rank[0][tid]] = tid;
+    if constexpr (kMixed)
+      if (tid < n) p.qorder[sm.o.r.rank[4][tid]] = tid;
     if (tid < nb) {
       p.bwd_order[sm.o.r.rank[1][tid]] = tid;
       sm.o.r.key[3][tid] = unit_key(tid, sm.o.r.rank[2][sm.bgrp[tid]]);
@@ -780,7 +895,7 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
   } else {
     int n2 = 1024;
     while (n2 < n) n2 <<= 1;
-    bitonic_sort<3>(key, n2, sm.o.sort);
+    bitonic_sort(key, n2, sm.o.sort);
     // tiles of the groups ranked before each group
     int cnt = 0, unused = 0, g = 0;
     if (tid < p.G) {
@@ -796,10 +911,12 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
     for (int r = 0; r < 2; ++r) {
       const int t = tid + nthr * r;
       if (t < n) p.fwd_order[t] = int32_t(key[0][r] & 0xffffu);
+      if constexpr (kMixed)
+        if (t < n) p.qorder[t] = int32_t(key[3][r] & 0xffffu);
       if (t < nb) p.bwd_order[t] = int32_t(key[1][r] & 0xffffu);
       ukey[0][r] = t < nb ? unit_key(t, sm.before[sm.bgrp[t]]) : ~0u;
     }
-    bitonic_sort<1>(ukey, n2, sm.o.sort);
+    bitonic_sort(ukey, n2, sm.o.sort);
 #pragma unroll
     for (int r = 0; r < 2; ++r)
       if (tid + nthr * r < nb) sm.unit_tile[tid + nthr * r] = uint16_t(ukey[0][r] & 2047u);
@@ -814,9 +931,10 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
     const int slot = ng <= p.det_asc_max ? k_rel : ng - 1 - k_rel;
     p.bwd_units_det[p.Hkv * sm.before[g] + kvh * ng + slot] = (kvh << 24) | i;
   }
-  if (tid < 16)   // (words from 4 on, except the backward tile count: dynamic-scheduling counters)
+  if (tid < 16)   // (words 4 to 7: dynamic-scheduling counters)
     p.header[tid] = tid == kHdrNumTiles ? n
-                    : tid == kHdrNumSegments ? p.nseg : tid == kHdrNumBTiles ? nb : 0;
+                    : tid == kHdrNumSegments ? p.nseg : tid == kHdrNumBTiles ? nb
+                    : kMixed && tid == kHdrNumQTiles ? n - sm.no_qtile : 0;
 }
 
 }  // namespace
@@ -912,6 +1030,9 @@ cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cu
   p.bwd_units_det = reinterpret_cast<int32_t*>(ws + l.bwd_units_det);
   p.Hkv = plan->prob.num_kv_heads;
   p.key_end = reinterpret_cast<int32_t*>(ws + l.key_end);
+  p.qtiles = plan->mixed ? reinterpret_cast<QTile*>(ws + l.qtiles) : nullptr;
+  p.qorder = reinterpret_cast<int32_t*>(ws + l.qorder);
+  p.grid_gain = reinterpret_cast<long long*>(ws + l.grid_gain);
   // a third of the SMs (the backward runs one CTA per SM), at most 48 tiles = 6144 tokens
   static DeviceSetup setup[kMaxDevices];
   DeviceSetup* dev = device_setup(setup);
@@ -935,13 +1056,17 @@ cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cu
     // rows <= G <= N and G + N <= 2048: kDescFused entries always suffice
     cudaError_t e = cudaSuccess;
     if (!dev->configured) {
-      auto opt_in = [&](auto kern) {
-        if (e == cudaSuccess)
-          e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(FusedSmem));
+      auto opt_in = [&](auto kern, size_t bytes) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
       };
-      opt_in(plan_fused_kernel<1>);
-      opt_in(plan_fused_kernel<kDescSmall>);
-      opt_in(plan_fused_kernel<kDescFused>);
+      auto both = [&](auto n_c) {
+        constexpr size_t kN = decltype(n_c)::value;
+        opt_in(plan_fused_kernel<kN, false>, sizeof(FusedSmem<false>));
+        opt_in(plan_fused_kernel<kN, true>, sizeof(FusedSmem<true>));
+      };
+      both(std::integral_constant<size_t, 1>{});
+      both(std::integral_constant<size_t, kDescSmall>{});
+      both(std::integral_constant<size_t, kDescFused>{});
       if (e != cudaSuccess) return e;
       dev->configured = true;
     }
@@ -949,8 +1074,11 @@ cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cu
       constexpr size_t kN = decltype(n_c)::value;
       DescBlock<kN> blk;
       if (host_desc) fill_desc(host_desc, n_desc, blk.v);
-      e = launch_kernel(true, plan_fused_kernel<kN>, dim3(1), dim3(mt <= kFusedSmallTiles ? 256 : 1024),
-                            sizeof(FusedSmem), stream, blk, p);
+      const dim3 threads(mt <= kFusedSmallTiles ? 256 : 1024);
+      e = plan->mixed ? launch_kernel(true, plan_fused_kernel<kN, true>, dim3(1), threads,
+                                      sizeof(FusedSmem<true>), stream, blk, p)
+                      : launch_kernel(true, plan_fused_kernel<kN, false>, dim3(1), threads,
+                                      sizeof(FusedSmem<false>), stream, blk, p);
     };
     if (!host_desc) go(std::integral_constant<size_t, 1>{});
     else if (n_all <= kDescSmall) go(std::integral_constant<size_t, kDescSmall>{});
