@@ -277,10 +277,10 @@ __global__ void __launch_bounds__(1024) rows_pack_kernel(RowsPtrs p, int tables_
 constexpr int kMaxAssignRanks = 1024;
 
 template <int kPerLane>
-__global__ void __launch_bounds__(32)
-assign_greedy_kernel(int R, int ranks, const long long* __restrict__ cost,
-                     const int32_t* __restrict__ order, int32_t* __restrict__ rank_of_row,
-                     long long* __restrict__ rank_cost) {
+__device__ __forceinline__ void assign_one_by_one(int R, int ranks, const long long* __restrict__ cost,
+                                                  const int32_t* __restrict__ order,
+                                                  int32_t* __restrict__ rank_of_row,
+                                                  long long* __restrict__ rank_cost) {
   constexpr long long kInf = 0x7fffffffffffffffLL;
   const int lane = threadIdx.x;
   long long load[kPerLane];
@@ -332,6 +332,88 @@ assign_greedy_kernel(int R, int ranks, const long long* __restrict__ cost,
   for (int j = 0; j < kPerLane; ++j)
     if (id[j] < ranks) rank_cost[id[j]] = load[j];
 }
+template <int kPerLane>
+__global__ void __launch_bounds__(32)
+assign_greedy_kernel(int R, int ranks, const long long* __restrict__ cost,
+                     const int32_t* __restrict__ order, int32_t* __restrict__ rank_of_row,
+                     long long* __restrict__ rank_cost) {
+  assign_one_by_one<kPerLane>(R, ranks, cost, order, rank_of_row, rank_cost);
+}
+
+// Up to 32 ranks: a round assigns as many rows as the sorted list of ranks allows at once.  Row i of
+// the round goes to rank i of the list while that rank is still before all the ranks that have got
+// a row in this round -- with loads closer together than a row's cost, as they soon are, that is
+// every rank.  Load and rank are one 64-bit word (for sums of costs below 2^58, else one row at a
+// time); the list is sorted again by counting, every lane comparing its word with the others', kN at
+// most, read from shared memory in one go.  Bound by that chain.
+// Building the rows of 4096 groups and dealing the 972 rows out to 8 ranks took 150 us with one row
+// at a time, now 126 (122 rounds instead of 972 steps).
+constexpr int kBatchRows = 1024, kBatchThreads = 256;
+template <int kN>
+__global__ void __launch_bounds__(kBatchThreads)
+assign_batch_kernel(int R, int ranks, const long long* __restrict__ cost,
+                    const int32_t* __restrict__ order, int32_t* __restrict__ rank_of_row,
+                    long long* __restrict__ rank_cost) {
+  using Key = unsigned long long;
+  __shared__ Key s_cost[kBatchRows];
+  __shared__ int32_t s_row[kBatchRows];
+  __shared__ alignas(16) Key s_key[32];
+  __shared__ Key s_sorted[32];
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (R > 0 && (cost[order[R - 1]] < 0 || cost[order[0]] >= (1LL << 58) / R)) {
+    if (tid < 32) assign_one_by_one<1>(R, ranks, cost, order, rank_of_row, rank_cost);
+    return;
+  }
+  Key key = lane < ranks ? Key(lane) : ~Key(0);
+  for (int base = 0; base < R; base += kBatchRows) {
+    const int m = min(kBatchRows, R - base);
+    __syncthreads();
+    for (int i = tid; i < m; i += kBatchThreads) {
+      s_row[i] = order[base + i];
+      s_cost[i] = Key(cost[s_row[i]]) << 5;
+    }
+    __syncthreads();
+    if (tid >= 32) continue;
+    auto exchange = [&]() {   // the list sorted again: my place is the number of words before mine
+      __syncwarp();
+      s_key[lane] = key;
+      __syncwarp();
+      int before = 0;
+#pragma unroll
+      for (int i = 0; i < kN; i += 2) {
+        const ulonglong2 o = *reinterpret_cast<const ulonglong2*>(&s_key[i]);
+        before += int(o.x < key) + int(o.y < key);
+      }
+      if (lane < ranks) s_sorted[before] = key;
+      __syncwarp();
+      if (lane < ranks) key = s_sorted[lane];
+    };
+    Key c = lane < m ? s_cost[lane] : 0;
+    for (int pos = 0; pos < m;) {
+      const bool there = lane < ranks && pos + lane < m;
+      const Key next = key + c, last = __shfl_sync(0xffffffffu, key, ranks - 1);
+      int count = ranks;
+      // every rank is in time if the last one is before all that have got a row
+      if (!__all_sync(0xffffffffu, lane >= ranks || (there && next > last))) {
+        __syncwarp();
+        s_key[lane] = there ? next : ~Key(0);
+        __syncwarp();
+        bool in_time = there;
+        for (int i = 0; i < ranks - 1; ++i) in_time = in_time && (i >= lane || key < s_key[i]);
+        const uint32_t fits = __ballot_sync(0xffffffffu, in_time);
+        count = fits == 0xffffffffu ? 32 : __ffs(~fits) - 1;   // (the first row always fits)
+      }
+      if (lane < count) {
+        rank_of_row[s_row[pos + lane]] = int(key & 31u);
+        key = next;
+      }
+      pos += count;
+      c = pos + lane < m ? s_cost[pos + lane] : 0;
+      exchange();
+    }
+  }
+  if (tid < ranks) rank_cost[key & 31u] = static_cast<long long>(key >> 5);
+}
 
 // More ranks than the lanes' registers hold: the loads in shared memory, the lanes sharing the
 // search for the least one.
@@ -379,11 +461,12 @@ cudaError_t launch_assign_rows(int R, const long long* row_cost, int ranks, int3
                                int* launches) {
   rank_kernel<long long><<<(R + kRankKeys - 1) / kRankKeys, kRankKeys * kRankSlices, 0, stream>>>(
       R, row_cost, order);
-  auto greedy = ranks <= 32    ? assign_greedy_kernel<1>
+  auto greedy = ranks <= 8     ? assign_batch_kernel<8>
+                : ranks <= 32  ? assign_batch_kernel<32>
                 : ranks <= 64  ? assign_greedy_kernel<2>
                 : ranks <= 128 ? assign_greedy_kernel<4>
                                : assign_greedy_smem_kernel;
-  greedy<<<1, 32, 0, stream>>>(R, ranks, row_cost, order, rank_of_row, rank_cost);
+  greedy<<<1, ranks <= 32 ? kBatchThreads : 32, 0, stream>>>(R, ranks, row_cost, order, rank_of_row, rank_cost);
   if (launches) *launches = 2;
   return cudaGetLastError();
 }

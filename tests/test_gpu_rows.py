@@ -145,3 +145,19 @@ def test_assign_rows_at_the_edges_of_the_lane_lists(rows, ranks):
     assert np.array_equal(order.cpu().numpy(), want[0])
     assert np.array_equal(rank_of_row.cpu().numpy(), want[1])
     assert np.array_equal(rank_cost.cpu().numpy(), want[2])
+
+
+@pytest.mark.parametrize("kind", ["equal", "zeros", "doubling", "huge", "mixed"])
+@pytest.mark.parametrize("rows,ranks", [(1, 32), (31, 31), (1024, 8), (1025, 32), (2500, 5)])
+def test_assign_rows_in_rounds(rows, ranks, kind):
+    """Several rows a round: costs where all ranks take one, where only the first does, and sums too
+    large for load and rank in one word."""
+    from paper_2602_24082_b200 import binding as B
+    rng = np.random.default_rng(rows + ranks)
+    cost = {"equal": np.full(rows, 17), "zeros": np.where(rng.random(rows) < 0.5, 0, 3),
+            "doubling": 1 << (np.arange(rows) % 40), "huge": rng.integers(1 << 46, (1 << 62) // rows, rows),
+            "mixed": rng.integers(0, 1 << rng.integers(1, 30, rows))}[kind].astype(np.int64)
+    order, rank_of_row, rank_cost = B.pp_assign_rows(torch.from_numpy(cost).cuda(), ranks)
+    want = R.assign_rows(cost, ranks)
+    for got, exact in zip((order, rank_of_row, rank_cost), want):
+        assert np.array_equal(got.cpu().numpy(), exact)
