@@ -855,19 +855,18 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
       const int k_rel = (un.tile.start - un.tile.grp_start) / kTile;
       int dep_lo = 0;
       // Passing the turn on needs the reductions of the tile to be complete (a wait of a
-      // microsecond or two), so it is deferred: the counter of iteration i is published after
-      // the reductions of iteration i + 1 have been issued -- the next key tile gets to the
-      // same query tile a whole query tile's worth of iterations later -- or at once whenever
-      // this unit finds that it has to wait for its own turn.
+      // microsecond or two), so it is deferred: the counter of iteration i is published in
+      // iteration i + 1, as soon as that tile is out of tensor memory and before this unit can come
+      // to wait for its own turn -- the next key tile gets to the same query tile a whole query
+      // tile's worth of iterations later.
       int32_t* pend = nullptr;
-      // What the turns order are reductions performed in L2: ours are complete (waited for, so
-      // performed) before the store below is issued, and the next unit issues its own behind the
-      // load that sees it.  Nobody reads the sums before the kernel ends, so neither side needs
-      // a fence -- which would cost this warp about a thousand cycles per tile.
-      auto publish = [&](int32_t* p) {
-        const int mine = k_rel + 1;
-        asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(mine) : "memory");
-      };
+      // What the turns order are reductions of the async proxy.  Ours are complete, and so visible to
+      // this thread, behind the bulk wait; the release hands that on, and the next unit issues
+      // its own behind the acquire that sees it and a proxy fence.  Release and acquire cost this
+      // warp about a thousand cycles each, the first while the tile behind it waits in registers and
+      // not in tensor memory (with the release at the end of the iteration four 4800-token groups,
+      // 28 / 4 heads, take 2306 us, here 2220; eight 1100-token groups, 32 / 8, 438 and 415).
+      auto publish = [&](int32_t* p) { store_release_gpu(p, k_rel + 1); };
       for (int it = 0; it < un.n_it; ++it, q_advance<kDet>(qi, unit_heads<kSplit>(prm, un), un.nq)) {
         const QTile qt = q_tile_at<kSplit>(prm, un, qi);
         const uint32_t g = gc + it;
@@ -878,9 +877,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
           // the last prompt tile follows the lowest response tile that adds to this query tile
           if (qi.hh == 0 && qi.qt > 0 && k_rel == un.tile.npc - 1 && k_rel + qi.qt >= un.tile.npc)
             dep_lo = prm.tiles[un.tidx + qi.qt].dep_lo;
-          // read the counter now: the answer (normally already the expected one) is back by the
-          // time the first box of the tile is staged
-          asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(seen_early) : "l"(sem) : "memory");
+          // read the counter now, under the wait for the tile (normally it has the expected value)
+          seen_early = load_acquire_gpu(sem);
         }
         wait_bar(bar(kDqFull), g & 1, abort_flag, prm.header, 80);
         tc_fence_after();
@@ -897,6 +895,13 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(kDqDrained));
+        if (kDet && leader) {
+          if (pend) {
+            bulk_wait_group<0>();
+            publish(pend);
+          }
+          pend = sem;
+        }
         if (row >= qt.len) {  // rows past the tile's end belong to other tokens: add zero
 #pragma unroll
           for (int i = 0; i < DV; ++i) w[i] = 0u;
@@ -926,16 +931,9 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                                                                                           : k_rel + 2);
               bool ok = seen_early == expect;
               for (uint32_t spin = 0; !ok && spin < (1u << 22); ++spin) {
-                int seen;
-                asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(sem) : "memory");
-                if (seen == expect) {
+                if (load_acquire_gpu(sem) == expect) {
                   ok = true;
                   break;
-                }
-                if (pend) {  // about to wait: do not keep the unit below waiting for us
-                  bulk_wait_group<0>();
-                  publish(pend);
-                  pend = nullptr;
                 }
                 if ((spin & 0xff) == 0xff && *abort_flag) break;
                 __nanosleep(20);
@@ -945,17 +943,11 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                   prm.header[1] = 81;
                 *abort_flag = 1;
               }
+              fence_proxy_async_global();
             }
             if (32 * quarter < qt.len) tma_reduce_add_3d(&tm_dq, buf, c * 32, qt.h, qt.start + 32 * quarter);
             bulk_commit_group();
           }
-        }
-        if (kDet && sem) {
-          if (pend) {  // the previous tile's boxes (all but this tile's DV / 32 groups) have landed
-            bulk_wait_group<DV / 32>();
-            publish(pend);
-          }
-          pend = sem;
         }
       }
       if (kDet && pend) {

@@ -1,0 +1,27 @@
+"""Orders between threads that no run can show to hold: where one is missing, equal runs still agree
+on the chip at hand.  They are read from the kernels' sources."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2602_24082_b200", "csrc")
+
+
+def _source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def test_turns_of_the_deterministic_backward_are_released_and_acquired():
+    """The reductions of one key tile come before those of the next: complete -> release -> acquire ->
+    proxy fence -> issued, on every path."""
+    assert ".relaxed." not in _source("pp_bwd.cu") + _source("pp_ptx.cuh")
+    main = _source("pp_bwd.cu")
+    dq = main[main.index("kBwdRegsDq, kBwdRegsLaunch>"):]
+    assert dq.count("load_acquire_gpu(sem)") == 2
+    assert re.search(r"auto publish = [^;]*store_release_gpu\(p, k_rel \+ 1\);", dq)
+    for call in re.finditer(r"publish\(pend\);", dq):
+        assert re.search(r"bulk_wait_group<[^>]*>\(\);\s*$", dq[:call.start()])
+    # published before the unit waits for its next turn: no unit below waits for one that waits itself
+    assert dq.index("publish(pend);") < dq.index("if (kDet && sem && c == 0)")
+    turn, reduce = dq.index("if (kDet && sem && c == 0)"), dq.index("tma_reduce_add_3d(")
+    assert re.search(r"fence_proxy_async_global\(\);\s*}\s*if \(32 \* quarter < qt.len\) $", dq[turn:reduce])
