@@ -740,6 +740,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         };
         if (full) ds_all(std::false_type{}); else ds_all(std::true_type{});
         fence_proxy_async_smem();
+        tc_fence_before();   // (the dQ tile overwrites the columns dP was loaded from)
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(kDsReady));
       }

@@ -25,3 +25,14 @@ def test_turns_of_the_deterministic_backward_are_released_and_acquired():
     assert dq.index("publish(pend);") < dq.index("if (kDet && sem && c == 0)")
     turn, reduce = dq.index("if (kDet && sem && c == 0)"), dq.index("tma_reduce_add_3d(")
     assert re.search(r"fence_proxy_async_global\(\);\s*}\s*if \(32 \* quarter < qt.len\) $", dq[turn:reduce])
+
+
+def test_tensor_memory_is_handed_back_behind_a_fence():
+    """One lane arrives for its warp: what the other lanes did to tensor memory is ordered before it by
+    their own fence and the warp barrier."""
+    main = _source("pp_bwd.cu")
+    for bar in ("kPReady", "kDsReady", "kDqDrained", "kDkvFree"):
+        places = [m.start() for m in re.finditer(r"mbar_arrive\(bar\(%s\)\)" % bar, main)]
+        assert places
+        for at in places:
+            assert re.search(r"tc_fence_before\(\);\s*__syncwarp\(\);\s*if \(lane == 0\) $", main[:at]), bar
