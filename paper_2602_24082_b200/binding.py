@@ -252,7 +252,9 @@ def pp_build_plan(desc: Sequence[np.ndarray], num_q_heads: int, num_kv_heads: in
         # (None: the arrays have to be converted first, below)
         handle = ext.build_plan(tuple(desc), num_q_heads, num_kv_heads, head_dim, total_tokens, workspace)
         if handle is not None:
-            return Plan(handle, workspace, (desc, None), num_q_heads, num_kv_heads, head_dim, total_tokens)
+            # (views of these arrays: the caller's container may be filled with others)
+            keep = tuple(map(memoryview, desc))
+            return Plan(handle, workspace, (keep, None), num_q_heads, num_kv_heads, head_dim, total_tokens)
     dev_arrays = device_arrays
     if desc_on_device and dev_arrays is None:
         dev_arrays = [torch.from_numpy(np.ascontiguousarray(a, dtype=np.int32)).to(device) for a in desc]
