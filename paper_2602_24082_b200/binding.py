@@ -243,14 +243,14 @@ def pp_build_plan(desc: Sequence[np.ndarray], num_q_heads: int, num_kv_heads: in
                   workspace: Optional[torch.Tensor] = None) -> Plan:
     """Builds a plan.  ``device_arrays`` (int32 CUDA tensors) and ``workspace`` (uint8 CUDA
     tensor of at least the queried size) let a caller re-plan every step without allocating."""
-    ext = _ext
+    ext, desc = _ext, tuple(desc)
     if ext is None:
         if not torch.cuda.is_available():
             raise RuntimeError("pp_build_plan needs a CUDA device (there is no CPU fallback)")
         ext = _step_calls()
     if workspace is not None and device_arrays is None and not desc_on_device:
         # (None: the arrays have to be converted first, below)
-        handle = ext.build_plan(tuple(desc), num_q_heads, num_kv_heads, head_dim, total_tokens, workspace)
+        handle = ext.build_plan(desc, num_q_heads, num_kv_heads, head_dim, total_tokens, workspace)
         if handle is not None:
             # (views of these arrays: the caller's container may be filled with others)
             keep = tuple(map(memoryview, desc))

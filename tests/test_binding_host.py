@@ -35,3 +35,14 @@ def test_a_plan_is_that_of_the_arrays_at_the_call(builds):
     assert (p.num_rows, p.num_groups, p.num_responses, p.total_tokens) == (2, 2, 3, 25)
     want, _ = B.make_problem(arrays(), 4, 2, 64, 25)
     assert plan.bwd_scratch_bytes == B.pp_plan_workspace_bytes(want)[2]
+
+
+@pytest.mark.parametrize("dtype", [np.int32, np.int64])
+def test_descriptors_may_come_from_an_iterator(builds, monkeypatch, dtype):
+    """An iterator can be gone through once, whichever way its arrays are taken."""
+    monkeypatch.setattr(B, "_call", lambda index, where, fn, problem, *rest: builds.append(problem.num_responses))
+    workspace = types.SimpleNamespace(is_cuda=True, get_device=lambda: 0, data_ptr=lambda: 0, numel=lambda: 0,
+                                      is_contiguous=lambda: True)
+    plan = B.pp_build_plan((np.asarray(a, dtype) for a in DESC), 4, 2, 64, 25, workspace=workspace)
+    assert builds == [tuple(DESC)] if dtype is np.int32 else builds == [3]
+    assert plan.problem.num_groups == 2
