@@ -261,8 +261,8 @@ def pp_build_plan(desc: Sequence[np.ndarray], num_q_heads: int, num_kv_heads: in
     problem, keep = make_problem(desc, num_q_heads, num_kv_heads, head_dim, total_tokens, dev_arrays)
     if workspace is None:
         workspace = torch.empty(pp_plan_workspace_bytes(problem)[0], dtype=torch.uint8, device=device)
-    elif not workspace.is_cuda:
-        raise ValueError("workspace: expected a CUDA tensor")
+    elif not (workspace.is_cuda and workspace.is_contiguous()):
+        raise ValueError("workspace: expected a contiguous CUDA tensor")
     handle = ctypes.c_void_p(0)
     try:
         _call(workspace.get_device(), "pp_build_plan", _build_plan, problem, workspace.data_ptr(),

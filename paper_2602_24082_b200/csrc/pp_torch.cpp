@@ -41,13 +41,17 @@ struct Dims {
   int64_t T, Hq, Hkv, D;
 };
 
-// The tensor of `o` if it is a contiguous CUDA tensor of that type and shape; otherwise the
-// Python check is called to raise, and null comes back.
+// The tensor of `o` if it is a contiguous CUDA tensor of that type and shape, on the device of `on`
+// (if given); otherwise the Python check is called to raise, and null comes back.
 const at::Tensor* take(PyObject* o, at::ScalarType type, const char* type_name, at::IntArrayRef shape,
-                       const char* name) {
+                       const char* name, const at::Tensor* on = nullptr) {
   if (THPVariable_Check(o)) {
     const at::Tensor& t = THPVariable_Unpack(o);
-    if (t.is_cuda() && t.scalar_type() == type && t.sizes() == shape && t.is_contiguous()) return &t;
+    if (t.is_cuda() && t.scalar_type() == type && t.sizes() == shape && t.is_contiguous()) {
+      if (!on || t.device() == on->device()) return &t;
+      PyErr_Format(PyExc_ValueError, "%s: on another device than q", name);
+      return nullptr;
+    }
   }
   PyObject* torch = PyImport_ImportModule("torch");
   PyObject* dtype = torch ? PyObject_GetAttrString(torch, type_name) : nullptr;
@@ -59,6 +63,16 @@ const at::Tensor* take(PyObject* o, at::ScalarType type, const char* type_name, 
   Py_XDECREF(tup);
   Py_XDECREF(dtype);
   Py_XDECREF(torch);
+  return nullptr;
+}
+
+// A buffer the caller provides, sized by its elements: a contiguous CUDA tensor.
+const at::Tensor* take_buffer(PyObject* o, const char* name, const at::Tensor* on = nullptr) {
+  if (THPVariable_Check(o)) {
+    const at::Tensor& t = THPVariable_Unpack(o);
+    if (t.is_cuda() && t.is_contiguous() && (!on || t.device() == on->device())) return &t;
+  }
+  PyErr_Format(PyExc_ValueError, "%s: expected a contiguous CUDA tensor%s", name, on ? " on q's device" : "");
   return nullptr;
 }
 
@@ -142,12 +156,12 @@ PyObject* build_plan(PyObject*, PyObject* const* a, Py_ssize_t n) {
     release();
     return nullptr;
   }
-  const at::Tensor& ws = THPVariable_Unpack(a[5]);
-  if (!ws.is_cuda()) {
+  const at::Tensor* w = take_buffer(a[5], "workspace");
+  if (!w) {
     release();
-    PyErr_SetString(PyExc_ValueError, "workspace: expected a CUDA tensor");
     return nullptr;
   }
+  const at::Tensor& ws = *w;
   const c10::cuda::CUDAGuard guard(ws.device());
   const pp_stream_t s = stream_of(ws.get_device());
   pp_plan* plan = nullptr;
@@ -184,22 +198,23 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (!take_dims(a, handle, d)) return nullptr;
   const int64_t qs[3] = {d.T, d.Hq, d.D}, ks[3] = {d.T, d.Hkv, d.D}, ls[2] = {d.Hq, d.T};
   const at::Tensor *q, *k, *v;
-  if (!(q = take(a[5], kBf16, "bfloat16", qs, "q")) || !(k = take(a[6], kBf16, "bfloat16", ks, "k")) ||
-      !(v = take(a[7], kBf16, "bfloat16", ks, "v")))
+  if (!(q = take(a[5], kBf16, "bfloat16", qs, "q")) || !(k = take(a[6], kBf16, "bfloat16", ks, "k", q)) ||
+      !(v = take(a[7], kBf16, "bfloat16", ks, "v", q)))
     return nullptr;
   const double scale = PyFloat_AsDouble(a[8]);
   if (scale == -1.0 && PyErr_Occurred()) return nullptr;
-  if (a[9] != Py_None && !take(a[9], kBf16, "bfloat16", qs, "o")) return nullptr;
-  if (a[10] != Py_None && !take(a[10], kF32, "float32", ls, "lse")) return nullptr;
+  if (a[9] != Py_None && !take(a[9], kBf16, "bfloat16", qs, "o", q)) return nullptr;
+  if (a[10] != Py_None && !take(a[10], kF32, "float32", ls, "lse", q)) return nullptr;
   const c10::cuda::CUDAGuard guard(q->device());
   const at::Tensor o = a[9] == Py_None ? at::empty(qs, q->options()) : THPVariable_Unpack(a[9]);
   const at::Tensor lse = a[10] == Py_None ? at::empty(ls, q->options().dtype(kF32)) : THPVariable_Unpack(a[10]);
   void* sp = nullptr;
   size_t sn = 0;
   if (a[11] != Py_None) {
-    const at::Tensor& t = THPVariable_Unpack(a[11]);
-    sp = t.data_ptr();
-    sn = size_t(t.numel());
+    const at::Tensor* t = take_buffer(a[11], "scratch", q);
+    if (!t) return nullptr;
+    sp = t->data_ptr();
+    sn = size_t(t->numel());
   }
   const pp_stream_t s = stream_of(q->get_device());
   const void *qp = q->data_ptr(), *kp = k->data_ptr(), *vp = v->data_ptr();
@@ -228,26 +243,31 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (!take_dims(a, handle, d)) return nullptr;
   const int64_t qs[3] = {d.T, d.Hq, d.D}, ks[3] = {d.T, d.Hkv, d.D}, ls[2] = {d.Hq, d.T};
   const at::Tensor *q, *k, *v, *o, *lse, *d_o;
-  if (!(q = take(a[5], kBf16, "bfloat16", qs, "q")) || !(k = take(a[6], kBf16, "bfloat16", ks, "k")) ||
-      !(v = take(a[7], kBf16, "bfloat16", ks, "v")) || !(o = take(a[8], kBf16, "bfloat16", qs, "o")) ||
-      !(lse = take(a[9], kF32, "float32", ls, "lse")) || !(d_o = take(a[10], kBf16, "bfloat16", qs, "d_o")))
+  if (!(q = take(a[5], kBf16, "bfloat16", qs, "q")) || !(k = take(a[6], kBf16, "bfloat16", ks, "k", q)) ||
+      !(v = take(a[7], kBf16, "bfloat16", ks, "v", q)) || !(o = take(a[8], kBf16, "bfloat16", qs, "o", q)) ||
+      !(lse = take(a[9], kF32, "float32", ls, "lse", q)) || !(d_o = take(a[10], kBf16, "bfloat16", qs, "d_o", q)))
     return nullptr;
   const double scale = PyFloat_AsDouble(a[11]);
   if (scale == -1.0 && PyErr_Occurred()) return nullptr;
   const int det = PyObject_IsTrue(a[16]);
   if (det < 0) return nullptr;
+  if ((a[12] != Py_None && !take(a[12], kBf16, "bfloat16", qs, "d_q", q)) ||
+      (a[13] != Py_None && !take(a[13], kBf16, "bfloat16", ks, "d_k", q)) ||
+      (a[14] != Py_None && !take(a[14], kBf16, "bfloat16", ks, "d_v", q)))
+    return nullptr;
+  const at::Tensor* scratch = take_buffer(a[15], "scratch", q);
+  if (!scratch) return nullptr;
   const c10::cuda::CUDAGuard guard(q->device());
   auto out = [&](PyObject* x, const at::Tensor& like, at::IntArrayRef shape) {
     return x == Py_None ? at::empty(shape, like.options()) : THPVariable_Unpack(x);
   };
   const at::Tensor dq = out(a[12], *q, qs), dk = out(a[13], *k, ks), dv = out(a[14], *v, ks);
-  const at::Tensor& sc = THPVariable_Unpack(a[15]);
   const pp_stream_t s = stream_of(q->get_device());
   const void *qp = q->data_ptr(), *kp = k->data_ptr(), *vp = v->data_ptr(), *op = o->data_ptr(),
              *gp = d_o->data_ptr();
   const float* lp = static_cast<const float*>(lse->data_ptr());
-  void *dqp = dq.data_ptr(), *dkp = dk.data_ptr(), *dvp = dv.data_ptr(), *sp = sc.data_ptr();
-  const size_t sn = size_t(sc.numel());
+  void *dqp = dq.data_ptr(), *dkp = dk.data_ptr(), *dvp = dv.data_ptr(), *sp = scratch->data_ptr();
+  const size_t sn = size_t(scratch->numel());
   int rc;
   Py_BEGIN_ALLOW_THREADS
   rc = (det ? api.bwd_det : api.bwd)(static_cast<const pp_plan*>(handle), qp, kp, vp, op, lp, gp, float(scale),

@@ -59,6 +59,38 @@ def test_unsuitable_tensors_are_refused(what, bad):
         B.pp_attn_bwd(plan, args["q"], args["k"], args["v"], o, lse, do, 0.125)
 
 
+@pytest.mark.parametrize("bad", [lambda t: t.float(), lambda t: t[:-1].contiguous(), lambda t: t[:, :1].contiguous(),
+                                 lambda t: t.cpu(), lambda t: t.transpose(0, 1).contiguous().transpose(0, 1),
+                                 lambda t: t.float().cpu().numpy()],
+                         ids=["type", "tokens", "heads", "cpu", "strides", "array"])
+def test_unsuitable_outputs_are_refused(bad):
+    """Before anything is launched: no gradient changes."""
+    B, plan, (q, k, v, do) = _inputs()
+    o, lse = B.pp_attn_fwd(plan, q, k, v, 0.125)
+    with pytest.raises(ValueError, match="^o: expected contiguous CUDA"):
+        B.pp_attn_fwd(plan, q, k, v, 0.125, o=bad(o))
+    out = {n: torch.full_like(t, 7.0) for n, t in (("d_q", q), ("d_k", k), ("d_v", v))}
+    for n, t in out.items():
+        with pytest.raises(ValueError, match=f"^{n}: expected contiguous CUDA"):
+            B.pp_attn_bwd(plan, q, k, v, o, lse, do, 0.125, **{**out, n: bad(t)})
+    assert all(bool((t == 7.0).all()) for t in out.values())
+
+
+@pytest.mark.parametrize("bad", [lambda t: t.cpu(), lambda t: t[:1].expand(t.numel()), lambda t: t.cpu().numpy()],
+                         ids=["cpu", "strides", "array"])
+def test_unsuitable_buffers_are_refused(bad):
+    B, plan, (q, k, v, do) = _inputs()
+    o, lse = B.pp_attn_fwd(plan, q, k, v, 0.125)
+    plan._bwd_scratch = bad(plan.bwd_scratch())
+    with pytest.raises(ValueError, match="^scratch: expected a contiguous CUDA"):
+        B.pp_attn_fwd(plan, q, k, v, 0.125, for_backward=True)
+    with pytest.raises(ValueError, match="^scratch: expected a contiguous CUDA"):
+        B.pp_attn_bwd(plan, q, k, v, o, lse, do, 0.125)
+    for desc in (W1.descriptors(), [a.tolist() for a in W1.descriptors()]):
+        with pytest.raises((ValueError, AttributeError)):
+            B.pp_build_plan(desc, 4, 2, 64, W1.total_tokens, workspace=bad(plan.workspace))
+
+
 def test_library_errors_are_raised():
     B, plan, (q, k, v, do) = _inputs()
     with pytest.raises(B.PPError) as e:
