@@ -1044,7 +1044,7 @@ cudaError_t launch_bwd_t(const pp_plan* plan, const void* o, const float* lse, c
   const size_t n4 = T * Hq * DV / 4;
   unsigned fb = unsigned((n4 + 256 * kFinUnroll - 1) / (256 * kFinUnroll));
   const SumParts sp = {prm.parts, prm.header, prm.tiles, prm.dk, prm.dv, prm.lg_split, pb.num_kv_heads, DV};
-  const unsigned sum_blocks = prm.lg_split ? unsigned(plan->max_tiles) * pb.num_kv_heads * 8 : 0;
+  const unsigned sum_blocks = prm.lg_split ? unsigned(max_btiles_of(pb)) * pb.num_kv_heads * 8 : 0;
   bwd_finalize_kernel<<<fb + sum_blocks, 256, 0, stream>>>(
       reinterpret_cast<const float4*>(prm.dq_acc), static_cast<uint2*>(dq), n4, prm.scale, fb, sp);
   if (e == cudaSuccess) e = cudaGetLastError();

@@ -75,7 +75,7 @@ struct PlanLayout {
   size_t tiles;      // Tile[max_tiles]
   size_t fwd_order;  // int32[max_tiles]
   size_t grp_btile0; // int32[G + 1]  first backward tile of each group
-  size_t btiles;     // BTile[max_tiles]  (at most T / 128 + G of them)
+  size_t btiles;     // BTile[max_tiles]  (at most max_btiles_of of them)
   size_t bwd_order;  // int32[max_tiles]  backward tiles, longest work first
   size_t tile_gwork; // int32[max_tiles]  backward work of the backward tile's whole group
   size_t tile_sgroup; // int32[max_tiles] super-group (block of consecutive groups)
@@ -117,6 +117,8 @@ inline int max_tiles_of(const pp_problem& p) {
   // sum over segments of ceil(len / 128) <= T / 128 + number of segments
   return p.total_tokens / kTile + p.num_groups + p.num_responses;
 }
+// The backward's tiles, cut per group: ceil(length / 128) each.
+inline int max_btiles_of(const pp_problem& p) { return p.total_tokens / kTile + p.num_groups; }
 
 // The forward's query tiles: those of the segments, or tiles of each group's 128-token grid, whose
 // rows may belong to several segments (a group keeps its segments' tiles where they are less
@@ -192,7 +194,7 @@ inline int bwd_split_log2(const pp_problem& p) {
   const double total = units * r * (m + 1) / 2;
   int best = 0;
   double best_time = 0;
-  for (int n = 0; n <= 3 && (1 << n) <= heads && max_tiles_of(p) < (1 << kPartShift); ++n) {
+  for (int n = 0; n <= 3 && (1 << n) <= heads && max_btiles_of(p) < (1 << kPartShift); ++n) {
     const double parts = units * (1 << n), share = (total + (n ? 3 : 2) * parts) / 148;
     const double time = share > longest / (1 << n) + 2 ? share : longest / (1 << n) + 2;
     if (n == 0 || time < 0.95 * best_time) {
@@ -211,11 +213,11 @@ inline BwdScratch bwd_scratch_layout(const pp_problem& p, int lg_split) {
   s.delta = off;  off = align_up(off + 4 * T * Hq, 256);
   s.lse2 = off;   off = align_up(off + 4 * T * Hq, 256);
   s.sem = off;
-  s.sem_bytes = 16 * size_t(max_tiles_of(p)) * Hq;
+  s.sem_bytes = 16 * size_t(max_btiles_of(p)) * Hq;
   off = align_up(off + s.sem_bytes, 256);
   s.parts = off;
   if (lg_split) {
-    const size_t parts = size_t(max_tiles_of(p)) * p.num_kv_heads << lg_split;
+    const size_t parts = size_t(max_btiles_of(p)) * p.num_kv_heads << lg_split;
     off = align_up(off + parts * 2 * kTile * D * 4, 256);
   }
   s.total = off;
