@@ -228,7 +228,8 @@ int pp_preference_loss(const pp_plan* plan, const float* token_logp, const float
  *
  *  - Limit: the scratch pp_plan_workspace_bytes reports for the plan's problem must not exceed
  *    pp_attn_bwd_noalloc_max_bytes (32 MiB, i.e. about T * Hq * D <= 8.2 M elements), not
- *    counting the room for partial dK and dV sums, which are only used where they fit too;
+ *    counting the turn counters of the deterministic variant, which this call has no use for,
+ *    and the room for partial dK and dV sums, which are only used where they fit too;
  *    larger problems are rejected with PP_ERR_STATIC_SCRATCH_LIMIT and nothing is launched.
  *  - Cost: every GPU on which the library is loaded holds those 32 MiB until the process exits.
  *  - The array used is the one on the device that holds the plan's workspace, and that device

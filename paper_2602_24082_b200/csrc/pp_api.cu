@@ -304,8 +304,8 @@ int pp_attn_bwd_noalloc(const pp_plan* plan, const void* q, const void* k, const
   if (!plan || !q || !k || !v || !o || !lse || !d_o || !d_q || !d_k || !d_v)
     return PP_ERR_INVALID_ARG;
   if (!(softmax_scale > 0.f) || softmax_scale > 1e30f) return PP_ERR_INVALID_ARG;
-  // (units stay whole where the parts do not fit)
-  if (pp::bwd_scratch_layout(plan->prob, 0).total > pp::kStaticScratchBytes) return PP_ERR_STATIC_SCRATCH_LIMIT;
+  // (no turn counters here; units stay whole where the parts do not fit)
+  if (pp::bwd_scratch_layout(plan->prob, 0).sem > pp::kStaticScratchBytes) return PP_ERR_STATIC_SCRATCH_LIMIT;
   const void* ptrs[] = {q, k, v, o, lse, d_o, d_q, d_k, d_v};
   for (const void* p : ptrs)
     if (!aligned16(p)) return PP_ERR_ALIGNMENT;

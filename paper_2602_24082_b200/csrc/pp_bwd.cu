@@ -1146,7 +1146,8 @@ cudaError_t launch_bwd_static(const pp_plan* plan, const void* q, const void* k,
   if (e != cudaSuccess) return e;
   // launch_bwd zeroes the fp32 dQ accumulator inside the scratch on every call and rewrites
   // Delta and the scaled LSE, so nothing of an earlier call's contents is read.
-  const int lg_split = plan->bwd_scratch <= kStaticScratchBytes ? plan->lg_split : 0;
+  const int lg_split =
+      bwd_scratch_layout(plan->prob, plan->lg_split).sem <= kStaticScratchBytes ? plan->lg_split : 0;
   return launch_bwd(plan, q, k, v, o, lse, d_o, scale, dq, dk, dv, scratch, lg_split, false, false,
                     stream, launches);
 }

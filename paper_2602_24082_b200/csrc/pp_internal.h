@@ -165,12 +165,12 @@ inline PlanLayout plan_layout(const pp_problem& p) {
   return l;
 }
 
-// Backward scratch: fp32 dQ accumulator [T][Hq][D], Delta [Hq][T], LSE*log2(e) [Hq][T], and
-// the turn counters of the deterministic variant, four per (query tile of the backward grid,
-// query head): one for each warp's 32 rows; and, where units are cut into
-// parts (below), the parts' fp32 dV and dK tiles.
+// Backward scratch: fp32 dQ accumulator [T][Hq][D], Delta [Hq][T], LSE*log2(e) [Hq][T]; where units
+// are cut into parts (below), the parts' fp32 dV and dK tiles; and, last because only the
+// deterministic variant has them, the turn counters, four per (query tile of the backward grid,
+// query head): one for each warp's 32 rows
 struct BwdScratch {
-  size_t dq_acc, delta, lse2, sem, sem_bytes, parts, total;
+  size_t dq_acc, delta, lse2, parts, sem, sem_bytes, total;
 };
 
 // A backward unit (a key tile and KV head against every (query tile, query head) that sees them)
@@ -212,14 +212,14 @@ inline BwdScratch bwd_scratch_layout(const pp_problem& p, int lg_split) {
   s.dq_acc = off; off = align_up(off + 4 * T * Hq * D, 256);
   s.delta = off;  off = align_up(off + 4 * T * Hq, 256);
   s.lse2 = off;   off = align_up(off + 4 * T * Hq, 256);
-  s.sem = off;
-  s.sem_bytes = 16 * size_t(max_btiles_of(p)) * Hq;
-  off = align_up(off + s.sem_bytes, 256);
   s.parts = off;
   if (lg_split) {
     const size_t parts = size_t(max_btiles_of(p)) * p.num_kv_heads << lg_split;
     off = align_up(off + parts * 2 * kTile * D * 4, 256);
   }
+  s.sem = off;
+  s.sem_bytes = 16 * size_t(max_btiles_of(p)) * Hq;
+  off = align_up(off + s.sem_bytes, 256);
   s.total = off;
   return s;
 }

@@ -46,6 +46,24 @@ def test_noalloc_backward_matches_regular_backward_twice():
         assert B.pp_last_launch_count() == 3
 
 
+def test_noalloc_does_not_count_the_turn_counters():
+    """1950 groups of two tokens: accumulator and statistics fit, with the counters of the deterministic
+    variant, which this call has no use for, the scratch is larger than the built-in one."""
+    from paper_2602_24082_b200 import binding as B
+    w = W.Workload("short", [[(1, (1,))] * 1950], 32, 8, 64, seed=4)
+    plan = B.plan_for(w)
+    limit = B.pp_attn_bwd_noalloc_max_bytes()
+    assert 4 * w.total_tokens * 32 * (64 + 2) <= limit < plan.bwd_scratch_bytes
+    q, k, v, do = (x.cuda() for x in w.tensors())
+    o, lse = B.pp_attn_fwd(plan, q, k, v, w.softmax_scale)
+    ref = B.pp_attn_bwd(plan, q, k, v, o, lse, do, w.softmax_scale)
+    got = [torch.full_like(x, 9.0) for x in ref]
+    B.pp_attn_bwd_noalloc(plan, q, k, v, o, lse, do, w.softmax_scale, *got)
+    torch.cuda.synchronize()
+    # every group is one key tile, so dQ is one sum here and as fixed as dK and dV
+    assert plan.status() == (0, 0) and all(torch.equal(a, b) for a, b in zip(got, ref))
+
+
 def test_noalloc_rejects_problems_beyond_the_builtin_scratch():
     from paper_2602_24082_b200 import binding as B
     limit = B.pp_attn_bwd_noalloc_max_bytes()
