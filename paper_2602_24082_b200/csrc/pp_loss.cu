@@ -45,14 +45,17 @@ __global__ void __launch_bounds__(kLossThreads)
 preference_loss_kernel(LossPtrs p, const float* __restrict__ logp, const float* __restrict__ ref,
                        float beta, float* __restrict__ resp_logp, float* resp_reward,
                        float* __restrict__ grp_loss, float* __restrict__ d_logp, int team_warps) {
-  __shared__ float s_sum[kLossWarps], s_ref[kLossWarps], s_grad[kLossWarps];
+  __shared__ double s_sum[kLossWarps], s_ref[kLossWarps];
+  __shared__ float s_grad[kLossWarps];
   if (p.header[0] != kStatusOk) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = blockIdx.x;
   const int x0 = p.grp_resp_off[g], x1 = p.grp_resp_off[g + 1], n = x1 - x0;
   const int sp = g + x0;  // the group's prompt segment; response x is segment g + 1 + x
   const int teams = kLossWarps / team_warps, team = warp / team_warps, in_team = warp % team_warps;
-  // 1. sequence log-probs and rewards, `teams` responses at a time
+  // 1. sequence log-probs and rewards, `teams` responses at a time.  A lane's own terms, a few dozen,
+  // are added in fp32, everything above in fp64: a reward is the small difference of two large sums, and
+  // every rounding of those is many times larger in it.
   for (int first = x0; first < x1; first += teams) {
     const int x = first + team;
     float s = 0.f, sr = 0.f;
@@ -66,23 +69,24 @@ preference_loss_kernel(LossPtrs p, const float* __restrict__ logp, const float* 
       else
         for_tokens(a, b, in_team, team_warps, [&](int t) { s += logp[t]; });
     }
+    double sum = s, sum_ref = sr;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      s += __shfl_xor_sync(0xffffffffu, s, o);
-      sr += __shfl_xor_sync(0xffffffffu, sr, o);
+      sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      sum_ref += __shfl_xor_sync(0xffffffffu, sum_ref, o);
     }
     if (lane == 0) {
-      s_sum[warp] = s;
-      s_ref[warp] = sr;
+      s_sum[warp] = sum;
+      s_ref[warp] = sum_ref;
     }
     __syncthreads();
     if (in_team == 0 && lane == 0 && x < x1) {
       for (int w = 1; w < team_warps; ++w) {
-        s += s_sum[warp + w];
-        sr += s_ref[warp + w];
+        sum += s_sum[warp + w];
+        sum_ref += s_ref[warp + w];
       }
-      resp_logp[x] = s;
-      resp_reward[x] = beta * (s - sr);
+      resp_logp[x] = float(sum);
+      resp_reward[x] = float(beta * (sum - sum_ref));
     }
     __syncthreads();
   }

@@ -50,3 +50,22 @@ def test_preference_loss_parity(w, with_ref):
         if seg == 0:
             prompt[st:st + ln] = True
     assert not grad[prompt].any()
+
+
+@pytest.mark.parametrize("rows", [[[(100, (8192, 5000, 33))]], [[(9, (4097, 4000))], [(300, (1, 7000))]],
+                                  [[(3, (150, 201)), (1, (7, 90, 8, 1))]] * 40, [[(5, (40, 30))]] * 5000],
+                         ids=["long", "two", "short", "many"])
+def test_sums_are_rounded_once(rows):
+    """Multiples of 2^-16 below 4: the few dozen terms of a lane add up exactly in fp32, a response's sum
+    does not fit 24 bits, so what comes out is the exact sum (and beta times the exact difference) rounded."""
+    from paper_2602_24082_b200 import binding as B
+    w = W.Workload("exact", rows, 1, 1, 64, seed=1)
+    rng = np.random.default_rng(3)
+    lp, ref = (-rng.integers(0, 1 << 18, w.total_tokens) / 65536.0 for _ in range(2))
+    plan = B.plan_for(w)
+    f32 = lambda x: torch.from_numpy(x.astype(np.float32)).cuda()
+    s, r, _, _ = B.pp_preference_loss(plan, f32(lp), f32(ref), 0.1)
+    spans = [(a, a + n) for a, n, _, _, seg in w.segments() if seg]
+    S, Sr = (np.array([x[a:b].sum() for a, b in spans]) for x in (lp, ref))
+    assert np.array_equal(s.cpu().numpy(), S.astype(np.float32))
+    assert np.array_equal(r.cpu().numpy(), (np.float64(np.float32(0.1)) * (S - Sr)).astype(np.float32))
