@@ -20,6 +20,13 @@ CASES = [
     W.Workload("mean400", [[(400, (511, 289, 400))], [(1, (799,))]], 1, 1, 64, seed=8),
     W.Workload("mean900", [[(900, (1023, 1, 1577))]], 1, 1, 64, seed=9),
     W.Workload("mean4096", [[(4096, (4095, 4097))]], 1, 1, 64, seed=10),
+    # every number of warps per group (16 up to 296 groups on 148 SMs, then 8, 4, 2, 1), a last block
+    # that is not full, more responses than a warp has lanes
+    W.Workload("gang8", [[(3, (40, 2)), (1, (1,) * 17), (300, (200,))]] * 149, 1, 1, 64, seed=11),
+    W.Workload("gang8-many", [[(3, (40, 2)), (1, (1,) * 33)]] * 401, 1, 1, 64, seed=15),
+    W.Workload("gang4", [[(150, (140, 2, 130))]] * 701, 1, 1, 64, seed=12),
+    W.Workload("gang2", [[(2, (3, 1)), (7, (130,)), (1, (1, 2, 3, 4))]] * 401, 1, 1, 64, seed=13),
+    W.Workload("gang1", [[(2, (3, 1)), (9, (35, 1, 70, 33))]] * 1201, 1, 1, 64, seed=14),
 ] + [W.random_structure(s) for s in range(8)]
 
 
