@@ -42,6 +42,8 @@ CASES = [
     ("d96", [[(90, (39, 127, 1, 1, 60))], [(1, (126, 1, 1, 300))], [(250, (6, 7, 8))]], 40, 8, 96),
     ("sorted-orders", _many(150, 1), 2, 1, 64),         # more than 512 tiles
     ("multi-kernel-plan", _many(520, 2), 1, 1, 64),     # more than 2048 tiles
+    # works of 1 to 24 key tiles, in groups of either kind of tile
+    ("multi-kernel-long", _many(300, 3) + [[(1500, (1400, 1, 90)), (2, (300, 1, 1))]] + _many(250, 4), 2, 2, 64),
 ]
 
 
