@@ -1,5 +1,5 @@
 """Thin binding of libpp_attn.so: argument marshalling only (the calls of a step -- plan,
-forward, backward -- through the CPython module _pp_torch, everything else through ctypes).
+forward, backward -- through the CPython module _pp_torch_*, everything else through ctypes).
 
 Every step of the path (plan building, forward, backward) runs in the library's CUDA
 kernels; PyTorch only provides device memory and the current stream.  There is no CPU
@@ -11,11 +11,14 @@ pp_attn_bwd.
 from __future__ import annotations
 
 import ctypes
+import importlib
 import os
 from typing import Optional, Sequence, Tuple
 
 import numpy as np
 import torch
+
+from .build import ext_module
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libpp_attn.so")
@@ -121,13 +124,14 @@ def _step_calls():
     global _ext
     if _ext is None:
         lib()
+        name = ext_module()
         try:
-            from . import _pp_torch
+            module = importlib.import_module("." + name, __package__)
         except ImportError as e:
-            raise RuntimeError("_pp_torch.so is missing or does not load: build it with "
+            raise RuntimeError(f"{name} is missing or does not load: build it with "
                                "`python -m paper_2602_24082_b200.build`") from e
-        _pp_torch.bind(LIB_PATH, PPError, _chk)
-        _ext = _pp_torch
+        module.bind(LIB_PATH, PPError, _chk)
+        _ext = module
     return _ext
 
 

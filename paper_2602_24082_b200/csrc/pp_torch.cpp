@@ -286,8 +286,12 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
 #define PP_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(name)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {PP_METHOD(bind), PP_METHOD(build_plan), PP_METHOD(fwd), PP_METHOD(bwd),
                          {nullptr, nullptr, 0, nullptr}};
-PyModuleDef module = {PyModuleDef_HEAD_INIT, "_pp_torch", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+#define PP_STR2(x) #x
+#define PP_STR(x) PP_STR2(x)
+#define PP_INIT2(x) PyInit_##x
+#define PP_INIT(x) PP_INIT2(x)
+PyModuleDef module = {PyModuleDef_HEAD_INIT, PP_STR(PP_MODULE), nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__pp_torch() { return PyModule_Create(&module); }
+PyMODINIT_FUNC PP_INIT(PP_MODULE)() { return PyModule_Create(&module); }   // (PP_MODULE: see build.py)
