@@ -36,6 +36,10 @@ FALLBACK_BF16_TFLOPS = 1590.0
 TARGET_CONFIGS = ["config1", "config2", "config3"] + [f"config4:{i}" for i in range(6)]
 HEADLINE = "config4:2"     # rho = 4, n = 2: the most useful FLOPs per step of all workloads
 
+# Measured beside the headline's step (headline_extras and the unpacked batches).
+ALSO = ("unpacked_padded", "unpacked_unpadded", "rope_qk", "preference_loss", "deterministic_bwd", "row_builder",
+        "row_assignment", "no_kernel_events", "graph_replay")
+
 # Paper figures (end-to-end training ratios on unnamed hardware): context only.
 PAPER_CONTEXT = {
     "training_time_reduction_at_least": 0.37,
@@ -444,7 +448,7 @@ class Runner:
         lbytes = 12.0 * T
         lg = lbytes / (statistics.median(lms) * 1e-3) / 1e9
         out["preference_loss"] = {"ms": statistics.median(lms), "bytes": lbytes,
-                                  "note": "latency-bound: one warp per group, 12 bytes per token",
+                                  "note": "latency-bound: 12 bytes per token",
                                   "roofline": {"bound": "hbm", "achieved": lg, "peak": self.hbm,
                                                "unit": "GB/s", "frac": lg / self.hbm}}
 
@@ -567,6 +571,46 @@ def rank_workload(name, rank, world, dev):
                "max_over_mean_rank_cost": float(rc.max() / rc.mean())}
 
 
+def rounded(x):
+    """Floats to six digits, in whatever holds them."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k_: rounded(v_) for k_, v_ in x.items()}
+    return [rounded(v_) for v_ in x] if isinstance(x, (list, tuple)) else x
+
+
+def result_line(head, per_config, world, dp=None) -> str:
+    """The JSON line: the headline workload's figures, and of the other workloads the throughput, the
+    step, the fractions of the peaks and the speedup over the unpacked batch."""
+    line = {
+        "metric": METRIC, "value": head["value"], "unit": UNIT, "n_gpus": world, "steps": head["steps"],
+        "warmup": head["warmup"], "ms_per_step": head["ms_per_step"], "higher_is_better": True,
+        "scaling": "weak", "vs_baseline": None, "dtype": "bf16", "data": "synthetic",
+    }
+    for k_ in ("config", "clocks", "gpu_launches", "tokens_per_s", "pct_of_peak", "roofline", "e2e", "cpu_baseline"):
+        line[k_] = head.get(k_)
+    line["roofline_fwd"] = {k_: head["roofline_fwd"][k_] for k_ in ("achieved", "frac", "avg_launch_ms")}
+    # what else is measured beside the step, in milliseconds
+    line["also_ms"] = {k_: v_.get("ms", v_.get("ms_per_step", v_.get("main_kernel_ms"))) for k_, v_ in head.items()
+                       if k_ in ALSO and isinstance(v_, dict)}
+    if dp:
+        line["data_parallel"] = dp
+    if per_config:
+        speedups = {n: [d.get(k_, {}).get("speedup_of_packed", 0.0) for k_ in ("unpacked_padded", "unpacked_unpadded")]
+                    for n, d in per_config.items()}
+        line["per_config"] = {n: {"value": d["value"], "ms_per_step": d["ms_per_step"],
+                                  "pct_of_burst": d["pct_of_peak"]["measured_burst"],
+                                  "speedup_padded_unpadded": speedups[n]}
+                              for n, d in ((n, per_config[n]) for n in TARGET_CONFIGS if n in per_config)}
+        pct = {n: per_config[n]["pct_of_peak"] for n in line["per_config"]}
+        line["min_pct_of_peak_over_configs"] = {
+            kind: min(p[kind] for p in pct.values()) for kind in ("measured_burst", "measured_sustained", "nominal")}
+        line["min_pct_of_peak_over_configs"]["config"] = min(pct, key=lambda n: pct[n]["measured_burst"])
+        line["packed_faster_than_unpacked_on_every_config"] = all(min(speedups[n]) > 1.0 for n in line["per_config"])
+    return json.dumps(rounded(line), separators=(",", ":"))
+
+
 def run_ours(args):
     import torch
     import torch.distributed as dist
@@ -597,35 +641,14 @@ def run_ours(args):
         args.no_cpu_baseline = True
     head = runner.measure(head_name, w, headline=not args.quick)
     if rank == 0:
-        line = {
-            "metric": METRIC, "value": head["value"], "unit": UNIT, "n_gpus": world, "steps": head["steps"],
-            "warmup": head["warmup"], "ms_per_step": head["ms_per_step"], "higher_is_better": True,
-            "scaling": "weak", "vs_baseline": None, "dtype": "bf16", "data": "synthetic",
-        }
-        for k_, v_ in head.items():
-            if k_ not in line:
-                line[k_] = v_
-        if dp:
-            line["data_parallel"] = dp
-        line.setdefault("cpu_baseline", None)
-        line["paper_context"] = PAPER_CONTEXT
+        # the details go to stderr, one line per workload: the result line stays short enough to be
+        # kept whole by whoever records it
         if per_config:
-            slim = lambda d: {k_: d[k_] for k_ in ("value", "unit", "ms_per_step", "steps", "clocks", "pct_of_peak",
-                                                   "tokens_per_s", "roofline", "roofline_fwd",
-                                                   "outside_main_kernels_ms", "unpacked_padded",
-                                                   "unpacked_unpadded", "paper_cost_model_mean", "config")
-                              if k_ in d}
             per_config[head_name] = head
-            line["per_config"] = {n: slim(per_config[n]) for n in TARGET_CONFIGS if n in per_config}
-            pct = {n: per_config[n]["pct_of_peak"] for n in line["per_config"]}
-            line["min_pct_of_peak_over_configs"] = {
-                kind: min(p[kind] for p in pct.values()) for kind in ("measured_burst", "measured_sustained", "nominal")}
-            line["min_pct_of_peak_over_configs"]["config"] = min(pct, key=lambda n: pct[n]["measured_burst"])
-            line["packed_faster_than_unpacked_on_every_config"] = all(
-                per_config[n].get("unpacked_padded", {}).get("speedup_of_packed", 0) > 1.0 and
-                per_config[n].get("unpacked_unpadded", {}).get("speedup_of_packed", 0) > 1.0
-                for n in line["per_config"])
-        print(json.dumps(line))
+        for n, d in (per_config or {head_name: head}).items():
+            print(json.dumps({n: d}), file=sys.stderr)
+        print(json.dumps({"paper_context": PAPER_CONTEXT}), file=sys.stderr)
+        print(result_line(head, per_config, world, dp))
     if world > 1:
         dist.destroy_process_group()
 

@@ -38,3 +38,38 @@ def test_headline_and_target_workloads_are_the_nine_full_size_ones():
     for n in bench.TARGET_CONFIGS:
         b, how = bench.dram_traffic(n)
         assert b and b > 1e8 and "ncu" in how
+
+
+def test_the_result_line_is_short_and_holds_the_agreed_keys():
+    """Nine workloads, every figure at full length."""
+    sys.path.insert(0, ROOT)
+    import bench
+    x = 1234.5678901234567
+    roof = {"kernel": "bwd_kernel (dS/dQ/dK/dV main)", "bound": "tensor", "achieved": x, "peak": x, "unit": "TFLOP/s",
+            "frac": x, "peak_kind": "of measured (sustained)", "frac_of_burst_peak": x, "frac_of_sustained_peak": x,
+            "traffic": x * 1e7, "traffic_source": "ncu capture of the two DRAM counters (1 pass)",
+            "traffic_unit": "bytes (dram read + write per launch)", "algorithmic_flops_per_launch": x * 1e10,
+            "avg_launch_ms": x}
+    unpacked = {"ms_per_step": x, "tokens": 123998, "speedup_of_packed": 1.8, "useful_pair_ratio": x}
+    one = lambda n: {"metric": bench.METRIC, "value": x, "unit": bench.UNIT, "steps": 20, "warmup": 5, "ms_per_step": x,
+                     "ms_min_median": [x, x], "config": bench.workload_config(bench.get_workload(n), n),
+                     "clocks": {"sm_mhz": 1462.0, "sm_max_mhz": 1965, "reasons": ["sw_power_cap"], "samples": 106},
+                     "gpu_launches": 100, "tokens_per_s": x * 1e6, "roofline": roof, "roofline_fwd": roof,
+                     "pct_of_peak": {"measured_burst": x, "measured_sustained": x, "nominal": x},
+                     "outside_main_kernels_ms": x, "unpacked_padded": unpacked, "unpacked_unpadded": unpacked,
+                     "paper_cost_model_mean": {"attention_cost_ratio": x, "memory_ratio": x}}
+    per = {n: one(n) for n in bench.TARGET_CONFIGS}
+    head = per[bench.HEADLINE]
+    extra = {"ms": x, "bytes": x * 1e8, "note": "n" * 90, "roofline": {"achieved": x, "peak": x, "unit": "GB/s", "frac": x}}
+    head.update(e2e={"value": x, "unit": bench.UNIT, "h2d_bytes_per_step": 10 ** 9, "d2h_bytes_per_step": 10 ** 9},
+                cpu_baseline={"value": x, "unit": bench.UNIT, "cores": 16, "kind": "oracle", "sample": "s" * 140},
+                **{k: extra for k in ("rope_qk", "preference_loss", "deterministic_bwd", "head_dim_96", "row_builder",
+                                      "row_assignment", "no_kernel_events", "graph_replay")})
+    text = bench.result_line(head, per, 1)
+    assert len(text) < 4000 and "\n" not in text
+    d = json.loads(text)
+    for key in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                "vs_baseline", "dtype", "data", "config", "clocks", "e2e", "gpu_launches"):
+        assert key in d
+    assert abs(d["value"] - x) < 1e-5 * x and list(d["per_config"]) == bench.TARGET_CONFIGS
+    assert d["packed_faster_than_unpacked_on_every_config"] is True
