@@ -193,10 +193,13 @@ def test_device_side_validation_reports_status():
 
 
 @pytest.mark.parametrize("segs,length", [(127, 1), (128, 1), (256, 1), (257, 1), (129, 130), (512, 1), (513, 1),
-                                         (1024, 1), (1025, 1), (300, 300), (2040, 1)])
+                                         (1024, 1), (1025, 1), (300, 300), (2032, 1), (2040, 1),
+                                         (150, 1000), (24, 8500)])
 def test_one_block_plan_at_the_edges_of_its_sorts_and_blocks(segs, length):
-    """Blocks of 256 and 1024 threads, orders by rank counting (up to 512 tiles) and by sorting:
-    the multi-kernel path's orders are reproduced exactly (longest first, ties by index)."""
+    """Blocks of 256 and 1024 threads, orders by rank counting (up to 512 tiles) and by sorting, one key
+    per thread and two (above 1024 tiles; the last two cases with segments' tiles, the others of that
+    size with mixed ones): the multi-kernel path's orders are reproduced exactly (longest first, ties by
+    index)."""
     from paper_2602_24082_b200 import binding as B
     rng = np.random.default_rng(segs)
     rows, left = [], segs
@@ -209,7 +212,8 @@ def test_one_block_plan_at_the_edges_of_its_sorts_and_blocks(segs, length):
         left -= 1 + n
     w = W.Workload("edges", rows, 6, 3, 64, seed=1)
     plan = B.plan_for(w)
-    assert plan.status() == (0, 0)
+    one_block = w.total_tokens // 128 + segs <= 2048      # (2040 segments of one token: just beyond)
+    assert plan.status() == (0, 0) and (B.pp_last_launch_count() == 1) == one_block == (segs != 2040)
     tiles, fwd_order, bwd_order, key_end = plan.read()
     btiles = plan.read_bwd_tiles()
     nb = len(btiles)
