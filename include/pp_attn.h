@@ -81,7 +81,9 @@ int pp_plan_workspace_bytes(const pp_problem* problem, size_t* plan_bytes,
  * descriptors into query/key tiles of 128 tokens aligned to segment starts, each with the
  * key ranges it must visit -- the prompt range and the part of its own segment before it
  * (class FULL: no masking), then its own diagonal tile (class DIAG: causal masking) --
- * while tiles of sibling responses are never listed (class SKIP is implicit).  The same
+ * while tiles of sibling responses are never listed (class SKIP is implicit).  (Where a batch
+ * has many short segments the forward runs over other query tiles instead, 128-token tiles of each
+ * group whose rows may belong to several segments; the tables below stay those of the segments.)  The same
  * tiles, read as key tiles, carry the contiguous query range [start, vis_end) that sees
  * them, for the backward pass.  Tiles are ordered longest-work-first for the forward pass;
  * the backward pass processes (tile, KV head) units group by group (largest group first,
@@ -144,7 +146,9 @@ int pp_plan_read(const pp_plan* plan, pp_stream_t stream, int32_t* num_tiles, in
 
 /*
  * Forward (Sec. 3.2): O = softmax(mask(scale * Q K^T)) V and LSE, per row and query head.
- * q, k, v, o: bf16 device pointers; lse: fp32 device pointer.  The forward itself needs no
+ * q, k, v, o: bf16 device pointers; lse: fp32 device pointer.  Inputs are finite: whole tiles are
+ * multiplied, hidden keys with a weight of zero, so that a NaN or an infinity in one token may
+ * reach other rows of its group (here and in the backward).  The forward itself needs no
  * scratch: d_scratch may be NULL.  Training callers may pass the buffer they are going to give
  * pp_attn_bwd as its scratch (256-byte aligned, at least the backward size reported by
  * pp_plan_workspace_bytes; PP_ERR_WORKSPACE_TOO_SMALL / PP_ERR_ALIGNMENT otherwise): the
@@ -175,10 +179,9 @@ int pp_attn_bwd(const pp_plan* plan, const void* q, const void* k, const void* v
  * verify run against run).  pp_attn_bwd adds the per-key-tile contributions to a query tile's
  * dQ in whatever order the CTAs reach it, so dQ can differ in the last bits between runs; here
  * the key tiles of a group take turns in descending tile order -- the order in which the units,
- * each walking its query tiles upwards from its own tile, reach a query tile anyway -- (one
- * counter per query tile and head inside d_scratch; units handed out one (group, KV head) set
- * after the other and in descending tile order inside a set, so that no CTA waits for work
- * that has not started).  dK, dV and the forward are reproducible in both variants.
+ * each walking its query tiles upwards from its own tile, reach a query tile anyway -- (counters
+ * per query tile and head inside d_scratch; units handed out one (group, KV head) set after
+ * the other, inside a set in an order in which some CTA always can go on).  dK, dV and the forward are reproducible in both variants.
  * Same arguments, sizes and errors as pp_attn_bwd; a turn that does not come within a bounded
  * number of polls sets the plan's status word (PP_ERR_PLAN_STATUS from pp_plan_status).
  */

@@ -10,7 +10,7 @@
 //                Per query tile: S^T = K Q^T and dP^T = V dO^T (tensor memory), P^T =
 //                exp2(S^T - LSE), dS^T = P^T (dP^T - Delta) in registers (thread = key row),
 //                dV += P^T dO, dK += dS^T Q, dQ_tile = dS K.  Only dQ leaves the CTA per tile:
-//                it is added into an fp32 accumulator with vector reductions.
+//                it is added into an fp32 accumulator with TMA reductions.
 //   finalize   : dQ = bf16(scale * accumulator)
 #include <algorithm>
 #include <mutex>

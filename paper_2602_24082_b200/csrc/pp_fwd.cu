@@ -12,7 +12,8 @@
 //   warps 18-19 optional: clear the backward's fp32 dQ accumulator for the unit's rows
 // A work unit is (query tile, KV head, pair of query heads of that KV head): both slots see
 // the same keys and the same mask, so every K / V tile staged in shared memory feeds two
-// S tiles.  While one slot's warpgroup does its exponentials the tensor core works on the
+// S tiles.  (The last head of an odd number of heads per KV head, and every head where there is one
+// per KV head, is a unit of its own, with slot 1 empty.)  While one slot's warpgroup does its exponentials the tensor core works on the
 // other slot (order: PV_0(j), QK_0(j+1), PV_1(j), QK_1(j+1), ...).  P (bf16) overwrites columns
 // [0,32) and [64,96) of its S tile in tensor memory (each half-row thread inside the columns it
 // has read itself) and is the A operand of the second MMA; V is
@@ -50,15 +51,13 @@ enum FwdBar : int {
   kQEmpty = 2,  // [2]
   kKFull = 4,   // [2] per K / V stage: full
   kKEmpty = 6,  // [2]                 empty
-  kVFull = 8,   // (unused)
-  kVEmpty = 10,
-  kSFull = 12,  // [2] per slot
-  kPFull = 14,
-  kODone = 16,
-  kOFree = 18,
-  kSchedFullF = 20,   // [2] unit ids handed from the producer to the other roles
-  kSchedEmptyF = 22,  // [2] 17 arrivals: MMA thread + 16 softmax warps
-  kNumFwdBars = 24
+  kSFull = 8,   // [2] per slot
+  kPFull = 10,
+  kODone = 12,
+  kOFree = 14,
+  kSchedFullF = 16,   // [2] unit ids handed from the producer to the other roles
+  kSchedEmptyF = 18,  // [2] 17 arrivals: MMA thread + 16 softmax warps (+ 2 clearing warps)
+  kNumFwdBars = 20
 };
 
 template <int D>

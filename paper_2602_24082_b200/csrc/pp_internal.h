@@ -128,8 +128,8 @@ inline int max_btiles_of(const pp_problem& p) { return p.total_tokens / kTile + 
 // more than 0.3 to the number of tiles and there are more units than run in two waves anyway.
 // Whole steps, segments -> grid, at (added tiles, units per SM): (2.6, 5) 139 -> 97 us, (1.4, 8)
 // 148 -> 118, (0.42, 54) 1805 -> 1524, (0.45, 13) 326 -> 289, (0.72, 1.8) 66 -> 63; but (0.27, 9)
-// 170 -> 173, (0.36, 1.6) 105 -> 112, (1.25, 0.4) 49 -> 52.  By sizes alone, so that every way of
-// running a problem sums in the same order.
+// 170 -> 173, (0.36, 1.6) 105 -> 112, (1.25, 0.4) 49 -> 52.  By sizes alone, 148 SMs whatever part of a
+// device there is, so that every way of running a problem sums in the same order.
 inline bool fwd_mixed_tiles(const pp_problem& p) {
   const int pairs = (p.num_q_heads / p.num_kv_heads + 1) / 2;
   const double grid = p.total_tokens / double(kTile) + 0.5 * p.num_groups, added = 0.5 * p.num_responses;
@@ -179,8 +179,10 @@ struct BwdScratch {
 // cut into 2^n parts by query heads, which CTAs process independently; each part leaves its dV and
 // dK in fp32 in the scratch and the finalize kernel adds them up in order.  n minimises the
 // estimated time in iterations, the longer of the longest part and everything's share per SM, with
-// two iterations of overhead for a unit and three for a part; it depends on sizes alone, so that
-// every way of running a problem sums in the same order.  Whole steps, units whole -> cut (us):
+// two iterations of overhead for a unit and three for a part; it depends on sizes alone (148 SMs
+// whatever part of a device there is), so that every way of running a problem sums in the same order.
+// It knows the mean group, not the longest: one long group among many short ones may get fewer parts
+// than would suit it.  Whole steps, units whole -> cut (us):
 // 276 tokens, 8 heads on 1 KV head 99 -> 56; 573, 32 on 4 102 -> 53; 8999, 7 on 1 183 -> 114; 3999,
 // 4 on 1 in one group 251 -> 113; 2753, 2 on 1 50 -> 44.  From about 148 units' worth of balanced
 // work on, parts only add their overhead and fp32 traffic, and the rule leaves units whole.

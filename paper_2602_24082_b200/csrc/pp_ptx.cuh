@@ -101,14 +101,6 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tmap, int 
       : "memory");
 }
 
-// Ask the TMA unit to bring a tile into L2 ahead of the load that will need it.
-__device__ __forceinline__ void tma_prefetch_l2_3d(const void* tmap, int c0, int c1, int c2) {
-  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(
-                   reinterpret_cast<uint64_t>(tmap)),
-               "r"(c0), "r"(c1), "r"(c2)
-               : "memory");
-}
-
 // 3-D tiled reduction shared -> global (element-wise add), tracked by bulk async-groups.
 __device__ __forceinline__ void tma_reduce_add_3d(const void* tmap, uint32_t src, int c0, int c1,
                                                   int c2) {
@@ -183,7 +175,7 @@ __device__ __forceinline__ uint32_t make_sdesc_lo(uint32_t smem_addr, uint32_t l
   return ((smem_addr & 0x3FFFFu) >> 4) | (((lbo_bytes >> 4) & 0x3FFFu) << 16);
 }
 
-// Shared-memory operands are given by the LOW word of their matrix descriptor (see make_sdesc):
+// Shared-memory operands are given by the LOW word of their matrix descriptor (see make_sdesc_lo):
 // the high word is the same for every tile here, so the issuing thread handles one register per
 // operand and k-step instead of two.
 // D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate, one CTA.
@@ -332,11 +324,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   uint32_t r;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
   return r;
-}
-__device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float c, float d) {
-  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c),
-               "f"(d)
-               : "memory");
 }
 
 }  // namespace pp
