@@ -866,7 +866,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
       // its own behind the acquire that sees it and a proxy fence.  Release and acquire cost this
       // warp about a thousand cycles each, the first while the tile behind it waits in registers and
       // not in tensor memory (with the release at the end of the iteration four 4800-token groups,
-      // 28 / 4 heads, take 2306 us, here 2220; eight 1100-token groups, 32 / 8, 438 and 415).
+      // 28 / 4 heads, take 2306 us, here 2207; eight 1100-token groups, 32 / 8, 438 and 415).  It is this
+      // variant's longest chain: two rows of 32768 tokens take 25.6 ms, by default 20.0.
       auto publish = [&](int32_t* p) { store_release_gpu(p, k_rel + 1); };
       for (int it = 0; it < un.n_it; ++it, q_advance<kDet>(qi, unit_heads<kSplit>(prm, un), un.nq)) {
         const QTile qt = q_tile_at<kSplit>(prm, un, qi);
