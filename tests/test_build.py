@@ -9,9 +9,9 @@ from paper_2602_24082_b200 import build as B
 
 
 def test_a_module_built_for_another_torch_or_python_is_not_up_to_date(monkeypatch):
+    B.build()
     started = []
     monkeypatch.setattr(B.subprocess, "Popen", lambda cmd, **kw: started.append(cmd))
-    B.build()                      # (built by now, whatever was there: nothing to start)
     assert B._start_ext(False) is None and not started
     here = B.ext_path()
     monkeypatch.setattr(torch, "__version__", torch.__version__ + ".post1")
