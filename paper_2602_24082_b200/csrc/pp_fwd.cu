@@ -45,6 +45,7 @@ struct FwdParams {
 constexpr int kFwdThreads = 640;
 constexpr uint32_t kFwdTmemCols = 512;
 constexpr float kRescaleThreshold = 8.f;  // log2 units
+constexpr int kEarlySteps = 3;            // of a half row's four 16-key steps of P, those handed over first
 
 enum FwdBar : int {
   kQFull = 0,   // [2] per slot
@@ -57,7 +58,8 @@ enum FwdBar : int {
   kOFree = 14,
   kSchedFullF = 16,   // [2] unit ids handed from the producer to the other roles
   kSchedEmptyF = 18,  // [2] 17 arrivals: MMA thread + 16 softmax warps (+ 2 clearing warps)
-  kNumFwdBars = 20
+  kPRest = 20,        // [2] per slot: the late columns of P (kPFull: the early ones)
+  kNumFwdBars = 22
 };
 
 template <int D>
@@ -65,8 +67,8 @@ struct FwdSmem {
   static constexpr int kTileBytes = 128 * D * 2;
   static constexpr int kQ = 0, kK = 2 * kTileBytes, kV = 4 * kTileBytes, kBars = 6 * kTileBytes;
   static constexpr int kSched = kBars + 256;          // two decoded unit records of 8 ints
-  static constexpr int kXch = kSched + 64;            // float [2 slots][2 buffers][128 rows][2 halves]
-  static constexpr int kTotal = kXch + 4096 + 1024;   // + slack to align the base to 1024 B
+  static constexpr int kXch = kSched + 64;            // float [2 slots][3 buffers][128 rows][2 halves]
+  static constexpr int kTotal = kXch + 6144 + 1024;   // + slack to align the base to 1024 B
 };
 
 struct KvTile {
@@ -157,7 +159,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
 
   if (tid == 0) {
     for (int i = 0; i < kNumFwdBars; ++i) {
-      const bool wg_count = (i >= kPFull && i < kPFull + 2) || (i >= kOFree && i < kOFree + 2);
+      const bool wg_count = (i >= kPFull && i < kPFull + 2) || (i >= kOFree && i < kOFree + 2) || i >= kPRest;
       const bool sched_empty = (i >= kSchedEmptyF && i < kSchedEmptyF + 2);
       // unit records are released by the MMA thread, the 16 softmax warps and, when the dQ
       // accumulator is cleared here, the two clearing warps
@@ -296,20 +298,35 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         }
         mma_commit(bar(kSFull + s));
       };
-      auto issue_pv = [&](int s, uint32_t vstage, int k_len, bool first, bool last) {
+      // P arrives in two parts: of the four k-steps (16 keys each) of each half row the first
+      // kEarlySteps, then the others
+      auto issue_pv = [&](int s, uint32_t vstage, int k_len, bool first, bool last, uint32_t par) {
         const uint32_t b = dv0 + vstage * kStageStep;
         const uint32_t tS = tmem + s * 128, tO = tmem + 256 + s * 128;
         if (k_len == kTile && !first) {
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)
-            mma_ts(tO, tS + (kk < 4 ? kk * 8 : 64 + (kk - 4) * 8), b + mnmajor_off(kk), idesc_o, 1);
+            if ((kk & 3) < kEarlySteps)
+              mma_ts(tO, tS + (kk < 4 ? kk * 8 : 64 + (kk - 4) * 8), b + mnmajor_off(kk), idesc_o, 1);
+          wait_bar(bar(kPRest + s), par, abort_flag, prm.header, 39);
+          tc_fence_after();
+#pragma unroll
+          for (int kk = 0; kk < 8; ++kk)
+            if ((kk & 3) >= kEarlySteps)
+              mma_ts(tO, tS + (kk < 4 ? kk * 8 : 64 + (kk - 4) * 8), b + mnmajor_off(kk), idesc_o, 1);
         } else {
           const int ksteps = (k_len + 15) >> 4;
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)
-            if (kk < ksteps)
+            if ((kk & 3) < kEarlySteps && kk < ksteps)
               mma_ts(tO, tS + (kk < 4 ? kk * 8 : 64 + (kk - 4) * 8), b + mnmajor_off(kk), idesc_o,
                      !first || (kk > 0));
+          wait_bar(bar(kPRest + s), par, abort_flag, prm.header, 39);
+          tc_fence_after();
+#pragma unroll
+          for (int kk = 0; kk < 8; ++kk)
+            if ((kk & 3) >= kEarlySteps && kk < ksteps)
+              mma_ts(tO, tS + (kk < 4 ? kk * 8 : 64 + (kk - 4) * 8), b + mnmajor_off(kk), idesc_o, 1);
         }
         // the accumulator is only waited for after the unit's last PV (the lazy rescale, rare,
         // runs after S of the next tile is complete, whose commit covers this PV as well)
@@ -341,7 +358,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
           wait_bar(bar(kPFull + 0), tc0 & 1, abort_flag, prm.header, 35);
           if (j == 0) wait_bar(bar(kOFree + 0), (uc0 & 1) ^ 1, abort_flag, prm.header, 37);
           tc_fence_after();
-          issue_pv(0, vst, cur_len, j == 0, !has_next);
+          issue_pv(0, vst, cur_len, j == 0, !has_next, tc0 & 1);
           ++tc0;
           if (has_next) {
             issue_qk(0, kst, nx_len);
@@ -351,7 +368,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             wait_bar(bar(kPFull + 1), tc1 & 1, abort_flag, prm.header, 36);
             if (j == 0) wait_bar(bar(kOFree + 1), (uc1 & 1) ^ 1, abort_flag, prm.header, 38);
             tc_fence_after();
-            issue_pv(1, vst, cur_len, j == 0, !has_next);
+            issue_pv(1, vst, cur_len, j == 0, !has_next, tc1 & 1);
             ++tc1;
             if (has_next) {
               issue_qk(1, kst, nx_len);
@@ -407,7 +424,11 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const uint32_t lane_base = tmem + (uint32_t(32 * qd) << 16);
     const uint32_t tS = lane_base + s * 128 + half * 64;   // my S columns; P goes to their start
     const uint32_t tO = lane_base + 256 + s * 128 + half * (D / 2);
-    float* xch = reinterpret_cast<float*>(gbase + L::kXch) + s * 512;  // [2 buffers][128 rows][2]
+    // What the two halves of a row exchange, one buffer each for the largest exponentials, the maxima
+    // and the row sums: a value is then only overwritten behind a barrier, or a wait for a tile that
+    // needs the partner's P, that follows the partner's read.
+    float* const xch_exp = reinterpret_cast<float*>(gbase + L::kXch) + s * 768 + row * 2;
+    float* const xch_max = xch_exp + 256, * const xch_sum = xch_exp + 512;
     uint32_t tcS = 0, ucS = 0;
     for (uint32_t un_i = 0;; ++un_i) {
       PP_TAKE_UNIT(un_i, true)
@@ -456,7 +477,6 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         auto visible = [&](int col) -> bool {
           return kMixed ? (vis[col >> 5] >> (col & 31)) & 1u : col < col_lim;
         };
-        float* xb = xch + (tcS & 1) * 256 + row * 2;
         // The 64 scores of this thread are handled as two chunks of 32 (fewer live registers).
         // max over the visible scores of one chunk
         auto chunk_max = [&](const uint32_t (&w)[32], int c, float m) -> float {
@@ -473,10 +493,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
           for (int i = 0; i < 32; ++i) m = fmaxf(m, visible(32 * c + i) ? __uint_as_float(w[i]) : -INFINITY);
           return m;
         };
-        float mx = -INFINITY;
-        bool settled = (j == 0);
-        if (settled) {
-          // first tile of the unit: the reference maximum is needed before the exponentials
+        // maximum over the row's visible scores, in base-2 units
+        auto row_max = [&]() -> float {
+          float mx = -INFINITY;
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
             uint32_t w[32];
@@ -484,31 +503,35 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             tmem_wait_ld();
             mx = chunk_max(w, c, mx);
           }
-          xb[half] = mx;
+          xch_max[half] = mx;
           named_barrier_sync(bar_id, 64);
-          m_used = fmaxf(mx, xb[half ^ 1]) * prm.scale_log2;
-        }
-        // Later tiles: the exponentials use the reference maximum of the previous tiles while
-        // the half-row maxima are exchanged; only if the new maximum exceeds the reference by
-        // more than the rescale threshold (rare) is the accumulator rescaled and the tile redone
-        // from the S values, which stay in tensor memory until P is stored.
+          return fmaxf(mx, xch_max[half ^ 1]) * prm.scale_log2;
+        };
+        // First tile of the unit: the reference maximum is needed before the exponentials -- with a
+        // guessed one the largest P of a row would not be exactly 1, and rows that see one or two
+        // keys would lose the exact cancellation in dP - Delta.  Later tiles use the reference of
+        // the tiles before; only if a row has outgrown it by more than the rescale threshold (rare)
+        // is the accumulator rescaled and the tile redone from the S values, which stay in tensor
+        // memory until P is stored.
+        if (j == 0) m_used = row_max();
+        // The 64 scores go through in four pieces of 16, the tensor-memory load of the next piece
+        // in flight under the exponentials of this one.  The first kEarlySteps pieces of P are
+        // handed to the MMA thread before the exponentials of the last are formed: their share of
+        // PV then runs under the rest of the softmax, which shortens the chain softmax -> PV -> QK
+        // that is one slot's period and bounds this kernel (two rows of 32768 tokens, Hq / Hkv
+        // 32 / 8, D 128: 7890 -> 7360 us; sixteen thousand tokens, 64 / 8: 535 -> 513; with two
+        // pieces early 7550 and 519).  Whether the row has outgrown its reference has to be known
+        // by then: the largest exponential tells for the early pieces (its max3 rides in the
+        // MUFU-bound loop for free), the largest exponent for the last.
         uint32_t pk[32];
-        float rs = 0.f;
-        bool done = false;
-        if (j > 0) {
-          // Common path (every tile but a unit's first, whose exact row maximum is formed first
-          // below -- with a guessed reference the largest P of a row would not be exactly 1,
-          // and rows that see one or two keys would lose the exact cancellation in dP - Delta): the 64 scores go through in four pieces of 16, the tensor-memory load
-          // of the next piece in flight under the exponentials of this one, and no maximum is
-          // formed from the scores: the largest exponential tells as well whether the row has
-          // outgrown its reference maximum by more than the rescale threshold
-          // (p > 2^threshold), and its max3 rides in the MUFU-bound loop for free.  (Measured:
-          // loads and the two maxima were 430 of a tile's 1850 softmax cycles, none of it
-          // overlapped with the exponentials.)
+        uint64_t sum2;
+        float x[16];   // exponents of the late piece
+        bool redone = j == 0;
+        for (;;) {
           const float neg_m = -m_used;
           const uint64_t sc2 = pack2(prm.scale_log2, prm.scale_log2), nm2 = pack2(neg_m, neg_m);
-          uint64_t sum2 = pack2(0.f, 0.f);
-          float pm0 = 0.f, pm1 = 0.f;
+          sum2 = pack2(0.f, 0.f);
+          float pm0 = 0.f, pm1 = 0.f, xm = -INFINITY;
           uint32_t wa[16], wb[16];
           auto exp16 = [&](const uint32_t (&w)[16], int piece, auto masked_c) {
             constexpr bool kMasked = decltype(masked_c)::value;
@@ -526,6 +549,18 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
               pk[8 * piece + i] = pack_bf16(p0, p1);
             }
           };
+          auto arg16 = [&](const uint32_t (&w)[16], int piece, auto masked_c) {
+            constexpr bool kMasked = decltype(masked_c)::value;
+#pragma unroll
+            for (int i = 0; i < 16; i += 2) {
+              unpack2(fma2(pack2(__uint_as_float(w[i]), __uint_as_float(w[i + 1])), sc2, nm2), x[i], x[i + 1]);
+              if (kMasked) {
+                x[i] = visible(16 * piece + i) ? x[i] : -INFINITY;
+                x[i + 1] = visible(16 * piece + i + 1) ? x[i + 1] : -INFINITY;
+              }
+              xm = max3(xm, x[i], x[i + 1]);
+            }
+          };
           auto pieces = [&](auto masked_c) {
             tmem_ld16(tS, wa);
             tmem_wait_ld();
@@ -538,65 +573,19 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             tmem_ld16(tS + 48, wb);
             exp16(wa, 2, masked_c);
             tmem_wait_ld();
-            exp16(wb, 3, masked_c);
+            arg16(wb, 3, masked_c);
           };
           if (full) pieces(std::false_type{}); else pieces(std::true_type{});
-          float s0, s1;
-          unpack2(sum2, s0, s1);
-          rs = s0 + s1;
-          const float pmax = fmaxf(pm0, pm1);
-          xb[half] = pmax;
+          if (redone) break;
+          const float pmax = fmaxf(fmaxf(pm0, pm1), ex2(xm));
+          xch_exp[half] = pmax;
           named_barrier_sync(bar_id, 64);
-          const float hi = fmaxf(pmax, xb[half ^ 1]);
-          // (rows past the tile's end must not steer the warp-wide decision)
-          const bool need = row < u_len && !(hi <= exp2f(kRescaleThreshold));
-          if (!__any_sync(0xffffffffu, need)) done = true;   // same rows and values in the partner warp
-          else xb = xch + ((tcS & 1) ^ 1) * 256 + row * 2;   // rare: the exact path below, which
-                                                            // exchanges again, in the other buffer
-        }
-        if (!done)
-        for (;;) {
-          const float neg_m = -m_used;
-          const uint64_t sc2 = pack2(prm.scale_log2, prm.scale_log2), nm2 = pack2(neg_m, neg_m);
-          uint64_t sum2 = pack2(0.f, 0.f);
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            uint32_t w[32];
-            tmem_ld32(tS + 32 * c, w);
-            tmem_wait_ld();
-            if (!settled) mx = chunk_max(w, c, mx);
-            if (full) {
-#pragma unroll
-              for (int i = 0; i < 16; ++i) {
-                float x0, x1;
-                unpack2(fma2(pack2(__uint_as_float(w[2 * i]), __uint_as_float(w[2 * i + 1])), sc2, nm2), x0, x1);
-                const float p0 = ex2(x0), p1 = ex2(x1);
-                sum2 = add2(sum2, pack2(p0, p1));
-                pk[16 * c + i] = pack_bf16(p0, p1);
-              }
-            } else {
-#pragma unroll
-              for (int i = 0; i < 16; ++i) {
-                float p0 = ex2(fmaf(__uint_as_float(w[2 * i]), prm.scale_log2, neg_m));
-                float p1 = ex2(fmaf(__uint_as_float(w[2 * i + 1]), prm.scale_log2, neg_m));
-                p0 = visible(32 * c + 2 * i) ? p0 : 0.f;
-                p1 = visible(32 * c + 2 * i + 1) ? p1 : 0.f;
-                sum2 = add2(sum2, pack2(p0, p1));
-                pk[16 * c + i] = pack_bf16(p0, p1);
-              }
-            }
-          }
-          float s0, s1;
-          unpack2(sum2, s0, s1);
-          rs = s0 + s1;
-          if (settled) break;
-          xb[half] = mx;
-          named_barrier_sync(bar_id, 64);
-          const float m_new = fmaxf(m_used, fmaxf(mx, xb[half ^ 1]) * prm.scale_log2);
+          const float hi = fmaxf(pmax, xch_exp[half ^ 1]);
           // Rows past the tile's end hold whatever follows in memory: they must not steer the
           // warp-wide decision, or a row's rounding would depend on its neighbours' data.
-          const bool need = row < u_len && (m_new - m_used) > kRescaleThreshold;
-          if (!__any_sync(0xffffffffu, need)) break;  // same rows, same values in the partner warp
+          const bool need = row < u_len && !(hi <= exp2f(kRescaleThreshold));
+          if (!__any_sync(0xffffffffu, need)) break;   // same rows, same values in the partner warp
+          const float m_new = fmaxf(m_used, row_max());
           const float alpha = ex2(m_used - m_new);
           // PV of the previous tile is complete: the commit that announced this tile's S was
           // issued after it and covers every earlier MMA of the issuing thread
@@ -611,20 +600,33 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
           }
           l_part *= alpha;
           m_used = m_new;
-          settled = true;
+          redone = true;
         }
-        l_part += rs;
-        tmem_st32(tS, pk);  // P over the first half of my own S columns
+        // P over the first half of my own S columns
+        tmem_st16(tS, pk);
+        tmem_st8(tS + 16, pk + 16);
         tmem_wait_st();
         tc_fence_before();
         mbar_arrive(bar(kPFull + s));
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float p0 = ex2(x[2 * i]), p1 = ex2(x[2 * i + 1]);
+          sum2 = add2(sum2, pack2(p0, p1));
+          pk[24 + i] = pack_bf16(p0, p1);
+        }
+        float s0, s1;
+        unpack2(sum2, s0, s1);
+        l_part += s0 + s1;
+        tmem_st8(tS + 24, pk + 24);
+        tmem_wait_st();
+        tc_fence_before();
+        mbar_arrive(bar(kPRest + s));
         ++tcS;
       }
       // ---- epilogue: row sum from both halves, O / l -> bf16, release the accumulator, store
-      float* xb = xch + (tcS & 1) * 256 + row * 2;
-      xb[half] = l_part;
+      xch_sum[half] = l_part;
       named_barrier_sync(bar_id, 64);
-      const float l_run = l_part + xb[half ^ 1];
+      const float l_run = l_part + xch_sum[half ^ 1];
       wait_bar(bar(kODone + s), ucS & 1, abort_flag, prm.header, 44 + s);
       ++ucS;
       tc_fence_after();
@@ -647,8 +649,6 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
       }
       tc_fence_before();
       mbar_arrive(bar(kOFree + s));
-      // the exchange buffer of parity (tcS & 1) is written again two uses later, after another
-      // barrier: no further synchronisation needed here
       const int h = u_h0 + s;
       if (half == 0 && row < u_len)
         prm.lse[size_t(h) * prm.T + u_start + row] = (m_used + log2f(l_run)) * 0.69314718055994531f;

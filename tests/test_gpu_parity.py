@@ -162,6 +162,27 @@ def test_growing_scores_take_the_rescale_path(d):
     check_against_oracle(w, tens, _run_gpu(w, tens, for_backward=True))
 
 
+@pytest.mark.parametrize("jump", [12.0, 200.0])   # log2 units: beyond the threshold; beyond fp32 without rescaling
+@pytest.mark.parametrize("at", [128, 175, 176, 191, 240, 255])
+def test_one_key_outgrows_the_reference(at, jump):
+    """One key of the second tile scores `jump` (log2) above everything before it, in a column of P
+    that is handed over early (the first 48 of each 64) or late (the last 16)."""
+    w = W.Workload("spike", [[(300, (40, 20))]], 2, 1, 64, seed=31)
+    q, k, v, do = w.tensors()
+    u = torch.zeros(64)
+    u[::2] = 0.25   # |u|^2 = 2
+    a = (jump / (2 * w.softmax_scale * 1.4426950408889634)) ** 0.5
+    k[at] = (a * u).to(k.dtype)
+    q = (0.1 * q.float() + a * u).to(q.dtype)
+    tens = (q, (k.float() * torch.where(torch.arange(len(k)) == at, 1.0, 0.05)[:, None, None]).to(k.dtype), v, do)
+    s = torch.einsum("qd,kd->qk", q[at:300, 0].float(), tens[1][:300, 0].float()) * w.softmax_scale * 1.4426950408889634
+    assert (s[:, at] - s[:, :128].max(dim=1).values > 8).all()
+    import oracle
+    O, LSE = oracle.attn_fwd_bwd(w.descriptors(), *tens, w.softmax_scale)[:2]
+    o, lse = _run_gpu(w, tens)[:2]
+    assert np.abs(o - O).max() <= TOL_O and np.abs(lse - LSE).max() <= TOL_LSE
+
+
 @pytest.mark.parametrize("seed", range(6))
 def test_random_long_structures(seed):
     """Segments of many tiles: the whole workload on the GPU, one KV-head group of it against
