@@ -139,8 +139,11 @@ int pp_plan_read_bwd_tiles(const pp_plan* plan, pp_stream_t stream, int32_t* num
                            int32_t* btiles);
 /* Backward processing order: max_tiles * Hkv records (kv_head << 24) | backward tile, of which
  * the first num_bwd_tiles * Hkv are valid.  Units of one group are adjacent (they stream the
- * same Q / dO tiles through L2), groups with the most work first.  Synchronises `stream`. */
+ * same Q / dO tiles through L2), groups with the most work first.  (With three or more query heads
+ * per KV head pp_attn_bwd takes the same units in smaller blocks; pp_plan_read_bwd_sched gives
+ * the order it takes them in.)  Synchronises `stream`. */
 int pp_plan_read_bwd_units(const pp_plan* plan, pp_stream_t stream, int32_t* units);
+int pp_plan_read_bwd_sched(const pp_plan* plan, pp_stream_t stream, int32_t* units);
 int pp_plan_read(const pp_plan* plan, pp_stream_t stream, int32_t* num_tiles, int32_t* tiles,
                  int32_t* fwd_order, int32_t* bwd_order, int32_t* key_end);
 

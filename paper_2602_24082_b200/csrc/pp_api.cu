@@ -169,15 +169,24 @@ int pp_destroy_plan(pp_plan* plan) {
 
 int pp_plan_max_tiles(const pp_plan* plan) { return plan ? plan->max_tiles : PP_ERR_INVALID_ARG; }
 
-int pp_plan_read_bwd_units(const pp_plan* plan, pp_stream_t stream, int32_t* units) {
-  if (!plan || !units) return PP_ERR_INVALID_ARG;
+static int read_units(const pp_plan* plan, size_t list, pp_stream_t stream, int32_t* units) {
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const size_t n = size_t(plan->max_tiles) * plan->prob.num_kv_heads;
-  if (cudaMemcpyAsync(units, plan->ws + plan->lay.bwd_units, n * 4, cudaMemcpyDeviceToHost, s) !=
-          cudaSuccess ||
+  if (cudaMemcpyAsync(units, plan->ws + list, n * 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return PP_ERR_CUDA;
   return PP_OK;
+}
+
+int pp_plan_read_bwd_units(const pp_plan* plan, pp_stream_t stream, int32_t* units) {
+  if (!plan || !units) return PP_ERR_INVALID_ARG;
+  return read_units(plan, plan->lay.bwd_units, stream, units);
+}
+
+int pp_plan_read_bwd_sched(const pp_plan* plan, pp_stream_t stream, int32_t* units) {
+  if (!plan || !units) return PP_ERR_INVALID_ARG;
+  return read_units(plan, pp::bwd_takes_sched(plan->prob) ? plan->lay.bwd_sched : plan->lay.bwd_units, stream,
+                    units);
 }
 
 int pp_plan_read_bwd_tiles(const pp_plan* plan, pp_stream_t stream, int32_t* num_tiles,

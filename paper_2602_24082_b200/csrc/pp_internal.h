@@ -79,7 +79,9 @@ struct PlanLayout {
   size_t bwd_order;  // int32[max_tiles]  backward tiles, longest work first
   size_t tile_gwork; // int32[max_tiles]  backward work of the backward tile's whole group
   size_t tile_sgroup; // int32[max_tiles] super-group (block of consecutive groups)
+  size_t tile_sblock; // int32[max_tiles] ... and its block in bwd_sched
   size_t bwd_units;  // int32[max_tiles * Hkv]  (kv head << 24) | backward tile, processing order
+  size_t bwd_sched;  // the same units in smaller blocks (bwd_takes_sched): what the kernel then takes
   size_t bwd_units_det;  // the same units, one (group, KV head) set after the other and inside a
                          //   set by descending tile index: the order of the deterministic backward
   size_t key_end;    // int32[T]
@@ -154,6 +156,8 @@ inline PlanLayout plan_layout(const pp_problem& p) {
   l.bwd_order = off; off = align_up(off + sizeof(int32_t) * size_t(mt), 256);
   l.tile_gwork = off; off = align_up(off + sizeof(int32_t) * size_t(mt), 256);
   l.tile_sgroup = off; off = align_up(off + sizeof(int32_t) * size_t(mt), 256);
+  l.tile_sblock = off; off = align_up(off + sizeof(int32_t) * size_t(mt), 256);
+  l.bwd_sched = off; off = align_up(off + sizeof(int32_t) * size_t(mt) * size_t(p.num_kv_heads), 256);
   l.bwd_units = off; off = align_up(off + sizeof(int32_t) * size_t(mt) * size_t(p.num_kv_heads), 256);
   l.bwd_units_det = off;
   off = align_up(off + sizeof(int32_t) * size_t(mt) * size_t(p.num_kv_heads), 256);
@@ -205,6 +209,24 @@ inline int bwd_split_log2(const pp_problem& p) {
     }
   }
   return best;
+}
+
+// Which order the backward takes its units in.  Both go through the groups by decreasing work, in
+// blocks of groups inside which the longest units come first.  With blocks of 600 units
+// (bwd_units) the 148 units that run at a time may be the longest of all of a block's groups, and with r
+// query heads per KV head a block's Q, dO and dQ accumulator are 600 r * 128 KB at D 128: far beyond
+// L2, so that a (query tile, head) is fetched, and its accumulator written back, for nearly every
+// other key tile.  Blocks of 150 units, with the last 200 in one block to balance the end
+// (bwd_sched), take a third to a half of that traffic (a model of L2 with 80 MB of least-recently-used tiles, which gives
+// the 600s' measured 0.93, 5.4 and 5.9 GB as 0.93, 5.9 and 5.7: 0.5, 3.9 and 2.2).  Main kernel, 600s
+// -> these: 9241 tokens, 32 / 8 heads 262 -> 250 us; 16384, 64 / 8 1361 -> 1230; 20187, 28 / 4 1818 ->
+// 1742; 16384, 32 / 8, D 64 456 -> 400; 36000 in short groups, 16 / 2 277 -> 243; 16760, 32 / 8 307 ->
+// 272; two rows of 32768, 32 / 8 19320 -> 19220.  With one and two heads per KV head a block's data is
+// that much smaller, and the smaller blocks only cost balance: 8 / 8 258 -> 265, 16 / 8 278 -> 276, 754 -> 740.
+// Up to 200 units both are one block.
+constexpr int kSchedBlockUnits = 150, kSchedTailUnits = 200;
+inline bool bwd_takes_sched(const pp_problem& p) {
+  return p.num_q_heads / p.num_kv_heads >= 3 && (long long)max_btiles_of(p) * p.num_kv_heads > kSchedTailUnits;
 }
 
 inline BwdScratch bwd_scratch_layout(const pp_problem& p, int lg_split) {

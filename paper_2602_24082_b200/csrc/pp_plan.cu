@@ -39,7 +39,9 @@ struct PlanPtrs {
   int32_t* bwd_order;
   int32_t* tile_gwork;
   int32_t* tile_sgroup;
+  int32_t* tile_sblock;
   int32_t* bwd_units;
+  int32_t* bwd_sched;   // null: not wanted
   int32_t* bwd_units_det;
   int Hkv;
   int32_t* key_end;
@@ -421,6 +423,13 @@ __global__ void plan_fwd_order_kernel(PlanPtrs p) {
 // the balancing.  A tile's group is identified by the group's first token.
 constexpr int kSuperGroupUnits = 600;
 
+// The blocks of the order that the kernel takes with several query heads per KV head
+// (bwd_takes_sched, which has the reasons): `later` = units of the groups ranked behind the tile's own,
+// of `total`.  (At most 1002 blocks, which the one-block plan's sort keys have room for.)
+__device__ __forceinline__ int sched_block(int later, int total) {
+  return later < kSchedTailUnits ? 0 : 1 + (later - kSchedTailUnits) / max(kSchedBlockUnits, total / 1000);
+}
+
 // bwd_order (plain longest-first list of the backward tiles) and each tile's group work
 __device__ __forceinline__ void plan_gwork_body(const PlanPtrs& p, int t, int n) {
   const BTile me = p.btiles[t];
@@ -436,11 +445,14 @@ __device__ __forceinline__ void plan_gwork_body(const PlanPtrs& p, int t, int n)
 
 __device__ __forceinline__ void plan_sgroup_body(const PlanPtrs& p, int t, int n) {
   const int gs = p.btiles[t].grp_start, gw = p.tile_gwork[t];
-  int rest = 0;  // tiles of this group and of the groups that come later
+  int rest = 0, later = 0;  // tiles of this group and of the groups that come later; of those alone
   for (int u = 0; u < n; ++u) {
     const int ogs = p.btiles[u].grp_start, ow = p.tile_gwork[u];
-    rest += (ogs == gs) || (ow < gw) || (ow == gw && ogs > gs);
+    const bool behind = (ow < gw) || (ow == gw && ogs > gs);
+    rest += (ogs == gs) || behind;
+    later += behind;
   }
+  p.tile_sblock[t] = sched_block(p.Hkv * later, p.Hkv * n);
   // counted from the END of the list, so the last block is never a small leftover whose
   // long units would start late: blocks are processed in decreasing index
   p.tile_sgroup[t] = (p.Hkv * rest - 1) / kSuperGroupUnits;
@@ -454,6 +466,15 @@ __device__ __forceinline__ void plan_units_body(const PlanPtrs& p, int t, int n)
     pos += (osg > sg) || (osg == sg && ((ob > wb) || (ob == wb && u < t)));
   }
   for (int kvh = 0; kvh < p.Hkv; ++kvh) p.bwd_units[p.Hkv * pos + kvh] = (kvh << 24) | t;
+  if (p.bwd_sched) {
+    const int sb = p.tile_sblock[t];
+    pos = 0;
+    for (int u = 0; u < n; ++u) {
+      const int osb = p.tile_sblock[u], ob = p.btiles[u].work;
+      pos += (osb > sb) || (osb == sb && ((ob > wb) || (ob == wb && u < t)));
+    }
+    for (int kvh = 0; kvh < p.Hkv; ++kvh) p.bwd_sched[p.Hkv * pos + kvh] = (kvh << 24) | t;
+  }
   // Deterministic order: one (group, KV head) set after the other, groups by decreasing work.
   // The tiles add to a query tile's dQ in descending order, so a unit waits for the unit of the
   // next tile.  Inside a set the units go out in ascending tile order (longest first, as in the
@@ -543,8 +564,9 @@ struct FusedSmem {
   union alignas(16) {   // (keys are read as uint4)
     uint32_t sort[2][kMixed ? 4 : 3][kFusedMaxTiles];
     struct {
-      uint32_t key[kMixed ? 5 : 4][kRankTiles];      // forward tiles, backward tiles, groups, backward units,
-      int32_t rank[kMixed ? 5 : 4][kRankTiles];      //   query tiles (groups: backward tiles of the groups before)
+      // forward tiles, backward tiles, groups, backward units in both orders, query tiles (groups:
+      uint32_t key[kMixed ? 6 : 5][kRankTiles];
+      int32_t rank[kMixed ? 6 : 5][kRankTiles];      //   backward tiles of the groups before)
     } r;
   } o;
   int32_t desc[kDescFused];
@@ -559,7 +581,7 @@ struct FusedSmem {
   uint16_t bgrp[kFusedMaxTiles];
   int32_t grid_gain[kMixed ? kFusedMaxTiles / 2 : 1];
   uint16_t qwork[kMixed ? kFusedMaxTiles : 2];       // work of the query tiles, 0 where there is none
-  uint16_t unit_tile[kFusedMaxTiles];   // backward tiles in the order of their units
+  uint16_t unit_tile[2][kFusedMaxTiles];   // backward tiles in the orders of their units
   int32_t warp_sum[2][32];
   int32_t status, detail, no_qtile;
 };
@@ -917,36 +939,46 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
     const int sg = (p.Hkv * (nb - ranked_before) - 1) / kSuperGroupUnits;
     return uint32_t(511 - sg) << 23 | uint32_t(4095 - sm.wb[t]) << 11 | uint32_t(t);
   };
+  auto sched_key = [&](int t, int ranked_before) {   // (a tile's work is 1 .. 2048)
+    const int g = sm.bgrp[t], later = nb - ranked_before - (sm.btile0[g + 1] - sm.btile0[g]);
+    return uint32_t(1023 - sched_block(p.Hkv * later, p.Hkv * nb)) << 22 | uint32_t(2048 - sm.wb[t]) << 11 |
+           uint32_t(t);
+  };
   if (by_rank) {   // (blocks of 256 threads have at most 256 tiles: one per thread)
     for (int t = tid; t < kRankTiles; t += nthr) {
       sm.o.r.key[0][t] = t == tid ? key[0][0] : ~0u;
       sm.o.r.key[1][t] = t == tid ? key[1][0] : ~0u;
       sm.o.r.key[2][t] = t == tid ? key[2][0] : ~0u;
-      sm.o.r.key[3][t] = ~0u;
-      sm.o.r.rank[0][t] = sm.o.r.rank[1][t] = sm.o.r.rank[2][t] = sm.o.r.rank[3][t] = 0;
+      sm.o.r.key[3][t] = sm.o.r.key[4][t] = ~0u;
+      for (int a = 0; a < 5; ++a) sm.o.r.rank[a][t] = 0;
       if constexpr (kMixed) {
-        sm.o.r.key[4][t] = t == tid ? key[3][0] : ~0u;
-        sm.o.r.rank[4][t] = 0;
+        sm.o.r.key[5][t] = t == tid ? key[3][0] : ~0u;
+        sm.o.r.rank[5][t] = 0;
       }
     }
     __syncthreads();
     rank_count<false>(sm.o.r.key[0], n, sm.o.r.rank[0], nullptr);
     rank_count<false>(sm.o.r.key[1], nb, sm.o.r.rank[1], nullptr);
     rank_count<true>(sm.o.r.key[2], p.G, sm.o.r.rank[2], sm.btile0);
-    if constexpr (kMixed) rank_count<false>(sm.o.r.key[4], n, sm.o.r.rank[4], nullptr);
+    if constexpr (kMixed) rank_count<false>(sm.o.r.key[5], n, sm.o.r.rank[5], nullptr);
     __syncthreads();
     if (tid < n) p.fwd_order[sm.o.r.rank[0][tid]] = tid;
     if constexpr (kMixed)
-      if (tid < n) p.qorder[sm.o.r.rank[4][tid]] = tid;
+      if (tid < n) p.qorder[sm.o.r.rank[5][tid]] = tid;
     if (tid < nb) {
       p.bwd_order[sm.o.r.rank[1][tid]] = tid;
       sm.o.r.key[3][tid] = unit_key(tid, sm.o.r.rank[2][sm.bgrp[tid]]);
+      if (p.bwd_sched) sm.o.r.key[4][tid] = sched_key(tid, sm.o.r.rank[2][sm.bgrp[tid]]);
     }
     if (tid < p.G) sm.before[tid] = sm.o.r.rank[2][tid];
     __syncthreads();
     rank_count<false>(sm.o.r.key[3], nb, sm.o.r.rank[3], nullptr);
+    if (p.bwd_sched) rank_count<false>(sm.o.r.key[4], nb, sm.o.r.rank[4], nullptr);
     __syncthreads();
-    if (tid < nb) sm.unit_tile[sm.o.r.rank[3][tid]] = uint16_t(tid);
+    if (tid < nb) {
+      sm.unit_tile[0][sm.o.r.rank[3][tid]] = uint16_t(tid);
+      if (p.bwd_sched) sm.unit_tile[1][sm.o.r.rank[4][tid]] = uint16_t(tid);
+    }
     __syncthreads();
   } else {
     int n2 = 1024;
@@ -962,7 +994,7 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
     block_scan2(cnt, unused, sm.warp_sum);
     if (tid < p.G) sm.before[g] = cnt - mine;
     __syncthreads();
-    uint32_t ukey[1][2];
+    uint32_t ukey[2][2];
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const int t = tid + nthr * r;
@@ -971,17 +1003,22 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
         if (t < n) p.qorder[t] = int32_t(key[3][r] & 0xffffu);
       if (t < nb) p.bwd_order[t] = int32_t(key[1][r] & 0xffffu);
       ukey[0][r] = t < nb ? unit_key(t, sm.before[sm.bgrp[t]]) : ~0u;
+      ukey[1][r] = t < nb ? sched_key(t, sm.before[sm.bgrp[t]]) : ~0u;
     }
     bitonic_sort(ukey, n2, sm.o.sort);
 #pragma unroll
-    for (int r = 0; r < 2; ++r)
-      if (tid + nthr * r < nb) sm.unit_tile[tid + nthr * r] = uint16_t(ukey[0][r] & 2047u);
+    for (int r = 0; r < 2; ++r) {
+      const int t = tid + nthr * r;
+      for (int a = 0; a < 2; ++a)
+        if (t < nb) sm.unit_tile[a][t] = uint16_t(ukey[a][r] & 2047u);
+    }
     __syncthreads();
   }
-  // ---- backward units, in both orders
+  // ---- backward units, in their orders
   for (int e = tid; e < nb * p.Hkv; e += nthr) {
     const int i = e / p.Hkv, kvh = e - i * p.Hkv;
-    p.bwd_units[e] = (kvh << 24) | int(sm.unit_tile[i]);
+    p.bwd_units[e] = (kvh << 24) | int(sm.unit_tile[0][i]);
+    if (p.bwd_sched) p.bwd_sched[e] = (kvh << 24) | int(sm.unit_tile[1][i]);
     // deterministic backward: set after set (see plan_units_body)
     const int g = sm.bgrp[i], ng = sm.btile0[g + 1] - sm.btile0[g], k_rel = i - sm.btile0[g];
     const int slot = ng <= p.det_asc_max ? k_rel : ng - 1 - k_rel;
@@ -1082,7 +1119,9 @@ cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cu
   p.bwd_order = reinterpret_cast<int32_t*>(ws + l.bwd_order);
   p.tile_gwork = reinterpret_cast<int32_t*>(ws + l.tile_gwork);
   p.tile_sgroup = reinterpret_cast<int32_t*>(ws + l.tile_sgroup);
+  p.tile_sblock = reinterpret_cast<int32_t*>(ws + l.tile_sblock);
   p.bwd_units = reinterpret_cast<int32_t*>(ws + l.bwd_units);
+  p.bwd_sched = bwd_takes_sched(plan->prob) ? reinterpret_cast<int32_t*>(ws + l.bwd_sched) : nullptr;
   p.bwd_units_det = reinterpret_cast<int32_t*>(ws + l.bwd_units_det);
   p.Hkv = plan->prob.num_kv_heads;
   p.key_end = reinterpret_cast<int32_t*>(ws + l.key_end);

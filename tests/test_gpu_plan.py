@@ -139,6 +139,39 @@ def test_backward_units_order(w):
     assert (units[:, 1].reshape(n, hkv) == units[:, 1].reshape(n, hkv)[:, :1]).all()
 
 
+@pytest.mark.parametrize("groups,length,hq,hkv", [
+    (1, 200, 3, 1), (9, 1100, 32, 8), (40, 300, 28, 4), (60, 1100, 8, 2), (150, 1200, 16, 4), (8, 1500, 4, 2),
+    (1100, 5, 6, 2), (12, 1000, 280, 70), (300, 650, 210, 70)])
+def test_order_the_backward_takes_its_units_in(groups, length, hq, hkv):
+    """From three query heads per KV head on: groups by decreasing work, the last 200 units in one block
+    and the others in blocks of 150 (larger beyond 1000 blocks), inside a block longest first with all
+    KV heads of a tile adjacent.  Below that: the order of read_bwd_units.  Plans in one block by
+    counting (up to 512 tiles) and by sorting, and of several kernels."""
+    from paper_2602_24082_b200 import binding as B
+    rng = np.random.default_rng(groups)
+    pick = lambda: int(rng.integers(1, 2 * length // 3 + 1))
+    w = W.Workload("sched", [[(pick(), (pick(), pick()))] for _ in range(groups)], hq, hkv, 64, seed=1)
+    plan = B.plan_for(w)
+    assert plan.status() == (0, 0)
+    btiles = plan.read_bwd_tiles()
+    n = len(btiles)
+    units = plan.read_bwd_sched(n)
+    if hq // hkv < 3:
+        assert np.array_equal(units, plan.read_bwd_units(n))
+        return
+    work, grp = btiles[:, 6].tolist(), btiles[:, 4].tolist()
+    gwork, gtiles = {}, {}
+    for g, x in zip(grp, work):
+        gwork[g], gtiles[g] = gwork.get(g, 0) + x, gtiles.get(g, 0) + 1
+    block, later = {}, 0
+    for g in sorted(gwork, key=lambda g: (gwork[g], -g)):     # from the last
+        block[g] = 0 if later < 200 else 1 + (later - 200) // max(150, hkv * n // 1000)
+        later += hkv * gtiles[g]
+    expect = sorted(range(n), key=lambda t: (-block[grp[t]], -work[t], t))
+    assert units[:, 1].tolist() == np.repeat(expect, hkv).tolist()
+    assert (units[:, 0].reshape(n, hkv) == np.arange(hkv)).all()
+
+
 def test_multi_kernel_plan_path_matches_fused_semantics():
     """> 2048 tiles forces the multi-kernel plan path; its tiles / orders obey the same
     rules (checked through the same dense-mask comparison on a prefix of the tokens)."""
