@@ -65,8 +65,9 @@ template <int D, bool kClear>
 __global__ void __launch_bounds__(32 * kPreWarps)
 bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o,
                       const float* __restrict__ lse, float* __restrict__ delta,
-                      float* __restrict__ lse2, float* __restrict__ dq_acc, int T, int Hq) {
+                      float* __restrict__ lse2, float* __restrict__ dq_acc, int T, int Hq, int4* sem, unsigned sem_n4) {
   launch_dependents();
+  dependency_wait();
   constexpr int kLanes = pre_lanes(D);    // lanes per row (D / 8 of them hold data)
   constexpr int kRows = 32 / kLanes;      // rows per warp and step
   const int lane = threadIdx.x & 31, sub = lane % kLanes, rin = lane / kLanes;
@@ -108,6 +109,8 @@ bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* 
       z[1] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < sem_n4; i += gridDim.x * blockDim.x)
+    sem[i] = make_int4(0, 0, 0, 0);   // turn counters (deterministic variant)
   if (writes) {
     delta[stat] = mine;
     lse2[stat] = my_lse * 1.4426950408889634f;
@@ -136,6 +139,7 @@ __global__ void __launch_bounds__(256)
 bwd_finalize_kernel(const float4* __restrict__ acc, uint2* __restrict__ dq, size_t n4, float scale,
                     unsigned dq_blocks, SumParts sp) {
   launch_dependents();
+  dependency_wait();
   if (blockIdx.x < dq_blocks) {
     const size_t i0 = size_t(blockIdx.x) * (256 * kFinUnroll) + threadIdx.x;
     float4 a[kFinUnroll];
@@ -352,6 +356,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   const long long t_kernel0 = clock64();
 #endif
 
+  launch_dependents();
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   if (base - raw + L::kUsed > L::kTotal) {  // cannot happen with an aligned base
@@ -1024,12 +1029,13 @@ cudaError_t launch_bwd_t(const pp_plan* plan, const void* o, const float* lse, c
   const pp_problem& pb = plan->prob;
   const size_t T = pb.total_tokens, Hq = pb.num_q_heads;
   const int num_sms = dev->num_sms;
+  const unsigned sem_n4 = prm.dq_sem ? unsigned(max_btiles_of(pb)) * pb.num_q_heads : 0;   // 16 bytes each
   const unsigned pre_blocks = unsigned(Hq * ((T + pre_tokens(DV) - 1) / pre_tokens(DV)));
   auto pre = dq_cleared ? bwd_preprocess_kernel<DV, false> : bwd_preprocess_kernel<DV, true>;
-  pre<<<pre_blocks, 32 * kPreWarps, 0, stream>>>(
-      static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse,
-      const_cast<float*>(prm.delta), const_cast<float*>(prm.lse2), prm.dq_acc, int(T), int(Hq));
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_kernel(pre_blocks <= kOverlapBlocks, pre, dim3(pre_blocks), dim3(32 * kPreWarps), 0, stream,
+                                static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse,
+                                const_cast<float*>(prm.delta), const_cast<float*>(prm.lse2), prm.dq_acc, int(T),
+                                int(Hq), reinterpret_cast<int4*>(prm.dq_sem), sem_n4);
   const long long units = ((long long)plan->max_tiles * pb.num_kv_heads) << prm.lg_split;
   dim3 grid(unsigned(std::min<long long>(units, num_sms)));
   ProfileEvents& ev = profile_events();
@@ -1046,9 +1052,9 @@ cudaError_t launch_bwd_t(const pp_plan* plan, const void* o, const float* lse, c
   unsigned fb = unsigned((n4 + 256 * kFinUnroll - 1) / (256 * kFinUnroll));
   const SumParts sp = {prm.parts, prm.header, prm.tiles, prm.dk, prm.dv, prm.lg_split, pb.num_kv_heads, DV};
   const unsigned sum_blocks = prm.lg_split ? unsigned(max_btiles_of(pb)) * pb.num_kv_heads * 8 : 0;
-  bwd_finalize_kernel<<<fb + sum_blocks, 256, 0, stream>>>(
-      reinterpret_cast<const float4*>(prm.dq_acc), static_cast<uint2*>(dq), n4, prm.scale, fb, sp);
-  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = launch_kernel(fb + sum_blocks <= kOverlapBlocks, bwd_finalize_kernel, dim3(fb + sum_blocks), dim3(256), 0, stream,
+                      reinterpret_cast<const float4*>(prm.dq_acc), static_cast<uint2*>(dq), n4, prm.scale, fb, sp);
   if (launches) *launches += 3;
   return e;
 }
@@ -1081,11 +1087,7 @@ cudaError_t launch_bwd(const pp_plan* plan, const void* q, const void* k, const 
   prm.parts = reinterpret_cast<float4*>(sc + sl.parts);
   prm.lg_split = lg_split;
   prm.dq_sem = nullptr;
-  if (deterministic) {
-    prm.dq_sem = reinterpret_cast<int32_t*>(sc + sl.sem);
-    cudaError_t me = cudaMemsetAsync(prm.dq_sem, 0, sl.sem_bytes, stream);
-    if (me != cudaSuccess) return me;
-  }
+  if (deterministic) prm.dq_sem = reinterpret_cast<int32_t*>(sc + sl.sem);
   prm.dk = static_cast<__nv_bfloat16*>(dk);
   prm.dv = static_cast<__nv_bfloat16*>(dv);
   prm.T = pb.total_tokens;

@@ -300,16 +300,19 @@ inline bool device_is_sm100() {
 }
 
 // Launches a kernel, with `overlap` so that it may start before the kernel in front of it on the
-// stream has ended (programmatic dependent launch): the plan, the forward and the backward main
-// kernel call dependency_wait before they touch global memory, the kernels in front of them in a
-// step (plan, preprocess, finalize) call launch_dependents first thing, and the launch (in the
+// stream has ended (programmatic dependent launch): the kernels of a step call launch_dependents
+// first thing and dependency_wait before they touch global memory, and the launch (in the
 // backward also barrier set-up, tensor-map fetches and tensor-memory allocation) runs under the
 // tail of the one before.  (Kernels that know nothing of this, in front or behind, see ordinary stream order.)
 // The persistent kernels take it up to kOverlapUnits units per SM: steps of 60 - 100 us gain 5 -
 // 9 % (144 ... 1054 tokens), one of 180 us 2.5 %, one of 500 us nothing, and a forward and
-// backward of 2600 and 1100 units (T 16384, 32 / 8 heads, D 64) lost 2 %.  The streaming kernels do
-// not take it: early blocks crowd the SMs that free up first (preprocess 30 -> 38 us at T 9241).
+// backward of 2600 and 1100 units (T 16384, 32 / 8 heads, D 64) lost 2 %.  The streaming kernels
+// (preprocess, finalize) take it up to kOverlapBlocks blocks, two per SM: 144 tokens, 1 / 1 heads,
+// 42.4 -> 38.6 us alone and 32.8 -> 30.3 in a row of steps, 300, 4 / 2 55.5 -> 51.7 and 44.6 -> 42.9,
+// 700, 8 / 8 50.0 -> 45.5 alone.  With more, early blocks crowd the SMs that free up first: up to eight
+// per SM 1000 tokens, 8 / 1 55.1 -> 61.2 in a row, preprocess 30 -> 38 us at T 9241.
 constexpr int kOverlapUnits = 4;
+constexpr unsigned kOverlapBlocks = 296;
 template <typename... P, typename... A>
 cudaError_t launch_kernel(bool overlap, void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t stream, A&&... args) {
