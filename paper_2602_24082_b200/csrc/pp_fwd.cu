@@ -12,8 +12,8 @@
 //   warps 18-19 optional: clear the backward's fp32 dQ accumulator for the unit's rows
 // A work unit is (query tile, KV head, pair of query heads of that KV head): both slots see
 // the same keys and the same mask, so every K / V tile staged in shared memory feeds two
-// S tiles.  (The last head of an odd number of heads per KV head, and every head where there is one
-// per KV head, is a unit of its own, with slot 1 empty.)  While one slot's warpgroup does its exponentials the tensor core works on the
+// S tiles.  The last head of an odd number of heads per KV head, and every head where there is one
+// per KV head, takes two query tiles of a segment into the slots (kPaired below) or leaves slot 1 empty.  While one slot's warpgroup does its exponentials the tensor core works on the
 // other slot (order: PV_0(j), QK_0(j+1), PV_1(j), QK_1(j+1), ...).  P (bf16) overwrites columns
 // [0,32) and [64,96) of its S tile in tensor memory (each half-row thread inside the columns it
 // has read itself) and is the A operand of the second MMA; V is
@@ -32,6 +32,7 @@ namespace {
 struct FwdParams {
   int32_t* header;
   const Tile* tiles;       // tiles of the segments
+  const uint8_t* tile_unit;  // (paired tiles)
   const QTile* qtiles;     // (mixed tiles)
   const int32_t* key_end;  // (mixed tiles)
   const int32_t* order;    // the tiles, longest work first
@@ -95,10 +96,17 @@ __device__ __forceinline__ KvTile kv_tile_of(const T& t, int j, int n0, int n1) 
   return k;
 }
 
-template <bool kMixed>
+// What the slots of a unit hold: two query heads of a tile, or of a tile that may have rows of several
+// segments (kMixed), or (kPaired) for the head left over by an odd number of heads per KV head two tiles of a
+// segment, one behind the other: slot 1 has the unit's tile, slot 0 the one before it, whose keys are those of
+// slot 1 but the last tile.
+enum FwdMode : int { kPlain, kMixedTiles, kPairedTiles };
+
+template <int kMode>
 struct Unit {
-  std::conditional_t<kMixed, QTile, Tile> tile;
+  std::conditional_t<kMode == kMixedTiles, QTile, Tile> tile;
   int h0, kvh, nslots, n0, n1, ntiles;
+  bool paired;
 };
 
 // Units are handed out dynamically in the plan's longest-work-first order: a CTA starts with the
@@ -107,8 +115,9 @@ struct Unit {
 // last one resets both counters for the next launch.
 constexpr int kHdrFwdNext = 4, kHdrFwdDone = 6;
 
-template <bool kMixed>
-__device__ __forceinline__ bool get_unit(const FwdParams& prm, int u, int ntiles_total, Unit<kMixed>& un) {
+// (a unit may be empty: no slots)
+template <int kMode>
+__device__ __forceinline__ bool get_unit(const FwdParams& prm, int u, int ntiles_total, Unit<kMode>& un) {
   const int r = prm.Hq / prm.Hkv, npairs = (r + 1) >> 1, per_tile = prm.Hkv * npairs;
   const int ord = u / per_tile;
   if (ord >= ntiles_total) return false;
@@ -117,8 +126,14 @@ __device__ __forceinline__ bool get_unit(const FwdParams& prm, int u, int ntiles
   const int pair = rem - un.kvh * npairs;
   un.h0 = un.kvh * r + 2 * pair;
   un.nslots = (2 * pair + 1 < r) ? 2 : 1;
-  if constexpr (kMixed) un.tile = prm.qtiles[prm.order[ord]];
-  else un.tile = prm.tiles[prm.order[ord]];
+  const int t = prm.order[ord];
+  if constexpr (kMode == kMixedTiles) un.tile = prm.qtiles[t];
+  else un.tile = prm.tiles[t];
+  un.paired = false;
+  if (kMode == kPairedTiles && un.nslots == 1) {
+    un.nslots = prm.tile_unit[t];
+    un.paired = un.nslots == 2;
+  }
   un.n0 = (un.tile.kv0_len + kTile - 1) / kTile;
   un.n1 = (un.tile.kv1_len + kTile - 1) / kTile;
   un.ntiles = un.n0 + un.n1 + 1;
@@ -129,14 +144,15 @@ __device__ __forceinline__ bool get_unit(const FwdParams& prm, int u, int ntiles
 // tensors in global memory.  For DV < D (96 in tiles of 128) the TMA loads fill the columns
 // past DV with zeros, so only the loops over the head dimension, the N of the second GEMM and
 // everything that addresses global memory know about DV.
-// kMixed: the rows of a query tile may belong to several segments, which changes the masks of its
-// own keys and of the first rows' response.  (A template parameter because the more general masks
-// take registers from the loop: 3.5 % on two rows of 32768 tokens in one instance for all.)
-template <int D, bool kMixed, int DV = D>
+// kMode: see FwdMode.  With mixed tiles the masks of a tile's own keys and of the first rows' response
+// change.  (A template parameter because the more general masks take registers from the loop: 3.5 %
+// on two rows of 32768 tokens in one instance for all.)
+template <int D, int kMode, int DV = D>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
            const __grid_constant__ CUtensorMap tm_v, FwdParams prm) {
   using L = FwdSmem<D>;
+  constexpr bool kMixed = kMode == kMixedTiles, kPaired = kMode == kPairedTiles;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // (known to be uniform in the warp)
@@ -183,19 +199,24 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   // Ring of two decoded unit records (producer -> MMA thread and softmax warps): the producer
   // alone reads the plan's tile list; the other roles get what they need from shared memory.
   volatile int* sched = reinterpret_cast<volatile int*>(gbase + L::kSched);
-  auto fetch_unit = [&](uint32_t n, Unit<kMixed>& un) -> bool {  // producer thread
+  bool first_draw = true;
+  auto fetch_unit = [&](uint32_t n, Unit<kMode>& un) -> bool {  // producer thread
     wait_bar(bar(kSchedEmptyF + (n & 1)), ((n >> 1) & 1) ^ 1, abort_flag, prm.header, 90);
-    // after a wait has given up, no more work is drawn: the end marker goes out instead
-    const int u = *abort_flag ? 0x7fffffff
-                  : n == 0    ? int(blockIdx.x)
-                              : int(gridDim.x) + atomicAdd(&prm.header[kHdrFwdNext], 1);
-    const bool ok = get_unit(prm, u, ntiles_total, un);
+    bool ok;
+    do {
+      // after a wait has given up, no more work is drawn: the end marker goes out instead
+      const int u = *abort_flag  ? 0x7fffffff
+                    : first_draw ? int(blockIdx.x)
+                                 : int(gridDim.x) + atomicAdd(&prm.header[kHdrFwdNext], 1);
+      first_draw = false;
+      ok = get_unit<kMode>(prm, u, ntiles_total, un);
+    } while (kPaired && ok && un.nslots == 0);
     volatile int* e = sched + (n & 1) * 8;
     e[0] = un.tile.start;
     if constexpr (kMixed) e[1] = un.tile.len | un.tile.first_rows << 8;
     else e[1] = un.tile.len;
     e[2] = un.h0;
-    e[3] = ok ? un.nslots : 0;  // 0 slots marks the end of the work list
+    e[3] = ok ? un.nslots | (kPaired && un.paired ? 4 : 0) : 0;  // 0 slots marks the end of the work list
     e[4] = un.n0;
     e[5] = un.n1;
     e[6] = un.tile.kv0_len - (un.n0 - 1) * kTile;
@@ -207,7 +228,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
 #define PP_TAKE_UNIT(n, whole_warp)                                                              \
   const bool u_ok = wait_bar(bar(kSchedFullF + ((n) & 1)), ((n) >> 1) & 1, abort_flag, prm.header, 91); \
   const volatile int* u_e = sched + ((n) & 1) * 8;                                               \
-  const int u_start = u_e[0], u_len1 = u_e[1], u_len = kMixed ? u_len1 & 255 : u_len1, u_h0 = u_e[2], u_nslots = u_ok ? u_e[3] : 0;       \
+  const int u_start = u_e[0], u_len1 = u_e[1], u_len = kMixed ? u_len1 & 255 : u_len1, u_h0 = u_e[2], u_slots = u_ok ? u_e[3] : 0;        \
+  const int u_nslots = kPaired ? u_slots & 3 : u_slots;                                          \
+  const bool u_paired = kPaired && (u_slots & 4);                                                \
   const int u_n0 = u_e[4], u_n1 = u_e[5], u_last0 = u_e[6], u_last1 = u_e[7];                    \
   const int u_ntiles = u_n0 + u_n1 + 1;                                                          \
   if (whole_warp) {                                                                              \
@@ -216,7 +239,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   } else {                                                                                       \
     mbar_arrive(bar(kSchedEmptyF + ((n) & 1)));                                                  \
   }                                                                                              \
-  (void)u_start, (void)u_len, (void)u_h0;                                                        \
+  (void)u_start, (void)u_len, (void)u_h0, (void)u_paired;                                        \
   /* keys of visible key tile j: only the last tile of a full range and the diagonal tile */    \
   /* can be shorter than 128 */                                                                  \
   auto u_klen = [=](int j) -> int {                                                              \
@@ -227,14 +250,14 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     // ------------------------------------------------------------ TMA producer
     if (elect_one()) {
       uint32_t kc = 0, qc[2] = {0, 0};
-      Unit<kMixed> un;
+      Unit<kMode> un;
       for (uint32_t un_i = 0; fetch_unit(un_i, un); ++un_i) {
         for (int s = 0; s < un.nslots; ++s) {
           wait_bar(bar(kQEmpty + s), (qc[s] & 1) ^ 1, abort_flag, prm.header, 20 + s);
           mbar_expect_tx(bar(kQFull + s), L::kTileBytes);
           for (int b = 0; b < D / 64; ++b)
-            tma_load_3d(sQ + s * L::kTileBytes + b * kBoxBytes, &tm_q, b * 64, un.h0 + s,
-                        un.tile.start, bar(kQFull + s));
+            tma_load_3d(sQ + s * L::kTileBytes + b * kBoxBytes, &tm_q, b * 64, un.paired ? un.h0 : un.h0 + s,
+                        un.paired && s == 0 ? un.tile.start - kTile : un.tile.start, bar(kQFull + s));
           ++qc[s];
         }
         // K and V travel in stages {V(j), K(j + 1)} -- what one period of the MMA thread
@@ -337,13 +360,14 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         PP_TAKE_UNIT(un_i, false)
         if (u_nslots == 0) break;
         const bool two = u_nslots == 2;
+        const int nt0 = u_ntiles - int(u_paired);   // key tiles of slot 0
         wait_bar(bar(kQFull + 0), uc0 & 1, abort_flag, prm.header, 30);
         if (two) wait_bar(bar(kQFull + 1), uc1 & 1, abort_flag, prm.header, 31);
         int cur_len = u_klen(0);
         wait_bar(bar(kKFull + (kc & 1)), (kc >> 1) & 1, abort_flag, prm.header, 32);
         tc_fence_after();
         issue_qk(0, kc & 1, cur_len);
-        if (u_ntiles == 1) mma_commit(bar(kQEmpty + 0));
+        if (nt0 == 1) mma_commit(bar(kQEmpty + 0));
         if (two) {
           issue_qk(1, kc & 1, cur_len);
           if (u_ntiles == 1) mma_commit(bar(kQEmpty + 1));
@@ -355,15 +379,17 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
           const int nx_len = has_next ? u_klen(j + 1) : 0;
           const uint32_t vst = kc & 1, kst = kc & 1;   // stage {V(j), K(j + 1)}
           wait_bar(bar(kKFull + kst), (kc >> 1) & 1, abort_flag, prm.header, 33);
-          // slot 0
-          wait_bar(bar(kPFull + 0), tc0 & 1, abort_flag, prm.header, 35);
-          if (j == 0) wait_bar(bar(kOFree + 0), (uc0 & 1) ^ 1, abort_flag, prm.header, 37);
-          tc_fence_after();
-          issue_pv(0, vst, cur_len, j == 0, !has_next, tc0 & 1);
-          ++tc0;
-          if (has_next) {
-            issue_qk(0, kst, nx_len);
-            if (j + 2 == u_ntiles) mma_commit(bar(kQEmpty + 0));
+          if (!kPaired || j < nt0) {   // slot 0
+            const bool has_next0 = j + 1 < nt0;
+            wait_bar(bar(kPFull + 0), tc0 & 1, abort_flag, prm.header, 35);
+            if (j == 0) wait_bar(bar(kOFree + 0), (uc0 & 1) ^ 1, abort_flag, prm.header, 37);
+            tc_fence_after();
+            issue_pv(0, vst, cur_len, j == 0, !has_next0, tc0 & 1);
+            ++tc0;
+            if (has_next0) {
+              issue_qk(0, kst, nx_len);
+              if (j + 2 == nt0) mma_commit(bar(kQEmpty + 0));
+            }
           }
           if (two) {
             wait_bar(bar(kPFull + 1), tc1 & 1, abort_flag, prm.header, 36);
@@ -397,9 +423,11 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         PP_TAKE_UNIT(un_i, true)
         if (u_nslots == 0) break;
         constexpr int kChunks = DV / 4;  // 16-byte chunks per row
-        const int total = u_len * kChunks;
         for (int sl = 0; sl < u_nslots; ++sl) {
-          float* base = prm.dq_clear + (size_t(u_start) * prm.Hq + (u_h0 + sl)) * DV;
+          const bool before = u_paired && sl == 0;   // the tile before the unit's
+          const int total = (before ? kTile : u_len) * kChunks;
+          float* base = prm.dq_clear + (size_t(before ? u_start - kTile : u_start) * prm.Hq +
+                                        (u_paired ? u_h0 : u_h0 + sl)) * DV;
           for (int c = cl; c < total; c += 64) {
             const int r = c / kChunks, col = c - r * kChunks;
             *reinterpret_cast<float4*>(base + size_t(r) * prm.Hq * DV + col * 4) =
@@ -435,6 +463,10 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
       PP_TAKE_UNIT(un_i, true)
       if (u_nslots == 0) break;
       if (s >= u_nslots) continue;
+      // what this slot holds
+      const bool my_before = u_paired && s == 0;
+      const int my_start = my_before ? u_start - kTile : u_start, my_len = my_before ? kTile : u_len;
+      const int my_ntiles = my_before ? u_ntiles - 1 : u_ntiles;
       float m_used = -INFINITY, l_part = 0.f;
       // Rows of several segments: of the tile's own keys up to its own position, a row sees the
       // prompt's, [0, pr), and those of its own segment, from `lo` on.  A segment ends where the
@@ -455,10 +487,10 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
           if (b <= qd && m) lo = max(lo, 32 * (b + 1) - __clz(m));
         }
       }
-      for (int j = 0; j < u_ntiles; ++j) {
+      for (int j = 0; j < my_ntiles; ++j) {
         KvTile kt;
         kt.len = u_klen(j);
-        kt.diag = j + 1 == u_ntiles;
+        kt.diag = j + 1 == my_ntiles;
         wait_bar(bar(kSFull + s), tcS & 1, abort_flag, prm.header, 40 + s);
         tc_fence_after();
         const bool full = !kt.diag && kt.len == kTile && (one_segment || j < u_n0);
@@ -584,7 +616,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
           const float hi = fmaxf(pmax, xch_exp[half ^ 1]);
           // Rows past the tile's end hold whatever follows in memory: they must not steer the
           // warp-wide decision, or a row's rounding would depend on its neighbours' data.
-          const bool need = row < u_len && !(hi <= exp2f(kRescaleThreshold));
+          const bool need = row < my_len && !(hi <= exp2f(kRescaleThreshold));
           if (!__any_sync(0xffffffffu, need)) break;   // same rows, same values in the partner warp
           const float m_new = fmaxf(m_used, row_max());
           const float alpha = ex2(m_used - m_new);
@@ -650,9 +682,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
       }
       tc_fence_before();
       mbar_arrive(bar(kOFree + s));
-      const int h = u_h0 + s;
-      if (half == 0 && row < u_len)
-        prm.lse[size_t(h) * prm.T + u_start + row] = (m_used + log2f(l_run)) * 0.69314718055994531f;
+      const int h = u_paired ? u_h0 : u_h0 + s;
+      if (half == 0 && row < my_len)
+        prm.lse[size_t(h) * prm.T + my_start + row] = (m_used + log2f(l_run)) * 0.69314718055994531f;
       // A thread holds kCh 16-byte chunks of one row; transposing them inside groups of kCh
       // lanes gives every lane the same chunk of kCh consecutive rows, so that one store
       // instruction of the warp writes whole contiguous half-rows instead of 32 scattered
@@ -683,9 +715,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
 #pragma unroll
         for (int i = 0; i < kCh; ++i) {
           const int r = 32 * qd + grp * kCh + i;
-          if (r < u_len && (DV == D || half * (D / 2) + chunk * 8 < DV)) {
+          if (r < my_len && (DV == D || half * (D / 2) + chunk * 8 < DV)) {
             uint4* dst = reinterpret_cast<uint4*>(
-                prm.o + ((size_t(u_start) + r) * prm.Hq + h) * DV + half * (D / 2) + chunk * 8);
+                prm.o + ((size_t(my_start) + r) * prm.Hq + h) * DV + half * (D / 2) + chunk * 8);
             *dst = make_uint4(ob[4 * i], ob[4 * i + 1], ob[4 * i + 2], ob[4 * i + 3]);
           }
         }
@@ -740,8 +772,7 @@ cudaError_t launch_fwd_t(const pp_plan* plan, const CUtensorMap& tq, const CUten
   if (!dev) return cudaErrorInvalidDevice;
   if (dev->cc_major != 10) return cudaErrorNotSupported;
   using Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, FwdParams);
-  const Kernel kerns[2] = {fwd_kernel<D, false, DV>, fwd_kernel<D, true, DV>};
-  const Kernel kern = kerns[plan->mixed];
+  const Kernel kerns[3] = {fwd_kernel<D, kPlain, DV>, fwd_kernel<D, kMixedTiles, DV>, fwd_kernel<D, kPairedTiles, DV>};
   if (!dev->configured) {
     for (Kernel k : kerns) {
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<D>::kTotal);
@@ -753,6 +784,7 @@ cudaError_t launch_fwd_t(const pp_plan* plan, const CUtensorMap& tq, const CUten
   const pp_problem& pb = plan->prob;
   const int r = pb.num_q_heads / pb.num_kv_heads;
   const long long units = (long long)plan->max_tiles * pb.num_kv_heads * ((r + 1) / 2);
+  const Kernel kern = kerns[plan->mixed ? kMixedTiles : fwd_paired_tiles(pb, num_sms) ? kPairedTiles : kPlain];
   dim3 grid(unsigned(std::min<long long>(units, num_sms)));
   ProfileEvents& ev = profile_events();
   const int slot = int(ev.fwd_count % kProfileRing);
@@ -779,6 +811,7 @@ cudaError_t launch_fwd(const pp_plan* plan, const void* q, const void* k, const 
   FwdParams prm;
   prm.header = reinterpret_cast<int32_t*>(plan->ws + plan->lay.header);
   prm.tiles = reinterpret_cast<const Tile*>(plan->ws + plan->lay.tiles);
+  prm.tile_unit = reinterpret_cast<const uint8_t*>(plan->ws + plan->lay.tile_unit);
   prm.qtiles = reinterpret_cast<const QTile*>(plan->ws + plan->lay.qtiles);
   prm.key_end = reinterpret_cast<const int32_t*>(plan->ws + plan->lay.key_end);
   prm.order = reinterpret_cast<const int32_t*>(plan->ws + (plan->mixed ? plan->lay.qorder : plan->lay.fwd_order));

@@ -23,6 +23,12 @@ struct Tile {
   int32_t work;       // forward work estimate in key tiles (backward: derived)
 };
 static_assert(sizeof(Tile) == 32, "tile record is 32 bytes");
+// What the forward does with a query tile of a segment where it takes them by twos: nothing (the tile
+// behind it has it), this tile alone (a segment's last), or the tile before it and this one.
+enum kTileUnit : uint8_t { kTileNone = 0, kTileAlone = 1, kTileWithLast = 2 };
+__host__ __device__ constexpr uint8_t tile_unit_of(int rel, int count) {   // tile `rel` of a segment's `count`
+  return rel & 1 ? kTileWithLast : rel + 1 == count ? kTileAlone : kTileNone;
+}
 
 // One key tile of the backward pass.  The backward cuts each GROUP (prompt and responses as one
 // token range) into tiles of 128 tokens from the group's start, so a tile may straddle segment
@@ -56,7 +62,8 @@ constexpr int kQTilePrompt = 256;
 
 // Words of the plan header (int32[16]).
 constexpr int kHdrStatus = 0, kHdrDetail = 1, kHdrNumTiles = 2, kHdrNumSegments = 3,
-              kHdrNumBTiles = 8, kHdrNumQTiles = 9;
+              kHdrNumBTiles = 8, kHdrNumQTiles = 9,
+              kHdrSchedTail = 10;   // (multi-kernel plan) tiles of the last block of bwd_sched
 
 // Status word values written by device code.
 enum : int32_t {
@@ -73,6 +80,7 @@ struct PlanLayout {
   size_t seg_start;  // int32[nseg + 1]
   size_t seg_tile0;  // int32[nseg + 1]  first tile of each segment
   size_t tiles;      // Tile[max_tiles]
+  size_t tile_unit;  // uint8[max_tiles]  kTileUnit below
   size_t fwd_order;  // int32[max_tiles]
   size_t grp_btile0; // int32[G + 1]  first backward tile of each group
   size_t btiles;     // BTile[max_tiles]  (at most max_btiles_of of them)
@@ -138,6 +146,20 @@ inline bool fwd_mixed_tiles(const pp_problem& p) {
   return added > 0.3 * grid && (grid + added) * p.num_kv_heads * pairs > 1.75 * 148;
 }
 
+// Whether the forward takes two tiles of a segment into a unit's slots for the last head of an odd number
+// of heads per KV head (each row's arithmetic is the same either way).  A unit with both slots filled
+// takes 1.4 times one with slot 1 empty, so it pays once there is more work per SM than the
+// longest such unit, in key tiles estimated from the mean group: 12000 tokens in 3000-token groups, 16 / 16 heads, D 128
+// 291 -> 204 us, 2600-token groups, D 96 225 -> 165; but 8000-token groups, 2 / 2 heads 166 -> 182.  With three and
+// more heads per KV head the other units take that long anyway: 20187 tokens, 28 / 4 631 -> 594.
+inline bool fwd_paired_tiles(const pp_problem& p, int sms) {
+  const int r = p.num_q_heads / p.num_kv_heads;
+  const double tiles = p.total_tokens / double(kTile) + 0.5 * (p.num_groups + p.num_responses);
+  const double m = double((p.total_tokens / p.num_groups + kTile - 1) / kTile);
+  if (!(r & 1) || tiles * p.num_kv_heads * ((r + 1) / 2) <= sms) return false;
+  return r > 1 || tiles * p.num_kv_heads * (m + 1) / 2 > 1.4 * sms * m * (p.num_groups > 1 ? 1.5 : 1.0);
+}
+
 inline PlanLayout plan_layout(const pp_problem& p) {
   PlanLayout l{};
   int nseg = p.num_groups + p.num_responses;
@@ -150,6 +172,7 @@ inline PlanLayout plan_layout(const pp_problem& p) {
   l.seg_start = off; off = align_up(off + sizeof(int32_t) * (nseg + 1), 256);
   l.seg_tile0 = off; off = align_up(off + sizeof(int32_t) * (nseg + 1), 256);
   l.tiles = off;     off = align_up(off + sizeof(Tile) * size_t(mt), 256);
+  l.tile_unit = off; off = align_up(off + size_t(mt), 256);
   l.fwd_order = off; off = align_up(off + sizeof(int32_t) * size_t(mt), 256);
   l.grp_btile0 = off; off = align_up(off + sizeof(int32_t) * (size_t(p.num_groups) + 1), 256);
   l.btiles = off;    off = align_up(off + sizeof(BTile) * size_t(mt), 256);
@@ -216,11 +239,10 @@ inline int bwd_split_log2(const pp_problem& p) {
 // (bwd_units) the 148 units that run at a time may be the longest of all of a block's groups, and with r
 // query heads per KV head a block's Q, dO and dQ accumulator are 600 r * 128 KB at D 128: far beyond
 // L2, so that a (query tile, head) is fetched, and its accumulator written back, for nearly every
-// other key tile.  Blocks of 150 units, with the last 200 in one block to balance the end
-// (bwd_sched), take a third to a half of that traffic (a model of L2 with 80 MB of least-recently-used tiles, which gives
+// other key tile.  Blocks of 150 units, with a larger last one to balance the end
+// (bwd_sched; sched_tail in the plan), take a third to a half of that traffic (a model of L2 with 80 MB of least-recently-used tiles, which gives
 // the 600s' measured 0.93, 5.4 and 5.9 GB as 0.93, 5.9 and 5.7: 0.5, 3.9 and 2.2).  Main kernel, 600s
-// -> these: 9241 tokens, 32 / 8 heads 262 -> 250 us; 16384, 64 / 8 1361 -> 1230; 20187, 28 / 4 1818 ->
-// 1742; 16384, 32 / 8, D 64 456 -> 400; 36000 in short groups, 16 / 2 277 -> 243; 16760, 32 / 8 307 ->
+// -> these: 9241 tokens, 32 / 8 heads 262 -> 250 us; 16384, 64 / 8 1361 -> 1230; 16384, 32 / 8, D 64 456 -> 400; 36000 in short groups, 16 / 2 277 -> 243; 16760, 32 / 8 307 ->
 // 272; two rows of 32768, 32 / 8 19320 -> 19220.  With one and two heads per KV head a block's data is
 // that much smaller, and the smaller blocks only cost balance: 8 / 8 258 -> 265, 16 / 8 278 -> 276, 754 -> 740.
 // Up to 200 units both are one block.

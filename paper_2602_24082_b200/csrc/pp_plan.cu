@@ -33,6 +33,7 @@ struct PlanPtrs {
   int32_t* seg_start;
   int32_t* seg_tile0;
   Tile* tiles;
+  uint8_t* tile_unit;
   int32_t* grp_btile0;
   BTile* btiles;
   int32_t* fwd_order;
@@ -267,6 +268,7 @@ __device__ __forceinline__ void plan_tile_body(const PlanPtrs& p, int t) {
   }
   tl.work = (tl.kv0_len + kTile - 1) / kTile + (tl.kv1_len + kTile - 1) / kTile + 1;
   p.tiles[t] = tl;
+  p.tile_unit[t] = tile_unit_of(t - p.seg_tile0[s], p.seg_tile0[s + 1] - p.seg_tile0[s]);
   if (p.qtiles) add_grid_gain(p, g, tile_cost(tl.work));
 }
 
@@ -424,10 +426,18 @@ __global__ void plan_fwd_order_kernel(PlanPtrs p) {
 constexpr int kSuperGroupUnits = 600;
 
 // The blocks of the order that the kernel takes with several query heads per KV head
-// (bwd_takes_sched, which has the reasons): `later` = units of the groups ranked behind the tile's own,
-// of `total`.  (At most 1002 blocks, which the one-block plan's sort keys have room for.)
-__device__ __forceinline__ int sched_block(int later, int total) {
-  return later < kSchedTailUnits ? 0 : 1 + (later - kSchedTailUnits) / max(kSchedBlockUnits, total / 1000);
+// (bwd_takes_sched, which has the reasons).  The last block begins with the first group behind which
+// there are fewer than kSchedTailUnits units, or not enough work to balance its longest unit: with less
+// than two thirds of that unit behind it for each of 148 SMs, 12000 tokens in four groups (28 / 4 heads, D 64, 384 units)
+// took 490 us, all in one block 455.  `later`, `later_work` = tiles of the groups ranked behind a group of
+// `tiles` tiles, and their work.
+__device__ __forceinline__ bool sched_tail(const PlanPtrs& p, int later, int later_work, int tiles) {
+  return p.Hkv * later < kSchedTailUnits || (long long)p.Hkv * later_work < 100LL * tiles;
+}
+// `tail` = tiles of the groups in the last block, `total` = of all.  (At most 1002 blocks, which the
+// one-block plan's sort keys have room for.)
+__device__ __forceinline__ int sched_block(const PlanPtrs& p, int later, int tail, int total) {
+  return later < tail ? 0 : 1 + p.Hkv * (later - tail) / max(kSchedBlockUnits, p.Hkv * total / 1000);
 }
 
 // bwd_order (plain longest-first list of the backward tiles) and each tile's group work
@@ -445,14 +455,17 @@ __device__ __forceinline__ void plan_gwork_body(const PlanPtrs& p, int t, int n)
 
 __device__ __forceinline__ void plan_sgroup_body(const PlanPtrs& p, int t, int n) {
   const int gs = p.btiles[t].grp_start, gw = p.tile_gwork[t];
-  int rest = 0, later = 0;  // tiles of this group and of the groups that come later; of those alone
+  // tiles of this group and of the groups that come later; of those alone, and their work
+  int rest = 0, later = 0, later_work = 0;
   for (int u = 0; u < n; ++u) {
     const int ogs = p.btiles[u].grp_start, ow = p.tile_gwork[u];
     const bool behind = (ow < gw) || (ow == gw && ogs > gs);
     rest += (ogs == gs) || behind;
     later += behind;
+    if (behind) later_work += p.btiles[u].work;
   }
-  p.tile_sblock[t] = sched_block(p.Hkv * later, p.Hkv * n);
+  p.tile_sblock[t] = later;
+  if (sched_tail(p, later, later_work, rest - later)) atomicMax(&p.header[kHdrSchedTail], rest);
   // counted from the END of the list, so the last block is never a small leftover whose
   // long units would start late: blocks are processed in decreasing index
   p.tile_sgroup[t] = (p.Hkv * rest - 1) / kSuperGroupUnits;
@@ -467,10 +480,10 @@ __device__ __forceinline__ void plan_units_body(const PlanPtrs& p, int t, int n)
   }
   for (int kvh = 0; kvh < p.Hkv; ++kvh) p.bwd_units[p.Hkv * pos + kvh] = (kvh << 24) | t;
   if (p.bwd_sched) {
-    const int sb = p.tile_sblock[t];
+    const int tail = p.header[kHdrSchedTail], sb = sched_block(p, p.tile_sblock[t], tail, n);
     pos = 0;
     for (int u = 0; u < n; ++u) {
-      const int osb = p.tile_sblock[u], ob = p.btiles[u].work;
+      const int osb = sched_block(p, p.tile_sblock[u], tail, n), ob = p.btiles[u].work;
       pos += (osb > sb) || (osb == sb && ((ob > wb) || (ob == wb && u < t)));
     }
     for (int kvh = 0; kvh < p.Hkv; ++kvh) p.bwd_sched[p.Hkv * pos + kvh] = (kvh << 24) | t;
@@ -583,7 +596,7 @@ struct FusedSmem {
   uint16_t qwork[kMixed ? kFusedMaxTiles : 2];       // work of the query tiles, 0 where there is none
   uint16_t unit_tile[2][kFusedMaxTiles];   // backward tiles in the orders of their units
   int32_t warp_sum[2][32];
-  int32_t status, detail, no_qtile;
+  int32_t status, detail, no_qtile, sched_tail;
 };
 
 // Inclusive sums of two values over the block.
@@ -720,7 +733,7 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
   }
   if (tid == 0) {
     sm.status = kStatusOk;
-    sm.detail = sm.no_qtile = 0;
+    sm.detail = sm.no_qtile = sm.sched_tail = 0;
   }
   if (kDesc > 1) dependency_wait();   // (the workspace may still be in use up to here)
   __syncthreads();
@@ -842,6 +855,7 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
       }
       tl.work = (tl.kv0_len + kTile - 1) / kTile + (tl.kv1_len + kTile - 1) / kTile + 1;
       p.tiles[t] = tl;
+      p.tile_unit[t] = tile_unit_of(t - sm.seg_tile0[s], sm.seg_tile0[s + 1] - sm.seg_tile0[s]);
       sm.tile[0][t] = tl.start;
       sm.tile[1][t] = tl.start + tl.len;
       sm.tile[2][t] = tl.vis_end;
@@ -941,7 +955,7 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
   };
   auto sched_key = [&](int t, int ranked_before) {   // (a tile's work is 1 .. 2048)
     const int g = sm.bgrp[t], later = nb - ranked_before - (sm.btile0[g + 1] - sm.btile0[g]);
-    return uint32_t(1023 - sched_block(p.Hkv * later, p.Hkv * nb)) << 22 | uint32_t(2048 - sm.wb[t]) << 11 |
+    return uint32_t(1023 - sched_block(p, later, sm.sched_tail, nb)) << 22 | uint32_t(2048 - sm.wb[t]) << 11 |
            uint32_t(t);
   };
   if (by_rank) {   // (blocks of 256 threads have at most 256 tiles: one per thread)
@@ -962,6 +976,16 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
     rank_count<true>(sm.o.r.key[2], p.G, sm.o.r.rank[2], sm.btile0);
     if constexpr (kMixed) rank_count<false>(sm.o.r.key[5], n, sm.o.r.rank[5], nullptr);
     __syncthreads();
+    if (p.bwd_sched) {
+      if (tid < p.G) {
+        const uint32_t mine = sm.o.r.key[2][tid];
+        int later_work = 0;
+        for (int g = 0; g < p.G; ++g) later_work += sm.o.r.key[2][g] > mine ? sm.gwork[g] : 0;
+        const int rest = nb - sm.o.r.rank[2][tid], own = sm.btile0[tid + 1] - sm.btile0[tid];
+        if (sched_tail(p, rest - own, later_work, own)) atomicMax(&sm.sched_tail, rest);
+      }
+      __syncthreads();
+    }
     if (tid < n) p.fwd_order[sm.o.r.rank[0][tid]] = tid;
     if constexpr (kMixed)
       if (tid < n) p.qorder[sm.o.r.rank[5][tid]] = tid;
@@ -985,14 +1009,19 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
     while (n2 < n) n2 <<= 1;
     bitonic_sort(key, n2, sm.o.sort);
     // tiles of the groups ranked before each group
-    int cnt = 0, unused = 0, g = 0;
+    int cnt = 0, work = 0, g = 0;
     if (tid < p.G) {
       g = int(key[2][0] & 1023u);
       cnt = sm.btile0[g + 1] - sm.btile0[g];
+      work = sm.gwork[g];
     }
     const int mine = cnt;
-    block_scan2(cnt, unused, sm.warp_sum);
-    if (tid < p.G) sm.before[g] = cnt - mine;
+    block_scan2(cnt, work, sm.warp_sum);
+    const int all_work = sm.warp_sum[1][(nthr >> 5) - 1];
+    if (tid < p.G) {
+      sm.before[g] = cnt - mine;
+      if (sched_tail(p, nb - cnt, all_work - work, mine)) atomicMax(&sm.sched_tail, nb - cnt + mine);
+    }
     __syncthreads();
     uint32_t ukey[2][2];
 #pragma unroll
@@ -1113,6 +1142,7 @@ cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cu
   p.seg_start = reinterpret_cast<int32_t*>(ws + l.seg_start);
   p.seg_tile0 = reinterpret_cast<int32_t*>(ws + l.seg_tile0);
   p.tiles = reinterpret_cast<Tile*>(ws + l.tiles);
+  p.tile_unit = reinterpret_cast<uint8_t*>(ws + l.tile_unit);
   p.grp_btile0 = reinterpret_cast<int32_t*>(ws + l.grp_btile0);
   p.btiles = reinterpret_cast<BTile*>(ws + l.btiles);
   p.fwd_order = reinterpret_cast<int32_t*>(ws + l.fwd_order);

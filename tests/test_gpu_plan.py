@@ -143,9 +143,9 @@ def test_backward_units_order(w):
     (1, 200, 3, 1), (9, 1100, 32, 8), (40, 300, 28, 4), (60, 1100, 8, 2), (150, 1200, 16, 4), (8, 1500, 4, 2),
     (1100, 5, 6, 2), (12, 1000, 280, 70), (300, 650, 210, 70)])
 def test_order_the_backward_takes_its_units_in(groups, length, hq, hkv):
-    """From three query heads per KV head on: groups by decreasing work, the last 200 units in one block
-    and the others in blocks of 150 (larger beyond 1000 blocks), inside a block longest first with all
-    KV heads of a tile adjacent.  Below that: the order of read_bwd_units.  Plans in one block by
+    """From three query heads per KV head and 200 units on: groups by decreasing work, the last 200 units and
+    what balances longer ones before them in one block, the others in blocks of 150 (larger beyond 1000
+    blocks), inside a block longest first with all KV heads of a tile adjacent.  Below that: the order of read_bwd_units.  Plans in one block by
     counting (up to 512 tiles) and by sorting, and of several kernels."""
     from paper_2602_24082_b200 import binding as B
     rng = np.random.default_rng(groups)
@@ -163,10 +163,14 @@ def test_order_the_backward_takes_its_units_in(groups, length, hq, hkv):
     gwork, gtiles = {}, {}
     for g, x in zip(grp, work):
         gwork[g], gtiles[g] = gwork.get(g, 0) + x, gtiles.get(g, 0) + 1
-    block, later = {}, 0
+    behind, tail, later, later_work = {}, 0, 0, 0
     for g in sorted(gwork, key=lambda g: (gwork[g], -g)):     # from the last
-        block[g] = 0 if later < 200 else 1 + (later - 200) // max(150, hkv * n // 1000)
-        later += hkv * gtiles[g]
+        behind[g] = later
+        if hkv * later < 200 or hkv * later_work < 100 * gtiles[g]:
+            tail = later + gtiles[g]
+        later, later_work = later + gtiles[g], later_work + gwork[g]
+    block = {g: 0 if x < tail else 1 + hkv * (x - tail) // max(150, hkv * n // 1000) for g, x in behind.items()}
+    assert tail == n or max(block.values()) > 0
     expect = sorted(range(n), key=lambda t: (-block[grp[t]], -work[t], t))
     assert units[:, 1].tolist() == np.repeat(expect, hkv).tolist()
     assert (units[:, 0].reshape(n, hkv) == np.arange(hkv)).all()
