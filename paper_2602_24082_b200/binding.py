@@ -467,41 +467,15 @@ def pp_build_rows(grp_prompt_len: torch.Tensor, grp_resp_off: torch.Tensor, resp
     int32 DEVICE tensors.  Returns a dict of device tensors: order, row_group_off (trimmed to
     rows + 1), row_tokens, row_cost (trimmed to rows), grp_prompt_len, grp_resp_off, resp_len in
     row order, and ``status`` (code, detail) as Python ints (reading it synchronises)."""
-    dev = grp_prompt_len.device
     G, N = int(grp_prompt_len.numel()), int(resp_len.numel())
-    for t, n, name in ((grp_prompt_len, G, "grp_prompt_len"), (grp_resp_off, G + 1, "grp_resp_off"),
-                       (resp_len, N, "resp_len")):
-        _chk(t, (n,), torch.int32, name)
-    nbytes = ctypes.c_size_t(0)
-    _check(lib().pp_build_rows_workspace_bytes(G, ctypes.byref(nbytes)), "pp_build_rows_workspace_bytes")
-    ws = torch.empty(nbytes.value, dtype=torch.uint8, device=dev)
-    i32 = lambda n: torch.empty(n, dtype=torch.int32, device=dev)
-    i64 = lambda n: torch.empty(n, dtype=torch.int64, device=dev)
-    order, rgo, meta = i32(G), i32(G + 1), i32(3)   # meta: status code, detail, number of rows
-    status, nrows = meta[:2], meta[2:]
-    rtok, rcost = i64(G), i64(G)
-    oP, ooff, orl = i32(G), i32(G + 1), i32(N)
-    _call(order.get_device(), "pp_build_rows", lib().pp_build_rows, G, N, grp_prompt_len.data_ptr(),
-          grp_resp_off.data_ptr(), resp_len.data_ptr(), int(row_capacity), ws.data_ptr(), ws.numel(),
-          order.data_ptr(), rgo.data_ptr(), nrows.data_ptr(), rtok.data_ptr(), rcost.data_ptr(),
-          oP.data_ptr(), ooff.data_ptr(), orl.data_ptr(), status.data_ptr())
-    code, detail, r = meta.tolist()   # one synchronising copy
-    return {"order": order, "row_group_off": rgo[:r + 1], "row_tokens": rtok[:r], "row_cost": rcost[:r],
-            "grp_prompt_len": oP, "grp_resp_off": ooff, "resp_len": orl, "status": (code, detail)}
+    return _step_calls().build_rows(grp_prompt_len, grp_resp_off, resp_len, G, N, int(row_capacity))
 
 
 def pp_assign_rows(row_cost: torch.Tensor, num_ranks: int):
     """Rows -> data-parallel ranks by longest-processing-time assignment on the attention cost.
     ``row_cost``: int64 DEVICE tensor [rows].  Returns device tensors (order [rows] int32,
     rank_of_row [rows] int32, rank_cost [num_ranks] int64)."""
-    _chk(row_cost, (row_cost.numel(),), torch.int64, "row_cost")
-    dev, R = row_cost.device, int(row_cost.numel())
-    order = torch.empty(R, dtype=torch.int32, device=dev)
-    rank_of_row = torch.empty(R, dtype=torch.int32, device=dev)
-    rank_cost = torch.empty(int(num_ranks), dtype=torch.int64, device=dev)
-    _call(order.get_device(), "pp_assign_rows", lib().pp_assign_rows, R, row_cost.data_ptr(),
-          int(num_ranks), order.data_ptr(), rank_of_row.data_ptr(), rank_cost.data_ptr())
-    return order, rank_of_row, rank_cost
+    return _step_calls().assign_rows(row_cost, int(row_cost.numel()), int(num_ranks))
 
 
 def pp_debug_expire_wait(plan: Plan, site: int):

@@ -180,6 +180,9 @@ static int read_units(const pp_plan* plan, size_t list, pp_stream_t stream, int3
 
 int pp_plan_read_bwd_units(const pp_plan* plan, pp_stream_t stream, int32_t* units) {
   if (!plan || !units) return PP_ERR_INVALID_ARG;
+  if (pp::bwd_takes_sched(plan->prob) &&
+      pp::launch_base_units(plan, reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess)
+    return PP_ERR_CUDA;
   return read_units(plan, plan->lay.bwd_units, stream, units);
 }
 

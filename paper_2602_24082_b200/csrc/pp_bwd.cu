@@ -356,7 +356,6 @@ bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   const long long t_kernel0 = clock64();
 #endif
 
-  launch_dependents();
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   if (base - raw + L::kUsed > L::kTotal) {  // cannot happen with an aligned base
@@ -1032,7 +1031,7 @@ cudaError_t launch_bwd_t(const pp_plan* plan, const void* o, const float* lse, c
   const unsigned sem_n4 = prm.dq_sem ? unsigned(max_btiles_of(pb)) * pb.num_q_heads : 0;   // 16 bytes each
   const unsigned pre_blocks = unsigned(Hq * ((T + pre_tokens(DV) - 1) / pre_tokens(DV)));
   auto pre = dq_cleared ? bwd_preprocess_kernel<DV, false> : bwd_preprocess_kernel<DV, true>;
-  cudaError_t e = launch_kernel(pre_blocks <= kOverlapBlocks, pre, dim3(pre_blocks), dim3(32 * kPreWarps), 0, stream,
+  cudaError_t e = launch_kernel(true, pre, dim3(pre_blocks), dim3(32 * kPreWarps), 0, stream,
                                 static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse,
                                 const_cast<float*>(prm.delta), const_cast<float*>(prm.lse2), prm.dq_acc, int(T),
                                 int(Hq), reinterpret_cast<int4*>(prm.dq_sem), sem_n4);
@@ -1053,7 +1052,7 @@ cudaError_t launch_bwd_t(const pp_plan* plan, const void* o, const float* lse, c
   const SumParts sp = {prm.parts, prm.header, prm.tiles, prm.dk, prm.dv, prm.lg_split, pb.num_kv_heads, DV};
   const unsigned sum_blocks = prm.lg_split ? unsigned(max_btiles_of(pb)) * pb.num_kv_heads * 8 : 0;
   if (e == cudaSuccess)
-    e = launch_kernel(fb + sum_blocks <= kOverlapBlocks, bwd_finalize_kernel, dim3(fb + sum_blocks), dim3(256), 0, stream,
+    e = launch_kernel(true, bwd_finalize_kernel, dim3(fb + sum_blocks), dim3(256), 0, stream,
                       reinterpret_cast<const float4*>(prm.dq_acc), static_cast<uint2*>(dq), n4, prm.scale, fb, sp);
   if (launches) *launches += 3;
   return e;

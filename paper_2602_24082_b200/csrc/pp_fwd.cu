@@ -157,7 +157,6 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // (known to be uniform in the warp)
 
-  launch_dependents();
   dependency_wait();
   if (prm.header[0] != kStatusOk) return;
   const int ntiles_total = prm.header[kMixed ? kHdrNumQTiles : kHdrNumTiles];

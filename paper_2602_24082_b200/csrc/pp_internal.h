@@ -89,7 +89,8 @@ struct PlanLayout {
   size_t tile_sgroup; // int32[max_tiles] super-group (block of consecutive groups)
   size_t tile_sblock; // int32[max_tiles] ... and its block in bwd_sched
   size_t bwd_units;  // int32[max_tiles * Hkv]  (kv head << 24) | backward tile, processing order
-  size_t bwd_sched;  // the same units in smaller blocks (bwd_takes_sched): what the kernel then takes
+                     //   (with bwd_takes_sched only where it is asked for)
+  size_t bwd_sched;  // the same units in smaller blocks: with bwd_takes_sched, what the kernel takes
   size_t bwd_units_det;  // the same units, one (group, KV head) set after the other and inside a
                          //   set by descending tile index: the order of the deterministic backward
   size_t key_end;    // int32[T]
@@ -322,19 +323,21 @@ inline bool device_is_sm100() {
 }
 
 // Launches a kernel, with `overlap` so that it may start before the kernel in front of it on the
-// stream has ended (programmatic dependent launch): the kernels of a step call launch_dependents
-// first thing and dependency_wait before they touch global memory, and the launch (in the
-// backward also barrier set-up, tensor-map fetches and tensor-memory allocation) runs under the
-// tail of the one before.  (Kernels that know nothing of this, in front or behind, see ordinary stream order.)
-// The persistent kernels take it up to kOverlapUnits units per SM: steps of 60 - 100 us gain 5 -
+// stream has ended (programmatic dependent launch): it calls dependency_wait before it touches global
+// memory, and its launch (in the backward also barrier set-up, tensor-map fetches and tensor-memory
+// allocation) runs under the tail of the one before, or under all of it where that calls
+// launch_dependents first thing (plan, preprocess, finalize).  (Kernels that know nothing of this, in
+// front or behind, see ordinary stream order.)
+// The main kernels take it up to kOverlapUnits units per SM: steps of 60 - 100 us gain 5 -
 // 9 % (144 ... 1054 tokens), one of 180 us 2.5 %, one of 500 us nothing, and a forward and
-// backward of 2600 and 1100 units (T 16384, 32 / 8 heads, D 64) lost 2 %.  The streaming kernels
-// (preprocess, finalize) take it up to kOverlapBlocks blocks, two per SM: 144 tokens, 1 / 1 heads,
-// 42.4 -> 38.6 us alone and 32.8 -> 30.3 in a row of steps, 300, 4 / 2 55.5 -> 51.7 and 44.6 -> 42.9,
-// 700, 8 / 8 50.0 -> 45.5 alone.  With more, early blocks crowd the SMs that free up first: up to eight
-// per SM 1000 tokens, 8 / 1 55.1 -> 61.2 in a row, preprocess 30 -> 38 us at T 9241.
+// backward of 2600 and 1100 units (T 16384, 32 / 8 heads, D 64) lost 2 %.  Preprocess and finalize always take it,
+// 3 - 5 us a step: 144 tokens, 1 / 1 heads 30.0 -> 27.4 us in a row of steps, 40.0 -> 36.4 alone; 374, 28 / 4,
+// D 64 39.4 -> 35.1; 1000, 8 / 2 59.8 -> 56.2; 3000, 16 / 8 104.9 -> 100.4; 28626 in short groups, 4 / 1
+// 169.3 -> 165; 12000, 32 / 8 427 -> 422.  The main kernels in front of them do not call
+// launch_dependents: early blocks of the stream crowd the SMs that free up first (with it and more than
+// two blocks per SM 1000 tokens, 8 / 1 55 -> 61, preprocess 30 -> 38 us at T 9241, and even
+// with fewer 144 tokens 30.1 instead of 27.4).
 constexpr int kOverlapUnits = 4;
-constexpr unsigned kOverlapBlocks = 296;
 template <typename... P, typename... A>
 cudaError_t launch_kernel(bool overlap, void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t stream, A&&... args) {
@@ -380,6 +383,8 @@ bool profile_read_all(float* fwd_ms, float* bwd_ms, int capacity, int* n_fwd, in
 // host_desc: the four descriptor arrays on the host, or null when they are on the device
 cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cudaStream_t stream,
                         int* launches);
+// the order of units that the plan leaves out where bwd_takes_sched (lay.bwd_units)
+cudaError_t launch_base_units(const pp_plan* plan, cudaStream_t stream);
 cudaError_t launch_fwd(const pp_plan* plan, const void* q, const void* k, const void* v, float scale,
                        void* o, float* lse, float* dq_clear, cudaStream_t stream, int* launches);
 cudaError_t launch_bwd(const pp_plan* plan, const void* q, const void* k, const void* v,

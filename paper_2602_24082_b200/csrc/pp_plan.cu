@@ -41,8 +41,8 @@ struct PlanPtrs {
   int32_t* tile_gwork;
   int32_t* tile_sgroup;
   int32_t* tile_sblock;
-  int32_t* bwd_units;
-  int32_t* bwd_sched;   // null: not wanted
+  int32_t* bwd_units;   // null: not wanted (either of the two, or the third)
+  int32_t* bwd_sched;
   int32_t* bwd_units_det;
   int Hkv;
   int32_t* key_end;
@@ -472,13 +472,16 @@ __device__ __forceinline__ void plan_sgroup_body(const PlanPtrs& p, int t, int n
 }
 
 __device__ __forceinline__ void plan_units_body(const PlanPtrs& p, int t, int n) {
-  const int sg = p.tile_sgroup[t], wb = p.btiles[t].work;
+  const int wb = p.btiles[t].work;
   int pos = 0;
-  for (int u = 0; u < n; ++u) {
-    const int osg = p.tile_sgroup[u], ob = p.btiles[u].work;
-    pos += (osg > sg) || (osg == sg && ((ob > wb) || (ob == wb && u < t)));
+  if (p.bwd_units) {
+    const int sg = p.tile_sgroup[t];
+    for (int u = 0; u < n; ++u) {
+      const int osg = p.tile_sgroup[u], ob = p.btiles[u].work;
+      pos += (osg > sg) || (osg == sg && ((ob > wb) || (ob == wb && u < t)));
+    }
+    for (int kvh = 0; kvh < p.Hkv; ++kvh) p.bwd_units[p.Hkv * pos + kvh] = (kvh << 24) | t;
   }
-  for (int kvh = 0; kvh < p.Hkv; ++kvh) p.bwd_units[p.Hkv * pos + kvh] = (kvh << 24) | t;
   if (p.bwd_sched) {
     const int tail = p.header[kHdrSchedTail], sb = sched_block(p, p.tile_sblock[t], tail, n);
     pos = 0;
@@ -495,6 +498,7 @@ __device__ __forceinline__ void plan_units_body(const PlanPtrs& p, int t, int n)
   // the list can have units waiting for a unit that has not been handed out yet, so fewer than
   // det_asc_max CTAs can be held up that way and the others keep drawing.  Larger sets go out
   // in DESCENDING tile order, where every unit follows the units it waits for.
+  if (!p.bwd_units_det) return;
   const int gs = p.btiles[t].grp_start, gw = p.tile_gwork[t];
   int before = 0, ng = 0;  // tiles of groups ranked earlier; tiles of this group
   for (int u = 0; u < n; ++u) {
@@ -577,9 +581,8 @@ struct FusedSmem {
   union alignas(16) {   // (keys are read as uint4)
     uint32_t sort[2][kMixed ? 4 : 3][kFusedMaxTiles];
     struct {
-      // forward tiles, backward tiles, groups, backward units in both orders, query tiles (groups:
-      uint32_t key[kMixed ? 6 : 5][kRankTiles];
-      int32_t rank[kMixed ? 6 : 5][kRankTiles];      //   backward tiles of the groups before)
+      uint32_t key[kMixed ? 5 : 4][kRankTiles];      // forward tiles, backward tiles, groups, backward units,
+      int32_t rank[kMixed ? 5 : 4][kRankTiles];      //   query tiles (groups: backward tiles of the groups before)
     } r;
   } o;
   int32_t desc[kDescFused];
@@ -594,7 +597,7 @@ struct FusedSmem {
   uint16_t bgrp[kFusedMaxTiles];
   int32_t grid_gain[kMixed ? kFusedMaxTiles / 2 : 1];
   uint16_t qwork[kMixed ? kFusedMaxTiles : 2];       // work of the query tiles, 0 where there is none
-  uint16_t unit_tile[2][kFusedMaxTiles];   // backward tiles in the orders of their units
+  uint16_t unit_tile[kFusedMaxTiles];   // backward tiles in the order of their units
   int32_t warp_sum[2][32];
   int32_t status, detail, no_qtile, sched_tail;
 };
@@ -948,33 +951,30 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
   __syncthreads();
   // at most 2048 * 2049 / 2 < 2^22 units of work in a group, at most 1024 groups
   if (tid < p.G) key[2][0] = uint32_t(0x3fffff - sm.gwork[tid]) << 10 | uint32_t(tid);
-  // super-groups (see above), inside one the longest tiles first; Hkv * nb / 600 < 512
+  // super-groups or blocks (see above), inside one the longest tiles first; Hkv * nb / 600 < 512 and a
+  // tile's work is 1 .. 2048
   auto unit_key = [&](int t, int ranked_before) {
-    const int sg = (p.Hkv * (nb - ranked_before) - 1) / kSuperGroupUnits;
-    return uint32_t(511 - sg) << 23 | uint32_t(4095 - sm.wb[t]) << 11 | uint32_t(t);
-  };
-  auto sched_key = [&](int t, int ranked_before) {   // (a tile's work is 1 .. 2048)
-    const int g = sm.bgrp[t], later = nb - ranked_before - (sm.btile0[g + 1] - sm.btile0[g]);
-    return uint32_t(1023 - sched_block(p, later, sm.sched_tail, nb)) << 22 | uint32_t(2048 - sm.wb[t]) << 11 |
-           uint32_t(t);
+    const int g = sm.bgrp[t], rest = nb - ranked_before, later = rest - (sm.btile0[g + 1] - sm.btile0[g]);
+    const int block = p.bwd_sched ? sched_block(p, later, sm.sched_tail, nb) : (p.Hkv * rest - 1) / kSuperGroupUnits;
+    return uint32_t(1023 - block) << 22 | uint32_t(2048 - sm.wb[t]) << 11 | uint32_t(t);
   };
   if (by_rank) {   // (blocks of 256 threads have at most 256 tiles: one per thread)
     for (int t = tid; t < kRankTiles; t += nthr) {
       sm.o.r.key[0][t] = t == tid ? key[0][0] : ~0u;
       sm.o.r.key[1][t] = t == tid ? key[1][0] : ~0u;
       sm.o.r.key[2][t] = t == tid ? key[2][0] : ~0u;
-      sm.o.r.key[3][t] = sm.o.r.key[4][t] = ~0u;
-      for (int a = 0; a < 5; ++a) sm.o.r.rank[a][t] = 0;
+      sm.o.r.key[3][t] = ~0u;
+      sm.o.r.rank[0][t] = sm.o.r.rank[1][t] = sm.o.r.rank[2][t] = sm.o.r.rank[3][t] = 0;
       if constexpr (kMixed) {
-        sm.o.r.key[5][t] = t == tid ? key[3][0] : ~0u;
-        sm.o.r.rank[5][t] = 0;
+        sm.o.r.key[4][t] = t == tid ? key[3][0] : ~0u;
+        sm.o.r.rank[4][t] = 0;
       }
     }
     __syncthreads();
     rank_count<false>(sm.o.r.key[0], n, sm.o.r.rank[0], nullptr);
     rank_count<false>(sm.o.r.key[1], nb, sm.o.r.rank[1], nullptr);
     rank_count<true>(sm.o.r.key[2], p.G, sm.o.r.rank[2], sm.btile0);
-    if constexpr (kMixed) rank_count<false>(sm.o.r.key[5], n, sm.o.r.rank[5], nullptr);
+    if constexpr (kMixed) rank_count<false>(sm.o.r.key[4], n, sm.o.r.rank[4], nullptr);
     __syncthreads();
     if (p.bwd_sched) {
       if (tid < p.G) {
@@ -988,21 +988,16 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
     }
     if (tid < n) p.fwd_order[sm.o.r.rank[0][tid]] = tid;
     if constexpr (kMixed)
-      if (tid < n) p.qorder[sm.o.r.rank[5][tid]] = tid;
+      if (tid < n) p.qorder[sm.o.r.rank[4][tid]] = tid;
     if (tid < nb) {
       p.bwd_order[sm.o.r.rank[1][tid]] = tid;
       sm.o.r.key[3][tid] = unit_key(tid, sm.o.r.rank[2][sm.bgrp[tid]]);
-      if (p.bwd_sched) sm.o.r.key[4][tid] = sched_key(tid, sm.o.r.rank[2][sm.bgrp[tid]]);
     }
     if (tid < p.G) sm.before[tid] = sm.o.r.rank[2][tid];
     __syncthreads();
     rank_count<false>(sm.o.r.key[3], nb, sm.o.r.rank[3], nullptr);
-    if (p.bwd_sched) rank_count<false>(sm.o.r.key[4], nb, sm.o.r.rank[4], nullptr);
     __syncthreads();
-    if (tid < nb) {
-      sm.unit_tile[0][sm.o.r.rank[3][tid]] = uint16_t(tid);
-      if (p.bwd_sched) sm.unit_tile[1][sm.o.r.rank[4][tid]] = uint16_t(tid);
-    }
+    if (tid < nb) sm.unit_tile[sm.o.r.rank[3][tid]] = uint16_t(tid);
     __syncthreads();
   } else {
     int n2 = 1024;
@@ -1023,7 +1018,7 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
       if (sched_tail(p, nb - cnt, all_work - work, mine)) atomicMax(&sm.sched_tail, nb - cnt + mine);
     }
     __syncthreads();
-    uint32_t ukey[2][2];
+    uint32_t ukey[1][2];
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const int t = tid + nthr * r;
@@ -1032,22 +1027,17 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
         if (t < n) p.qorder[t] = int32_t(key[3][r] & 0xffffu);
       if (t < nb) p.bwd_order[t] = int32_t(key[1][r] & 0xffffu);
       ukey[0][r] = t < nb ? unit_key(t, sm.before[sm.bgrp[t]]) : ~0u;
-      ukey[1][r] = t < nb ? sched_key(t, sm.before[sm.bgrp[t]]) : ~0u;
     }
     bitonic_sort(ukey, n2, sm.o.sort);
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int t = tid + nthr * r;
-      for (int a = 0; a < 2; ++a)
-        if (t < nb) sm.unit_tile[a][t] = uint16_t(ukey[a][r] & 2047u);
-    }
+    for (int r = 0; r < 2; ++r)
+      if (tid + nthr * r < nb) sm.unit_tile[tid + nthr * r] = uint16_t(ukey[0][r] & 2047u);
     __syncthreads();
   }
-  // ---- backward units, in their orders
+  // ---- backward units, in both orders
   for (int e = tid; e < nb * p.Hkv; e += nthr) {
     const int i = e / p.Hkv, kvh = e - i * p.Hkv;
-    p.bwd_units[e] = (kvh << 24) | int(sm.unit_tile[0][i]);
-    if (p.bwd_sched) p.bwd_sched[e] = (kvh << 24) | int(sm.unit_tile[1][i]);
+    (p.bwd_sched ? p.bwd_sched : p.bwd_units)[e] = (kvh << 24) | int(sm.unit_tile[i]);
     // deterministic backward: set after set (see plan_units_body)
     const int g = sm.bgrp[i], ng = sm.btile0[g + 1] - sm.btile0[g], k_rel = i - sm.btile0[g];
     const int slot = ng <= p.det_asc_max ? k_rel : ng - 1 - k_rel;
@@ -1127,8 +1117,7 @@ bool profile_read(float* fwd_ms, float* bwd_ms) {
   return ok;
 }
 
-cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cudaStream_t stream,
-                        int* launches) {
+static PlanPtrs plan_ptrs(const pp_plan* plan) {
   PlanPtrs p;
   char* ws = plan->ws;
   const PlanLayout& l = plan->lay;
@@ -1150,8 +1139,9 @@ cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cu
   p.tile_gwork = reinterpret_cast<int32_t*>(ws + l.tile_gwork);
   p.tile_sgroup = reinterpret_cast<int32_t*>(ws + l.tile_sgroup);
   p.tile_sblock = reinterpret_cast<int32_t*>(ws + l.tile_sblock);
-  p.bwd_units = reinterpret_cast<int32_t*>(ws + l.bwd_units);
-  p.bwd_sched = bwd_takes_sched(plan->prob) ? reinterpret_cast<int32_t*>(ws + l.bwd_sched) : nullptr;
+  const bool sched = bwd_takes_sched(plan->prob);
+  p.bwd_units = sched ? nullptr : reinterpret_cast<int32_t*>(ws + l.bwd_units);
+  p.bwd_sched = sched ? reinterpret_cast<int32_t*>(ws + l.bwd_sched) : nullptr;
   p.bwd_units_det = reinterpret_cast<int32_t*>(ws + l.bwd_units_det);
   p.Hkv = plan->prob.num_kv_heads;
   p.key_end = reinterpret_cast<int32_t*>(ws + l.key_end);
@@ -1159,18 +1149,37 @@ cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cu
   p.qorder = reinterpret_cast<int32_t*>(ws + l.qorder);
   p.work_at = p.bwd_units_det;
   p.grid_gain = reinterpret_cast<long long*>(ws + l.grid_gain);
-  // a third of the SMs (the backward runs one CTA per SM), at most 48 tiles = 6144 tokens
-  static DeviceSetup setup[kMaxDevices];
-  DeviceSetup* dev = device_setup(setup);
-  if (!dev) return cudaErrorInvalidDevice;
-  // (a set of the backward is held up with all its parts)
-  p.det_asc_max = std::min(48, dev->num_sms / 3) >> plan->lg_split;
+  p.det_asc_max = 0;
   p.num_rows = plan->prob.num_rows;
   p.G = plan->prob.num_groups;
   p.N = plan->prob.num_responses;
   p.T = plan->prob.total_tokens;
   p.nseg = plan->nseg;
   p.max_tiles = plan->max_tiles;
+  return p;
+}
+
+cudaError_t launch_base_units(const pp_plan* plan, cudaStream_t stream) {
+  PlanPtrs p = plan_ptrs(plan);
+  p.bwd_units = reinterpret_cast<int32_t*>(plan->ws + plan->lay.bwd_units);
+  p.bwd_sched = p.bwd_units_det = nullptr;
+  p.qtiles = nullptr;
+  const int blocks = (p.max_tiles + 127) / 128;
+  plan_gwork_kernel<<<blocks, 128, 0, stream>>>(p);
+  plan_sgroup_kernel<<<blocks, 128, 0, stream>>>(p);
+  plan_units_kernel<<<blocks, 128, 0, stream>>>(p);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cudaStream_t stream,
+                        int* launches) {
+  PlanPtrs p = plan_ptrs(plan);
+  // a third of the SMs (the backward runs one CTA per SM), at most 48 tiles = 6144 tokens
+  static DeviceSetup setup[kMaxDevices];
+  DeviceSetup* dev = device_setup(setup);
+  if (!dev) return cudaErrorInvalidDevice;
+  // (a set of the backward is held up with all its parts)
+  p.det_asc_max = std::min(48, dev->num_sms / 3) >> plan->lg_split;
 
   const int mt = plan->max_tiles;
   // Host descriptors: up to kDescLarge entries travel as a kernel argument, which keeps the call

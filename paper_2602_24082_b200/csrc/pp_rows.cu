@@ -6,7 +6,11 @@
 // the order, the rows, each row's tokens and visible query-key pairs (the attention cost of
 // Sec. 3.2.1, for balancing data-parallel ranks) and the descriptor arrays in row order, ready
 // for pp_build_plan with descriptors on the device.  Integer work only; microseconds.
+#include <algorithm>
+#include <type_traits>
+
 #include "pp_internal.h"
+#include "pp_ptx.cuh"
 
 namespace pp {
 namespace {
@@ -18,10 +22,12 @@ struct RowsPtrs {
   const int32_t* prompt_len;
   const int32_t* resp_off;
   const int32_t* resp_len;
-  int32_t* tok;      // [G] tokens per group, saturated (a group above the capacity is an error)
+  int2* tok;         // [G] tokens (negative: why the group is refused, kTokBad or kTokTooLong) and responses
+                     //   per group; in the space of nxt and jump_a
   long long* cost;   // [G] visible pairs per group
-  long long* pre;    // [G] inclusive prefix sums of the sorted groups' tokens
-  long long* pre_cost;  // [G] ... and of their visible pairs
+  // in sorted order:
+  long long* pre;    // [G] tokens, then (where they do not fit shared memory) their inclusive prefix sums
+  long long* pre_cost;  // [G] ... and visible pairs
   int32_t* nxt;      // [G] end of the row that would start at each sorted position
   int32_t* jump_a;   // [G] pointer-doubling buffers, used when they do not fit shared memory
   int32_t* jump_b;   // [G]
@@ -37,32 +43,30 @@ struct RowsPtrs {
   int32_t* status;   // [2]: code, detail
 };
 
-__device__ __forceinline__ void rows_fail(int32_t* status, int32_t code, int32_t detail) {
-  if (atomicCAS(&status[0], kRowsOk, code) == kRowsOk) status[1] = detail;
-}
+constexpr int32_t kTokBad = -1, kTokTooLong = -2;
 
 // tokens and visible pairs of every group: P (P + 1) / 2 for the causal prompt, and
 // R P + R (R + 1) / 2 for a response that sees the whole prompt and itself causally
 __global__ void rows_measure_kernel(RowsPtrs p) {
+  launch_dependents();
+  dependency_wait();
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= p.G) return;
   const long long P = p.prompt_len[g];
   const int x0 = p.resp_off[g], x1 = p.resp_off[g + 1];
-  if (P < 1 || x1 <= x0 || x0 < 0 || x1 > p.N) {
-    rows_fail(p.status, kRowsBadGroup, g);
-    p.tok[g] = 0;
-    p.cost[g] = 0;
-    return;
-  }
+  bool ok = !(P < 1 || x1 <= x0 || x0 < 0 || x1 > p.N);
   long long t = P, u = P * (P + 1) / 2;
-  for (int x = x0; x < x1; ++x) {
-    const long long R = p.resp_len[x];
-    if (R < 1) rows_fail(p.status, kRowsBadGroup, g);
-    t += R;
-    u += R * P + R * (R + 1) / 2;
+  if (ok) {
+#pragma unroll 4
+    for (int x = x0; x < x1; ++x) {
+      const long long R = p.resp_len[x];
+      ok = ok && R >= 1;
+      t += R;
+      u += R * P + R * (R + 1) / 2;
+    }
   }
-  if (t > p.capacity) rows_fail(p.status, kRowsTooLong, g);
-  p.tok[g] = int32_t(t < 0x7fffffff ? t : 0x7fffffff);
+  const int32_t tok = !ok ? kTokBad : t > p.capacity ? kTokTooLong : int32_t(t);
+  p.tok[g] = make_int2(tok, tok > 0 ? x1 - x0 : 0);
   p.cost[g] = u;
 }
 
@@ -70,197 +74,282 @@ __global__ void rows_measure_kernel(RowsPtrs p) {
 // is quadratic, so what matters is to spread it: a block ranks 32 keys, each of its 32 warps
 // counts a slice of every staged chunk (all lanes read the same key: broadcast reads), and the
 // partial counts are added at the end.  (One thread per key and 256 keys per block left 132 SMs
-// idle: 72 us for 4096 groups, now 7.)
+// idle: 72 us for 4096 groups, now 7.)  For groups the responses before each are counted along, and the
+// group goes to its place here, on many SMs: one block that gathered it in sorted order was bound by its
+// SM's memory pipe.
 constexpr int kRankKeys = 32, kRankSlices = 32, kRankChunk = 2048;
+__device__ __forceinline__ long long key_of(long long k) { return k; }
+__device__ __forceinline__ int32_t key_of(int2 k) { return k.x; }
+// what a key before mine adds: 1, and in the upper half its responses
+__device__ __forceinline__ int32_t weight_of(long long) { return 1; }
+__device__ __forceinline__ long long weight_of(int2 k) { return static_cast<long long>(k.y) << 32 | 1; }
 
-template <typename Key>
+template <typename Item>
 __global__ void __launch_bounds__(kRankKeys * kRankSlices)
-rank_kernel(int n, const Key* __restrict__ keys, int32_t* __restrict__ order) {
-  __shared__ Key s_key[kRankChunk];
-  __shared__ int32_t s_count[kRankSlices][kRankKeys];
+rank_kernel(int n, const Item* __restrict__ items, int32_t* __restrict__ order, RowsPtrs p) {
+  constexpr bool kGroups = sizeof(Item) == sizeof(int2) && !std::is_same_v<Item, long long>;
+  using Key = decltype(key_of(Item{}));
+  using Sum = decltype(weight_of(Item{}));
+  __shared__ Item s_item[kRankChunk];
+  __shared__ Sum s_sum[kRankSlices][kRankKeys];
+  __shared__ int3 s_copy[kRankKeys];   // first response, number of them, where they go
+  launch_dependents();
+  dependency_wait();
   const int tid = threadIdx.x, item = tid % kRankKeys, slice = tid / kRankKeys;
   const int first = blockIdx.x * kRankKeys, g = first + item;
-  const Key mine = g < n ? keys[g] : 0;
-  int count = 0;
+  const bool emits = tid < kRankKeys && g < n;
+  const Key mine = g < n ? key_of(items[g]) : Key(0);
+  int32_t prompt = 0, x0 = 0, n_resp = 0;
+  long long cost = 0;
+  if (kGroups && emits) {
+    prompt = p.prompt_len[g];
+    x0 = p.resp_off[g];
+    n_resp = p.tok[g].y;
+    cost = p.cost[g];
+  }
+  Sum sum = 0;
   for (int base = 0; base < n; base += kRankChunk) {
     const int here = min(kRankChunk, n - base);
-    for (int i = tid; i < here; i += kRankKeys * kRankSlices) s_key[i] = keys[base + i];
+    for (int i = tid; i < here; i += kRankKeys * kRankSlices) s_item[i] = items[base + i];
     __syncthreads();
     constexpr int kPer = kRankChunk / kRankSlices;
     const int lo = slice * kPer, hi = min(lo + kPer, here);
     if (base + hi <= first) {          // slices before or behind my block's keys: one comparison
 #pragma unroll 16
-      for (int i = lo; i < hi; ++i) count += s_key[i] >= mine;
+      for (int i = lo; i < hi; ++i) sum += key_of(s_item[i]) >= mine ? weight_of(s_item[i]) : 0;
     } else if (base + lo >= first + kRankKeys) {
 #pragma unroll 16
-      for (int i = lo; i < hi; ++i) count += s_key[i] > mine;
+      for (int i = lo; i < hi; ++i) sum += key_of(s_item[i]) > mine ? weight_of(s_item[i]) : 0;
     } else {
-      for (int i = lo; i < hi; ++i) count += s_key[i] > mine || (s_key[i] == mine && base + i < g);
+      for (int i = lo; i < hi; ++i)
+        sum += key_of(s_item[i]) > mine || (key_of(s_item[i]) == mine && base + i < g) ? weight_of(s_item[i]) : 0;
     }
     __syncthreads();
   }
-  s_count[slice][item] = count;
+  s_sum[slice][item] = sum;
+  if (kGroups && tid < kRankKeys) s_copy[tid] = make_int3(0, 0, 0);
   __syncthreads();
-  if (tid < kRankKeys && g < n) {
-    int rank = 0;
+  if (emits) {
+    Sum before = 0;
 #pragma unroll
-    for (int k = 0; k < kRankSlices; ++k) rank += s_count[k][tid];
+    for (int k = 0; k < kRankSlices; ++k) before += s_sum[k][tid];
+    const int rank = int(before & 0xffffffff);
     order[rank] = g;
+    if constexpr (kGroups) {
+      const int y0 = int(before >> 32);
+      p.pre[rank] = mine;
+      p.pre_cost[rank] = cost;
+      p.out_prompt_len[rank] = prompt;
+      p.out_resp_off[rank] = y0;
+      if (rank == n - 1) p.out_resp_off[n] = y0 + n_resp;
+      // (only with a refused group elsewhere can the sum of the others go beyond N)
+      s_copy[tid] = make_int3(x0, y0 >= 0 ? max(min(n_resp, p.N - y0), 0) : 0, y0);
+    }
+  }
+  if constexpr (kGroups) {
+    __syncthreads();
+    const int3 c = s_copy[slice];   // a warp per group
+    for (int x = item; x < c.y; x += 32) p.out_resp_len[c.z + x] = p.resp_len[c.x + x];
   }
 }
 
-// Inclusive block-wide sums of three values per thread (two barriers).
-struct Sum3 {
-  long long a, b;
-  int32_t c;
+// Inclusive block-wide sums of one or two values per thread of a block of 1024 (two barriers).
+template <int kN>
+struct Sums {
+  long long v[kN];
 };
-__device__ __forceinline__ Sum3 block_scan(Sum3 v, Sum3* s_warp) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+template <int kN>
+__device__ __forceinline__ Sums<kN> warp_scan(Sums<kN> s) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
-    const long long a = __shfl_up_sync(0xffffffffu, v.a, d), b = __shfl_up_sync(0xffffffffu, v.b, d);
-    const int32_t c = __shfl_up_sync(0xffffffffu, v.c, d);
-    if (lane >= d) {
-      v.a += a;
-      v.b += b;
-      v.c += c;
-    }
-  }
-  if (lane == 31) s_warp[warp] = v;
-  __syncthreads();
-  if (warp == 0) {   // the block has 32 warps
-    Sum3 w = s_warp[lane];
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const long long a = __shfl_up_sync(0xffffffffu, w.a, d), b = __shfl_up_sync(0xffffffffu, w.b, d);
-      const int32_t c = __shfl_up_sync(0xffffffffu, w.c, d);
-      if (lane >= d) {
-        w.a += a;
-        w.b += b;
-        w.c += c;
-      }
+    for (int a = 0; a < kN; ++a) {
+      const long long x = __shfl_up_sync(0xffffffffu, s.v[a], d);
+      if (lane >= d) s.v[a] += x;
     }
-    s_warp[lane] = w;
   }
+  return s;
+}
+// `all` receives the block's totals.
+template <int kN>
+__device__ __forceinline__ Sums<kN> block_scan(Sums<kN> s, Sums<kN>* s_warp, Sums<kN>& all) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  s = warp_scan(s);
+  __syncthreads();   // (s_warp may still be read from the scan before)
+  if (lane == 31) s_warp[warp] = s;
   __syncthreads();
-  if (warp) {
-    v.a += s_warp[warp - 1].a;
-    v.b += s_warp[warp - 1].b;
-    v.c += s_warp[warp - 1].c;
+  const Sums<kN> w = warp_scan(s_warp[lane]);   // every warp for itself
+#pragma unroll
+  for (int a = 0; a < kN; ++a) {
+    const long long before = __shfl_sync(0xffffffffu, w.v[a], warp ? warp - 1 : 0);
+    if (warp) s.v[a] += before;
+    all.v[a] = __shfl_sync(0xffffffffu, w.v[a], 31);
   }
-  return v;
+  return s;
 }
 
-// One block: prefix sums over the sorted groups, next-fit rows, row costs, reordered
-// descriptors.  It is all latency, so dependent loads are issued for several groups at once and
-// whatever is searched or chased -- the token sums, the pointer-doubling tables -- lives in
-// shared memory up to kPackSmemGroups groups (20 bytes each).  4096 groups: 47 us with the tables
-// in global memory and shared-memory scans of ten rounds per 1024 groups, now 38.
+// One block: prefix sums over the sorted groups, next-fit rows, row costs.  Bound by what one SM's
+// shared-memory pipe and barriers allow, so the sums come from kPer consecutive positions per thread, read as
+// vectors and scanned once for 1024 kPer of them; searches and jumps take neighbouring positions in
+// neighbouring lanes, kPer of them side by side; and up to kPackSmemGroups groups all that is
+// searched or chased lives in shared memory (28 bytes each).  4096 groups: @PACK@.
 constexpr int kPackSmemGroups = 8192;
+constexpr size_t pack_smem(int G) { return size_t(16) * ((G + 1) & ~1) + size_t(12) * G; }
 
-__global__ void __launch_bounds__(1024) rows_pack_kernel(RowsPtrs p, int tables_in_smem) {
-  extern __shared__ long long s_tables[];
-  __shared__ Sum3 s_warp[32];
-  __shared__ Sum3 s_total;
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  if (p.status[0] != kRowsOk) {
-    if (tid == 0) *p.num_rows = 0;
+template <int kPer, bool kSmem>
+__global__ void __launch_bounds__(1024) rows_pack_kernel(RowsPtrs p) {
+  extern __shared__ __align__(16) long long s_tables[];
+  __shared__ Sums<2> s_warp[32];
+  __shared__ Sums<1> s_warp1[32];
+  __shared__ int32_t s_bad;
+  const int tid = threadIdx.x, G = p.G;
+  constexpr int kThreads = 1024, kChunk = kThreads * kPer;
+  const int Gp = (G + 1) & ~1;   // (tables begin on 16 bytes)
+  long long* pre = kSmem ? s_tables : p.pre;
+  long long* pre_cost = kSmem ? s_tables + Gp : p.pre_cost;
+  int32_t* s_int = reinterpret_cast<int32_t*>(s_tables + 2 * Gp);
+  int32_t* ja = kSmem ? s_int : p.jump_a;
+  int32_t* jb = kSmem ? s_int + G : p.jump_b;
+  int32_t* mark = kSmem ? s_int + 2 * G : p.mark;
+  if (tid == 0) s_bad = 0x7fffffff;
+  launch_dependents();
+  dependency_wait();
+  // (refused groups have negative tokens and stand last)
+  if (p.pre[G - 1] < 0) {
+    __syncthreads();
+    for (int g = tid; g < G; g += kThreads)
+      if (p.tok[g].x < 0) atomicMin(&s_bad, g);
+    __syncthreads();
+    if (tid == 0) {
+      p.status[0] = p.tok[s_bad].x == kTokBad ? kRowsBadGroup : kRowsTooLong;
+      p.status[1] = s_bad;
+      *p.num_rows = 0;
+    }
     return;
   }
-  long long* pre = tables_in_smem ? s_tables : p.pre;
-  int32_t* s_int = reinterpret_cast<int32_t*>(s_tables + p.G);
-  int32_t* ja = tables_in_smem ? s_int : p.jump_a;
-  int32_t* jb = tables_in_smem ? s_int + p.G : p.jump_b;
-  int32_t* mark = tables_in_smem ? s_int + 2 * p.G : p.mark;
-  // tokens, pairs and response counts in sorted order
-#pragma unroll 4
-  for (int i = tid; i < p.G; i += nthr) {
-    const int g = p.order[i];
-    pre[i] = p.tok[g];
-    p.pre_cost[i] = p.cost[g];
-    p.out_prompt_len[i] = p.prompt_len[g];
-    const int x0 = p.resp_off[g];
-    ja[i] = x0;
-    jb[i] = p.resp_off[g + 1] - x0;
-  }
-  // inclusive scans of tokens and pairs and exclusive scan of response counts, in sorted order
-  // (every thread scans what it has gathered itself: no barrier in between)
-  Sum3 carry = {0, 0, 0};
-  for (int base = 0; base < p.G; base += nthr) {
-    const int i = base + tid;
-    Sum3 v = {0, 0, 0};
-    if (i < p.G) v = {pre[i], p.pre_cost[i], jb[i]};
-    const int32_t n_resp = v.c;
-    const Sum3 w = block_scan(v, s_warp);
-    if (i < p.G) {
-      pre[i] = carry.a + w.a;
-      p.pre_cost[i] = carry.b + w.b;
-      p.out_resp_off[i] = carry.c + w.c - n_resp;
+  // inclusive sums of tokens and pairs
+  Sums<2> carry = {};
+  for (int base = 0; base < G; base += kChunk) {
+    const int i0 = base + tid * kPer;
+    long long t[kPer], c[kPer];
+    if (kPer > 1 && i0 + kPer <= G) {
+#pragma unroll
+      for (int k = 0; k < kPer; k += 2) {
+        const longlong2 a = *reinterpret_cast<const longlong2*>(p.pre + i0 + k);
+        const longlong2 b = *reinterpret_cast<const longlong2*>(p.pre_cost + i0 + k);
+        t[k] = a.x;
+        t[k + 1] = a.y;
+        c[k] = b.x;
+        c[k + 1] = b.y;
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) {
+        t[k] = i0 + k < G ? p.pre[i0 + k] : 0;
+        c[k] = i0 + k < G ? p.pre_cost[i0 + k] : 0;
+      }
     }
-    if (tid == nthr - 1) s_total = w;
-    __syncthreads();
-    carry.a += s_total.a;
-    carry.b += s_total.b;
-    carry.c += s_total.c;
-  }
-  if (tid == 0) p.out_resp_off[p.G] = carry.c;
-  // the responses' lengths, four loads in flight per thread
-  for (int i = tid; i < p.G; i += nthr) {
-    const int x0 = ja[i], n = jb[i], y0 = p.out_resp_off[i];
-#pragma unroll 4
-    for (int x = 0; x < n; ++x) p.out_resp_len[y0 + x] = p.resp_len[x0 + x];
+#pragma unroll
+    for (int k = 1; k < kPer; ++k) {
+      t[k] += t[k - 1];
+      c[k] += c[k - 1];
+    }
+    Sums<2> all;
+    const Sums<2> w = block_scan<2>({t[kPer - 1], c[kPer - 1]}, s_warp, all);
+    const long long t0 = carry.v[0] + w.v[0] - t[kPer - 1], c0 = carry.v[1] + w.v[1] - c[kPer - 1];
+    if (kPer > 1 && i0 + kPer <= G) {
+#pragma unroll
+      for (int k = 0; k < kPer; k += 2) {
+        *reinterpret_cast<longlong2*>(pre + i0 + k) = make_longlong2(t0 + t[k], t0 + t[k + 1]);
+        *reinterpret_cast<longlong2*>(pre_cost + i0 + k) = make_longlong2(c0 + c[k], c0 + c[k + 1]);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < kPer; ++k)
+        if (i0 + k < G) {
+          pre[i0 + k] = t0 + t[k];
+          pre_cost[i0 + k] = c0 + c[k];
+        }
+    }
+    carry.v[0] += all.v[0];
+    carry.v[1] += all.v[1];
   }
   __syncthreads();
-  // Next fit in parallel.  nxt[s] = where the row that starts at sorted position s ends: the
-  // largest e whose tokens still fit (every group fits alone, so e > s).  The row starts are
-  // the positions reachable from 0 through nxt; they are marked by pointer doubling (after
+  // Next fit in parallel.  The row that starts at sorted position s ends at the largest e whose tokens
+  // still fit (every group fits alone, so e > s).  The row starts are
+  // the positions reachable from 0 that way; they are marked by pointer doubling (after
   // round r every start within 2^r hops is marked), then numbered by a prefix count.
-  for (int s = tid; s < p.G; s += nthr) {
-    const long long base = s ? pre[s - 1] : 0;
-    int lo = s + 1, hi = p.G;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (pre[mid - 1] - base <= p.capacity) lo = mid; else hi = mid - 1;
+  const int top = 1 << (31 - __clz(G));
+  for (int base = 0; base < G; base += kChunk) {
+    int at[kPer];
+    long long limit[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      at[k] = min(base + tid + kThreads * k, G);
+      limit[k] = (at[k] ? pre[at[k] - 1] : 0) + p.capacity;
     }
-    p.nxt[s] = lo;
-    ja[s] = lo;
-    mark[s] = (s == 0);
+    for (int w = top; w > 0; w >>= 1) {
+#pragma unroll
+      for (int k = 0; k < kPer; ++k)
+        if (at[k] + w <= G && pre[at[k] + w - 1] <= limit[k]) at[k] += w;
+    }
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int s = base + tid + kThreads * k;
+      if (s < G) {
+        p.nxt[s] = at[k];
+        ja[s] = at[k];
+        mark[s] = s == 0;
+      }
+    }
   }
-  for (int hop = 1; hop < p.G; hop <<= 1) {
-    __syncthreads();
-    for (int s = tid; s < p.G; s += nthr) {
-      const int to = ja[s];
-      jb[s] = to < p.G ? ja[to] : p.G;
+  __syncthreads();
+  // (marking runs along with the doubling: a mark set in this round by another thread only
+  // marks further positions that are reachable as well; once the doubled hop from 0 has left the
+  // list, all are marked)
+  for (bool last = false; !last;) {
+    last = ja[0] >= G;
+#pragma unroll 4
+    for (int s = tid; s < G; s += kThreads) {
+      const int to = ja[s], m = mark[s];
+      jb[s] = to < G ? ja[to] : G;
+      if (to < G && m) mark[to] = 1;
     }
-    // (marking runs along with the doubling: a mark set in this round by another thread only
-    // marks further positions that are reachable as well)
-    for (int s = tid; s < p.G; s += nthr)
-      if (mark[s] && ja[s] < p.G) mark[ja[s]] = 1;
     __syncthreads();
     int32_t* t = ja;
     ja = jb;
     jb = t;
   }
-  __syncthreads();
   // number the marked positions (exclusive scan of the marks) and emit the rows
   int32_t rows = 0;
-  for (int base = 0; base < p.G; base += nthr) {
-    const int i = base + tid;
-    const int32_t m = i < p.G ? mark[i] : 0;
-    const Sum3 w = block_scan({0, 0, m}, s_warp);
-    if (m) {
-      const int r = rows + w.c - 1, e = p.nxt[i] - 1;
-      p.row_group_off[r] = i;
-      p.row_tokens[r] = pre[e] - (i ? pre[i - 1] : 0);
-      p.row_cost[r] = p.pre_cost[e] - (i ? p.pre_cost[i - 1] : 0);
+  for (int base = 0; base < G; base += kChunk) {
+    const int i0 = base + tid * kPer;
+    int32_t m[kPer], mine = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      m[k] = i0 + k < G ? mark[i0 + k] : 0;
+      mine += m[k];
     }
-    if (tid == nthr - 1) s_total = w;
-    __syncthreads();
-    rows += s_total.c;
+    Sums<1> all;
+    const Sums<1> w = block_scan<1>({mine}, s_warp1, all);
+    int r = rows + int(w.v[0]) - mine;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k)
+      if (m[k]) {
+        const int i = i0 + k, e = p.nxt[i] - 1;
+        p.row_group_off[r] = i;
+        p.row_tokens[r] = pre[e] - (i ? pre[i - 1] : 0);
+        p.row_cost[r] = pre_cost[e] - (i ? pre_cost[i - 1] : 0);
+        ++r;
+      }
+    rows += int(all.v[0]);
   }
   if (tid == 0) {
-    p.row_group_off[rows] = p.G;
+    p.row_group_off[rows] = G;
     *p.num_rows = rows;
+    p.status[0] = kRowsOk;
+    p.status[1] = 0;
   }
 }
 
@@ -332,87 +421,108 @@ __device__ __forceinline__ void assign_one_by_one(int R, int ranks, const long l
   for (int j = 0; j < kPerLane; ++j)
     if (id[j] < ranks) rank_cost[id[j]] = load[j];
 }
-template <int kPerLane>
-__global__ void __launch_bounds__(32)
-assign_greedy_kernel(int R, int ranks, const long long* __restrict__ cost,
-                     const int32_t* __restrict__ order, int32_t* __restrict__ rank_of_row,
-                     long long* __restrict__ rank_cost) {
-  assign_one_by_one<kPerLane>(R, ranks, cost, order, rank_of_row, rank_cost);
-}
-
-// Up to 32 ranks: a round assigns as many rows as the sorted list of ranks allows at once.  Row i of
-// the round goes to rank i of the list while that rank is still before all the ranks that have got
+// Up to 128 ranks: a round assigns as many rows as the sorted order of the ranks allows at once.  Row i of
+// the round goes to the rank at place i while that rank is still before all the ranks that have got
 // a row in this round -- with loads closer together than a row's cost, as they soon are, that is
-// every rank.  Load and rank are one 64-bit word (for sums of costs below 2^58, else one row at a
-// time); the list is sorted again by counting, every lane comparing its word with the others', kN at
-// most, read from shared memory in one go.  Bound by that chain.
-// Building the rows of 4096 groups and dealing the 972 rows out to 8 ranks took 150 us with one row
-// at a time, now 126 (122 rounds instead of 972 steps).
+// every rank.  A thread keeps one rank, whose load and number are one 64-bit word (for sums of costs
+// below 2^56, else one row at a time); its place is the number of words before its own, all kN read from shared
+// memory side by side.  Bound by that chain, word -> place -> cost -> word.  972 rows: @GREEDY@.
 constexpr int kBatchRows = 1024, kBatchThreads = 256;
-template <int kN>
+template <int kN>   // ranks at most; a multiple of 32 threads work, one warp without barriers
 __global__ void __launch_bounds__(kBatchThreads)
 assign_batch_kernel(int R, int ranks, const long long* __restrict__ cost,
                     const int32_t* __restrict__ order, int32_t* __restrict__ rank_of_row,
                     long long* __restrict__ rank_cost) {
   using Key = unsigned long long;
+  constexpr int kWork = kN < 32 ? 32 : kN;
   __shared__ Key s_cost[kBatchRows];
   __shared__ int32_t s_row[kBatchRows];
-  __shared__ alignas(16) Key s_key[32];
-  __shared__ Key s_sorted[32];
-  const int tid = threadIdx.x, lane = tid & 31;
-  if (R > 0 && (cost[order[R - 1]] < 0 || cost[order[0]] >= (1LL << 58) / R)) {
-    if (tid < 32) assign_one_by_one<1>(R, ranks, cost, order, rank_of_row, rank_cost);
+  __shared__ alignas(16) Key s_key[kN];
+  __shared__ alignas(16) Key s_next[kN];
+  __shared__ int32_t s_count;
+  dependency_wait();
+  const int tid = threadIdx.x;
+  if (R > 0 && (cost[order[R - 1]] < 0 || cost[order[0]] >= (1LL << 56) / R)) {
+    if (tid < 32) assign_one_by_one<(kN + 31) / 32>(R, ranks, cost, order, rank_of_row, rank_cost);
     return;
   }
-  Key key = lane < ranks ? Key(lane) : ~Key(0);
+  auto sync = [&]() {
+    if constexpr (kWork == 32) __syncwarp(); else named_barrier_sync(1, kWork);
+  };
+  const bool mine = tid < ranks;
+  Key key = mine ? Key(tid) : ~Key(0);
   for (int base = 0; base < R; base += kBatchRows) {
     const int m = min(kBatchRows, R - base);
     __syncthreads();
     for (int i = tid; i < m; i += kBatchThreads) {
       s_row[i] = order[base + i];
-      s_cost[i] = Key(cost[s_row[i]]) << 5;
+      s_cost[i] = Key(cost[s_row[i]]) << 7;
     }
     __syncthreads();
-    if (tid >= 32) continue;
-    auto exchange = [&]() {   // the list sorted again: my place is the number of words before mine
-      __syncwarp();
-      s_key[lane] = key;
-      __syncwarp();
-      int before = 0;
-#pragma unroll
+    if (tid >= kWork) continue;
+    for (int pos = 0; pos < m;) {
+      if (tid < kN) s_key[tid] = key;
+      if (tid == 0) s_count = min(ranks, m - pos);
+      sync();
+      int place = 0;
+#pragma unroll 16
       for (int i = 0; i < kN; i += 2) {
         const ulonglong2 o = *reinterpret_cast<const ulonglong2*>(&s_key[i]);
-        before += int(o.x < key) + int(o.y < key);
+        place += int(o.x < key) + int(o.y < key);
       }
-      if (lane < ranks) s_sorted[before] = key;
-      __syncwarp();
-      if (lane < ranks) key = s_sorted[lane];
-    };
-    Key c = lane < m ? s_cost[lane] : 0;
-    for (int pos = 0; pos < m;) {
-      const bool there = lane < ranks && pos + lane < m;
-      const Key next = key + c, last = __shfl_sync(0xffffffffu, key, ranks - 1);
-      int count = ranks;
-      // every rank is in time if the last one is before all that have got a row
-      if (!__all_sync(0xffffffffu, lane >= ranks || (there && next > last))) {
-        __syncwarp();
-        s_key[lane] = there ? next : ~Key(0);
-        __syncwarp();
-        bool in_time = there;
-        for (int i = 0; i < ranks - 1; ++i) in_time = in_time && (i >= lane || key < s_key[i]);
-        const uint32_t fits = __ballot_sync(0xffffffffu, in_time);
-        count = fits == 0xffffffffu ? 32 : __ffs(~fits) - 1;   // (the first row always fits)
+      const bool there = mine && pos + place < m;
+      const Key next = there ? key + s_cost[pos + place] : key;
+      // every rank is in time if all that get a row end up behind the last one
+      bool all_in_time = false;
+      if constexpr (kWork == 32) {
+        const int last = __ffs(__ballot_sync(0xffffffffu, mine && place == ranks - 1)) - 1;
+        const Key last_key = __shfl_sync(0xffffffffu, key, last);
+        all_in_time = __all_sync(0xffffffffu, !there || next > last_key);
       }
-      if (lane < count) {
-        rank_of_row[s_row[pos + lane]] = int(key & 31u);
+      int count = min(ranks, m - pos);
+      if (!all_in_time) {
+        if (mine) s_next[place] = there ? next : ~Key(0);
+        sync();
+        Key least = ~Key(0);   // of the ranks that get a row before this one
+#pragma unroll 16
+        for (int i = 0; i < kN; i += 2) {
+          const ulonglong2 o = *reinterpret_cast<const ulonglong2*>(&s_next[i]);
+          if (i < place && o.x < least) least = o.x;
+          if (i + 1 < place && o.y < least) least = o.y;
+        }
+        if (there && key > least) atomicMin(&s_count, place);
+        sync();
+        count = s_count;
+      }
+      if (there && place < count) {
+        rank_of_row[s_row[pos + place]] = tid;
         key = next;
       }
       pos += count;
-      c = pos + lane < m ? s_cost[pos + lane] : 0;
-      exchange();
+      sync();
     }
   }
-  if (tid < ranks) rank_cost[key & 31u] = static_cast<long long>(key >> 5);
+  if (mine) rank_cost[tid] = static_cast<long long>(key >> 7);
+}
+
+// One rank: all rows and their sum.
+__global__ void __launch_bounds__(1024)
+assign_single_kernel(int R, const long long* __restrict__ cost, int32_t* __restrict__ rank_of_row,
+                     long long* __restrict__ rank_cost) {
+  __shared__ unsigned long long s_sum;
+  if (threadIdx.x == 0) s_sum = 0;
+  dependency_wait();
+  __syncthreads();
+  unsigned long long sum = 0;
+  for (int i = threadIdx.x; i < R; i += blockDim.x) {
+    sum += static_cast<unsigned long long>(cost[i]);
+    rank_of_row[i] = 0;
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+  if ((threadIdx.x & 31) == 0) atomicAdd(&s_sum, sum);
+  __syncthreads();
+  if (threadIdx.x == 0) *rank_cost = static_cast<long long>(s_sum);
 }
 
 // More ranks than the lanes' registers hold: the loads in shared memory, the lanes sharing the
@@ -422,6 +532,7 @@ assign_greedy_smem_kernel(int R, int ranks, const long long* __restrict__ cost,
                           const int32_t* __restrict__ order, int32_t* __restrict__ rank_of_row,
                           long long* __restrict__ rank_cost) {
   __shared__ long long s_load[kMaxAssignRanks];
+  dependency_wait();
   const int lane = threadIdx.x;
   for (int k = lane; k < ranks; k += 32) s_load[k] = 0;
   __syncwarp();
@@ -459,16 +570,23 @@ assign_greedy_smem_kernel(int R, int ranks, const long long* __restrict__ cost,
 cudaError_t launch_assign_rows(int R, const long long* row_cost, int ranks, int32_t* order,
                                int32_t* rank_of_row, long long* rank_cost, cudaStream_t stream,
                                int* launches) {
-  rank_kernel<long long><<<(R + kRankKeys - 1) / kRankKeys, kRankKeys * kRankSlices, 0, stream>>>(
-      R, row_cost, order);
-  auto greedy = ranks <= 8     ? assign_batch_kernel<8>
-                : ranks <= 32  ? assign_batch_kernel<32>
-                : ranks <= 64  ? assign_greedy_kernel<2>
-                : ranks <= 128 ? assign_greedy_kernel<4>
-                               : assign_greedy_smem_kernel;
-  greedy<<<1, ranks <= 32 ? kBatchThreads : 32, 0, stream>>>(R, ranks, row_cost, order, rank_of_row, rank_cost);
+  const unsigned blocks = unsigned((R + kRankKeys - 1) / kRankKeys);
+  cudaError_t e = launch_kernel(true, rank_kernel<long long>, dim3(blocks), dim3(kRankKeys * kRankSlices), 0,
+                                stream, R, row_cost, order, RowsPtrs{});
+  if (e != cudaSuccess) return e;
+  if (ranks == 1) {
+    e = launch_kernel(true, assign_single_kernel, dim3(1), dim3(1024), 0, stream, R, row_cost, rank_of_row, rank_cost);
+  } else {
+    auto greedy = ranks <= 8     ? assign_batch_kernel<8>
+                  : ranks <= 32  ? assign_batch_kernel<32>
+                  : ranks <= 64  ? assign_batch_kernel<64>
+                  : ranks <= 128 ? assign_batch_kernel<128>
+                                 : assign_greedy_smem_kernel;
+    e = launch_kernel(true, greedy, dim3(1), dim3(ranks <= 128 ? kBatchThreads : 32), 0, stream, R, ranks, row_cost,
+                      order, rank_of_row, rank_cost);
+  }
   if (launches) *launches = 2;
-  return cudaGetLastError();
+  return e;
 }
 
 size_t rows_workspace_bytes(int G) {
@@ -498,7 +616,7 @@ cudaError_t launch_build_rows(int G, int N, const int32_t* prompt_len, const int
   p.jump_a = reinterpret_cast<int32_t*>(w + 3 * a8 + a4);
   p.jump_b = reinterpret_cast<int32_t*>(w + 3 * a8 + 2 * a4);
   p.mark = reinterpret_cast<int32_t*>(w + 3 * a8 + 3 * a4);
-  p.tok = reinterpret_cast<int32_t*>(w + 3 * a8 + 4 * a4);
+  p.tok = reinterpret_cast<int2*>(w + 3 * a8);
   p.order = order;
   p.row_group_off = row_group_off;
   p.num_rows = num_rows;
@@ -508,25 +626,33 @@ cudaError_t launch_build_rows(int G, int N, const int32_t* prompt_len, const int
   p.out_resp_off = out_resp_off;
   p.out_resp_len = out_resp_len;
   p.status = status;
-  cudaError_t e = cudaMemsetAsync(status, 0, 8, stream);
-  if (e != cudaSuccess) return e;
-  rows_measure_kernel<<<(G + 255) / 256, 256, 0, stream>>>(p);
-  rank_kernel<int32_t><<<(G + kRankKeys - 1) / kRankKeys, kRankKeys * kRankSlices, 0, stream>>>(
-      G, p.tok, order);
   // per device: the opt-in to more than 48 KB of dynamic shared memory
   static DeviceSetup setup[kMaxDevices];
   DeviceSetup* dev = device_setup(setup);
   if (!dev) return cudaErrorInvalidDevice;
+  cudaError_t e = cudaSuccess;
   if (!dev->configured) {
-    e = cudaFuncSetAttribute(rows_pack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             20 * kPackSmemGroups);
-    if (e != cudaSuccess) return e;
+    for (auto kern : {rows_pack_kernel<1, true>, rows_pack_kernel<2, true>, rows_pack_kernel<4, true>,
+                      rows_pack_kernel<8, true>}) {
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               int(pack_smem(kPackSmemGroups)));
+      if (e != cudaSuccess) return e;
+    }
     dev->configured = true;
   }
-  const bool in_smem = G <= kPackSmemGroups;
-  rows_pack_kernel<<<1, 1024, in_smem ? size_t(20) * G : 0, stream>>>(p, in_smem);
+  e = launch_kernel(true, rows_measure_kernel, dim3((G + 255) / 256), dim3(256), 0, stream, p);
+  if (e == cudaSuccess)
+    e = launch_kernel(true, rank_kernel<int2>, dim3((G + kRankKeys - 1) / kRankKeys),
+                      dim3(kRankKeys * kRankSlices), 0, stream, G, p.tok, order, p);
+  auto pack = G <= 1024            ? rows_pack_kernel<1, true>
+              : G <= 2048            ? rows_pack_kernel<2, true>
+              : G <= 4096            ? rows_pack_kernel<4, true>
+              : G <= kPackSmemGroups ? rows_pack_kernel<8, true>
+                                     : rows_pack_kernel<8, false>;
+  if (e == cudaSuccess)
+    e = launch_kernel(true, pack, dim3(1), dim3(1024), G <= kPackSmemGroups ? pack_smem(G) : 0, stream, p);
   if (launches) *launches = 3;
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace pp

@@ -1,13 +1,15 @@
-// The calls of a training step as CPython functions on torch tensors: argument checks, output
+// The calls of a training step, and the row builder's, as CPython functions on torch tensors: argument checks, output
 // allocation, current device and stream, and the C ABI call, without interpreter code or ctypes
 // in between.  On small steps the host is what a call costs (a 144-token step has 28 us of
 // kernels): plan, forward and backward took 12.6, 11.1 and 18.7 us through ctypes, of which 4.8,
-// 3.7 and 10.1 were the library's own; now 4.4, 5.2 and 12.5.
+// 3.7 and 10.1 were the library's own; now 4.4, 5.2 and 12.5.  Building and dealing out the rows of 4096 groups
+// @ROWHOST@.
 // Only marshalling lives here; everything is computed by libpp_attn.so, whose entry points are
 // looked up once (bind).  Anything unusual -- a tensor that fails a check, descriptors that are not
 // contiguous int32 arrays, an error code -- goes back to the Python side, which raises.
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
+#include <cuda_runtime_api.h>
 #include <dlfcn.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <torch/types.h>
@@ -20,6 +22,9 @@ struct Api {
   decltype(&pp_build_plan) build_plan = nullptr;
   decltype(&pp_attn_fwd) fwd = nullptr;
   decltype(&pp_attn_bwd) bwd = nullptr, bwd_det = nullptr;
+  decltype(&pp_build_rows_workspace_bytes) rows_bytes = nullptr;
+  decltype(&pp_build_rows) build_rows = nullptr;
+  decltype(&pp_assign_rows) assign_rows = nullptr;
 } api;
 PyObject* g_error = nullptr;  // PPError(code, where)
 PyObject* g_chk = nullptr;    // _chk(tensor, shape, dtype, name): raises what is wrong with it
@@ -105,7 +110,10 @@ PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
   x.fwd = reinterpret_cast<decltype(x.fwd)>(dlsym(lib, "pp_attn_fwd"));
   x.bwd = reinterpret_cast<decltype(x.bwd)>(dlsym(lib, "pp_attn_bwd"));
   x.bwd_det = reinterpret_cast<decltype(x.bwd_det)>(dlsym(lib, "pp_attn_bwd_deterministic"));
-  if (!x.build_plan || !x.fwd || !x.bwd || !x.bwd_det) {
+  x.rows_bytes = reinterpret_cast<decltype(x.rows_bytes)>(dlsym(lib, "pp_build_rows_workspace_bytes"));
+  x.build_rows = reinterpret_cast<decltype(x.build_rows)>(dlsym(lib, "pp_build_rows"));
+  x.assign_rows = reinterpret_cast<decltype(x.assign_rows)>(dlsym(lib, "pp_assign_rows"));
+  if (!x.build_plan || !x.fwd || !x.bwd || !x.bwd_det || !x.rows_bytes || !x.build_rows || !x.assign_rows) {
     PyErr_SetString(PyExc_RuntimeError, "libpp_attn.so lacks an entry point");
     return nullptr;
   }
@@ -283,8 +291,89 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   PP_GUARD_END
 }
 
+// build_rows(prompt_len, resp_off, resp_len, groups, responses, capacity) -> dict
+PyObject* build_rows(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  if (!nargs(n, 6, "build_rows")) return nullptr;
+  PP_GUARD_BEGIN
+  const int64_t G = PyLong_AsLongLong(a[3]), N = PyLong_AsLongLong(a[4]), capacity = PyLong_AsLongLong(a[5]);
+  if (PyErr_Occurred()) return nullptr;
+  const int64_t gs[1] = {G}, os[1] = {G + 1}, ns[1] = {N};
+  const at::Tensor *P, *off, *R;
+  if (!(P = take(a[0], at::kInt, "int32", gs, "grp_prompt_len")) ||
+      !(off = take(a[1], at::kInt, "int32", os, "grp_resp_off")) || !(R = take(a[2], at::kInt, "int32", ns, "resp_len")))
+    return nullptr;
+  size_t bytes = 0;
+  if (const int rc = api.rows_bytes(int32_t(G), &bytes)) return raise_code(rc, "pp_build_rows_workspace_bytes");
+  const c10::cuda::CUDAGuard guard(P->device());
+  const auto i32 = P->options(), i64 = P->options().dtype(at::kLong);
+  const at::Tensor ws = at::empty({int64_t(bytes)}, P->options().dtype(at::kByte));
+  const at::Tensor order = at::empty({G}, i32), rgo = at::empty({G + 1}, i32), rtok = at::empty({G}, i64),
+                   rcost = at::empty({G}, i64), op = at::empty({G}, i32), ooff = at::empty({G + 1}, i32),
+                   orl = at::empty({N}, i32);
+  // status code, detail and number of rows: written by the kernel to page-locked memory, which is read
+  // behind the synchronisation that the number of rows needs anyway, without a copy
+  const at::Tensor meta = at::empty({3}, at::TensorOptions().dtype(at::kInt).pinned_memory(true));
+  const volatile int32_t* m = meta.data_ptr<int32_t>();
+  void* dm = nullptr;
+  if (cudaHostGetDevicePointer(&dm, meta.data_ptr(), 0) != cudaSuccess) {
+    PyErr_SetString(PyExc_RuntimeError, "page-locked memory is not mapped into the device");
+    return nullptr;
+  }
+  const c10::cuda::CUDAStream stream = c10::cuda::getCurrentCUDAStream(P->get_device());
+  int32_t* meta_dev = static_cast<int32_t*>(dm);
+  int rc;
+  cudaError_t e = cudaSuccess;
+  const int32_t *pp = P->data_ptr<int32_t>(), *po = off->data_ptr<int32_t>(), *pr = R->data_ptr<int32_t>();
+  Py_BEGIN_ALLOW_THREADS
+  rc = api.build_rows(int32_t(G), int32_t(N), pp, po, pr, int32_t(capacity), ws.data_ptr(), bytes,
+                      order.data_ptr<int32_t>(), rgo.data_ptr<int32_t>(), meta_dev + 2, rtok.data_ptr<int64_t>(),
+                      rcost.data_ptr<int64_t>(), op.data_ptr<int32_t>(), ooff.data_ptr<int32_t>(),
+                      orl.data_ptr<int32_t>(), meta_dev, reinterpret_cast<pp_stream_t>(stream.stream()));
+  if (rc == PP_OK) e = cudaStreamSynchronize(stream.stream());
+  Py_END_ALLOW_THREADS
+  if (rc) return raise_code(rc, "pp_build_rows");
+  if (e != cudaSuccess) {
+    PyErr_SetString(PyExc_RuntimeError, cudaGetErrorString(e));
+    return nullptr;
+  }
+  const int64_t rows = m[2];
+  const int code = m[0], detail = m[1];
+  return Py_BuildValue("{sNsNsNsNsNsNsNs(ii)}", "order", THPVariable_Wrap(order), "row_group_off",
+                       THPVariable_Wrap(rgo.narrow(0, 0, rows + 1)), "row_tokens",
+                       THPVariable_Wrap(rtok.narrow(0, 0, rows)), "row_cost",
+                       THPVariable_Wrap(rcost.narrow(0, 0, rows)), "grp_prompt_len", THPVariable_Wrap(op),
+                       "grp_resp_off", THPVariable_Wrap(ooff), "resp_len", THPVariable_Wrap(orl), "status", code, detail);
+  PP_GUARD_END
+}
+
+// assign_rows(row_cost, rows, ranks) -> (order, rank_of_row, rank_cost)
+PyObject* assign_rows(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  if (!nargs(n, 3, "assign_rows")) return nullptr;
+  PP_GUARD_BEGIN
+  const int64_t R = PyLong_AsLongLong(a[1]), ranks = PyLong_AsLongLong(a[2]);
+  if (PyErr_Occurred()) return nullptr;
+  const int64_t rs[1] = {R};
+  const at::Tensor* cost = take(a[0], at::kLong, "int64", rs, "row_cost");
+  if (!cost) return nullptr;
+  const c10::cuda::CUDAGuard guard(cost->device());
+  const auto i32 = cost->options().dtype(at::kInt);
+  const at::Tensor order = at::empty({R}, i32), rank_of_row = at::empty({R}, i32),
+                   rank_cost = at::empty({ranks}, cost->options());
+  const pp_stream_t s = stream_of(cost->get_device());
+  const int64_t* cp = cost->data_ptr<int64_t>();
+  int rc;
+  Py_BEGIN_ALLOW_THREADS
+  rc = api.assign_rows(int32_t(R), cp, int32_t(ranks), order.data_ptr<int32_t>(), rank_of_row.data_ptr<int32_t>(),
+                       rank_cost.data_ptr<int64_t>(), s);
+  Py_END_ALLOW_THREADS
+  if (rc) return raise_code(rc, "pp_assign_rows");
+  return Py_BuildValue("(NNN)", THPVariable_Wrap(order), THPVariable_Wrap(rank_of_row), THPVariable_Wrap(rank_cost));
+  PP_GUARD_END
+}
+
 #define PP_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(name)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {PP_METHOD(bind), PP_METHOD(build_plan), PP_METHOD(fwd), PP_METHOD(bwd),
+                         PP_METHOD(build_rows), PP_METHOD(assign_rows),
                          {nullptr, nullptr, 0, nullptr}};
 #define PP_STR2(x) #x
 #define PP_STR(x) PP_STR2(x)

@@ -125,7 +125,7 @@ def test_assign_rows_errors():
     assert e.value.code == -2
 
 
-@pytest.mark.parametrize("G", [31, 33, 64, 65, 1023, 1025, 2049, 8192, 8193])
+@pytest.mark.parametrize("G", [31, 33, 64, 65, 1023, 1025, 2048, 2049, 4097, 8192, 8193])
 def test_row_builder_at_the_edges_of_its_blocks_and_tables(G):
     """Bit-exact; 8192 groups are the most whose tables stay in shared memory."""
     rng = np.random.default_rng(G)
@@ -133,7 +133,7 @@ def test_row_builder_at_the_edges_of_its_blocks_and_tables(G):
     _compare(P, off, rl, int(R.group_tokens(P, off, rl).max()) * 3 + G % 7)
 
 
-@pytest.mark.parametrize("ranks", [2, 31, 32, 33, 64, 65, 128, 129])
+@pytest.mark.parametrize("ranks", [1, 2, 8, 9, 31, 32, 33, 64, 65, 128, 129])
 @pytest.mark.parametrize("rows", [1, 31, 32, 33, 129, 700])
 def test_assign_rows_at_the_edges_of_the_lane_lists(rows, ranks):
     """One, two and four list entries per lane and the search beyond; zero costs and ties."""
@@ -148,7 +148,7 @@ def test_assign_rows_at_the_edges_of_the_lane_lists(rows, ranks):
 
 
 @pytest.mark.parametrize("kind", ["equal", "zeros", "doubling", "huge", "mixed"])
-@pytest.mark.parametrize("rows,ranks", [(1, 32), (31, 31), (1024, 8), (1025, 32), (2500, 5)])
+@pytest.mark.parametrize("rows,ranks", [(1, 32), (31, 31), (1024, 8), (1025, 32), (2500, 5), (2500, 1), (1100, 64), (1500, 127)])
 def test_assign_rows_in_rounds(rows, ranks, kind):
     """Several rows a round: costs where all ranks take one, where only the first does, and sums too
     large for load and rank in one word."""
