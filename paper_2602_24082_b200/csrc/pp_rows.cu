@@ -193,7 +193,8 @@ __device__ __forceinline__ Sums<kN> block_scan(Sums<kN> s, Sums<kN>* s_warp, Sum
 // shared-memory pipe and barriers allow, so the sums come from kPer consecutive positions per thread, read as
 // vectors and scanned once for 1024 kPer of them; searches and jumps take neighbouring positions in
 // neighbouring lanes, kPer of them side by side; and up to kPackSmemGroups groups all that is
-// searched or chased lives in shared memory (28 bytes each).  4096 groups: @PACK@.
+// searched or chased lives in shared memory (28 bytes each).  4096 groups: 38 us with
+// gathers and every phase strided over global memory and scans of 1024, now 18.
 constexpr int kPackSmemGroups = 8192;
 constexpr size_t pack_smem(int G) { return size_t(16) * ((G + 1) & ~1) + size_t(12) * G; }
 
@@ -356,13 +357,14 @@ __global__ void __launch_bounds__(1024) rows_pack_kernel(RowsPtrs p) {
 // ---------------------------------------------------------------- rows -> data-parallel ranks
 // Longest-processing-time assignment: rows in order of decreasing cost (ties by index), each to
 // the rank with the least cost so far (ties to the lowest rank).  The order comes from rank
-// counting over all rows; the greedy pass is sequential by nature and runs in one warp.  What
-// bounds it is the chain from one row's assignment to the next one's, so the ranks are kept
+// counting over all rows; the greedy pass is sequential by nature and runs in one block: in rounds
+// (assign_batch_kernel below) or, where the sums are too large for those, one row at a time in one warp.  What
+// bounds the latter is the chain from one row's assignment to the next one's, so the ranks are kept
 // sorted by (load, rank) across the lanes' registers, kPerLane entries each: a step takes the
 // first entry, adds the row's cost and inserts it again -- every lane compares its entries with
 // the new one and keeps, shifts or replaces them -- so the chain is one broadcast, one add and
-// one compare.  Rows are fetched and results written 32 at a time.  (Searching all loads in shared
-// memory for the least one with a five-step butterfly took 345 ns a row, now 67 with up to 32 ranks, 98 with 64, 120 with 128.)
+// one compare.  Rows are fetched and results written 32 at a time.  (67 ns a row with up to 32 ranks, 98
+// with 64, 120 with 128; searching all loads in shared memory for the least one, as beyond 128, 345.)
 constexpr int kMaxAssignRanks = 1024;
 
 template <int kPerLane>
@@ -426,7 +428,9 @@ __device__ __forceinline__ void assign_one_by_one(int R, int ranks, const long l
 // a row in this round -- with loads closer together than a row's cost, as they soon are, that is
 // every rank.  A thread keeps one rank, whose load and number are one 64-bit word (for sums of costs
 // below 2^56, else one row at a time); its place is the number of words before its own, all kN read from shared
-// memory side by side.  Bound by that chain, word -> place -> cost -> word.  972 rows: @GREEDY@.
+// memory side by side.  Bound by that chain, word -> place -> cost -> word.  972 rows to 8 ranks:
+// 35 us with the list sorted again every round, now 32; building and dealing out to 64 ranks 177 us with
+// one row at a time, now 68.
 constexpr int kBatchRows = 1024, kBatchThreads = 256;
 template <int kN>   // ranks at most; a multiple of 32 threads work, one warp without barriers
 __global__ void __launch_bounds__(kBatchThreads)

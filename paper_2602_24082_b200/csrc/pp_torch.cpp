@@ -2,8 +2,9 @@
 // allocation, current device and stream, and the C ABI call, without interpreter code or ctypes
 // in between.  On small steps the host is what a call costs (a 144-token step has 28 us of
 // kernels): plan, forward and backward took 12.6, 11.1 and 18.7 us through ctypes, of which 4.8,
-// 3.7 and 10.1 were the library's own; now 4.4, 5.2 and 12.5.  Building and dealing out the rows of 4096 groups
-// @ROWHOST@.
+// 3.7 and 10.1 were the library's own; now 4.4, 5.2 and 12.5.  The call that builds
+// the rows of 4096 groups took 94 us through ctypes with a copy of the row count, now 56 (13 of the difference
+// are its packing kernel's), the one that deals them out 19.5, now 13.
 // Only marshalling lives here; everything is computed by libpp_attn.so, whose entry points are
 // looked up once (bind).  Anything unusual -- a tensor that fails a check, descriptors that are not
 // contiguous int32 arrays, an error code -- goes back to the Python side, which raises.
