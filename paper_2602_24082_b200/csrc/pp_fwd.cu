@@ -19,7 +19,8 @@
 // has read itself) and is the A operand of the second MMA; V is
 // its MN-major B operand straight from the TMA layout.  O is rescaled lazily: only when a
 // row's running maximum grew by more than 2^8 since the value used for scaling.
-// TMEM: S0 | S1 | O0 | O1, 128 columns each.
+// TMEM: S0 | S1 | O0 | O1, 128 columns each.  At D = 64 narrower accumulators leave room for P beside S (kOwnP
+// below): S0 | S1 | P0 | P1 | O0 | O1, and a slot's next QK is issued as soon as its scores are read.
 // Query tiles are those of the segments or, with many short ones, mixed tiles (kMixed below).
 #include <algorithm>
 #include <type_traits>
@@ -60,7 +61,9 @@ enum FwdBar : int {
   kSchedFullF = 16,   // [2] unit ids handed from the producer to the other roles
   kSchedEmptyF = 18,  // [2] 17 arrivals: MMA thread + 16 softmax warps (+ 2 clearing warps)
   kPRest = 20,        // [2] per slot: the late columns of P (kPFull: the early ones)
-  kNumFwdBars = 22
+  kSFree = 22,        // [2] per slot, with columns of its own for P: the scores are read
+  kPFree = 24,        // [2]                                          PV has read P
+  kNumFwdBars = 26
 };
 
 template <int D>
@@ -153,6 +156,12 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
            const __grid_constant__ CUtensorMap tm_v, FwdParams prm) {
   using L = FwdSmem<D>;
   constexpr bool kMixed = kMode == kMixedTiles, kPaired = kMode == kPairedTiles;
+  // P in columns of its own: the chain of a slot is then softmax -> QK -> softmax, without PV.
+  // 16384 tokens, 32 / 8 heads 214 -> 205 us, 12000, 16 / 16 heads 184 -> 170, 28 / 4 190 -> 180.  Not with
+  // mixed tiles, whose units are short: 12000 tokens in short segments, 32 / 8 heads 98.3 -> 100.4.
+  constexpr bool kOwnP = D == 64 && !kMixed;
+  constexpr uint32_t kTmemP = kOwnP ? 256 : 0, kTmemPStep = kOwnP ? 64 : 128, kPHalf = kOwnP ? 32 : 64;
+  constexpr uint32_t kTmemO = kOwnP ? 384 : 256, kTmemOStep = kOwnP ? 64 : 128;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // (known to be uniform in the warp)
@@ -175,7 +184,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
 
   if (tid == 0) {
     for (int i = 0; i < kNumFwdBars; ++i) {
-      const bool wg_count = (i >= kPFull && i < kPFull + 2) || (i >= kOFree && i < kOFree + 2) || i >= kPRest;
+      const bool wg_count = (i >= kPFull && i < kPFull + 2) || (i >= kOFree && i < kOFree + 2) ||
+                            (i >= kPRest && i < kPFree);
       const bool sched_empty = (i >= kSchedEmptyF && i < kSchedEmptyF + 2);
       // unit records are released by the MMA thread, the 16 softmax warps and, when the dQ
       // accumulator is cleared here, the two clearing warps
@@ -325,34 +335,36 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
       // kEarlySteps, then the others
       auto issue_pv = [&](int s, uint32_t vstage, int k_len, bool first, bool last, uint32_t par) {
         const uint32_t b = dv0 + vstage * kStageStep;
-        const uint32_t tS = tmem + s * 128, tO = tmem + 256 + s * 128;
+        const uint32_t tP = tmem + kTmemP + s * kTmemPStep, tO = tmem + kTmemO + s * kTmemOStep;
+        auto p_at = [&](int kk) { return tP + (kk < 4 ? kk * 8 : kPHalf + (kk - 4) * 8); };
         if (k_len == kTile && !first) {
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)
             if ((kk & 3) < kEarlySteps)
-              mma_ts(tO, tS + (kk < 4 ? kk * 8 : 64 + (kk - 4) * 8), b + mnmajor_off(kk), idesc_o, 1);
+              mma_ts(tO, p_at(kk), b + mnmajor_off(kk), idesc_o, 1);
           wait_bar(bar(kPRest + s), par, abort_flag, prm.header, 39);
           tc_fence_after();
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)
             if ((kk & 3) >= kEarlySteps)
-              mma_ts(tO, tS + (kk < 4 ? kk * 8 : 64 + (kk - 4) * 8), b + mnmajor_off(kk), idesc_o, 1);
+              mma_ts(tO, p_at(kk), b + mnmajor_off(kk), idesc_o, 1);
         } else {
           const int ksteps = (k_len + 15) >> 4;
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)
             if ((kk & 3) < kEarlySteps && kk < ksteps)
-              mma_ts(tO, tS + (kk < 4 ? kk * 8 : 64 + (kk - 4) * 8), b + mnmajor_off(kk), idesc_o,
+              mma_ts(tO, p_at(kk), b + mnmajor_off(kk), idesc_o,
                      !first || (kk > 0));
           wait_bar(bar(kPRest + s), par, abort_flag, prm.header, 39);
           tc_fence_after();
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)
             if ((kk & 3) >= kEarlySteps && kk < ksteps)
-              mma_ts(tO, tS + (kk < 4 ? kk * 8 : 64 + (kk - 4) * 8), b + mnmajor_off(kk), idesc_o, 1);
+              mma_ts(tO, p_at(kk), b + mnmajor_off(kk), idesc_o, 1);
         }
         // the accumulator is only waited for after the unit's last PV (the lazy rescale, rare,
         // runs after S of the next tile is complete, whose commit covers this PV as well)
+        if (kOwnP) mma_commit(bar(kPFree + s));
         if (last) mma_commit(bar(kODone + s));
       };
       for (uint32_t un_i = 0;; ++un_i) {
@@ -380,23 +392,35 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
           wait_bar(bar(kKFull + kst), (kc >> 1) & 1, abort_flag, prm.header, 33);
           if (!kPaired || j < nt0) {   // slot 0
             const bool has_next0 = j + 1 < nt0;
+            if (kOwnP && has_next0) {
+              wait_bar(bar(kSFree + 0), tc0 & 1, abort_flag, prm.header, 27);
+              tc_fence_after();
+              issue_qk(0, kst, nx_len);
+              if (j + 2 == nt0) mma_commit(bar(kQEmpty + 0));
+            }
             wait_bar(bar(kPFull + 0), tc0 & 1, abort_flag, prm.header, 35);
             if (j == 0) wait_bar(bar(kOFree + 0), (uc0 & 1) ^ 1, abort_flag, prm.header, 37);
             tc_fence_after();
             issue_pv(0, vst, cur_len, j == 0, !has_next0, tc0 & 1);
             ++tc0;
-            if (has_next0) {
+            if (!kOwnP && has_next0) {
               issue_qk(0, kst, nx_len);
               if (j + 2 == nt0) mma_commit(bar(kQEmpty + 0));
             }
           }
           if (two) {
+            if (kOwnP && has_next) {
+              wait_bar(bar(kSFree + 1), tc1 & 1, abort_flag, prm.header, 28);
+              tc_fence_after();
+              issue_qk(1, kst, nx_len);
+              if (j + 2 == u_ntiles) mma_commit(bar(kQEmpty + 1));
+            }
             wait_bar(bar(kPFull + 1), tc1 & 1, abort_flag, prm.header, 36);
             if (j == 0) wait_bar(bar(kOFree + 1), (uc1 & 1) ^ 1, abort_flag, prm.header, 38);
             tc_fence_after();
             issue_pv(1, vst, cur_len, j == 0, !has_next, tc1 & 1);
             ++tc1;
-            if (has_next) {
+            if (!kOwnP && has_next) {
               issue_qk(1, kst, nx_len);
               if (j + 2 == u_ntiles) mma_commit(bar(kQEmpty + 1));
             }
@@ -451,7 +475,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const int bar_id = 1 + s * 4 + qd;        // named barrier shared with the partner warp
     const uint32_t lane_base = tmem + (uint32_t(32 * qd) << 16);
     const uint32_t tS = lane_base + s * 128 + half * 64;   // my S columns; P goes to their start
-    const uint32_t tO = lane_base + 256 + s * 128 + half * (D / 2);
+    const uint32_t tP = lane_base + kTmemP + s * kTmemPStep + half * kPHalf;   //   or to its own
+    const uint32_t tO = lane_base + kTmemO + s * kTmemOStep + half * (D / 2);
     // What the two halves of a row exchange, one buffer each for the largest exponentials, the maxima
     // and the row sums: a value is then only overwritten behind a barrier, or a wait for a tile that
     // needs the partner's P, that follows the partner's read.
@@ -620,7 +645,12 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
           const float m_new = fmaxf(m_used, row_max());
           const float alpha = ex2(m_used - m_new);
           // PV of the previous tile is complete: the commit that announced this tile's S was
-          // issued after it and covers every earlier MMA of the issuing thread
+          // issued after it and covers every earlier MMA of the issuing thread (but with columns of P's own
+          // that QK came first)
+          if (kOwnP) {
+            wait_bar(bar(kPFree + s), (tcS & 1) ^ 1, abort_flag, prm.header, 48);
+            tc_fence_after();
+          }
 #pragma unroll 1
           for (int c = 0; c < D / 16; ++c) {  // eight columns at a time
             uint32_t w[8];
@@ -634,9 +664,15 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
           m_used = m_new;
           redone = true;
         }
-        // P over the first half of my own S columns
-        tmem_st16(tS, pk);
-        tmem_st8(tS + 16, pk + 16);
+        if (kOwnP) {
+          tc_fence_before();
+          mbar_arrive(bar(kSFree + s));
+          wait_bar(bar(kPFree + s), (tcS & 1) ^ 1, abort_flag, prm.header, 48);   // (long complete)
+          tc_fence_after();
+        }
+        // P over the first half of my own S columns, or to its own
+        tmem_st16(tP, pk);
+        tmem_st8(tP + 16, pk + 16);
         tmem_wait_st();
         tc_fence_before();
         mbar_arrive(bar(kPFull + s));
@@ -649,7 +685,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         float s0, s1;
         unpack2(sum2, s0, s1);
         l_part += s0 + s1;
-        tmem_st8(tS + 24, pk + 24);
+        tmem_st8(tP + 24, pk + 24);
         tmem_wait_st();
         tc_fence_before();
         mbar_arrive(bar(kPRest + s));
