@@ -59,6 +59,7 @@ __global__ void __launch_bounds__(kLossThreads)
 preference_loss_kernel(LossPtrs p, const float* __restrict__ logp, const float* __restrict__ ref,
                        float beta, float* __restrict__ resp_logp, float* resp_reward,
                        float* __restrict__ grp_loss, float* __restrict__ d_logp, int team_warps) {
+  dependency_wait();
   // (two buffers each, in turn: one barrier per round)
   __shared__ double s_sum[2][kLossWarps], s_ref[2][kLossWarps];
   __shared__ float s_grad[2][kLossWarps];
@@ -182,9 +183,8 @@ cudaError_t launch_preference_loss(const pp_plan* plan, const float* logp, const
               : gang_warps == 4 ? preference_loss_kernel<4>
               : gang_warps == 2 ? preference_loss_kernel<2>
                                 : preference_loss_kernel<1>;
-  kern<<<(p.G + gangs - 1) / gangs, kLossThreads, 0, stream>>>(p, logp, ref, beta, resp_logp, resp_reward,
-                                                              grp_loss, d_logp, team_warps);
-  return cudaGetLastError();
+  return launch_kernel(true, kern, dim3((p.G + gangs - 1) / gangs), dim3(kLossThreads), 0, stream, p, logp, ref, beta,
+                       resp_logp, resp_reward, grp_loss, d_logp, team_warps);
 }
 
 }  // namespace pp

@@ -8,7 +8,8 @@
 //   x'[i]       = x[i] cos a - x[i + D/2] sin a
 //   x'[i + D/2] = x[i + D/2] cos a + x[i] sin a
 // Both kernels are HBM-bound: one pass over Q and K (read + write, bf16), 4 bytes per token
-// for the ids.
+// for the ids.  On small batches their launches count: overlapped with the kernel in front (launch_kernel), ids,
+// embedding and preference loss of 325 tokens took 26.6 us, now 24.3, of 6000 36.3 and 31.3, of 65536 231 and 226.
 #include "pp_internal.h"
 #include "pp_ptx.cuh"
 
@@ -44,6 +45,8 @@ __device__ __forceinline__ int position_of(const SegPtrs& p, int t) {
 }
 
 __global__ void position_ids_kernel(SegPtrs p, int32_t* __restrict__ pos) {
+  launch_dependents();
+  dependency_wait();
   if (p.header[0] != kStatusOk) return;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < p.T) pos[t] = position_of(p, t);
@@ -56,6 +59,7 @@ template <int D>
 __global__ void __launch_bounds__(256)
 rope_kernel(SegPtrs p, __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, int Hq,
             int Hkv, float log2_base) {
+  dependency_wait();
   if (p.header[0] != kStatusOk) return;
   const int lane = threadIdx.x & 31;
   const int t = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -105,8 +109,7 @@ SegPtrs seg_ptrs(const pp_plan* plan) {
 
 cudaError_t launch_position_ids(const pp_plan* plan, int32_t* pos, cudaStream_t stream) {
   SegPtrs p = seg_ptrs(plan);
-  position_ids_kernel<<<(p.T + 255) / 256, 256, 0, stream>>>(p, pos);
-  return cudaGetLastError();
+  return launch_kernel(true, position_ids_kernel, dim3((p.T + 255) / 256), dim3(256), 0, stream, p, pos);
 }
 
 cudaError_t launch_rope(const pp_plan* plan, void* q, void* k, float base, cudaStream_t stream) {
@@ -114,19 +117,9 @@ cudaError_t launch_rope(const pp_plan* plan, void* q, void* k, float base, cudaS
   const pp_problem& pb = plan->prob;
   const float log2_base = log2f(base);
   const unsigned blocks = unsigned((p.T + 7) / 8);
-  if (pb.head_dim == 128)
-    rope_kernel<128><<<blocks, 256, 0, stream>>>(p, static_cast<__nv_bfloat16*>(q),
-                                                 static_cast<__nv_bfloat16*>(k), pb.num_q_heads,
-                                                 pb.num_kv_heads, log2_base);
-  else if (pb.head_dim == 96)
-    rope_kernel<96><<<blocks, 256, 0, stream>>>(p, static_cast<__nv_bfloat16*>(q),
-                                                static_cast<__nv_bfloat16*>(k), pb.num_q_heads,
-                                                pb.num_kv_heads, log2_base);
-  else
-    rope_kernel<64><<<blocks, 256, 0, stream>>>(p, static_cast<__nv_bfloat16*>(q),
-                                                static_cast<__nv_bfloat16*>(k), pb.num_q_heads,
-                                                pb.num_kv_heads, log2_base);
-  return cudaGetLastError();
+  auto kern = pb.head_dim == 128 ? rope_kernel<128> : pb.head_dim == 96 ? rope_kernel<96> : rope_kernel<64>;
+  return launch_kernel(true, kern, dim3(blocks), dim3(256), 0, stream, p, static_cast<__nv_bfloat16*>(q),
+                       static_cast<__nv_bfloat16*>(k), pb.num_q_heads, pb.num_kv_heads, log2_base);
 }
 
 }  // namespace pp
