@@ -141,7 +141,7 @@ int pp_plan_read_bwd_tiles(const pp_plan* plan, pp_stream_t stream, int32_t* num
  * the first num_bwd_tiles * Hkv are valid.  Units of one group are adjacent (they stream the
  * same Q / dO tiles through L2), groups with the most work first.  (With three or more query heads
  * per KV head pp_attn_bwd takes the same units in smaller blocks; pp_plan_read_bwd_sched gives
- * the order it takes them in.)  Synchronises `stream`. */
+ * the order it takes them in.)  Neither call writes to the plan.  Synchronises `stream`. */
 int pp_plan_read_bwd_units(const pp_plan* plan, pp_stream_t stream, int32_t* units);
 int pp_plan_read_bwd_sched(const pp_plan* plan, pp_stream_t stream, int32_t* units);
 int pp_plan_read(const pp_plan* plan, pp_stream_t stream, int32_t* num_tiles, int32_t* tiles,

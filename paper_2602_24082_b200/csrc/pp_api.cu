@@ -169,27 +169,58 @@ int pp_destroy_plan(pp_plan* plan) {
 
 int pp_plan_max_tiles(const pp_plan* plan) { return plan ? plan->max_tiles : PP_ERR_INVALID_ARG; }
 
-static int read_units(const pp_plan* plan, size_t list, pp_stream_t stream, int32_t* units) {
+int pp_plan_read_bwd_sched(const pp_plan* plan, pp_stream_t stream, int32_t* units) {
+  if (!plan || !units) return PP_ERR_INVALID_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const size_t n = size_t(plan->max_tiles) * plan->prob.num_kv_heads;
-  if (cudaMemcpyAsync(units, plan->ws + list, n * 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+  if (cudaMemcpyAsync(units, plan->ws + plan->lay.bwd_units, n * 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return PP_ERR_CUDA;
   return PP_OK;
 }
 
-int pp_plan_read_bwd_units(const pp_plan* plan, pp_stream_t stream, int32_t* units) {
-  if (!plan || !units) return PP_ERR_INVALID_ARG;
-  if (pp::bwd_takes_sched(plan->prob) &&
-      pp::launch_base_units(plan, reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess)
-    return PP_ERR_CUDA;
-  return read_units(plan, plan->lay.bwd_units, stream, units);
+// The order in super-groups from the backward's tiles (plan_sgroup_body and plan_units_body): groups by
+// decreasing work, blocks of 600 units from the end, in a block the longest tiles first.
+static void super_group_units(const pp::BTile* tiles, int n, int Hkv, int32_t* units) {
+  struct Group {
+    int first, tiles;
+    long long work;
+  };
+  std::vector<Group> groups;   // (a group's tiles are consecutive)
+  for (int t = 0; t < n; ++t) {
+    if (t == 0 || tiles[t].grp_start != tiles[t - 1].grp_start) groups.push_back({t, 0, 0});
+    ++groups.back().tiles;
+    groups.back().work += tiles[t].work;
+  }
+  std::stable_sort(groups.begin(), groups.end(), [](const Group& a, const Group& b) { return a.work > b.work; });
+  std::vector<int> block(n), order(n);
+  long long rest = n;
+  for (const Group& g : groups) {
+    std::fill_n(block.begin() + g.first, g.tiles, int((Hkv * rest - 1) / pp::kSuperGroupUnits));
+    rest -= g.tiles;
+  }
+  for (int t = 0; t < n; ++t) order[t] = t;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+    return block[a] != block[b] ? block[a] > block[b] : tiles[a].work > tiles[b].work;
+  });
+  for (int i = 0; i < n; ++i)
+    for (int kvh = 0; kvh < Hkv; ++kvh) units[size_t(i) * Hkv + kvh] = (kvh << 24) | order[i];
 }
 
-int pp_plan_read_bwd_sched(const pp_plan* plan, pp_stream_t stream, int32_t* units) {
+int pp_plan_read_bwd_units(const pp_plan* plan, pp_stream_t stream, int32_t* units) {
   if (!plan || !units) return PP_ERR_INVALID_ARG;
-  return read_units(plan, pp::bwd_takes_sched(plan->prob) ? plan->lay.bwd_sched : plan->lay.bwd_units, stream,
-                    units);
+  if (!pp::bwd_takes_sched(plan->prob)) return pp_plan_read_bwd_sched(plan, stream, units);
+  // only the smaller blocks are in the workspace, which a reader does not write to
+  try {
+    std::vector<pp::BTile> tiles(plan->max_tiles);
+    int32_t n = 0;
+    const int rc = pp_plan_read_bwd_tiles(plan, stream, &n, reinterpret_cast<int32_t*>(tiles.data()));
+    if (rc == PP_ERR_CUDA) return rc;
+    if (rc == PP_OK) super_group_units(tiles.data(), n, plan->prob.num_kv_heads, units);
+  } catch (const std::bad_alloc&) {
+    return PP_ERR_CUDA;
+  }
+  return PP_OK;   // (a refused plan has no units)
 }
 
 int pp_plan_read_bwd_tiles(const pp_plan* plan, pp_stream_t stream, int32_t* num_tiles,

@@ -1083,8 +1083,7 @@ cudaError_t launch_bwd(const pp_plan* plan, const void* q, const void* k, const 
   prm.header = reinterpret_cast<int32_t*>(plan->ws + plan->lay.header);
   prm.tiles = reinterpret_cast<const BTile*>(plan->ws + plan->lay.btiles);
   prm.order = reinterpret_cast<const int32_t*>(
-      plan->ws + (deterministic ? plan->lay.bwd_units_det
-                  : bwd_takes_sched(pb) ? plan->lay.bwd_sched : plan->lay.bwd_units));
+      plan->ws + (deterministic ? plan->lay.bwd_units_det : plan->lay.bwd_units));
   prm.key_end = reinterpret_cast<const int32_t*>(plan->ws + plan->lay.key_end);
   prm.delta = reinterpret_cast<float*>(sc + sl.delta);
   prm.lse2 = reinterpret_cast<float*>(sc + sl.lse2);

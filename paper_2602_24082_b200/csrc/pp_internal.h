@@ -63,7 +63,7 @@ constexpr int kQTilePrompt = 256;
 // Words of the plan header (int32[16]).
 constexpr int kHdrStatus = 0, kHdrDetail = 1, kHdrNumTiles = 2, kHdrNumSegments = 3,
               kHdrNumBTiles = 8, kHdrNumQTiles = 9,
-              kHdrSchedTail = 10;   // (multi-kernel plan) tiles of the last block of bwd_sched
+              kHdrSchedTail = 10;   // (multi-kernel plan) tiles of the last of the smaller blocks
 
 // Status word values written by device code.
 enum : int32_t {
@@ -87,10 +87,9 @@ struct PlanLayout {
   size_t bwd_order;  // int32[max_tiles]  backward tiles, longest work first
   size_t tile_gwork; // int32[max_tiles]  backward work of the backward tile's whole group
   size_t tile_sgroup; // int32[max_tiles] super-group (block of consecutive groups)
-  size_t tile_sblock; // int32[max_tiles] ... and its block in bwd_sched
+  size_t tile_sblock; // int32[max_tiles] tiles of the groups behind the tile's, for its smaller block
   size_t bwd_units;  // int32[max_tiles * Hkv]  (kv head << 24) | backward tile, processing order
-                     //   (with bwd_takes_sched only where it is asked for)
-  size_t bwd_sched;  // the same units in smaller blocks: with bwd_takes_sched, what the kernel takes
+                     //   (in super-groups or, with bwd_takes_sched, in smaller blocks)
   size_t bwd_units_det;  // the same units, one (group, KV head) set after the other and inside a
                          //   set by descending tile index: the order of the deterministic backward
   size_t key_end;    // int32[T]
@@ -181,7 +180,6 @@ inline PlanLayout plan_layout(const pp_problem& p) {
   l.tile_gwork = off; off = align_up(off + sizeof(int32_t) * size_t(mt), 256);
   l.tile_sgroup = off; off = align_up(off + sizeof(int32_t) * size_t(mt), 256);
   l.tile_sblock = off; off = align_up(off + sizeof(int32_t) * size_t(mt), 256);
-  l.bwd_sched = off; off = align_up(off + sizeof(int32_t) * size_t(mt) * size_t(p.num_kv_heads), 256);
   l.bwd_units = off; off = align_up(off + sizeof(int32_t) * size_t(mt) * size_t(p.num_kv_heads), 256);
   l.bwd_units_det = off;
   off = align_up(off + sizeof(int32_t) * size_t(mt) * size_t(p.num_kv_heads), 256);
@@ -237,17 +235,17 @@ inline int bwd_split_log2(const pp_problem& p) {
 
 // Which order the backward takes its units in.  Both go through the groups by decreasing work, in
 // blocks of groups inside which the longest units come first.  With blocks of 600 units
-// (bwd_units) the 148 units that run at a time may be the longest of all of a block's groups, and with r
+// (super-groups) the 148 units that run at a time may be the longest of all of a block's groups, and with r
 // query heads per KV head a block's Q, dO and dQ accumulator are 600 r * 128 KB at D 128: far beyond
 // L2, so that a (query tile, head) is fetched, and its accumulator written back, for nearly every
 // other key tile.  Blocks of 150 units, with a larger last one to balance the end
-// (bwd_sched; sched_tail in the plan), take a third to a half of that traffic (a model of L2 with 80 MB of least-recently-used tiles, which gives
+// (sched_tail in the plan), take a third to a half of that traffic (a model of L2 with 80 MB of least-recently-used tiles, which gives
 // the 600s' measured 0.93, 5.4 and 5.9 GB as 0.93, 5.9 and 5.7: 0.5, 3.9 and 2.2).  Main kernel, 600s
 // -> these: 9241 tokens, 32 / 8 heads 262 -> 250 us; 16384, 64 / 8 1361 -> 1230; 16384, 32 / 8, D 64 456 -> 400; 36000 in short groups, 16 / 2 277 -> 243; 16760, 32 / 8 307 ->
 // 272; two rows of 32768, 32 / 8 19320 -> 19220.  With one and two heads per KV head a block's data is
 // that much smaller, and the smaller blocks only cost balance: 8 / 8 258 -> 265, 16 / 8 278 -> 276, 754 -> 740.
 // Up to 200 units both are one block.
-constexpr int kSchedBlockUnits = 150, kSchedTailUnits = 200;
+constexpr int kSuperGroupUnits = 600, kSchedBlockUnits = 150, kSchedTailUnits = 200;
 inline bool bwd_takes_sched(const pp_problem& p) {
   return p.num_q_heads / p.num_kv_heads >= 3 && (long long)max_btiles_of(p) * p.num_kv_heads > kSchedTailUnits;
 }
@@ -383,8 +381,6 @@ bool profile_read_all(float* fwd_ms, float* bwd_ms, int capacity, int* n_fwd, in
 // host_desc: the four descriptor arrays on the host, or null when they are on the device
 cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cudaStream_t stream,
                         int* launches);
-// the order of units that the plan leaves out where bwd_takes_sched (lay.bwd_units)
-cudaError_t launch_base_units(const pp_plan* plan, cudaStream_t stream);
 cudaError_t launch_fwd(const pp_plan* plan, const void* q, const void* k, const void* v, float scale,
                        void* o, float* lse, float* dq_clear, cudaStream_t stream, int* launches);
 cudaError_t launch_bwd(const pp_plan* plan, const void* q, const void* k, const void* v,

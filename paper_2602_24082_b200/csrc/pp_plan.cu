@@ -41,8 +41,8 @@ struct PlanPtrs {
   int32_t* tile_gwork;
   int32_t* tile_sgroup;
   int32_t* tile_sblock;
-  int32_t* bwd_units;   // null: not wanted (either of the two, or the third)
-  int32_t* bwd_sched;
+  int32_t* bwd_units;
+  bool sched;           // in the smaller blocks (bwd_takes_sched)
   int32_t* bwd_units_det;
   int Hkv;
   int32_t* key_end;
@@ -423,7 +423,6 @@ __global__ void plan_fwd_order_kernel(PlanPtrs p) {
 // into one super-group, i.e. a plain longest-first list; large ones keep the working set of the
 // concurrently running units near one group's Q / dO.  Dynamic scheduling in the kernel does
 // the balancing.  A tile's group is identified by the group's first token.
-constexpr int kSuperGroupUnits = 600;
 
 // The blocks of the order that the kernel takes with several query heads per KV head
 // (bwd_takes_sched, which has the reasons).  The last block begins with the first group behind which
@@ -474,23 +473,20 @@ __device__ __forceinline__ void plan_sgroup_body(const PlanPtrs& p, int t, int n
 __device__ __forceinline__ void plan_units_body(const PlanPtrs& p, int t, int n) {
   const int wb = p.btiles[t].work;
   int pos = 0;
-  if (p.bwd_units) {
+  if (!p.sched) {
     const int sg = p.tile_sgroup[t];
     for (int u = 0; u < n; ++u) {
       const int osg = p.tile_sgroup[u], ob = p.btiles[u].work;
       pos += (osg > sg) || (osg == sg && ((ob > wb) || (ob == wb && u < t)));
     }
-    for (int kvh = 0; kvh < p.Hkv; ++kvh) p.bwd_units[p.Hkv * pos + kvh] = (kvh << 24) | t;
-  }
-  if (p.bwd_sched) {
+  } else {
     const int tail = p.header[kHdrSchedTail], sb = sched_block(p, p.tile_sblock[t], tail, n);
-    pos = 0;
     for (int u = 0; u < n; ++u) {
       const int osb = sched_block(p, p.tile_sblock[u], tail, n), ob = p.btiles[u].work;
       pos += (osb > sb) || (osb == sb && ((ob > wb) || (ob == wb && u < t)));
     }
-    for (int kvh = 0; kvh < p.Hkv; ++kvh) p.bwd_sched[p.Hkv * pos + kvh] = (kvh << 24) | t;
   }
+  for (int kvh = 0; kvh < p.Hkv; ++kvh) p.bwd_units[p.Hkv * pos + kvh] = (kvh << 24) | t;
   // Deterministic order: one (group, KV head) set after the other, groups by decreasing work.
   // The tiles add to a query tile's dQ in descending order, so a unit waits for the unit of the
   // next tile.  Inside a set the units go out in ascending tile order (longest first, as in the
@@ -498,7 +494,6 @@ __device__ __forceinline__ void plan_units_body(const PlanPtrs& p, int t, int n)
   // the list can have units waiting for a unit that has not been handed out yet, so fewer than
   // det_asc_max CTAs can be held up that way and the others keep drawing.  Larger sets go out
   // in DESCENDING tile order, where every unit follows the units it waits for.
-  if (!p.bwd_units_det) return;
   const int gs = p.btiles[t].grp_start, gw = p.tile_gwork[t];
   int before = 0, ng = 0;  // tiles of groups ranked earlier; tiles of this group
   for (int u = 0; u < n; ++u) {
@@ -955,7 +950,7 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
   // tile's work is 1 .. 2048
   auto unit_key = [&](int t, int ranked_before) {
     const int g = sm.bgrp[t], rest = nb - ranked_before, later = rest - (sm.btile0[g + 1] - sm.btile0[g]);
-    const int block = p.bwd_sched ? sched_block(p, later, sm.sched_tail, nb) : (p.Hkv * rest - 1) / kSuperGroupUnits;
+    const int block = p.sched ? sched_block(p, later, sm.sched_tail, nb) : (p.Hkv * rest - 1) / kSuperGroupUnits;
     return uint32_t(1023 - block) << 22 | uint32_t(2048 - sm.wb[t]) << 11 | uint32_t(t);
   };
   if (by_rank) {   // (blocks of 256 threads have at most 256 tiles: one per thread)
@@ -976,7 +971,7 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
     rank_count<true>(sm.o.r.key[2], p.G, sm.o.r.rank[2], sm.btile0);
     if constexpr (kMixed) rank_count<false>(sm.o.r.key[4], n, sm.o.r.rank[4], nullptr);
     __syncthreads();
-    if (p.bwd_sched) {
+    if (p.sched) {
       if (tid < p.G) {
         const uint32_t mine = sm.o.r.key[2][tid];
         int later_work = 0;
@@ -1037,7 +1032,7 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
   // ---- backward units, in both orders
   for (int e = tid; e < nb * p.Hkv; e += nthr) {
     const int i = e / p.Hkv, kvh = e - i * p.Hkv;
-    (p.bwd_sched ? p.bwd_sched : p.bwd_units)[e] = (kvh << 24) | int(sm.unit_tile[i]);
+    p.bwd_units[e] = (kvh << 24) | int(sm.unit_tile[i]);
     // deterministic backward: set after set (see plan_units_body)
     const int g = sm.bgrp[i], ng = sm.btile0[g + 1] - sm.btile0[g], k_rel = i - sm.btile0[g];
     const int slot = ng <= p.det_asc_max ? k_rel : ng - 1 - k_rel;
@@ -1117,7 +1112,8 @@ bool profile_read(float* fwd_ms, float* bwd_ms) {
   return ok;
 }
 
-static PlanPtrs plan_ptrs(const pp_plan* plan) {
+cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cudaStream_t stream,
+                        int* launches) {
   PlanPtrs p;
   char* ws = plan->ws;
   const PlanLayout& l = plan->lay;
@@ -1139,9 +1135,8 @@ static PlanPtrs plan_ptrs(const pp_plan* plan) {
   p.tile_gwork = reinterpret_cast<int32_t*>(ws + l.tile_gwork);
   p.tile_sgroup = reinterpret_cast<int32_t*>(ws + l.tile_sgroup);
   p.tile_sblock = reinterpret_cast<int32_t*>(ws + l.tile_sblock);
-  const bool sched = bwd_takes_sched(plan->prob);
-  p.bwd_units = sched ? nullptr : reinterpret_cast<int32_t*>(ws + l.bwd_units);
-  p.bwd_sched = sched ? reinterpret_cast<int32_t*>(ws + l.bwd_sched) : nullptr;
+  p.bwd_units = reinterpret_cast<int32_t*>(ws + l.bwd_units);
+  p.sched = bwd_takes_sched(plan->prob);
   p.bwd_units_det = reinterpret_cast<int32_t*>(ws + l.bwd_units_det);
   p.Hkv = plan->prob.num_kv_heads;
   p.key_end = reinterpret_cast<int32_t*>(ws + l.key_end);
@@ -1149,31 +1144,12 @@ static PlanPtrs plan_ptrs(const pp_plan* plan) {
   p.qorder = reinterpret_cast<int32_t*>(ws + l.qorder);
   p.work_at = p.bwd_units_det;
   p.grid_gain = reinterpret_cast<long long*>(ws + l.grid_gain);
-  p.det_asc_max = 0;
   p.num_rows = plan->prob.num_rows;
   p.G = plan->prob.num_groups;
   p.N = plan->prob.num_responses;
   p.T = plan->prob.total_tokens;
   p.nseg = plan->nseg;
   p.max_tiles = plan->max_tiles;
-  return p;
-}
-
-cudaError_t launch_base_units(const pp_plan* plan, cudaStream_t stream) {
-  PlanPtrs p = plan_ptrs(plan);
-  p.bwd_units = reinterpret_cast<int32_t*>(plan->ws + plan->lay.bwd_units);
-  p.bwd_sched = p.bwd_units_det = nullptr;
-  p.qtiles = nullptr;
-  const int blocks = (p.max_tiles + 127) / 128;
-  plan_gwork_kernel<<<blocks, 128, 0, stream>>>(p);
-  plan_sgroup_kernel<<<blocks, 128, 0, stream>>>(p);
-  plan_units_kernel<<<blocks, 128, 0, stream>>>(p);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cudaStream_t stream,
-                        int* launches) {
-  PlanPtrs p = plan_ptrs(plan);
   // a third of the SMs (the backward runs one CTA per SM), at most 48 tiles = 6144 tokens
   static DeviceSetup setup[kMaxDevices];
   DeviceSetup* dev = device_setup(setup);

@@ -176,6 +176,21 @@ def test_order_the_backward_takes_its_units_in(groups, length, hq, hkv):
     assert (units[:, 0].reshape(n, hkv) == np.arange(hkv)).all()
 
 
+@pytest.mark.parametrize("rows,hq,hkv", [([[(700, (300, 200))]] * 40, 8, 2), ([[(60, (20, 11))]] * 1500, 6, 2), ([[(300, (90,))]] * 3, 2, 2)])
+def test_reading_a_plan_does_not_write_to_it(rows, hq, hkv):
+    """Both orders of the backward's units, also where only one of them is in the workspace: the plan may be
+    in use on another stream meanwhile."""
+    from paper_2602_24082_b200 import binding as B
+    plan = B.plan_for(W.Workload("read", rows, hq, hkv, 64, seed=2))
+    assert plan.status() == (0, 0)
+    before = plan.workspace.clone()
+    n = len(plan.read_bwd_tiles())
+    for units in (plan.read_bwd_units(n), plan.read_bwd_sched(n)):
+        assert sorted(map(tuple, units.tolist())) == [(h, t) for h in range(hkv) for t in range(n)]
+    plan.read()
+    assert torch.equal(plan.workspace, before)
+
+
 def test_multi_kernel_plan_path_matches_fused_semantics():
     """> 2048 tiles forces the multi-kernel plan path; its tiles / orders obey the same
     rules (checked through the same dense-mask comparison on a prefix of the tokens)."""
