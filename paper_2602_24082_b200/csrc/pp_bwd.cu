@@ -63,9 +63,9 @@ __host__ __device__ constexpr int pre_tokens(int d) { return kPreWarps * kPreUnr
 
 template <int D, bool kClear>
 __global__ void __launch_bounds__(32 * kPreWarps)
-bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o,
-                      const float* __restrict__ lse, float* __restrict__ delta,
-                      float* __restrict__ lse2, float* __restrict__ dq_acc, int T, int Hq, int4* sem, unsigned sem_n4) {
+bwd_preprocess_kernel(const __nv_bfloat16* o, const __nv_bfloat16* d_o,
+                      const float* lse, float* delta,
+                      float* lse2, float* dq_acc, int T, int Hq, int4* sem, unsigned sem_n4) {
   launch_dependents();
   dependency_wait();
   constexpr int kLanes = pre_lanes(D);    // lanes per row (D / 8 of them hold data)
@@ -138,7 +138,7 @@ struct SumParts {
 
 template <bool kParts>   // (an instance of its own: the stream alone needs fewer registers)
 __global__ void __launch_bounds__(256)
-bwd_finalize_kernel(const float4* __restrict__ acc, uint2* __restrict__ dq, size_t n4, float scale,
+bwd_finalize_kernel(const float4* acc, uint2* dq, size_t n4, float scale,
                     unsigned dq_blocks, SumParts sp) {
   launch_dependents();
   dependency_wait();

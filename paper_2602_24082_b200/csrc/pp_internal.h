@@ -326,6 +326,8 @@ inline bool device_is_sm100() {
 // allocation) runs under the tail of the one before, or under all of it where that calls
 // launch_dependents first thing (plan, preprocess, finalize).  (Kernels that know nothing of this, in
 // front or behind, see ordinary stream order.)
+// Such a kernel is resident while the one in front still writes what it will read: its pointers carry no
+// __restrict__, which would promise that those values do not change meanwhile.
 // The main kernels take it up to kOverlapUnits units per SM: steps of 60 - 100 us gain 5 -
 // 9 % (144 ... 1054 tokens), one of 180 us 2.5 %, one of 500 us nothing, and a forward and
 // backward of 2600 and 1100 units (T 16384, 32 / 8 heads, D 64) lost 2 %.  Preprocess and finalize always take it,

@@ -56,9 +56,9 @@ __device__ __forceinline__ void for_tokens(int a, int b, int w, int nw, F f) {
 
 template <int kGang>
 __global__ void __launch_bounds__(kLossThreads)
-preference_loss_kernel(LossPtrs p, const float* __restrict__ logp, const float* __restrict__ ref,
-                       float beta, float* __restrict__ resp_logp, float* resp_reward,
-                       float* __restrict__ grp_loss, float* __restrict__ d_logp, int team_warps) {
+preference_loss_kernel(LossPtrs p, const float* logp, const float* ref,
+                       float beta, float* resp_logp, float* resp_reward,
+                       float* grp_loss, float* d_logp, int team_warps) {
   dependency_wait();
   // (two buffers each, in turn: one barrier per round)
   __shared__ double s_sum[2][kLossWarps], s_ref[2][kLossWarps];

@@ -44,7 +44,7 @@ __device__ __forceinline__ int position_of(const SegPtrs& p, int t) {
   return prompt ? in_seg : p.grp_prompt_len[g] + in_seg;
 }
 
-__global__ void position_ids_kernel(SegPtrs p, int32_t* __restrict__ pos) {
+__global__ void position_ids_kernel(SegPtrs p, int32_t* pos) {
   launch_dependents();
   dependency_wait();
   if (p.header[0] != kStatusOk) return;
@@ -57,7 +57,7 @@ __global__ void position_ids_kernel(SegPtrs p, int32_t* __restrict__ pos) {
 // once per token and reused for every Q and K head.
 template <int D>
 __global__ void __launch_bounds__(256)
-rope_kernel(SegPtrs p, __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, int Hq,
+rope_kernel(SegPtrs p, __nv_bfloat16* q, __nv_bfloat16* k, int Hq,
             int Hkv, float log2_base) {
   dependency_wait();
   if (p.header[0] != kStatusOk) return;

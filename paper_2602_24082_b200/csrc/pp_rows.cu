@@ -86,7 +86,7 @@ __device__ __forceinline__ long long weight_of(int2 k) { return static_cast<long
 
 template <typename Item>
 __global__ void __launch_bounds__(kRankKeys * kRankSlices)
-rank_kernel(int n, const Item* __restrict__ items, int32_t* __restrict__ order, RowsPtrs p) {
+rank_kernel(int n, const Item* items, int32_t* order, RowsPtrs p) {
   constexpr bool kGroups = sizeof(Item) == sizeof(int2) && !std::is_same_v<Item, long long>;
   using Key = decltype(key_of(Item{}));
   using Sum = decltype(weight_of(Item{}));
@@ -368,10 +368,10 @@ __global__ void __launch_bounds__(1024) rows_pack_kernel(RowsPtrs p) {
 constexpr int kMaxAssignRanks = 1024;
 
 template <int kPerLane>
-__device__ __forceinline__ void assign_one_by_one(int R, int ranks, const long long* __restrict__ cost,
-                                                  const int32_t* __restrict__ order,
-                                                  int32_t* __restrict__ rank_of_row,
-                                                  long long* __restrict__ rank_cost) {
+__device__ __forceinline__ void assign_one_by_one(int R, int ranks, const long long* cost,
+                                                  const int32_t* order,
+                                                  int32_t* rank_of_row,
+                                                  long long* rank_cost) {
   constexpr long long kInf = 0x7fffffffffffffffLL;
   const int lane = threadIdx.x;
   long long load[kPerLane];
@@ -434,9 +434,9 @@ __device__ __forceinline__ void assign_one_by_one(int R, int ranks, const long l
 constexpr int kBatchRows = 1024, kBatchThreads = 256;
 template <int kN>   // ranks at most; a multiple of 32 threads work, one warp without barriers
 __global__ void __launch_bounds__(kBatchThreads)
-assign_batch_kernel(int R, int ranks, const long long* __restrict__ cost,
-                    const int32_t* __restrict__ order, int32_t* __restrict__ rank_of_row,
-                    long long* __restrict__ rank_cost) {
+assign_batch_kernel(int R, int ranks, const long long* cost,
+                    const int32_t* order, int32_t* rank_of_row,
+                    long long* rank_cost) {
   using Key = unsigned long long;
   constexpr int kWork = kN < 32 ? 32 : kN;
   __shared__ Key s_cost[kBatchRows];
@@ -511,8 +511,8 @@ assign_batch_kernel(int R, int ranks, const long long* __restrict__ cost,
 
 // One rank: all rows and their sum.
 __global__ void __launch_bounds__(1024)
-assign_single_kernel(int R, const long long* __restrict__ cost, int32_t* __restrict__ rank_of_row,
-                     long long* __restrict__ rank_cost) {
+assign_single_kernel(int R, const long long* cost, int32_t* rank_of_row,
+                     long long* rank_cost) {
   __shared__ unsigned long long s_sum;
   if (threadIdx.x == 0) s_sum = 0;
   dependency_wait();
@@ -532,9 +532,9 @@ assign_single_kernel(int R, const long long* __restrict__ cost, int32_t* __restr
 // More ranks than the lanes' registers hold: the loads in shared memory, the lanes sharing the
 // search for the least one.
 __global__ void __launch_bounds__(32)
-assign_greedy_smem_kernel(int R, int ranks, const long long* __restrict__ cost,
-                          const int32_t* __restrict__ order, int32_t* __restrict__ rank_of_row,
-                          long long* __restrict__ rank_cost) {
+assign_greedy_smem_kernel(int R, int ranks, const long long* cost,
+                          const int32_t* order, int32_t* rank_of_row,
+                          long long* rank_cost) {
   __shared__ long long s_load[kMaxAssignRanks];
   dependency_wait();
   const int lane = threadIdx.x;

@@ -36,3 +36,16 @@ def test_tensor_memory_is_handed_back_behind_a_fence():
         assert places
         for at in places:
             assert re.search(r"tc_fence_before\(\);\s*__syncwarp\(\);\s*if \(lane == 0\) $", main[:at]), bar
+
+
+def test_kernels_that_start_early_promise_nothing_about_their_inputs():
+    """A kernel that waits for the one in front is resident while its inputs are still written: pointers that
+    are restrict would let loads be moved before the wait."""
+    early = 0
+    for name in sorted(os.listdir(CSRC)):
+        if name.endswith(".cu"):
+            for kernel in _source(name).split("__global__")[1:]:
+                if "dependency_wait();" in kernel:
+                    early += 1
+                    assert "__restrict__" not in kernel, (name, kernel[:120])
+    assert early >= 12
