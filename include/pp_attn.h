@@ -144,6 +144,12 @@ int pp_plan_read_bwd_tiles(const pp_plan* plan, pp_stream_t stream, int32_t* num
  * the order it takes them in.)  Neither call writes to the plan.  Synchronises `stream`. */
 int pp_plan_read_bwd_units(const pp_plan* plan, pp_stream_t stream, int32_t* units);
 int pp_plan_read_bwd_sched(const pp_plan* plan, pp_stream_t stream, int32_t* units);
+/* How pp_attn_fwd takes its query tiles.  *mode: 0 = each tile of a segment by itself, 1 = tiles that
+ * may hold rows of several segments, 2 = as 0, but the head that an odd number of query heads per KV head
+ * leaves without a partner may take two tiles of a segment at a time; then tile_units (may be NULL;
+ * pp_plan_max_tiles entries) receives per tile 0 = taken with the tile behind it, 1 = alone, 2 = with the
+ * tile before it.  Synchronises `stream`. */
+int pp_plan_read_fwd_units(const pp_plan* plan, pp_stream_t stream, int32_t* mode, uint8_t* tile_units);
 int pp_plan_read(const pp_plan* plan, pp_stream_t stream, int32_t* num_tiles, int32_t* tiles,
                  int32_t* fwd_order, int32_t* bwd_order, int32_t* key_end);
 

@@ -30,7 +30,7 @@ EXPORTS = ["pp_plan_workspace_bytes", "pp_build_plan", "pp_plan_status", "pp_des
            "pp_last_launch_count", "pp_error_string", "pp_step_host_arena_bytes", "pp_step_host_runs",
            "pp_attn_step_host", "pp_profile_enable", "pp_profile_read", "pp_profile_read_all",
            "pp_attn_bwd_noalloc", "pp_attn_bwd_noalloc_max_bytes", "pp_plan_read_bwd_units",
-           "pp_plan_read_bwd_sched", "pp_plan_read_bwd_tiles", "pp_attn_bwd_deterministic",
+           "pp_plan_read_bwd_sched", "pp_plan_read_fwd_units", "pp_plan_read_bwd_tiles", "pp_attn_bwd_deterministic",
            "pp_position_ids", "pp_rope_qk", "pp_preference_loss",
            "pp_build_rows_workspace_bytes", "pp_build_rows", "pp_assign_rows",
            "pp_debug_expire_wait"]
@@ -76,6 +76,7 @@ def lib() -> ctypes.CDLL:
         L.pp_plan_max_tiles.argtypes = [vp]
         L.pp_plan_read_bwd_units.argtypes = [vp, vp, vp]
         L.pp_plan_read_bwd_sched.argtypes = [vp, vp, vp]
+        L.pp_plan_read_fwd_units.argtypes = [vp, vp, vp, vp]
         L.pp_plan_read_bwd_tiles.argtypes = [vp, vp, vp, vp]
         L.pp_plan_read.argtypes = [vp, vp, vp, vp, vp, vp, vp]
         L.pp_attn_fwd.argtypes = [vp, vp, vp, vp, ctypes.c_float, vp, vp, vp, sz, vp]
@@ -210,6 +211,14 @@ class Plan:
     def read_bwd_sched(self, num_tiles: int) -> np.ndarray:
         """The order in which pp_attn_bwd takes them."""
         return self._read_units("pp_plan_read_bwd_sched", num_tiles)
+
+    def read_fwd_units(self, num_tiles: int) -> Tuple[int, np.ndarray]:
+        """How pp_attn_fwd takes its query tiles: (mode, per tile what is taken with it in mode 2)."""
+        mode = ctypes.c_int32(0)
+        units = np.ones(lib().pp_plan_max_tiles(self.handle), dtype=np.uint8)
+        _check(lib().pp_plan_read_fwd_units(self.handle, _stream(), ctypes.byref(mode), units.ctypes.data),
+               "pp_plan_read_fwd_units")
+        return mode.value, units[:num_tiles]
 
     def _read_units(self, call: str, num_tiles: int) -> np.ndarray:
         mt = lib().pp_plan_max_tiles(self.handle)

@@ -107,7 +107,8 @@ static int build_plan(const pp_problem* problem, const pp_problem* whole, void* 
     if (rc) return rc;
   }
   // first call that touches a device: everything above is host-side validation
-  if (!pp::device_is_sm100()) return PP_ERR_UNSUPPORTED;
+  const int sms = pp::sm100_sms();
+  if (!sms) return PP_ERR_UNSUPPORTED;
   pp_plan* plan = new (std::nothrow) pp_plan;
   if (!plan) return PP_ERR_CUDA;
   plan->prob = *problem;
@@ -117,6 +118,7 @@ static int build_plan(const pp_problem* problem, const pp_problem* whole, void* 
   plan->lay = lay;
   plan->fwd_scratch = 0;
   plan->mixed = pp::fwd_mixed_tiles(*whole);
+  plan->paired = !plan->mixed && pp::fwd_paired_tiles(*problem, sms);
   plan->lg_split = pp::bwd_split_log2(*whole);
   plan->bwd_scratch = pp::bwd_scratch_layout(*problem, plan->lg_split).total;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
@@ -168,6 +170,18 @@ int pp_destroy_plan(pp_plan* plan) {
 }
 
 int pp_plan_max_tiles(const pp_plan* plan) { return plan ? plan->max_tiles : PP_ERR_INVALID_ARG; }
+
+int pp_plan_read_fwd_units(const pp_plan* plan, pp_stream_t stream, int32_t* mode, uint8_t* tile_units) {
+  if (!plan || !mode) return PP_ERR_INVALID_ARG;
+  *mode = plan->mixed ? 1 : plan->paired ? 2 : 0;
+  if (!plan->paired || !tile_units) return PP_OK;
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  if (cudaMemcpyAsync(tile_units, plan->ws + plan->lay.tile_unit, plan->max_tiles, cudaMemcpyDeviceToHost, s) !=
+          cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    return PP_ERR_CUDA;
+  return PP_OK;
+}
 
 int pp_plan_read_bwd_sched(const pp_plan* plan, pp_stream_t stream, int32_t* units) {
   if (!plan || !units) return PP_ERR_INVALID_ARG;

@@ -819,7 +819,7 @@ cudaError_t launch_fwd_t(const pp_plan* plan, const CUtensorMap& tq, const CUten
   const pp_problem& pb = plan->prob;
   const int r = pb.num_q_heads / pb.num_kv_heads;
   const long long units = (long long)plan->max_tiles * pb.num_kv_heads * ((r + 1) / 2);
-  const Kernel kern = kerns[plan->mixed ? kMixedTiles : fwd_paired_tiles(pb, num_sms) ? kPairedTiles : kPlain];
+  const Kernel kern = kerns[plan->mixed ? kMixedTiles : plan->paired ? kPairedTiles : kPlain];
   dim3 grid(unsigned(std::min<long long>(units, num_sms)));
   ProfileEvents& ev = profile_events();
   const int slot = int(ev.fwd_count % kProfileRing);

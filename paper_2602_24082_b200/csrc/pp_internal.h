@@ -24,7 +24,8 @@ struct Tile {
 };
 static_assert(sizeof(Tile) == 32, "tile record is 32 bytes");
 // What the forward does with a query tile of a segment where it takes them by twos: nothing (the tile
-// behind it has it), this tile alone (a segment's last), or the tile before it and this one.
+// behind it has it), this tile alone (a segment's last, and the longest: pair_pays), or the tile before it
+// and this one.
 enum kTileUnit : uint8_t { kTileNone = 0, kTileAlone = 1, kTileWithLast = 2 };
 __host__ __device__ constexpr uint8_t tile_unit_of(int rel, int count) {   // tile `rel` of a segment's `count`
   return rel & 1 ? kTileWithLast : rel + 1 == count ? kTileAlone : kTileNone;
@@ -63,7 +64,8 @@ constexpr int kQTilePrompt = 256;
 // Words of the plan header (int32[16]).
 constexpr int kHdrStatus = 0, kHdrDetail = 1, kHdrNumTiles = 2, kHdrNumSegments = 3,
               kHdrNumBTiles = 8, kHdrNumQTiles = 9,
-              kHdrSchedTail = 10;   // (multi-kernel plan) tiles of the last of the smaller blocks
+              kHdrSchedTail = 10,   // (multi-kernel plan) tiles of the last of the smaller blocks
+              kHdrFwdWork = 12;     // ... and the forward tiles' works, 64 bits
 
 // Status word values written by device code.
 enum : int32_t {
@@ -114,6 +116,7 @@ struct pp_plan {
   // scratch sizes
   size_t fwd_scratch, bwd_scratch;
   bool mixed;     // the forward runs over mixed query tiles (fwd_mixed_tiles)
+  bool paired;    // ... takes tiles of a segment by twos (fwd_paired_tiles)
   int lg_split;   // log2 of the parts each backward unit is cut into (bwd_split_log2)
   // backward scratch whose dQ accumulator the latest forward on this plan has cleared
   mutable const void* cleared_scratch = nullptr;
@@ -149,7 +152,8 @@ inline bool fwd_mixed_tiles(const pp_problem& p) {
 // Whether the forward takes two tiles of a segment into a unit's slots for the last head of an odd number
 // of heads per KV head (each row's arithmetic is the same either way).  A unit with both slots filled
 // takes 1.4 times one with slot 1 empty, so it pays once there is more work per SM than the
-// longest such unit, in key tiles estimated from the mean group: 12000 tokens in 3000-token groups, 16 / 16 heads, D 128
+// longest such unit, in key tiles estimated from the mean group (the plan, which knows the groups, leaves
+// those alone that are longer: pair_pays there): 12000 tokens in 3000-token groups, 16 / 16 heads, D 128
 // 291 -> 204 us, 2600-token groups, D 96 225 -> 165; but 8000-token groups, 2 / 2 heads 166 -> 182.  With three and
 // more heads per KV head the other units take that long anyway: 20187 tokens, 28 / 4 631 -> 594.
 inline bool fwd_paired_tiles(const pp_problem& p, int sms) {
@@ -314,10 +318,10 @@ inline DeviceSetup* device_setup(DeviceSetup* table) {
 }
 // The kernels are sm_100a code (tcgen05, tensor memory): any other device is refused before a
 // launch is attempted.  Checked once per device.
-inline bool device_is_sm100() {
+inline int sm100_sms() {   // SMs of the current device; 0 if it is another kind
   static DeviceSetup probe[kMaxDevices];
   DeviceSetup* d = device_setup(probe);
-  return d && d->cc_major == 10;
+  return d && d->cc_major == 10 ? d->num_sms : 0;
 }
 
 // Launches a kernel, with `overlap` so that it may start before the kernel in front of it on the

@@ -33,7 +33,10 @@ struct PlanPtrs {
   int32_t* seg_start;
   int32_t* seg_tile0;
   Tile* tiles;
-  uint8_t* tile_unit;
+  uint8_t* tile_unit;   // null: not wanted
+  int sms;
+  int pair_cost, unit_cost;  // tenths per key tile of a unit with two tiles and of all units of a query
+                             //   tile and KV head (see pair_pays)
   int32_t* grp_btile0;
   BTile* btiles;
   int32_t* fwd_order;
@@ -244,7 +247,21 @@ __device__ __forceinline__ void add_grid_gain(const PlanPtrs& p, int g, int gain
             static_cast<unsigned long long>(static_cast<long long>(gain)));
 }
 
-__device__ __forceinline__ void plan_tile_body(const PlanPtrs& p, int t) {
+// Whether two query tiles of a segment go into one unit, by the key tiles of the second and of the whole
+// forward: such a unit takes 1.4 times as long as that tile alone (1.6 times at head_dim 64), which must not
+// be longer than every SM's share of everything.  So the longest tiles of uneven batches stay alone.  All by
+// twos -> none -> by this rule: one group of 6000 tokens and thirty of 600, 3 / 3 heads, D 64 69.6 -> 53.2 -> 51.2
+// us; 14384 and forty of 600, 2 / 2, D 128 161.9 -> 149.5 -> 145.4; 20000 and a hundred of 300, 1 / 1
+// 212.8 -> 188.5 -> 188.4; the same, 2 / 2 225.4 -> 253.9 -> 204.8.  Even batches go by twos as before.
+__device__ __forceinline__ bool pair_pays(const PlanPtrs& p, int work, long long all_work) {
+  return (long long)p.pair_cost * p.sms * work <= p.Hkv * all_work * p.unit_cost;
+}
+// ... for a tile of `work` of which tile_unit_of says `unit` (the tile behind it has one key tile more)
+__device__ __forceinline__ uint8_t settled_unit(const PlanPtrs& p, uint8_t unit, int work, long long all_work) {
+  return pair_pays(p, work + (unit == kTileNone), all_work) ? unit : uint8_t(kTileAlone);
+}
+
+__device__ __forceinline__ int plan_tile_body(const PlanPtrs& p, int t) {
   int s = upper_segment(p.seg_tile0, p.nseg, t);
   // segments with zero tiles cannot exist (len >= 1), so seg_tile0 is strictly increasing
   int g = group_of_segment(p, s);
@@ -268,15 +285,21 @@ __device__ __forceinline__ void plan_tile_body(const PlanPtrs& p, int t) {
   }
   tl.work = (tl.kv0_len + kTile - 1) / kTile + (tl.kv1_len + kTile - 1) / kTile + 1;
   p.tiles[t] = tl;
-  p.tile_unit[t] = tile_unit_of(t - p.seg_tile0[s], p.seg_tile0[s + 1] - p.seg_tile0[s]);
+  if (p.tile_unit) p.tile_unit[t] = tile_unit_of(t - p.seg_tile0[s], p.seg_tile0[s + 1] - p.seg_tile0[s]);
   if (p.qtiles) add_grid_gain(p, g, tile_cost(tl.work));
+  return tl.work;
 }
 
 __global__ void plan_tiles_kernel(PlanPtrs p) {
   if (p.header[0] != kStatusOk) return;
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (p.qtiles && t < work_slots(p)) p.work_at[t] = 0;
-  if (t < p.header[2]) plan_tile_body(p, t);
+  const int work = t < p.header[2] ? plan_tile_body(p, t) : 0;
+  if (p.tile_unit) {
+    const int sum = __reduce_add_sync(0xffffffffu, work);
+    if ((threadIdx.x & 31) == 0)
+      atomicAdd(reinterpret_cast<unsigned long long*>(p.header + kHdrFwdWork), static_cast<unsigned long long>(sum));
+  }
 }
 
 __device__ __forceinline__ void plan_key_end_body(const PlanPtrs& p, int j) {
@@ -359,6 +382,8 @@ __device__ __forceinline__ void plan_fwd_order_body(const PlanPtrs& p, int t, in
     rf += (of > wf) || (of == wf && u < t);
   }
   p.fwd_order[rf] = t;
+  if (p.tile_unit)
+    p.tile_unit[t] = settled_unit(p, p.tile_unit[t], wf, *reinterpret_cast<const long long*>(p.header + kHdrFwdWork));
 }
 
 // The query tiles' order by counting: tiles per work (plan_fwd_order_kernel), where each work begins
@@ -594,7 +619,7 @@ struct FusedSmem {
   uint16_t qwork[kMixed ? kFusedMaxTiles : 2];       // work of the query tiles, 0 where there is none
   uint16_t unit_tile[kFusedMaxTiles];   // backward tiles in the order of their units
   int32_t warp_sum[2][32];
-  int32_t status, detail, no_qtile, sched_tail;
+  int32_t status, detail, no_qtile, sched_tail, fwd_work;
 };
 
 // Inclusive sums of two values over the block.
@@ -731,7 +756,7 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
   }
   if (tid == 0) {
     sm.status = kStatusOk;
-    sm.detail = sm.no_qtile = sm.sched_tail = 0;
+    sm.detail = sm.no_qtile = sm.sched_tail = sm.fwd_work = 0;
   }
   if (kDesc > 1) dependency_wait();   // (the workspace may still be in use up to here)
   __syncthreads();
@@ -829,6 +854,8 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
   constexpr int kOrders = kMixed ? 4 : 3;
   uint32_t key[kOrders][2];
   for (int a = 0; a < kOrders; ++a) key[a][0] = key[a][1] = ~0u;
+  uint8_t unit[2];
+  int work = 0;
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     const int t = tid + nthr * r;
@@ -853,17 +880,28 @@ plan_fused_kernel(const __grid_constant__ DescBlock<kDesc> blk, PlanPtrs p) {
       }
       tl.work = (tl.kv0_len + kTile - 1) / kTile + (tl.kv1_len + kTile - 1) / kTile + 1;
       p.tiles[t] = tl;
-      p.tile_unit[t] = tile_unit_of(t - sm.seg_tile0[s], sm.seg_tile0[s + 1] - sm.seg_tile0[s]);
+      unit[r] = tile_unit_of(t - sm.seg_tile0[s], sm.seg_tile0[s + 1] - sm.seg_tile0[s]);
       sm.tile[0][t] = tl.start;
       sm.tile[1][t] = tl.start + tl.len;
       sm.tile[2][t] = tl.vis_end;
       key[0][r] = uint32_t(0xffff - tl.work) << 16 | uint32_t(t);
       if constexpr (kMixed) atomicAdd(&sm.grid_gain[g], tile_cost(tl.work));
+      work += tl.work;
     }
+  }
+  if (!kMixed && p.tile_unit) {
+    work = __reduce_add_sync(0xffffffffu, work);
+    if (lane == 0) atomicAdd(&sm.fwd_work, work);
   }
   for (int s = tid; s <= p.nseg; s += nthr) p.seg_start[s] = sm.seg_start[s];
   __syncthreads();
   const int nb = sm.btile0[p.G];
+  if (!kMixed && p.tile_unit) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+      if (tid + nthr * r < n)
+        p.tile_unit[tid + nthr * r] = settled_unit(p, unit[r], 0xffff - int(key[0][r] >> 16), sm.fwd_work);
+  }
   QTile q[2];
   // ---- backward tiles; key_end (every key of a forward tile ends its visibility at vis_end)
 #pragma unroll
@@ -1127,7 +1165,7 @@ cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cu
   p.seg_start = reinterpret_cast<int32_t*>(ws + l.seg_start);
   p.seg_tile0 = reinterpret_cast<int32_t*>(ws + l.seg_tile0);
   p.tiles = reinterpret_cast<Tile*>(ws + l.tiles);
-  p.tile_unit = reinterpret_cast<uint8_t*>(ws + l.tile_unit);
+  p.tile_unit = plan->paired ? reinterpret_cast<uint8_t*>(ws + l.tile_unit) : nullptr;
   p.grp_btile0 = reinterpret_cast<int32_t*>(ws + l.grp_btile0);
   p.btiles = reinterpret_cast<BTile*>(ws + l.btiles);
   p.fwd_order = reinterpret_cast<int32_t*>(ws + l.fwd_order);
@@ -1156,6 +1194,9 @@ cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cu
   if (!dev) return cudaErrorInvalidDevice;
   // (a set of the backward is held up with all its parts)
   p.det_asc_max = std::min(48, dev->num_sms / 3) >> plan->lg_split;
+  p.sms = dev->num_sms;
+  p.pair_cost = plan->prob.head_dim == 64 ? 16 : 14;   // (two heads in a unit: as much)
+  p.unit_cost = 10 + p.pair_cost * (plan->prob.num_q_heads / plan->prob.num_kv_heads / 2);
 
   const int mt = plan->max_tiles;
   // Host descriptors: up to kDescLarge entries travel as a kernel argument, which keeps the call
