@@ -452,14 +452,17 @@ __global__ void plan_fwd_order_kernel(PlanPtrs p) {
 // The blocks of the order that the kernel takes with several query heads per KV head
 // (bwd_takes_sched, which has the reasons).  The last block begins with the first group behind which
 // there are fewer than kSchedTailUnits units, or not enough work to balance its longest unit: with less
-// than two thirds of that unit behind it for each of 148 SMs, 12000 tokens in four groups (28 / 4 heads, D 64, 384 units)
-// took 490 us, all in one block 455.  `later`, `later_work` = tiles of the groups ranked behind a group of
-// `tiles` tiles, and their work.
+// than two thirds of that unit behind it for each of 148 SMs, 12000 tokens in four groups (28 / 4 heads, D 64,
+// 384 units) took 490 us, all in one block 455.  But for that it does not grow beyond a super-group: of 21883
+// tokens, 10844 in one group, at 32 / 8 heads, D 96, it took all 1424 units, whose data L2 does not hold: main
+// kernel and streams 1648 us, with the limit 1580; 8000 tokens and eight groups of 1000, 32 / 8 1355 -> 1295.
+// `later`, `later_work` = tiles of the groups ranked behind a group of `tiles` tiles, and their work.
 __device__ __forceinline__ bool sched_tail(const PlanPtrs& p, int later, int later_work, int tiles) {
-  return p.Hkv * later < kSchedTailUnits || (long long)p.Hkv * later_work < 100LL * tiles;
+  return p.Hkv * later < kSchedTailUnits || ((long long)p.Hkv * later_work < 100LL * tiles &&
+                                             p.Hkv * (later + tiles) <= kSuperGroupUnits);
 }
-// `tail` = tiles of the groups in the last block, `total` = of all.  (At most 1002 blocks, which the
-// one-block plan's sort keys have room for.)
+// `tail` = tiles of the groups in the last block, `total` = of all.  (At most 1007 blocks -- the divisor is
+// rounded down and at least 150 --, which the one-block plan's sort keys have room for.)
 __device__ __forceinline__ int sched_block(const PlanPtrs& p, int later, int tail, int total) {
   return later < tail ? 0 : 1 + p.Hkv * (later - tail) / max(kSchedBlockUnits, p.Hkv * total / 1000);
 }

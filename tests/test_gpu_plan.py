@@ -144,13 +144,28 @@ def test_backward_units_order(w):
     (1100, 5, 6, 2), (12, 1000, 280, 70), (300, 650, 210, 70)])
 def test_order_the_backward_takes_its_units_in(groups, length, hq, hkv):
     """From three query heads per KV head and 200 units on: groups by decreasing work, the last 200 units and
-    what balances longer ones before them in one block, the others in blocks of 150 (larger beyond 1000
-    blocks), inside a block longest first with all KV heads of a tile adjacent.  Below that: the order of read_bwd_units.  Plans in one block by
-    counting (up to 512 tiles) and by sorting, and of several kernels."""
-    from paper_2602_24082_b200 import binding as B
+    what balances longer ones before them, up to 600 units, in one block, the others in blocks of 150 (larger
+    beyond 1000 blocks), inside a block longest first with all KV heads of a tile adjacent.  Below that: the
+    order of read_bwd_units.  Plans in one block by counting (up to 512 tiles) and by sorting, and of several
+    kernels."""
     rng = np.random.default_rng(groups)
     pick = lambda: int(rng.integers(1, 2 * length // 3 + 1))
-    w = W.Workload("sched", [[(pick(), (pick(), pick()))] for _ in range(groups)], hq, hkv, 64, seed=1)
+    _check_backward_order(W.Workload("sched", [[(pick(), (pick(), pick()))] for _ in range(groups)], hq, hkv, 64, seed=1))
+
+
+@pytest.mark.parametrize("lens,hq,hkv,blocks", [
+    ([10844] + [1380] * 8, 32, 8, {0, 1, 2, 3}),   # long units, and more than 600 of them in the first two groups
+    ([3000] * 4, 28, 4, {0, 1}), ([2900] * 7, 28, 4, {0, 1, 2})])
+def test_long_units_do_not_merge_more_than_600(lens, hq, hkv, blocks):
+    """A block that grows to balance a long unit stays within what L2 can serve."""
+    third = lambda x: (x - 2 * (x // 3), (x // 3, x // 3))
+    assert _check_backward_order(W.Workload("merge", [[third(x)] for x in lens], hq, hkv, 64, seed=1)) == blocks
+
+
+def _check_backward_order(w):
+    """Checks the order; returns the set of its blocks."""
+    from paper_2602_24082_b200 import binding as B
+    hq, hkv = w.num_q_heads, w.num_kv_heads
     plan = B.plan_for(w)
     assert plan.status() == (0, 0)
     btiles = plan.read_bwd_tiles()
@@ -158,7 +173,7 @@ def test_order_the_backward_takes_its_units_in(groups, length, hq, hkv):
     units = plan.read_bwd_sched(n)
     if hq // hkv < 3:
         assert np.array_equal(units, plan.read_bwd_units(n))
-        return
+        return {0}
     work, grp = btiles[:, 6].tolist(), btiles[:, 4].tolist()
     gwork, gtiles = {}, {}
     for g, x in zip(grp, work):
@@ -166,7 +181,7 @@ def test_order_the_backward_takes_its_units_in(groups, length, hq, hkv):
     behind, tail, later, later_work = {}, 0, 0, 0
     for g in sorted(gwork, key=lambda g: (gwork[g], -g)):     # from the last
         behind[g] = later
-        if hkv * later < 200 or hkv * later_work < 100 * gtiles[g]:
+        if hkv * later < 200 or (hkv * later_work < 100 * gtiles[g] and hkv * (later + gtiles[g]) <= 600):
             tail = later + gtiles[g]
         later, later_work = later + gtiles[g], later_work + gwork[g]
     block = {g: 0 if x < tail else 1 + hkv * (x - tail) // max(150, hkv * n // 1000) for g, x in behind.items()}
@@ -174,6 +189,7 @@ def test_order_the_backward_takes_its_units_in(groups, length, hq, hkv):
     expect = sorted(range(n), key=lambda t: (-block[grp[t]], -work[t], t))
     assert units[:, 1].tolist() == np.repeat(expect, hkv).tolist()
     assert (units[:, 0].reshape(n, hkv) == np.arange(hkv)).all()
+    return set(block.values())
 
 
 @pytest.mark.parametrize("rows,hq,hkv", [([[(700, (300, 200))]] * 40, 8, 2), ([[(60, (20, 11))]] * 1500, 6, 2), ([[(300, (90,))]] * 3, 2, 2)])
