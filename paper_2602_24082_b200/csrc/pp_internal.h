@@ -88,8 +88,8 @@ struct PlanLayout {
   size_t btiles;     // BTile[max_tiles]  (at most max_btiles_of of them)
   size_t bwd_order;  // int32[max_tiles]  backward tiles, longest work first
   size_t tile_gwork; // int32[max_tiles]  backward work of the backward tile's whole group
-  size_t tile_sgroup; // int32[max_tiles] super-group (block of consecutive groups)
-  size_t tile_sblock; // int32[max_tiles] tiles of the groups behind the tile's, for its smaller block
+  size_t tile_block; // int32[max_tiles] super-group (block of consecutive groups) or, for the smaller blocks,
+                     //   tiles of the groups behind the tile's
   size_t bwd_units;  // int32[max_tiles * Hkv]  (kv head << 24) | backward tile, processing order
                      //   (in super-groups or, with bwd_takes_sched, in smaller blocks)
   size_t bwd_units_det;  // the same units, one (group, KV head) set after the other and inside a
@@ -182,8 +182,7 @@ inline PlanLayout plan_layout(const pp_problem& p) {
   l.btiles = off;    off = align_up(off + sizeof(BTile) * size_t(mt), 256);
   l.bwd_order = off; off = align_up(off + sizeof(int32_t) * size_t(mt), 256);
   l.tile_gwork = off; off = align_up(off + sizeof(int32_t) * size_t(mt), 256);
-  l.tile_sgroup = off; off = align_up(off + sizeof(int32_t) * size_t(mt), 256);
-  l.tile_sblock = off; off = align_up(off + sizeof(int32_t) * size_t(mt), 256);
+  l.tile_block = off; off = align_up(off + sizeof(int32_t) * size_t(mt), 256);
   l.bwd_units = off; off = align_up(off + sizeof(int32_t) * size_t(mt) * size_t(p.num_kv_heads), 256);
   l.bwd_units_det = off;
   off = align_up(off + sizeof(int32_t) * size_t(mt) * size_t(p.num_kv_heads), 256);

@@ -42,8 +42,7 @@ struct PlanPtrs {
   int32_t* fwd_order;
   int32_t* bwd_order;
   int32_t* tile_gwork;
-  int32_t* tile_sgroup;
-  int32_t* tile_sblock;
+  int32_t* tile_block;
   int32_t* bwd_units;
   bool sched;           // in the smaller blocks (bwd_takes_sched)
   int32_t* bwd_units_det;
@@ -466,6 +465,16 @@ __device__ __forceinline__ bool sched_tail(const PlanPtrs& p, int later, int lat
 __device__ __forceinline__ int sched_block(const PlanPtrs& p, int later, int tail, int total) {
   return later < tail ? 0 : 1 + p.Hkv * (later - tail) / max(kSchedBlockUnits, p.Hkv * total / 1000);
 }
+// The values [lo, hi) of `later` that fall into the same block.  (The plan of several kernels compares every
+// pair of tiles: with a division for each, and groups' works added up tile by tile, a plan of 300000 tokens in
+// 1000 groups took 981 us, now 685.)
+__device__ __forceinline__ void sched_block_range(int Hkv, int later, int tail, int total, int& lo, int& hi) {
+  lo = 0, hi = tail;
+  if (later < tail) return;
+  const int unit = max(kSchedBlockUnits, Hkv * total / 1000), q = Hkv * (later - tail) / unit;
+  lo = tail + (q * unit + Hkv - 1) / Hkv;
+  hi = tail + ((q + 1) * unit + Hkv - 1) / Hkv;
+}
 
 // bwd_order (plain longest-first list of the backward tiles) and each tile's group work
 __device__ __forceinline__ void plan_gwork_body(const PlanPtrs& p, int t, int n) {
@@ -481,38 +490,37 @@ __device__ __forceinline__ void plan_gwork_body(const PlanPtrs& p, int t, int n)
 }
 
 __device__ __forceinline__ void plan_sgroup_body(const PlanPtrs& p, int t, int n) {
-  const int gs = p.btiles[t].grp_start, gw = p.tile_gwork[t];
-  // tiles of this group and of the groups that come later; of those alone, and their work
-  int rest = 0, later = 0, later_work = 0;
-  for (int u = 0; u < n; ++u) {
-    const int ogs = p.btiles[u].grp_start, ow = p.tile_gwork[u];
-    const bool behind = (ow < gw) || (ow == gw && ogs > gs);
-    rest += (ogs == gs) || behind;
-    later += behind;
-    if (behind) later_work += p.btiles[u].work;
+  const BTile me = p.btiles[t];
+  const int gw = p.tile_gwork[t];
+  // tiles and work of the groups that come later
+  int later = 0, later_work = 0;
+#pragma unroll 4
+  for (int g = 0; g < p.G; ++g) {
+    const int first = p.grp_btile0[g], ow = p.tile_gwork[first];
+    if (ow < gw || (ow == gw && first > t)) {
+      later += p.grp_btile0[g + 1] - first;
+      later_work += ow;
+    }
   }
-  p.tile_sblock[t] = later;
-  if (sched_tail(p, later, later_work, rest - later)) atomicMax(&p.header[kHdrSchedTail], rest);
-  // counted from the END of the list, so the last block is never a small leftover whose
-  // long units would start late: blocks are processed in decreasing index
-  p.tile_sgroup[t] = (p.Hkv * rest - 1) / kSuperGroupUnits;
+  const int own = (me.grp_end - me.grp_start + kTile - 1) / kTile, rest = later + own;
+  if (!p.sched) {
+    // counted from the END of the list, so the last block is never a small leftover whose
+    // long units would start late: blocks are processed in decreasing index
+    p.tile_block[t] = (p.Hkv * rest - 1) / kSuperGroupUnits;
+  } else {
+    p.tile_block[t] = later;
+    if (sched_tail(p, later, later_work, own)) atomicMax(&p.header[kHdrSchedTail], rest);
+  }
 }
 
 __device__ __forceinline__ void plan_units_body(const PlanPtrs& p, int t, int n) {
-  const int wb = p.btiles[t].work;
+  const int wb = p.btiles[t].work, mine = p.tile_block[t];
+  int lo = mine, hi = mine + 1;   // the values of tile_block in this tile's block
+  if (p.sched) sched_block_range(p.Hkv, mine, p.header[kHdrSchedTail], n, lo, hi);
   int pos = 0;
-  if (!p.sched) {
-    const int sg = p.tile_sgroup[t];
-    for (int u = 0; u < n; ++u) {
-      const int osg = p.tile_sgroup[u], ob = p.btiles[u].work;
-      pos += (osg > sg) || (osg == sg && ((ob > wb) || (ob == wb && u < t)));
-    }
-  } else {
-    const int tail = p.header[kHdrSchedTail], sb = sched_block(p, p.tile_sblock[t], tail, n);
-    for (int u = 0; u < n; ++u) {
-      const int osb = sched_block(p, p.tile_sblock[u], tail, n), ob = p.btiles[u].work;
-      pos += (osb > sb) || (osb == sb && ((ob > wb) || (ob == wb && u < t)));
-    }
+  for (int u = 0; u < n; ++u) {
+    const int other = p.tile_block[u], ob = p.btiles[u].work;
+    pos += (other >= hi) || (other >= lo && ((ob > wb) || (ob == wb && u < t)));
   }
   for (int kvh = 0; kvh < p.Hkv; ++kvh) p.bwd_units[p.Hkv * pos + kvh] = (kvh << 24) | t;
   // Deterministic order: one (group, KV head) set after the other, groups by decreasing work.
@@ -1174,8 +1182,7 @@ cudaError_t launch_plan(const pp_plan* plan, const int32_t* const* host_desc, cu
   p.fwd_order = reinterpret_cast<int32_t*>(ws + l.fwd_order);
   p.bwd_order = reinterpret_cast<int32_t*>(ws + l.bwd_order);
   p.tile_gwork = reinterpret_cast<int32_t*>(ws + l.tile_gwork);
-  p.tile_sgroup = reinterpret_cast<int32_t*>(ws + l.tile_sgroup);
-  p.tile_sblock = reinterpret_cast<int32_t*>(ws + l.tile_sblock);
+  p.tile_block = reinterpret_cast<int32_t*>(ws + l.tile_block);
   p.bwd_units = reinterpret_cast<int32_t*>(ws + l.bwd_units);
   p.sched = bwd_takes_sched(plan->prob);
   p.bwd_units_det = reinterpret_cast<int32_t*>(ws + l.bwd_units_det);

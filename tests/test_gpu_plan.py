@@ -162,6 +162,25 @@ def test_long_units_do_not_merge_more_than_600(lens, hq, hkv, blocks):
     assert _check_backward_order(W.Workload("merge", [[third(x)] for x in lens], hq, hkv, 64, seed=1)) == blocks
 
 
+def test_the_smaller_blocks_cost_a_large_plan_nothing():
+    """Plans of several kernels compare every pair of tiles: the two orders take about the same time."""
+    from paper_2602_24082_b200 import binding as B
+    times = []
+    for hq in (8, 32):
+        w = W.Workload("large", [[(400, (300, 300))]] * 1000, hq, 8, 128, seed=1)
+        ws = B.plan_for(w).workspace
+        best = 1e9
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            plan = B.pp_build_plan(w.descriptors(), hq, 8, 128, w.total_tokens, workspace=ws)
+            b.record()
+            assert plan.status() == (0, 0)
+            best = min(best, a.elapsed_time(b))
+        times.append(best)
+    assert times[1] <= 1.2 * times[0]
+
+
 def _check_backward_order(w):
     """Checks the order; returns the set of its blocks."""
     from paper_2602_24082_b200 import binding as B
