@@ -124,9 +124,16 @@ bwd_preprocess_kernel(const __nv_bfloat16* o, const __nv_bfloat16* d_o,
 // Hq = 32, D = 128 (227 MB): 44 us with one load per thread and a grid-stride loop, 38 / 33 with
 // 2 / 4 loads, 30 with the hints (7.5 TB/s, part of it from L2); T = 16384, Hq = 64: 154 -> 116.
 // Where units are cut into parts, the blocks behind these add up the parts of a (backward tile, KV
-// head), 32 rows of dV or dK each, all parts' loads in flight: 1556 tokens, 8 / 1 heads 41.5 -> 40.2 us a
-// step against four at a time, 251, 28 / 4 37.8 -> 37.0, 2830, 8 / 2 79.4 -> 79.1.
+// head), 32 rows of dV or dK each, with the loads of four or eight parts in flight (fin_parts).
 constexpr int kFinUnroll = 4;
+// Eight parts in flight shorten the sums, but take 78 registers instead of 40, which the whole stream pays
+// for: eight only where there are as many and the stream is about one wave of such blocks.
+// Whole steps, four -> eight: 251 tokens, 8 / 1 heads 33.9 -> 33.2 us, 1556 69.5 -> 68.7; backward with
+// preprocess and finalize, eight everywhere -> this rule: 14381 tokens, 14 / 2, D 96 212 -> 208, 5000, 28 / 4
+// 452 -> 448.
+inline int fin_parts(int lg_split, unsigned dq_blocks, int num_sms) {
+  return lg_split == 0 ? 0 : lg_split == 3 && dq_blocks <= 4u * num_sms ? 8 : 4;
+}
 struct SumParts {
   const float4* parts;
   const int32_t* header;
@@ -136,7 +143,7 @@ struct SumParts {
   int lg_split, Hkv, D;
 };
 
-template <bool kParts>   // (an instance of its own: the stream alone needs fewer registers)
+template <int kParts>   // (0: an instance of its own, the stream alone needs 26 registers)
 __global__ void __launch_bounds__(256)
 bwd_finalize_kernel(const float4* acc, uint2* dq, size_t n4, float scale,
                     unsigned dq_blocks, SumParts sp) {
@@ -171,18 +178,22 @@ bwd_finalize_kernel(const float4* acc, uint2* dq, size_t n4, float scale,
     const float4* src = sp.parts + ((size_t(unit) << sp.lg_split) * 2 + which) * (c4s * kTile) +
                         c * kTile + 32 * quarter + lane;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 x[8];   // (at most eight parts, all in flight)
+    constexpr int kIn = kParts ? kParts : 1;
+#pragma unroll 1
+    for (int first = 0; first < (1 << sp.lg_split); first += kIn) {
+      float4 x[kIn];
 #pragma unroll
-    for (int p = 0; p < 8; ++p)
-      if (p < (1 << sp.lg_split)) x[p] = src[size_t(p) * 2 * c4s * kTile];
+      for (int p = 0; p < kIn; ++p)
+        if (first + p < (1 << sp.lg_split)) x[p] = src[size_t(first + p) * 2 * c4s * kTile];
 #pragma unroll
-    for (int p = 0; p < 8; ++p)
-      if (p < (1 << sp.lg_split)) {
-        s.x += x[p].x;
-        s.y += x[p].y;
-        s.z += x[p].z;
-        s.w += x[p].w;
-      }
+      for (int p = 0; p < kIn; ++p)
+        if (first + p < (1 << sp.lg_split)) {
+          s.x += x[p].x;
+          s.y += x[p].y;
+          s.z += x[p].z;
+          s.w += x[p].w;
+        }
+    }
     s_out[lane][c] = make_uint2(pack_bf16(s.x * f, s.y * f), pack_bf16(s.z * f, s.w * f));
   }
   __syncthreads();
@@ -1057,8 +1068,10 @@ cudaError_t launch_bwd_t(const pp_plan* plan, const void* o, const float* lse, c
   unsigned fb = unsigned((n4 + 256 * kFinUnroll - 1) / (256 * kFinUnroll));
   const SumParts sp = {prm.parts, prm.header, prm.tiles, prm.dk, prm.dv, prm.lg_split, pb.num_kv_heads, DV};
   const unsigned sum_blocks = prm.lg_split ? unsigned(max_btiles_of(pb)) * pb.num_kv_heads * 8 : 0;
+  const int parts = fin_parts(prm.lg_split, fb, num_sms);
+  auto fin = parts == 8 ? bwd_finalize_kernel<8> : parts == 4 ? bwd_finalize_kernel<4> : bwd_finalize_kernel<0>;
   if (e == cudaSuccess)
-    e = launch_kernel(true, prm.lg_split ? bwd_finalize_kernel<true> : bwd_finalize_kernel<false>, dim3(fb + sum_blocks), dim3(256), 0, stream,
+    e = launch_kernel(true, fin, dim3(fb + sum_blocks), dim3(256), 0, stream,
                       reinterpret_cast<const float4*>(prm.dq_acc), static_cast<uint2*>(dq), n4, prm.scale, fb, sp);
   if (launches) *launches += 3;
   return e;

@@ -20,6 +20,7 @@ CASES = [
     ([[(640, (200, 73))]], 48, 8, 128, 4),                     # more parts than SMs, 1 or 2 heads each
     ([[(100, (90, 87))]], 64, 8, 128, 8),
     ([[(900, (700, 300, 148))]], 4, 1, 128, 4),                # units of 16 query tiles
+    ([[(1200, (700, 512))]], 8, 1, 128, 8),                    # dQ of more than 592 blocks: sums in two rounds
 ]
 
 
