@@ -540,7 +540,12 @@ assign_greedy_smem_kernel(int R, int ranks, const long long* cost,
   const int lane = threadIdx.x;
   for (int k = lane; k < ranks; k += 32) s_load[k] = 0;
   __syncwarp();
+  // (fetched ahead: the loads may not pass the stores of the row before; 3000 rows, 129 ranks 1264 -> 1115 us)
+  int row = order[0], row_next = R > 1 ? order[1] : 0;
+  long long c = cost[row];
   for (int i = 0; i < R; ++i) {
+    const long long c_next = i + 1 < R ? cost[row_next] : 0;
+    const int row_after = i + 2 < R ? order[i + 2] : 0;
     long long best = 0x7fffffffffffffffLL;
     int best_k = ranks;
     for (int k = lane; k < ranks; k += 32) {   // ascending k: the first minimum is kept
@@ -560,10 +565,12 @@ assign_greedy_smem_kernel(int R, int ranks, const long long* cost,
       }
     }
     if (lane == 0) {
-      const int row = order[i];
       rank_of_row[row] = best_k;
-      s_load[best_k] = best + cost[row];
+      s_load[best_k] = best + c;
     }
+    row = row_next;
+    row_next = row_after;
+    c = c_next;
     __syncwarp();
   }
   for (int k = lane; k < ranks; k += 32) rank_cost[k] = s_load[k];
