@@ -431,7 +431,43 @@ __device__ __forceinline__ void assign_one_by_one(int R, int ranks, const long l
 // memory side by side.  Bound by that chain, word -> place -> cost -> word.  972 rows to 8 ranks:
 // 35 us with the list sorted again every round, now 32; building and dealing out to 64 ranks 177 us with
 // one row at a time, now 68.
-constexpr int kBatchRows = 1024, kBatchThreads = 256;
+// Where ranks lie further apart than the rows are long, only the first few are in time: with more than 32 of
+// them a round that assigned less than a fifth of its places is followed by a stretch of rows one at a time, first
+// kStretchFirst, twice as many each time the round behind it is no better.  Rounds alone -> so: 300 rows, few long
+// ones, 33 ranks 98 -> 38 us (one at a time: 50), 3000 that fall by a ninth each, 100 ranks 636 -> 240 (350);
+// even costs are as fast as before with up to 64 ranks and 1 to 4 % slower with more.
+constexpr int kBatchRows = 1024, kBatchThreads = 256, kStretchFirst = 16, kStretchLast = 128;
+// One warp: the next rows one at a time.  `sorted`: the 32 kPerLane words in order, kPerLane to a lane; a row
+// takes the first, adds its cost and inserts it again.  The words return to key_of_rank.
+template <int kPerLane>
+__device__ __noinline__ void one_by_one_sorted(int rows, const unsigned long long* sorted, const unsigned long long* cost,
+                                                  const int32_t* row, int32_t* rank_of_row,
+                                                  unsigned long long* key_of_rank) {
+  constexpr unsigned long long kInf = ~0ull;
+  const int lane = threadIdx.x;
+  unsigned long long e[kPerLane];
+#pragma unroll
+  for (int j = 0; j < kPerLane; ++j) e[j] = sorted[lane * kPerLane + j];
+  for (int i = 0; i < rows; ++i) {
+    const unsigned long long least = __shfl_sync(0xffffffffu, e[0], 0), v = least + cost[i];
+    unsigned long long up = __shfl_down_sync(0xffffffffu, e[0], 1);   // the word behind my last one
+    if (lane == 31) up = kInf;
+    if (lane == 0) rank_of_row[row[i]] = int(least & 127u);
+    bool mine_before = lane == 0 || e[0] < v;   // (word 0 of lane 0 is taken out)
+#pragma unroll
+    for (int j = 0; j < kPerLane; ++j) {
+      const unsigned long long next = j + 1 < kPerLane ? e[j + 1] : up;
+      const bool next_before = next < v;
+      if (next_before) e[j] = next;
+      else if (mine_before) e[j] = v;
+      mine_before = next_before;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < kPerLane; ++j)
+    if (e[j] != kInf) key_of_rank[e[j] & 127u] = e[j];
+}
+
 template <int kN>   // ranks at most; a multiple of 32 threads work, one warp without barriers
 __global__ void __launch_bounds__(kBatchThreads)
 assign_batch_kernel(int R, int ranks, const long long* cost,
@@ -455,6 +491,7 @@ assign_batch_kernel(int R, int ranks, const long long* cost,
   };
   const bool mine = tid < ranks;
   Key key = mine ? Key(tid) : ~Key(0);
+  int count, stretch = 0, stretch_end;   // rows of the last round; rows one at a time, and their end
   for (int base = 0; base < R; base += kBatchRows) {
     const int m = min(kBatchRows, R - base);
     __syncthreads();
@@ -464,6 +501,8 @@ assign_batch_kernel(int R, int ranks, const long long* cost,
     }
     __syncthreads();
     if (tid >= kWork) continue;
+    count = kN;   // (the last round of a chunk says nothing)
+    stretch_end = -1;
     for (int pos = 0; pos < m;) {
       if (tid < kN) s_key[tid] = key;
       if (tid == 0) s_count = min(ranks, m - pos);
@@ -474,6 +513,22 @@ assign_batch_kernel(int R, int ranks, const long long* cost,
         const ulonglong2 o = *reinterpret_cast<const ulonglong2*>(&s_key[i]);
         place += int(o.x < key) + int(o.y < key);
       }
+      if constexpr (kN > 32) {
+        if (count < kN / 5) {
+          stretch = pos - count == stretch_end ? min(2 * stretch, kStretchLast) : kStretchFirst;
+          count = kN;
+          s_next[mine ? place : tid] = key;
+          sync();
+          const int rows = min(stretch, m - pos);
+          if (tid < 32) one_by_one_sorted<kN / 32>(rows, s_next, s_cost + pos, s_row + pos, rank_of_row, s_key);
+          sync();
+          if (mine) key = s_key[tid];
+          pos += rows;
+          stretch_end = pos;
+          sync();
+          continue;
+        }
+      }
       const bool there = mine && pos + place < m;
       const Key next = there ? key + s_cost[pos + place] : key;
       // every rank is in time if all that get a row end up behind the last one
@@ -483,7 +538,7 @@ assign_batch_kernel(int R, int ranks, const long long* cost,
         const Key last_key = __shfl_sync(0xffffffffu, key, last);
         all_in_time = __all_sync(0xffffffffu, !there || next > last_key);
       }
-      int count = min(ranks, m - pos);
+      count = min(ranks, m - pos);
       if (!all_in_time) {
         if (mine) s_next[place] = there ? next : ~Key(0);
         sync();

@@ -147,17 +147,41 @@ def test_assign_rows_at_the_edges_of_the_lane_lists(rows, ranks):
     assert np.array_equal(rank_cost.cpu().numpy(), want[2])
 
 
-@pytest.mark.parametrize("kind", ["equal", "zeros", "doubling", "huge", "mixed"])
-@pytest.mark.parametrize("rows,ranks", [(1, 32), (31, 31), (1024, 8), (1025, 32), (2500, 5), (2500, 1), (1100, 64), (1500, 127)])
+def _spread(rows):
+    """Costs that fall by a ninth from row to row, down to ones: the ranks end up far apart."""
+    return (1e11 * np.exp(-np.arange(rows) * 0.12)).astype(np.int64) + 1
+
+
+@pytest.mark.parametrize("kind", ["equal", "zeros", "doubling", "huge", "mixed", "spread", "giants"])
+@pytest.mark.parametrize("rows,ranks", [(1, 32), (31, 31), (1024, 8), (1025, 32), (2500, 5), (2500, 1), (1100, 64), (1500, 127),
+                                        (1100, 33), (2100, 65), (3000, 100), (1300, 128)])
 def test_assign_rows_in_rounds(rows, ranks, kind):
-    """Several rows a round: costs where all ranks take one, where only the first does, and sums too
-    large for load and rank in one word."""
+    """Several rows a round: costs where all ranks take one, where only the first few do (with more than 32
+    ranks rows then go one at a time for a while), and sums too large for load and rank in one word."""
     from paper_2602_24082_b200 import binding as B
     rng = np.random.default_rng(rows + ranks)
     cost = {"equal": np.full(rows, 17), "zeros": np.where(rng.random(rows) < 0.5, 0, 3),
             "doubling": 1 << (np.arange(rows) % 40), "huge": rng.integers(1 << 46, (1 << 62) // rows, rows),
-            "mixed": rng.integers(0, 1 << rng.integers(1, 30, rows))}[kind].astype(np.int64)
+            "mixed": rng.integers(0, 1 << rng.integers(1, 30, rows)), "spread": _spread(rows),
+            "giants": np.where(np.arange(rows) < ranks, _spread(rows), rng.integers(1000, 5000, rows))}[kind].astype(np.int64)
     order, rank_of_row, rank_cost = B.pp_assign_rows(torch.from_numpy(cost).cuda(), ranks)
     want = R.assign_rows(cost, ranks)
     for got, exact in zip((order, rank_of_row, rank_cost), want):
         assert np.array_equal(got.cpu().numpy(), exact)
+
+
+def test_ranks_far_apart_take_little_longer_than_even_ones():
+    from paper_2602_24082_b200 import binding as B
+    times = []
+    for cost in (np.arange(20000) + 1000, _spread(20000)):
+        c = torch.from_numpy(cost).cuda()
+        best = 1e9
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            B.pp_assign_rows(c, 33)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        times.append(best)
+    assert times[1] <= 2.4 * times[0]
