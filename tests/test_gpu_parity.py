@@ -162,20 +162,36 @@ def test_growing_scores_take_the_rescale_path(d):
     check_against_oracle(w, tens, _run_gpu(w, tens, for_backward=True))
 
 
+# one group of (300, (40, 20)): plain units; 8 such groups: mixed tiles; groups of 600: tiles of a segment by twos,
+# where the key lies before both tiles of a pair, inside the first and inside the second
+SPIKED = {"plain": ([[(300, (40, 20))]], 2, 1, 0), "mixed": ([[(300, (40, 20))]] * 8, 16, 8, 1),
+          "paired": ([[(600, (90,))]] * 3, 32, 32, 2)}
+
+
 @pytest.mark.parametrize("jump", [12.0, 200.0])   # log2 units: beyond the threshold; beyond fp32 without rescaling
-@pytest.mark.parametrize("at", [128, 175, 176, 191, 240, 255])
-def test_one_key_outgrows_the_reference(at, jump):
-    """One key of the second tile scores `jump` (log2) above everything before it, in a column of P
-    that is handed over early (the first 48 of each 64) or late (the last 16)."""
-    w = W.Workload("spike", [[(300, (40, 20))]], 2, 1, 64, seed=31)
+@pytest.mark.parametrize("mode,at", [("plain", a) for a in (128, 175, 176, 191, 240, 255)] +
+                         [("mixed", a) for a in (128, 175, 176, 255)] +
+                         [("paired", a) for a in (128, 176, 300, 383, 384, 511)])
+@pytest.mark.parametrize("d", [64, 96, 128])
+def test_one_key_outgrows_the_reference(d, mode, at, jump):
+    """One key behind the first tile scores `jump` (log2) above everything before it, in a column of P
+    that is handed over early (the first 48 of each 64) or late (the last 16); P has columns of its own at
+    head_dim 64 (not with mixed tiles) and lies over the scores otherwise."""
+    rows, hq, hkv, number = SPIKED[mode]
+    w = W.Workload("spike", rows, hq, hkv, d, seed=31)
+    from paper_2602_24082_b200 import binding as B
+    assert B.plan_for(w).read_fwd_units(0)[0] == number
     q, k, v, do = w.tensors()
-    u = torch.zeros(64)
-    u[::2] = 0.25   # |u|^2 = 2
-    a = (jump / (2 * w.softmax_scale * 1.4426950408889634)) ** 0.5
-    k[at] = (a * u).to(k.dtype)
+    u = torch.zeros(d)
+    u[::2] = 0.25   # |u|^2 = d / 32
+    a = (jump / (d / 32 * w.softmax_scale * 1.4426950408889634)) ** 0.5
+    spikes = torch.tensor(w.row_offsets()[:-1]) + at
     q = (0.1 * q.float() + a * u).to(q.dtype)
-    tens = (q, (k.float() * torch.where(torch.arange(len(k)) == at, 1.0, 0.05)[:, None, None]).to(k.dtype), v, do)
-    s = torch.einsum("qd,kd->qk", q[at:300, 0].float(), tens[1][:300, 0].float()) * w.softmax_scale * 1.4426950408889634
+    damped = 0.05 * k.float()
+    damped[spikes] = a * u
+    tens = (q, damped.to(k.dtype), v, do)
+    prompt = rows[0][0][0]
+    s = torch.einsum("qd,kd->qk", q[at:prompt, 0].float(), tens[1][:prompt, 0].float()) * w.softmax_scale * 1.4426950408889634
     assert (s[:, at] - s[:, :128].max(dim=1).values > 8).all()
     import oracle
     O, LSE = oracle.attn_fwd_bwd(w.descriptors(), *tens, w.softmax_scale)[:2]
