@@ -13,14 +13,14 @@
 // A work unit is (query tile, KV head, pair of query heads of that KV head): both slots see
 // the same keys and the same mask, so every K / V tile staged in shared memory feeds two
 // S tiles.  The last head of an odd number of heads per KV head, and every head where there is one
-// per KV head, takes two query tiles of a segment into the slots (kPaired below) or leaves slot 1 empty.  While one slot's warpgroup does its exponentials the tensor core works on the
-// other slot (order: PV_0(j), QK_0(j+1), PV_1(j), QK_1(j+1), ...).  P (bf16) overwrites columns
+// per KV head, takes two query tiles of a segment into the slots (kPaired below) or leaves slot 1 empty.
+// While one slot's warpgroup does its exponentials the tensor core works on the other slot (order: PV_0(j), QK_0(j+1), PV_1(j), QK_1(j+1), ...).  P (bf16) overwrites columns
 // [0,32) and [64,96) of its S tile in tensor memory (each half-row thread inside the columns it
 // has read itself) and is the A operand of the second MMA; V is
 // its MN-major B operand straight from the TMA layout.  O is rescaled lazily: only when a
 // row's running maximum grew by more than 2^8 since the value used for scaling.
-// TMEM: S0 | S1 | O0 | O1, 128 columns each.  At D = 64 narrower accumulators leave room for P beside S (kOwnP
-// below): S0 | S1 | P0 | P1 | O0 | O1, and a slot's next QK is issued as soon as its scores are read.
+// TMEM: S0 | S1 | O0 | O1, 128 columns each.  At D = 64 narrower accumulators leave room for P beside S
+// (kOwnP below): S0 | S1 | P0 | P1 | O0 | O1, and a slot's next QK is issued as soon as its scores are read.
 // Query tiles are those of the segments or, with many short ones, mixed tiles (kMixed below).
 #include <algorithm>
 #include <type_traits>
@@ -114,8 +114,8 @@ struct Unit {
 
 // Units are handed out dynamically in the plan's longest-work-first order: a CTA starts with the
 // unit of its own index, for later ones the producer draws from a global counter (header[4]) when
-// the CTA is ready for more; it passes them on through a two-entry shared-memory ring; header[6] counts finished CTAs and the
-// last one resets both counters for the next launch.
+// the CTA is ready for more; it passes them on through a two-entry shared-memory ring; header[6] counts
+// finished CTAs and the last one resets both counters for the next launch.
 constexpr int kHdrFwdNext = 4, kHdrFwdDone = 6;
 
 // (a unit may be empty: no slots)
@@ -237,7 +237,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
 #define PP_TAKE_UNIT(n, whole_warp)                                                              \
   const bool u_ok = wait_bar(bar(kSchedFullF + ((n) & 1)), ((n) >> 1) & 1, abort_flag, prm.header, 91); \
   const volatile int* u_e = sched + ((n) & 1) * 8;                                               \
-  const int u_start = u_e[0], u_len1 = u_e[1], u_len = kMixed ? u_len1 & 255 : u_len1, u_h0 = u_e[2], u_slots = u_ok ? u_e[3] : 0;        \
+  const int u_start = u_e[0], u_len1 = u_e[1], u_len = kMixed ? u_len1 & 255 : u_len1;           \
+  const int u_h0 = u_e[2], u_slots = u_ok ? u_e[3] : 0;                                          \
   const int u_nslots = kPaired ? u_slots & 3 : u_slots;                                          \
   const bool u_paired = kPaired && (u_slots & 4);                                                \
   const int u_n0 = u_e[4], u_n1 = u_e[5], u_last0 = u_e[6], u_last1 = u_e[7];                    \

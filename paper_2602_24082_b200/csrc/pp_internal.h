@@ -241,13 +241,14 @@ inline int bwd_split_log2(const pp_problem& p) {
 // (super-groups) the 148 units that run at a time may be the longest of all of a block's groups, and with r
 // query heads per KV head a block's Q, dO and dQ accumulator are 600 r * 128 KB at D 128: far beyond
 // L2, so that a (query tile, head) is fetched, and its accumulator written back, for nearly every
-// other key tile.  Blocks of 150 units, with a larger last one to balance the end
-// (sched_tail in the plan), take a third to a half of that traffic (a model of L2 with 80 MB of least-recently-used tiles, which gives
-// the 600s' measured 0.93, 5.4 and 5.9 GB as 0.93, 5.9 and 5.7: 0.5, 3.9 and 2.2).  Main kernel, 600s
-// -> these: 9241 tokens, 32 / 8 heads 262 -> 250 us; 16384, 64 / 8 1361 -> 1230; 16384, 32 / 8, D 64 456 -> 400; 36000 in short groups, 16 / 2 277 -> 243; 16760, 32 / 8 307 ->
-// 272; two rows of 32768, 32 / 8 19320 -> 19220.  With one and two heads per KV head a block's data is
-// that much smaller, and the smaller blocks only cost balance: 8 / 8 258 -> 265, 16 / 8 278 -> 276, 754 -> 740.
-// Up to 200 units both are one block.
+// other key tile.  Blocks of 150 units with a larger last one to balance the end (sched_tail in the plan)
+// move less where the groups are small against L2.  DRAM traffic of the main kernel, 600s -> these: 9241
+// tokens, 32 / 8 heads 0.93 -> 0.52 GB, 16384, 64 / 8 5.36 -> 3.31; 20187 in four long groups, 28 / 4, where the
+// last block grows to what it was, 5.90 -> 5.95; two rows of 32768 in groups as large as a block, 32 / 8,
+// between -15 and +3 %.  Times of it: 9241 tokens 262 -> 250 us; 16384, 64 / 8 1361 -> 1230; 16384, 32 / 8, D 64
+// 456 -> 400; 36000 in short groups, 16 / 2 277 -> 243; 16760, 32 / 8 307 -> 272; two rows of 32768, 32 / 8
+// 19320 -> 19220.  With one and two heads per KV head a block's data is that much smaller, and the smaller blocks
+// only cost balance: 8 / 8 258 -> 265, 16 / 8 278 -> 276, 754 -> 740.  Up to 200 units both are one block.
 constexpr int kSuperGroupUnits = 600, kSchedBlockUnits = 150, kSchedTailUnits = 200;
 inline bool bwd_takes_sched(const pp_problem& p) {
   return p.num_q_heads / p.num_kv_heads >= 3 && (long long)max_btiles_of(p) * p.num_kv_heads > kSchedTailUnits;
